@@ -75,6 +75,11 @@ enum {
                               lists into the sample's pivots), so that the second read comes from the L2.  Needs
                               n_pivot <= 16, d % 64 == 0, pivots chosen by score, else UNSUPPORTED. */
 
+#define DART_PATH_FLOW 7     /* steps 1-3 in one persistent launch that keeps the time between a row's two reads, and with it
+                              the bytes that pass between them, small enough for the L2 to serve the second.  Needs
+                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, no text pivots, else
+                              UNSUPPORTED.  The fastest path up to 16 pivots (AUTO takes it). */
+
 /* dart_opts.pivot_source: where step 2 takes the pivots from when the caller does not name them (pivots_in == NULL) */
 #define DART_PIVOTS_BY_SCORE 0 /* the n_pivot vision tokens of best score (dart_reduce) */
 #define DART_PIVOTS_MIXED 1    /* both modalities (Sec. 5.4; the pivot-selection table uses 4 visual and 4 text tokens):
@@ -180,7 +185,9 @@ typedef struct {
                               DART_PATH_FUSED: >= 2 cuts the second pass of a row tile into eight column chunks (one task each)
                               and keeps the first pass within `tune` steps of the second (low 12 bits).  One-pass kernel:
                               bit 0x1000 = one row tile per task, bit 0x2000 = two where they fit (default: two when every
-                              CTA gets at least two tasks).  All of them tuning options: same results. */
+                              CTA gets at least two tasks).  DART_PATH_FLOW: low 8 bits = how many MB of rows the scores may be ahead of
+                              the pivots, bits 12-14 = chunks of a row on their way per scoring warp, bits 16-20 = column
+                              slices (1, 2, 4, 8 or 16).  All of them tuning options: same results. */
 } dart_opts;
 
 /* Optional per-step outputs of dart_reduce_ex; every member is a device pointer or NULL. */
@@ -284,7 +291,8 @@ int dart_status(dart_ctx *ctx);
  * 10 sweep-1 tasks not all counted, 11/12 selection queue, 13 first pass held back; 40-55 the paired sweeps' waits (44 a
  * sample's lists not all counted in, 50 its pivots not published, 51 their norms not handed over, ...); 64-70 the one-pass
  * kernel's waits (stage not freed, tile not loaded (MMA / norms), accumulator not freed / not filled, norms not taken /
- * not ready); 80-86 the resident sweep's waits (83 = a sample's candidates not all published); 100 = a failed check of
+ * not ready); 80-86 the resident sweep's waits (83 = a sample's candidates not all published);
+ * 90-99, 101 the flow path's (90 a row's score not published, 91 a sample's pivots, ...); 100 = a failed check of
  * opts->pivots_in),
  * detail[1] = index of the step in the kernel's schedule (or the sample), detail[2] = CTA; for wait 1 also
  * detail[3] = sample.  For bug reports.

@@ -12,14 +12,15 @@
 #include "dart_onepass.cuh"
 #include "dart_resident.cuh"
 #include "dart_pair.cuh"
+#include "dart_flow.cuh"
 
 namespace {
 
 constexpr int kSweepChunks = 8;     // column chunks per row tile of the persistent sweep's second pass
 constexpr int kSweepChunkMaxP = 16; // ... for up to this many pivots
 
-enum Slot { SLOT_SCORE = 0, SLOT_PIVOT, SLOT_SIM, SLOT_RETAIN, SLOT_GATHER, SLOT_SWEEP, SLOT_ONEPASS, SLOT_RESIDENT, SLOT_PAIR, SLOT_COUNT };
-const char *const kSlotNames[SLOT_COUNT] = {"score", "pivot", "sim", "retain", "gather", "sweep", "onepass", "resident", "pair"};
+enum Slot { SLOT_SCORE = 0, SLOT_PIVOT, SLOT_SIM, SLOT_RETAIN, SLOT_GATHER, SLOT_SWEEP, SLOT_ONEPASS, SLOT_RESIDENT, SLOT_PAIR, SLOT_FLOW, SLOT_COUNT };
+const char *const kSlotNames[SLOT_COUNT] = {"score", "pivot", "sim", "retain", "gather", "sweep", "onepass", "resident", "pair", "flow"};
 
 typedef CUresult (*TensorMapEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                       const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -79,6 +80,13 @@ struct dart_ctx {
     bool pair_ok;
     unsigned long long *pair_cand; // [B_max][sm_count][16] candidate keys
     int32_t *pair_res;             // [B_max][32] resolved pivots and their norms
+    // flow path (csrc/dart_flow.cuh): words and counters that every call finds, and leaves, as the constructor sets them
+    bool flow_ok;
+    bool flow_dirty;               // a call ended between its launches: the next one sets them first
+    unsigned long long *flow_rec;  // [B_max][S_max] published scores; all kNoRec between calls
+    int *flow_cnt;                 // [B_max][row groups] zero between calls
+    int32_t *flow_pv;              // [B_max][32] published pivots; all kNoPivot between calls
+    size_t flow_part_n;            // floats of sim_share the slices' shares may take
     // pivots chosen inside the library from other sources than the vision tokens' scores (dart_opts.pivot_source)
     int32_t *pivot_src;            // [B_max][P_max]
     float *text_score;             // [2][B_max][S_max]: L1 scores, then sums of squares, of the text rows (before | after the block)
@@ -296,19 +304,23 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
 
 // Step 5b.  With independent pivots the rows are packed at the samples' offsets (cu_seqlens) instead of B equal blocks.
 void launch_gather(dart_ctx *ctx, int B, const void *hidden, int n_vis, int n_keep, const int32_t *out_idx, void *out_hidden,
-                   const dart_opts &o, cudaStream_t st)
+                   const dart_opts &o, cudaStream_t st, bool flow = false)
 {
     using namespace dart;
     const int S = ctx->S, d8 = ctx->desc.d / 8, S_out = S - n_vis + n_keep;
+    FlowState fs = {}; // the flow path's words and counters, put back by this launch
+    if (flow)
+        fs = FlowState{ctx->flow_rec, ctx->flow_cnt, ctx->flow_pv, (long long)B * n_vis, (long long)B * ((n_vis + flow::kRows - 1) / flow::kRows),
+                       (long long)B * flow::kMaxP};
     Prof pr(ctx, st, SLOT_GATHER);
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
     if (o.rule == DART_RULE_UNION)
         gather_varlen_kernel<<<grid, kGatherWarps * 32, 0, st>>>((const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
-                                                                ctx->status, (uint4 *)out_hidden);
+                                                                ctx->status, (uint4 *)out_hidden, fs);
     else
         gather_kernel<<<grid, kGatherWarps * 32, 0, st>>>((const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
-                                                         (uint4 *)out_hidden);
+                                                         (uint4 *)out_hidden, fs);
 }
 
 // Step 2 with the caller's pivots: checked and copied into the workspace.
@@ -356,6 +368,18 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
 
+int flow_tiles(int P) { return P <= 8 ? 1 : P <= 16 ? 2 : 4; } // pivot tiles of 8 the flow kernel is compiled for
+size_t flow_groups(const dart_ctx *ctx) { return (size_t)ctx->desc.B_max * ((ctx->desc.S_max + dart::flow::kRows - 1) / dart::flow::kRows); }
+
+// The words and counters of the flow path as every call expects to find them.
+int flow_reset(dart_ctx *ctx, cudaStream_t st)
+{
+    DART_CUDA(ctx, cudaMemsetAsync(ctx->flow_rec, 0xff, (size_t)ctx->desc.B_max * ctx->desc.S_max * sizeof(unsigned long long), st));
+    DART_CUDA(ctx, cudaMemsetAsync(ctx->flow_cnt, 0, flow_groups(ctx) * sizeof(int), st));
+    DART_CUDA(ctx, cudaMemsetAsync(ctx->flow_pv, 0xff, (size_t)ctx->desc.B_max * dart::flow::kMaxP * sizeof(int32_t), st));
+    return DART_OK;
+}
+
 // ---- fused path ------------------------------------------------------------------------------------
 int fused_setup(dart_ctx *ctx)
 {
@@ -378,10 +402,28 @@ int fused_setup(dart_ctx *ctx)
     ctx->counters_bytes = (size_t)D.B_max * 2 * sizeof(int);
     if (rc == DART_OK) rc = ws_alloc(ctx, (uint8_t **)&ctx->counters, ctx->counters_bytes);
     if (rc != DART_OK) return rc;
-    {   // shares of the similarities for up to 16 pivots; contexts that would need more than 1 GiB go without
-        const size_t n = (size_t)kSweepChunks * D.B_max * (D.P_max < kSweepChunkMaxP ? D.P_max : kSweepChunkMaxP) * D.S_max;
+    {   // shares of the similarities: the sweep's column chunks for up to 16 pivots, or the flow path's slices (four of them,
+        // more for small batches); contexts that would need more than 1 GiB go without
+        size_t n = (size_t)kSweepChunks * D.B_max * (D.P_max < kSweepChunkMaxP ? D.P_max : kSweepChunkMaxP) * D.S_max;
+        const size_t one = flow_groups(ctx) * dart::flow::kRows * 8 * flow_tiles(D.P_max < dart::flow::kMaxP ? D.P_max : dart::flow::kMaxP);
+        const size_t small = one * dart::flow::kMaxSlices < ((size_t)8 << 20) ? one * dart::flow::kMaxSlices : ((size_t)8 << 20);
+        ctx->flow_part_n = one * 4 > small ? one * 4 : small;
+        if (n < ctx->flow_part_n) n = ctx->flow_part_n;
         if (n * sizeof(float) <= ((size_t)1 << 30)) rc = ws_alloc(ctx, &ctx->sim_share, n);
         if (rc != DART_OK) return rc;
+        if (ctx->sim_share) {
+            rc = ws_alloc(ctx, &ctx->flow_rec, (size_t)D.B_max * D.S_max);
+            if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->flow_cnt, flow_groups(ctx));
+            if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->flow_pv, (size_t)D.B_max * dart::flow::kMaxP);
+            if (rc == DART_OK) rc = flow_reset(ctx, 0);
+            if (rc != DART_OK) return rc;
+            DART_CUDA(ctx, cudaStreamSynchronize(0)); // the first call may use a stream that does not wait for this one
+            const int smem = ctx->max_smem_optin - dart::flow::kStaticSmemReserve;
+            ctx->flow_ok =
+                cudaFuncSetAttribute(dart::flow::flow_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                cudaFuncSetAttribute(dart::flow::flow_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                cudaFuncSetAttribute(dart::flow::flow_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+        }
     }
     if (cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin - kStaticSmemReserve) !=
         cudaSuccess)
@@ -586,6 +628,108 @@ int launch_onepass_kernel(dart_ctx *ctx, int B, const void *src, bool scores_els
     return DART_OK;
 }
 
+
+// ---- flow path -------------------------------------------------------------------------------------
+bool flow_applies(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
+{
+    return ctx->flow_ok && P <= dart::flow::kMaxP && n_vis <= dart::flow::kMaxVis && !o.text_pivots && (long long)B * n_vis < (1ll << 29);
+}
+
+// Slices, ring depth, scorer slots and window of a call.  Returns false when the shape does not fit shared memory or the workspace.
+bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o, dart::flow::Params &p)
+{
+    namespace F = dart::flow;
+    const long long row_bytes = (long long)ctx->desc.d * 2, sample = row_bytes * n_vis, MB = 1ll << 20;
+    const int NT = flow_tiles(P), want_nsl = (o.tune >> 16) & 31, want_slot = (o.tune >> 12) & 7;
+    p.given = o.pivots_in != nullptr;
+    p.n_stream = ctx->sm_count - (p.given ? 0 : F::selectors(sample));
+    const size_t limit = (size_t)ctx->max_smem_optin - F::kStaticSmemReserve - 1024;
+    p.n_atoms = ctx->n_atoms, p.n_rg = (n_vis + F::kRows - 1) / F::kRows;
+    double best = 0;
+    p.nsl = 0;
+    for (int nsl = 1; nsl <= F::kMaxSlices && nsl <= p.n_atoms && nsl <= p.n_stream; nsl *= 2) {
+        const int na = (p.n_atoms + nsl - 1) / nsl;
+        if (F::pivot_bytes(NT, na) + 2 * (size_t)F::kStageBytes + (size_t)F::kScoreWarps * F::kChunkBytes > limit) continue;
+        if (na > F::kMaxItemAtoms && nsl < 4 && !want_nsl) continue; // an item's time is part of what lies between the two reads of a row
+        if ((size_t)B * p.n_rg * nsl * 8 * NT * F::kRows > ctx->flow_part_n) continue;
+        // the longest queue of items of any SM, in bytes plus what an item costs beside its bytes
+        const long long per = ((long long)B * p.n_rg + p.n_stream / nsl - 1) / (p.n_stream / nsl);
+        const double cost = (double)per * ((double)na * F::kAtomBytes + 16384.0);
+        if (want_nsl ? nsl == want_nsl : p.nsl == 0 || cost < best) best = cost, p.nsl = nsl;
+    }
+    if (p.nsl == 0 || F::selector_bytes(n_vis) > limit) return false;
+    p.na_max = (p.n_atoms + p.nsl - 1) / p.nsl;
+    p.pitch = (uint32_t)p.na_max * 128u + 16u;
+    p.n_slot = want_slot ? (want_slot < F::kMaxSlots ? want_slot : F::kMaxSlots) : p.given ? 4 : 2; // given pivots: nothing waits in the ring (measured 255 -> 186 us)
+    const size_t slot_bytes = (size_t)F::kScoreWarps * F::kChunkBytes, left = limit - F::pivot_bytes(NT, p.na_max);
+    while (p.n_slot > 1 && left < p.n_slot * slot_bytes + 3 * (size_t)F::kStageBytes) --p.n_slot;
+    const size_t n_st = (left - p.n_slot * slot_bytes) / F::kStageBytes;
+    p.n_st = (int)(n_st > (size_t)F::kMaxStages ? (size_t)F::kMaxStages : n_st);
+    // The scorers' lead over the last sample whose pivots are known, in bytes of rows: enough to keep them busy while a
+    // sample's last rows, its selection and its pivots' publication take their time (36 MB), but no more than the L2 keeps for
+    // the second read.  Measured at 256 x 2880 x 4096, us per launch: 32 MB 1557, 52 MB 1519, 60 MB 1395, 64 MB 1498, 72 MB
+    // 1593, 128 MB 2070 (both reads from HBM); at 64 x 4096 x 4096: 64 MB 579, 72 MB 552, 80 MB 605.
+    long long window = sample + 36 * MB < 72 * MB ? sample + 36 * MB : 72 * MB;
+    if (window < sample + 20 * MB) window = sample + 20 * MB;
+    if (o.tune & 0xff) window = (long long)(o.tune & 0xff) * MB > sample ? (long long)(o.tune & 0xff) * MB : sample;
+    window = window / row_bytes + 1;
+    p.window = (int)(window < (1ll << 29) ? window : (1ll << 29));
+    return true;
+}
+
+// Whether AUTO takes the flow path.  Pivots by score: up to 16 pivots it is the fastest path at every size measured, from one
+// sample of 130 tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.40 against 1.85 ms of
+// the sweep, 16 pivots 1.48 against 1.87).  Up to 32 pivots its multiplying warps bound it on large batches (256 x 2880 x
+// 4096: 2.05 against 1.91 ms of two passes; 32 x 2880 x 4096: 290 against 328 us).  Given pivots: it reads every row into an
+// SM twice where the one-pass kernel reads it once, but needs no launches before it and spreads a few samples over all SMs
+// (4 x 2880 x 4096: 44 against 58 us, 32 x 576 x 4096: 59 against 73, 32 x 2880 x 4096: 186 against 173).
+bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
+{
+    if (!flow_applies(ctx, B, n_vis, P, o)) return false;
+    const long long bytes = 2ll * ctx->desc.d * n_vis * B;
+    if (o.pivots_in ? bytes > 200000000ll : (P > 16 && bytes > 1000000000ll)) return false;
+    dart::flow::Params p = {};
+    return flow_config(ctx, B, n_vis, P, o, p);
+}
+
+// Steps 1-3 in one launch (csrc/dart_flow.cuh), then steps 4-5.
+int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, const int64_t *pos_in, int vis_offset, int n_vis,
+                int P, int n_keep, void *out_hidden, int32_t *out_idx, int64_t *out_pos, const dart_opts &o, const dart_debug *dbg,
+                cudaStream_t st)
+{
+    namespace F = dart::flow;
+    const void *keys = keys_in ? keys_in : hidden;
+    const int NT = flow_tiles(P);
+    F::Params p = {};
+    if (!flow_config(ctx, B, n_vis, P, o, p)) return DART_ERR_UNSUPPORTED;
+    p.B = B, p.S = ctx->S, p.vis_offset = vis_offset, p.n_vis = n_vis, p.P = P, p.d8 = ctx->desc.d / 8;
+    p.norm_kind = o.norm_kind, p.smallest = o.pivot_smallest, p.withhold = o.test_withhold_pivots;
+    p.wait_ns = o.wait_limit > 0 ? (unsigned long long)o.wait_limit * 1000ull : 2000000000ull;
+    p.keys = (const uint4 *)keys;
+    p.rec = ctx->flow_rec, p.part = ctx->sim_share, p.cnt = ctx->flow_cnt, p.pv_word = ctx->flow_pv, p.sim = ctx->sim;
+    if (dbg && (dbg->l1 || dbg->ssq)) p.l1 = ctx->l1, p.ssq = ctx->ssq;
+    p.pivot_idx = ctx->pivot_idx, p.status = ctx->status;
+    CUtensorMap tm;
+    int rc = encode_2d(ctx, &tm, keys, (uint64_t)ctx->desc.d, (uint64_t)B * ctx->S, F::kRows);
+    if (rc == DART_OK && ctx->flow_dirty) rc = flow_reset(ctx, st);
+    if (rc != DART_OK) return rc;
+    ctx->flow_dirty = true;
+    if (p.given) launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
+    {
+        Prof pr(ctx, st, SLOT_FLOW);
+        void *args[2] = {&tm, &p};
+        const void *fn = NT == 1 ? (const void *)F::flow_kernel<1> : NT == 2 ? (const void *)F::flow_kernel<2> : (const void *)F::flow_kernel<4>;
+        size_t smem = 1024 + (size_t)p.n_st * F::kStageBytes + (size_t)F::kScoreWarps * p.n_slot * F::kChunkBytes + F::pivot_bytes(NT, p.na_max);
+        if (smem < F::selector_bytes(n_vis)) smem = F::selector_bytes(n_vis);
+        // every CTA waits for scores that the others publish: co-residency is required
+        DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3(F::kThreads), args, smem, st));
+    }
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st, true);
+    DART_CUDA(ctx, cudaGetLastError());
+    ctx->flow_dirty = false;
+    return copy_debug(ctx, B, n_vis, P, dbg, st);
+}
 
 // The resident sweep applies when a sample's rows fit the chip: at most 8 pivots and, per CTA, no more octets of one
 // sample than the exchange warp has lane groups and tensor memory has slots.
@@ -811,9 +955,15 @@ int launch_reduce(dart_ctx *ctx, int B, const void *hidden, const void *keys, co
         if (!pair_applies(ctx, P) || o.pivots_in || (o.cosine_on_hidden && keys && keys != hidden)) return DART_ERR_UNSUPPORTED;
         return launch_pair(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
     }
+    if (o.path == DART_PATH_FLOW) {
+        if (!flow_applies(ctx, B, n_vis, P, o) || (o.cosine_on_hidden && keys && keys != hidden)) return DART_ERR_UNSUPPORTED;
+        return launch_flow(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
+    }
     if (o.cosine_on_hidden && keys && keys != hidden)
         return launch_two_pass(ctx, B, hidden, keys, hidden, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o,
                                dbg, fused, st);
+    if (o.path == DART_PATH_AUTO && flow_preferred(ctx, B, n_vis, P, o))
+        return launch_flow(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
     // AUTO takes the resident sweep for up to four samples: nothing has to be hidden behind other samples there, and
     // rows that stay on the chip save the second read and most of the sweep's waits (measured, 576 tokens: one
     // sample 80 us against 103 us, four samples 96 against 107, eight samples 118 against 113).
@@ -1010,6 +1160,11 @@ int dart_destroy(dart_ctx *ctx)
     cudaFree(ctx->status);
     cudaFree(ctx->counters);
     cudaFree(ctx->sim_share);
+    cudaFree(ctx->flow_rec);
+    cudaFree(ctx->flow_cnt);
+    cudaFree(ctx->flow_pv);
+    cudaFree(ctx->band);
+    cudaFree(ctx->band_n);
     cudaFree(ctx->res_cand);
     cudaFree(ctx->pair_cand);
     cudaFree(ctx->pair_res);
@@ -1050,7 +1205,7 @@ int dart_reduce_ex(dart_ctx *ctx, const void *hidden, const void *keys, const in
     if (o.norm_kind == 0) o.norm_kind = 1;
     if (o.norm_kind != 1 && o.norm_kind != 2) return DART_ERR_UNSUPPORTED;
     if (o.path != DART_PATH_AUTO && o.path != DART_PATH_STAGED && o.path != DART_PATH_FUSED && o.path != DART_PATH_TWO_PASS &&
-        o.path != DART_PATH_RESIDENT && o.path != DART_PATH_SPLIT && o.path != DART_PATH_PAIRED)
+        o.path != DART_PATH_RESIDENT && o.path != DART_PATH_SPLIT && o.path != DART_PATH_PAIRED && o.path != DART_PATH_FLOW)
         return DART_ERR_UNSUPPORTED;
     if (o.rule != DART_RULE_QUOTAS && o.rule != DART_RULE_GLOBAL && o.rule != DART_RULE_UNION) return DART_ERR_UNSUPPORTED;
     if (o.rule == DART_RULE_UNION) {
@@ -1263,7 +1418,7 @@ int dart_gather_rows(const void *src, const int32_t *idx, int B, int S, int S_ou
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
     gather_kernel<<<grid, kGatherWarps * 32, 0, (cudaStream_t)stream>>>((const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
-                                                                       nullptr, (uint4 *)out);
+                                                                       nullptr, (uint4 *)out, FlowState{});
     return cudaGetLastError() == cudaSuccess ? DART_OK : DART_ERR_CUDA;
 }
 

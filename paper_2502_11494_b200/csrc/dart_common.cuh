@@ -67,6 +67,22 @@ struct TileSplit {
     __host__ __device__ __forceinline__ int streamed(int i) const { return inv ? i * k : i + i / (k - 1) + 1; }
 };
 
+// What the flow path leaves behind in the workspace; the call's last kernel puts it back to the state that the next call
+// expects (words all ones, counters zero), whether the call succeeded or not.
+struct FlowState {
+    unsigned long long *rec;
+    int *cnt;
+    int32_t *pv;
+    long long n_rec, n_cnt, n_pv;
+    __device__ __forceinline__ void put_back() const
+    {
+        const long long n = (long long)gridDim.x * blockDim.x, t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        for (long long i = t; i < n_rec; i += n) rec[i] = ~0ull;
+        for (long long i = t; i < n_cnt; i += n) cnt[i] = 0;
+        for (long long i = t; i < n_pv; i += n) pv[i] = -1;
+    }
+};
+
 // ---- thread groups ---------------------------------------------------------------------------------
 // The selection helpers below run either on a whole CTA or on a group of warps inside one
 // (a named barrier), so that a few warps of a persistent kernel can select while others stream.

@@ -1,0 +1,671 @@
+// Flow path: steps 1-3 of a whole batch in ONE persistent launch for up to 32 pivots, built so that a key row's second read
+// comes from the L2 cache (or is already waiting in shared memory) instead of HBM.
+//
+// A row's similarities need the sample's pivots, and those need the norms of all the sample's rows: every row is read twice.
+// What decides where the second read is served from is how many bytes of other rows pass between the two reads:
+//   (time from a sample's first score to its pivots + time one second-pass item takes) x bandwidth.
+// So all of that is kept short here:
+//   - the scorers take one row per warp at a time, every SM on the same sample: a sample's rows are scored within a few
+//     microseconds of each other;
+//   - a row's score and sum of squares are published as ONE 64-bit word, and readers poll the words themselves: no counter,
+//     no fence, no second round trip;
+//   - a few CTAs do nothing but select pivots from those words: about 3 us a sample (5-6 us on an SM that also streams), and
+//     publish them the same way, word by word;
+//   - a second-pass item is 64 rows x 1/nsl of the columns: an SM's pivot tile is P x d/nsl (16 KB at 8 pivots, d = 4096, 4
+//     slices) instead of P x d, and the item takes about 2.5 us instead of the 20 us of a 128-row tile of full rows;
+//   - the item's rows are fetched into a ring before the pivots are known;
+//   - the scorers are held back to `window` rows beyond the samples that have their pivots.
+// The slices' shares of a dot product meet in global memory (L2): the SM that finishes a row group last adds them up in
+// slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
+// With the caller's pivots nothing is selected: first and second read then follow each other within the window.
+//
+// Per CTA (704 threads, one CTA per SM, cooperative launch):
+//   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
+//   warps 4-7    second pass: mma.sync.m16n8k16 (16 rows each; P <= 32 leaves the tensor pipe idle whatever the form, and
+//                64-row items do not fill the 128 rows of a tcgen05.mma)
+//   warp 8       producer: TMA tiles of 64 rows x 64 columns (128-byte swizzle), two per ring stage
+//   warps 9-12   combine: count the item, and if it is its row group's last, add up the slices and write the similarities
+//   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
+//   warp 21      watcher: how far the pivots of the batch have got, for the scorers' window
+// Every wait is bounded in time; on expiry the kernel records DART_ERR_TIMEOUT in the status word, lets the copies in flight
+// land and exits normally.
+#pragma once
+#include "dart_sweep.cuh"
+
+namespace dart {
+namespace flow {
+
+using sweep::Ctl;
+using sweep::mbar_arrive;
+using sweep::mbar_arrive_expect_tx;
+using sweep::mbar_init;
+using sweep::Ring;
+using sweep::smem_u32;
+using sweep::tma_load_2d;
+
+constexpr int kMaxP = 32;
+constexpr int kRows = 64;                  // rows of an item
+constexpr int kAtomCols = 64;              // 64 bf16 = 128 bytes = one swizzle row
+constexpr int kAtomBytes = kRows * 128;    // 8 KB
+constexpr int kAps = 2;                    // atoms per ring stage
+constexpr int kStageBytes = kAps * kAtomBytes;
+constexpr int kMaxStages = 13;
+constexpr int kPivWarps = 4;
+constexpr int kMulWarp0 = 4, kMulWarps = 4;
+constexpr int kProdWarp = 8;
+constexpr int kCombWarp0 = 9, kCombWarps = 4; // (an item is counted 2-3 us after its shares were written: two warps held the others up)
+constexpr int kScoreWarp0 = kCombWarp0 + kCombWarps, kScoreWarps = 8;
+constexpr int kWatchWarp = kScoreWarp0 + kScoreWarps;
+constexpr int kThreads = 32 * (kWatchWarp + 1);
+constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane and chunk of a row
+constexpr uint32_t kChunkBytes = kChunk * 512; // 4 KB: half a row of 4096 columns
+constexpr int kMaxSlots = 6;               // chunks of a row on their way per scorer
+constexpr int kSel = 512;                  // threads of a selector CTA that select
+constexpr int kPoll = 6;                   // words per selecting thread on their way at once: 3072 tokens
+constexpr int kMail = 2;                   // items on their way to each combine warp
+constexpr int kPvRing = 16;                // pivot lists kept for the combine warps: 2 pivot buffers + 8 items on their way, and slack
+constexpr int kMaxVis = 8192;              // a sample's keys in a selector's shared memory
+constexpr int kMaxSlices = 16;
+constexpr int kMaxItemAtoms = 16;          // items of at most 128 KB where the batch leaves the choice
+constexpr int kStaticSmemReserve = 6144;
+constexpr int32_t kNoPivot = -1;           // a pivot's word before it is published
+constexpr uint32_t kNoWord = ~0u;
+constexpr unsigned long long kNoRec = ~0ull; // a row's word before it is published (no sums produce it)
+enum { kWaitRec = 90, kWaitPivots, kWaitPivFree, kWaitPiv, kWaitStage, kWaitStageFree, kWaitMailFree, kWaitMail, kWaitCombRec,
+       kWaitWindow, kWaitChunk = 101 }; // (100 is taken by the check of given pivots)
+// Selector CTAs: a selection takes about 3 us, a sample streams at about 6 MB per us.
+__host__ inline int selectors(long long sample_bytes) { return sample_bytes >= (4 << 20) ? 4 : sample_bytes >= (2 << 20) ? 8 : 16; }
+
+struct Params {
+    int B, S, vis_offset, n_vis, P, d8; // d8: row width in 16-byte units
+    int n_atoms, n_rg, nsl, na_max;     // atoms per row; row groups per sample; column slices; atoms of the widest slice
+    int n_st, n_slot;                   // ring depth; chunks on their way per scorer
+    int n_stream;                       // CTAs that stream; the others select
+    int given;                          // the pivots are in pivot_idx already
+    int norm_kind, smallest, withhold;
+    int window;                         // rows the scorers may be ahead of `pos` (>= n_vis)
+    uint32_t pitch;                     // bytes between pivot rows in shared memory
+    unsigned long long wait_ns;
+    const uint4 *keys;                  // [B][S][d]
+    unsigned long long *rec;            // [B][n_vis] (score bits, sum-of-squares bits); kNoRec on entry, put back by the gather
+    float *part;                        // [B][n_rg][nsl][8 NT][64] the slices' shares of the dot products
+    int *cnt;                           // [B][n_rg] slices that have arrived; zero on entry, put back by the gather
+    float *sim;                         // [B][P][n_vis]
+    float *l1, *ssq;                    // [B][n_vis], NULL unless the caller wants them
+    int32_t *pivot_idx;                 // [B][P]
+    int32_t *pv_word;                   // [B][kMaxP] the same, published word by word; kNoPivot on entry, put back by the gather
+    int *status;
+};
+
+struct Shared {
+    unsigned long long full[kMaxStages], empty[kMaxStages];
+    unsigned long long chunk_full[kScoreWarps][kMaxSlots];
+    unsigned long long piv_full[2], piv_empty[2];
+    unsigned long long mail_full[kCombWarps][kMail], mail_empty[kCombWarps][kMail];
+    uint32_t group_best[32];          // selectors: best keys of groups of 16 threads
+    uint32_t n_list;
+    int32_t pv[kPvRing][kMaxP];       // pivots of the samples on their way, by the SM's own count of samples
+    int abort_flag;
+    volatile int pos;                 // rows (of the batch) whose samples have their pivots; given pivots: rows the second pass is through with
+};
+static_assert(sizeof(Shared) + 64 <= kStaticSmemReserve, "static shared memory exceeds its reserve");
+
+// shared memory of the two pivot buffers; of a selector (the list takes every token: with many equal scores many are at the floor)
+__host__ inline size_t pivot_bytes(int NT, int na_max) { return (size_t)2 * 8 * NT * ((size_t)na_max * 128 + 16); }
+__host__ inline size_t selector_bytes(int n_vis) { return (size_t)n_vis * 12; }
+
+__device__ __forceinline__ unsigned long long ld_rec(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_word(const void *p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_word(int32_t *p, int32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_rec(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// two fp32 additions / multiply-adds per instruction
+__device__ __forceinline__ void add2(unsigned long long &a, unsigned long long x)
+{
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(x));
+}
+__device__ __forceinline__ void fma2(unsigned long long &a, unsigned long long x)
+{
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a) : "l"(x));
+}
+__device__ __forceinline__ float sum2(unsigned long long a)
+{
+    return __uint_as_float((uint32_t)a) + __uint_as_float((uint32_t)(a >> 32));
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The items of one SM: slice sl = CTA % nsl, and of that slice every m-th (sample, row group), sample-major, m being the
+// number of SMs that share the slice.
+struct Items {
+    int sl, a0, na; // slice, its first atom and their number
+    int b, rg;      // current item
+    int n_rg, B, step;
+    __device__ explicit Items(const Params &p)
+    {
+        sl = (int)(blockIdx.x % (unsigned)p.nsl);
+        a0 = p.n_atoms * sl / p.nsl;
+        na = p.n_atoms * (sl + 1) / p.nsl - a0;
+        step = (p.n_stream - sl + p.nsl - 1) / p.nsl;
+        n_rg = p.n_rg, B = p.B;
+        const int first = (int)blockIdx.x / p.nsl;
+        b = first / n_rg, rg = first - b * n_rg;
+    }
+    __device__ __forceinline__ bool valid() const { return b < B; }
+    __device__ __forceinline__ void next()
+    {
+        rg += step;
+        if (rg >= n_rg) {
+            const int k = rg / n_rg;
+            b += k, rg -= k * n_rg;
+        }
+    }
+};
+
+// |x| and x^2 of a chunk of kChunk x 16 bytes
+__device__ __forceinline__ void add_chunk(const uint4 (&v)[kChunk], unsigned long long (&s)[2], unsigned long long (&q)[2])
+{
+#pragma unroll
+    for (int u = 0; u < kChunk; ++u) {
+        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t a = w[e] & 0x7fff7fffu; // both signs cleared: neither sum looks at them
+            unsigned long long x;
+            asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(a << 16), "r"(a & 0xffff0000u));
+            add2(s[e & 1], x);
+            fma2(q[e & 1], x);
+        }
+    }
+}
+
+// The scorers: warp w of SM c takes the batch's rows w * n_stream + c, + 8 * n_stream, ...  Every warp has p.n_slot slots of
+// shared memory for chunks of a row (4 KB each) and refills a slot itself as soon as it has read it.  (Straight into registers,
+// with three chunks' loads written ahead of the sums, the rows arrived at 2.5 TB/s: the loads did not stay ahead.)
+__device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
+{
+    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) - kScoreWarp0;
+    const int total = p.B * p.n_vis, stride = p.n_stream * kScoreWarps;
+    const int nc = (p.d8 + kChunk * 32 - 1) / (kChunk * 32); // chunks per row
+    unsigned long long policy;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+    slot0 += (uint32_t)(w * p.n_slot) * kChunkBytes;
+    int r = w * p.n_stream + (int)blockIdx.x, c = 0; // the chunk that is added up next
+    int rq = r, cq = 0;                               // the chunk that is requested next
+    int n_way = 0, in = 0, out = 0;                   // chunks on their way; the slot requested next, read next
+    uint32_t phase = 0;
+    auto allowed = [&](int row) { return row - sh.pos < p.window; };
+    auto wait_allowed = [&](int row) {
+        const long long t0 = clock64();
+        for (uint32_t it = 0;; ++it) {
+            if (allowed(row)) return true;
+            __nanosleep(40);
+            if ((it & 15u) == 15u) {
+                if (ctl.aborted()) return false;
+                if ((unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                    if (lane == 0) ctl.give_up(kWaitWindow, row);
+                    return false;
+                }
+            }
+        }
+    };
+    // Asks for chunks while there are free slots and their rows are within the window.  (It must not wait for the window: the
+    // rows on their way may be what moves it.)
+    auto refill = [&]() {
+        while (n_way < p.n_slot && rq < total && (cq > 0 || __all_sync(0xffffffffu, allowed(rq)))) {
+            if (lane == 0) {
+                const int b = rq / p.n_vis, j = rq - b * p.n_vis, n = min(kChunk * 32, p.d8 - cq * kChunk * 32);
+                const uint4 *src = p.keys + ((size_t)b * p.S + p.vis_offset + j) * (size_t)p.d8 + cq * kChunk * 32;
+                const uint32_t bar = smem_u32(&sh.chunk_full[w][in]);
+                mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
+                sweep::bulk_load(slot0 + (uint32_t)in * kChunkBytes, src, (uint32_t)n * 16u, bar, policy);
+            }
+            ++n_way;
+            if (++in == p.n_slot) in = 0;
+            if (++cq == nc) cq = 0, rq += stride;
+        }
+    };
+    unsigned long long s[2] = {0ull, 0ull}, q[2] = {0ull, 0ull};
+    bool ok = true;
+    while (r < total) {
+        refill();
+        if (n_way == 0) {
+            ok = __all_sync(0xffffffffu, wait_allowed(rq));
+            if (!ok) break;
+            continue;
+        }
+        ok = ctl.wait_bar(smem_u32(&sh.chunk_full[w][out]), phase, kWaitChunk, r);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const int n = p.d8 - c * kChunk * 32;
+        uint4 v[kChunk];
+#pragma unroll
+        for (int u = 0; u < kChunk; ++u)
+            v[u] = u * 32 + lane < n ? sweep::lds128(slot0 + (uint32_t)out * kChunkBytes + (uint32_t)(u * 32 + lane) * 16u) : make_uint4(0, 0, 0, 0);
+        add_chunk(v, s, q);
+        __syncwarp(); // the slot has been read
+        --n_way;
+        if (++out == p.n_slot) out = 0, phase ^= 1u;
+        if (++c == nc) {
+            const float l1 = warp_sum(sum2(s[0]) + sum2(s[1])), ssq = warp_sum(sum2(q[0]) + sum2(q[1]));
+            if (lane == 0 && !(p.withhold && r == 0)) {
+                st_rec(p.rec + r, ((unsigned long long)__float_as_uint(ssq) << 32) | __float_as_uint(l1));
+                if (p.l1) p.l1[r] = l1, p.ssq[r] = ssq;
+            }
+            s[0] = s[1] = q[0] = q[1] = 0ull;
+            c = 0, r += stride;
+        }
+    }
+    if (!ok && lane == 0) // let the copies on their way land before the CTA may exit
+        for (; n_way > 0; --n_way) {
+            ctl.wait_landed(smem_u32(&sh.chunk_full[w][out]), phase);
+            if (++out == p.n_slot) out = 0, phase ^= 1u;
+        }
+}
+
+// The selectors (CTAs that do nothing else): sample k, k + n_selectors, ... of the batch each.  512 threads read the sample's
+// words as they appear; the P-th best of 32 groups' best keys is a floor that few keys pass; those are ranked by counting.
+__device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, Shared &sh, uint32_t *skey, unsigned long long *list)
+{
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    auto any = [](bool x) { return sweep::group_any<1, kSel>(x); };
+    for (int b = (int)blockIdx.x - p.n_stream; b < p.B; b += (int)gridDim.x - p.n_stream) {
+        const uint32_t *rec = reinterpret_cast<const uint32_t *>(p.rec + (size_t)b * p.n_vis) + (p.norm_kind == 2 ? 1 : 0);
+        const long long t0 = clock64();
+        bool dead = false;
+        uint32_t best = 0; // larger = better
+        for (int j0 = t; j0 < p.n_vis && !dead; j0 += kSel * kPoll) {
+            uint32_t v[kPoll];
+#pragma unroll
+            for (int u = 0; u < kPoll; ++u) v[u] = j0 + u * kSel < p.n_vis ? ld_word(rec + 2 * (j0 + u * kSel)) : 0u;
+#pragma unroll
+            for (int u = 0; u < kPoll; ++u) {
+                const int j = j0 + u * kSel;
+                for (uint32_t spin = 0; v[u] == kNoWord && !dead; ++spin) { // not published yet
+                    __nanosleep(32);
+                    v[u] = ld_word(rec + 2 * j);
+                    if ((spin & 63u) == 63u) {
+                        dead = ctl.aborted();
+                        if (!dead && (unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                            ctl.give_up(kWaitRec, b);
+                            dead = true;
+                        }
+                    }
+                }
+                uint32_t k = order_key(__uint_as_float(v[u]));
+                if (p.smallest) k = ~k;
+                if (j < p.n_vis) {
+                    skey[j] = k;
+                    best = max(best, k);
+                }
+            }
+        }
+        uint32_t g = best; // best of 16 lanes
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+        if ((lane & 15) == 0) sh.group_best[2 * warp + (lane >> 4)] = g;
+        if (t == 0) sh.n_list = 0;
+        if (any(dead)) return;
+        // the floor: the P-th best of the 32 groups' best keys
+        const uint32_t x = sh.group_best[lane];
+        int gt = 0, ge = 0;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            const uint32_t y = __shfl_sync(0xffffffffu, x, u);
+            gt += y > x, ge += y >= x;
+        }
+        const uint32_t here = __ballot_sync(0xffffffffu, gt < p.P && ge >= p.P); // (samples of fewer tokens than groups: empty groups hold 0)
+        const uint32_t fl = __shfl_sync(0xffffffffu, x, __ffs(here) - 1);
+        if (best >= fl)
+            for (int j = t; j < p.n_vis; j += kSel) {
+                const uint32_t k = skey[j];
+                if (k >= fl) list[atomicAdd(&sh.n_list, 1u)] = ((unsigned long long)k << 32) | (0xffffffffu - (uint32_t)j); // equal scores: lower index first
+            }
+        any(false);
+        const int m = (int)sh.n_list;
+        for (int e = t; e < m; e += kSel) {
+            const unsigned long long mine = list[e];
+            int r = 0;
+            for (int u = 0; u < m; ++u) r += list[u] > mine ? 1 : 0;
+            if (r < p.P) {
+                const int32_t pv = (int32_t)(0xffffffffu - (uint32_t)mine);
+                st_word(p.pv_word + (size_t)b * kMaxP + r, pv);
+                p.pivot_idx[(size_t)b * p.P + r] = pv;
+            }
+        }
+        any(false); // the list may be filled again
+    }
+}
+
+// Pivots of the samples this SM has items of: their slice of the columns.
+template <int NT>
+__device__ __forceinline__ void take_pivots(const Params &p, const Ctl &ctl, Shared &sh, uint32_t piv0)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int seq = 0, last_b = -1;
+    for (Items it(p); it.valid(); it.next()) {
+        if (it.b == last_b) continue;
+        last_b = it.b;
+        const int b = it.b, buf = seq & 1;
+        bool ok = ctl.wait_bar(smem_u32(&sh.piv_empty[buf]), ((uint32_t)(seq >> 1) & 1u) ^ 1u, kWaitPivFree, b);
+        int pv = 0;
+        if (lane < p.P && ok) {
+            if (p.given) {
+                pv = p.pivot_idx[(size_t)b * p.P + lane];
+            } else {
+                const int32_t *word = p.pv_word + (size_t)b * kMaxP + lane;
+                const long long t0 = clock64();
+                for (uint32_t spin = 0; (pv = (int)ld_word(word)) == kNoPivot; ++spin) {
+                    __nanosleep(32);
+                    if ((spin & 31u) == 31u) {
+                        ok = !ctl.aborted();
+                        if (ok && (unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                            ctl.give_up(kWaitPivots, b);
+                            ok = false;
+                        }
+                        if (!ok) break;
+                    }
+                }
+            }
+        }
+        if (!__all_sync(0xffffffffu, ok)) return;
+        if (warp == 0 && lane < p.P) sh.pv[seq % kPvRing][lane] = pv;
+        // (ranks beyond P repeat the last pivot: their products are not used)
+        const int n_ch = it.na * 8;
+        for (int i = warp; i < 8 * NT; i += kPivWarps) {
+            const int row = __shfl_sync(0xffffffffu, pv, min(i, p.P - 1));
+            const uint4 *src = p.keys + ((size_t)b * p.S + p.vis_offset + row) * (size_t)p.d8 + it.a0 * 8;
+            const uint32_t dst = piv0 + (uint32_t)(buf * 8 * NT + i) * p.pitch;
+            for (int k = lane; k < n_ch; k += 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)k * 16u), "l"(src + k) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        mbar_arrive(smem_u32(&sh.piv_full[buf]));
+        ++seq;
+    }
+}
+
+// Second pass: 16 rows of the item per warp, all columns of the slice.
+template <int NT>
+__device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared &sh, uint32_t ring0, uint32_t piv0)
+{
+    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) - kMulWarp0;
+    const int row = 16 * w + (lane & 15);                     // tile row whose 16 bytes this lane addresses for ldmatrix
+    const uint32_t a_row = (uint32_t)row * 128u, a_sw = (uint32_t)(row & 7);
+    const uint32_t b_lane = (uint32_t)(lane & 7) * p.pitch + (uint32_t)(lane >> 3) * 16u;
+    const size_t part_item = (size_t)8 * NT * kRows;
+    Ring ring(p.n_st);
+    int seq = -1, last_b = -1, k = 0;
+    for (Items it(p); it.valid(); it.next(), ++k) {
+        if (it.b != last_b) {
+            if (seq >= 0 && lane == 0) mbar_arrive(smem_u32(&sh.piv_empty[seq & 1])); // (the warp has converged at the item's end)
+            ++seq;
+            last_b = it.b;
+            const bool ok = ctl.wait_bar(smem_u32(&sh.piv_full[seq & 1]), (uint32_t)(seq >> 1) & 1u, kWaitPiv, it.b);
+            if (!__all_sync(0xffffffffu, ok)) return;
+        }
+        if (p.given && w == 0 && lane == 0) sh.pos = it.b * p.n_vis + it.rg * kRows;
+        const uint32_t piv = piv0 + (uint32_t)((seq & 1) * 8 * NT) * p.pitch + b_lane;
+        float acc[NT][2][4];
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[n][h][e] = 0.f;
+        for (int a = 0; a < it.na; a += kAps) {
+            const bool ok = ctl.wait_bar(smem_u32(&sh.full[ring.stage]), ring.phase, kWaitStage, it.b);
+            if (!__all_sync(0xffffffffu, ok)) return;
+            // one atom: all its fragments are asked for before the first is multiplied
+            auto atom = [&](int h) {
+                const uint32_t tile = ring0 + (uint32_t)ring.stage * kStageBytes + (uint32_t)h * kAtomBytes + a_row;
+                const uint32_t pb = piv + (uint32_t)(a + h) * 128u;
+                uint32_t af[4][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) ldmatrix4(tile + ((((uint32_t)(2 * u) + (uint32_t)(lane >> 4)) ^ a_sw) << 4), af[u]);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    uint32_t b0[4], b1[4];
+                    ldmatrix4(pb + (uint32_t)n * 8u * p.pitch, b0);
+                    ldmatrix4(pb + (uint32_t)n * 8u * p.pitch + 64u, b1);
+                    mma_bf16(acc[n][0], af[0], b0[0], b0[1]);
+                    mma_bf16(acc[n][1], af[1], b0[2], b0[3]);
+                    mma_bf16(acc[n][0], af[2], b1[0], b1[1]);
+                    mma_bf16(acc[n][1], af[3], b1[2], b1[3]);
+                }
+            };
+            atom(0);
+            if (a + 1 < it.na) atom(1);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh.empty[ring.stage]));
+            ring.advance();
+        }
+        // the slice's share of the dot products: 8 consecutive rows of a pivot per 32 bytes
+        float *dst = p.part + (((size_t)it.b * p.n_rg + it.rg) * p.nsl + it.sl) * part_item + 16 * w + (lane >> 2);
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float *o = dst + (size_t)(8 * n + 2 * (lane & 3) + e) * kRows;
+                __stcg(o, acc[n][0][e] + acc[n][1][e]);
+                __stcg(o + 8, acc[n][0][2 + e] + acc[n][1][2 + e]);
+            }
+        const int c = k % kCombWarps, slot = k / kCombWarps % kMail;
+        const bool ok = ctl.wait_bar(smem_u32(&sh.mail_empty[c][slot]), ((uint32_t)(k / kCombWarps / kMail) & 1u) ^ 1u, kWaitMailFree, it.b);
+        if (!__all_sync(0xffffffffu, ok)) return;
+        if (lane == 0) mbar_arrive(smem_u32(&sh.mail_full[c][slot])); // release: the warp's stores are ordered before it
+    }
+    if (p.given && w == 0 && lane == 0) sh.pos = 0x3fffffff; // nothing holds the scorers back any more
+}
+
+// Watcher: how far the batch's pivots have got, for the scorers.  (Held back by the second pass of their own SM instead, the
+// scorers of an SM with one item more than the others delayed everybody's pivots: 8 us between the first and the last SM.)
+__device__ __forceinline__ void watch(const Params &p, const Ctl &ctl, Shared &sh)
+{
+    if ((threadIdx.x & 31) != 0 || p.given) return;
+    long long last = clock64();
+    for (int b = 0; b < p.B; ++b) {
+        const int32_t *word = p.pv_word + (size_t)b * kMaxP;
+        for (uint32_t spin = 0; (int32_t)ld_word(word) == kNoPivot; ++spin) {
+            __nanosleep(32);
+            if ((spin & 31u) == 31u && (ctl.aborted() || (unsigned long long)(clock64() - last) > ctl.limit_cycles)) return; // (the scorers report it)
+        }
+        sh.pos = (b + 1) * p.n_vis;
+        last = clock64();
+    }
+}
+
+// Producer: the items' rows into the ring, whether their pivots are known yet or not.
+__device__ __forceinline__ void produce(const Params &p, const Ctl &ctl, Shared &sh, uint32_t ring0, const CUtensorMap *tm)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    Ring ring(p.n_st);
+    long long issued = 0;
+    bool ok = true;
+    for (Items it(p); ok && it.valid(); it.next()) {
+        // (rows beyond the vision block, or beyond the tensor: their products are not used)
+        const int y = it.b * p.S + p.vis_offset + it.rg * kRows;
+        for (int a = 0; a < it.na; a += kAps) {
+            const int nh = min(kAps, it.na - a);
+            const uint32_t full = smem_u32(&sh.full[ring.stage]);
+            ok = ctl.wait_bar(smem_u32(&sh.empty[ring.stage]), ring.phase ^ 1u, kWaitStageFree, it.b);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive_expect_tx(full, (uint32_t)nh * kAtomBytes);
+            __syncwarp();
+            if (lane < nh)
+                tma_load_2d(ring0 + (uint32_t)ring.stage * kStageBytes + (uint32_t)lane * kAtomBytes, tm, (it.a0 + a + lane) * kAtomCols, y,
+                            full, policy);
+            ring.advance();
+            ++issued;
+        }
+    }
+    if ((!ok || ctl.aborted()) && lane == 0) // let the copies already issued land before the CTA may exit
+        for (long long i = issued > p.n_st ? issued - p.n_st : 0; i < issued; ++i)
+            ctl.wait_landed(smem_u32(&sh.full[i % p.n_st]), (uint32_t)((i / p.n_st) & 1));
+}
+
+// Combine: an item is counted once its shares are written; whoever counts a row group's last slice adds the shares up.
+template <int NT>
+__device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared &sh)
+{
+    const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - kCombWarp0;
+    const size_t part_item = (size_t)8 * NT * kRows;
+    int seq = -1, last_b = -1, k = 0;
+    auto rec_ssq = [&](const unsigned long long *rec, int b, float &ssq) { // the word may not be there yet when the pivots were given
+        unsigned long long v = ld_rec(rec);
+        if (v == kNoRec) {
+            const long long t0 = clock64();
+            for (uint32_t spin = 0; (v = ld_rec(rec)) == kNoRec; ++spin) {
+                __nanosleep(100);
+                if ((spin & 15u) == 15u) {
+                    if (ctl.aborted()) return false;
+                    if ((unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                        ctl.give_up(kWaitCombRec, b);
+                        return false;
+                    }
+                }
+            }
+        }
+        ssq = __uint_as_float((uint32_t)(v >> 32));
+        return true;
+    };
+    for (Items it(p); it.valid(); it.next(), ++k) {
+        if (it.b != last_b) ++seq, last_b = it.b;
+        if (k % kCombWarps != c) continue;
+        const int slot = k / kCombWarps % kMail;
+        bool ok = ctl.wait_bar(smem_u32(&sh.mail_full[c][slot]), (uint32_t)(k / kCombWarps / kMail) & 1u, kWaitMail, it.b);
+        if (!__all_sync(0xffffffffu, ok)) return;
+        const size_t group = (size_t)it.b * p.n_rg + it.rg;
+        int before = 0;
+        // release: the item's shares, written by the warps that filled the mailbox; acquire: the other slices' shares
+        if (lane == 0 && p.nsl > 1)
+            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(p.cnt + group) : "memory");
+        before = __shfl_sync(0xffffffffu, before, 0);
+        __syncwarp();
+        if (before == p.nsl - 1) {
+            const int j = it.rg * kRows + 2 * lane; // this lane's rows: j and j + 1
+            const unsigned long long *rec = p.rec + (size_t)it.b * p.n_vis;
+            float n0 = 0.f, n1 = 0.f, np = 0.f;
+            if (j < p.n_vis) ok = ok && rec_ssq(rec + j, it.b, n0);
+            if (j + 1 < p.n_vis) ok = ok && rec_ssq(rec + j + 1, it.b, n1);
+            if (lane < p.P) ok = ok && rec_ssq(rec + sh.pv[seq % kPvRing][lane], it.b, np);
+            if (!__all_sync(0xffffffffu, ok)) return;
+            n0 = sqrtf(n0), n1 = sqrtf(n1), np = sqrtf(np);
+            const float2 *src = reinterpret_cast<const float2 *>(p.part + group * p.nsl * part_item) + lane;
+            float *dst = p.sim + (size_t)it.b * p.P * p.n_vis + j;
+            for (int i0 = 0; i0 < p.P; i0 += 4) { // 4 pivots x 4 slices on their way at once
+                float2 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = make_float2(0.f, 0.f);
+                for (int s0 = 0; s0 < p.nsl; s0 += 4) {
+                    float2 x[4][4];
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            x[s][i] = s0 + s < p.nsl ? __ldcg(src + (((size_t)(s0 + s) * part_item + (size_t)(i0 + i) * kRows) >> 1)) : make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) // in slice order
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i].x += x[s][i].x, v[i].y += x[s][i].y;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float ni = __shfl_sync(0xffffffffu, np, i0 + i), d0 = ni * n0, d1 = ni * n1;
+                    if (i0 + i < p.P) { // dup = dot / (|pivot| |row|); a zero norm gives 0
+                        if (j < p.n_vis) dst[(size_t)(i0 + i) * p.n_vis] = d0 > 0.f ? v[i].x / d0 : 0.f;
+                        if (j + 1 < p.n_vis) dst[(size_t)(i0 + i) * p.n_vis + 1] = d1 > 0.f ? v[i].y / d1 : 0.f;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sh.mail_empty[c][slot]));
+    }
+}
+
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant__ CUtensorMap tm, const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    if (*p.status != 0) return; // an earlier kernel of this call failed (every CTA sees the same word: nobody waits)
+    const uint32_t ring0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t slot0 = ring0 + (uint32_t)p.n_st * kStageBytes;
+    const uint32_t piv0 = slot0 + (uint32_t)(kScoreWarps * p.n_slot) * kChunkBytes;
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(smem_raw); // (selectors have no ring)
+    uint32_t *skey = reinterpret_cast<uint32_t *>(list + p.n_vis);
+    const int warp = threadIdx.x >> 5;
+    // whoever waits for something nearest to what is missing has the shortest limit, so that it is the one that reports it
+    const unsigned long long limit = 2ull * p.wait_ns; // ns -> cycles at the highest SM clock: never shorter than asked
+    const Ctl ctl{&sh.abort_flag, p.status, warp < kPivWarps ? limit + limit / 8 : warp == kProdWarp ? limit + limit / 2 : limit + limit / 4};
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kMaxStages; ++s) {
+            mbar_init(smem_u32(&sh.full[s]), 1);
+            mbar_init(smem_u32(&sh.empty[s]), kMulWarps);
+        }
+        for (int w = 0; w < kScoreWarps; ++w)
+            for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&sh.chunk_full[w][s]), 1);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(smem_u32(&sh.piv_full[s]), kPivWarps * 32);
+            mbar_init(smem_u32(&sh.piv_empty[s]), kMulWarps);
+        }
+        for (int c = 0; c < kCombWarps; ++c)
+            for (int s = 0; s < kMail; ++s) {
+                mbar_init(smem_u32(&sh.mail_full[c][s]), kMulWarps);
+                mbar_init(smem_u32(&sh.mail_empty[c][s]), 1);
+            }
+        sh.abort_flag = 0;
+        sh.pos = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if ((int)blockIdx.x >= p.n_stream) {
+        if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, skey, list);
+    } else if (warp == kWatchWarp) {
+        watch(p, ctl, sh);
+    } else if (warp >= kScoreWarp0) {
+        score_rows(p, ctl, sh, slot0);
+    } else if (warp < kPivWarps) {
+        take_pivots<NT>(p, ctl, sh, piv0);
+    } else if (warp < kMulWarp0 + kMulWarps) {
+        multiply<NT>(p, ctl, sh, ring0, piv0);
+    } else if (warp == kProdWarp) {
+        produce(p, ctl, sh, ring0, &tm);
+    } else {
+        combine<NT>(p, ctl, sh);
+    }
+    __syncthreads(); // nobody leaves while a copy may still land in the CTA's shared memory
+}
+
+} // namespace flow
+} // namespace dart

@@ -1370,8 +1370,9 @@ pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restric
 // One warp per output row (as gather_kernel); rows at and beyond cu[B] do not exist.
 __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, const int32_t *__restrict__ cu, int B,
-                     int S, int d8, long long rows_cap, const int *__restrict__ status, uint4 *__restrict__ out_hidden)
+                     int S, int d8, long long rows_cap, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs)
 {
+    fs.put_back();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
     if (row >= rows_cap || *status != 0 || row >= cu[B]) return;
@@ -1394,8 +1395,9 @@ gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict
 
 __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, int S, int S_out, int d8,
-              long long rows_total, const int *__restrict__ status, uint4 *__restrict__ out_hidden)
+              long long rows_total, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs)
 {
+    fs.put_back();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
     if (row >= rows_total || (status && *status != 0)) return; // after a failed kernel out_idx is undefined

@@ -1,0 +1,114 @@
+"""The flow path (both reads of a row a few microseconds apart, pivots published word by word) against the oracle,
+through the C ABI (needs a B200)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import parity  # noqa: E402
+from paper_2502_11494_b200 import dart, workloads as W  # noqa: E402
+from test_gpu_parity import _np, compare, gaussian, run_gpu  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+FLOW = dart.DART_PATH_FLOW
+
+# (B, S, d, vis_offset, n_vis, P, Kp): row groups of 64, pivot tiles of 8/16/32, one to sixteen column slices
+SHAPES = [
+    (1, 16, 64, 0, 16, 1, 1),             # one group, one atom, one slice; most SMs hold nothing
+    (2, 50, 64, 3, 40, 32, 40),           # more pivots than groups of 16 selecting threads hold tokens; everything kept
+    (3, 200, 128, 7, 64, 8, 20),          # exactly one row group
+    (3, 200, 192, 7, 65, 9, 20),          # one row more; three atoms over two slices
+    (2, 333, 320, 17, 301, 7, 60),        # five atoms over four slices
+    (1, 700, 4096, 40, 576, 8, 64),       # sixteen slices
+    (40, 700, 1088, 40, 576, 17, 64),     # 17 atoms, the widest pivot tile
+    (2, 3000, 4096, 40, 2880, 16, 320),
+    (1, 3300, 256, 9, 3073, 5, 200),      # one token more than the selecting threads ask for at once
+    (2, 8200, 64, 4, 8192, 3, 700),       # the longest sample
+    (1, 9000, 192, 5, 4097, 32, 500),     # a last row group of one row
+    (3, 80, 8192, 2, 70, 12, 30),         # the widest rows
+    (300, 40, 64, 1, 33, 4, 9),           # more samples than SMs
+]
+
+
+@pytest.mark.parametrize("given", [False, True], ids=["by score", "given"])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_flow_matches_the_oracle(oracle, shape, given):
+    B, S, d, vo, nv, P, Kp = shape
+    k, h = gaussian(B, S, d, seed=1300 + sum(shape))
+    ctx = dart.Dart(B, S, d, P, Kp)
+    opts, piv = dart.dart_opts(path=FLOW), None
+    if given:
+        g = torch.Generator(device="cuda").manual_seed(5)
+        piv = torch.rand((B, nv), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
+        opts.pivots_in = piv.data_ptr()
+    try:
+        for tune in (0, 0x1001, 0x10000):   # default; the least window and one slot; one slice where it fits
+            opts.tune = tune
+            try:
+                res = ctx.reduce(h, k, vo, nv, P, Kp, debug=True, opts=opts)
+            except dart.DartError as e:     # one slice of wide rows does not fit shared memory beside the ring
+                assert tune == 0x10000 and d > 1024 and e.code == dart.DART_ERR_UNSUPPORTED
+                continue
+            torch.cuda.synchronize()
+            assert ctx.status() == dart.DART_OK, dart.dart_status_detail(ctx.handle)
+            if tune == 0:
+                kb, hb = W.bits(k), W.bits(h)
+                ora = oracle.reduce(hb, kb, vo, nv, P, Kp, pivots_in=None if piv is None else piv.cpu().numpy())
+                rep = parity.check_batch(ora, kb, hb, vo, nv, P, Kp, _np(res[0]), _np(res[1]), _np(res[2]),
+                                         dbg={n: _np(v) for n, v in res[3].items()}, pivots_given=given)
+                assert rep.exact >= rep.above_margin
+                assert rep.max_rel_l1 < 5e-5 and rep.max_rel_l2 < 5e-5 and rep.max_abs_sim < 2e-5
+                first = res
+            else:
+                assert torch.allclose(res[3]["sim"], first[3]["sim"], rtol=0, atol=4e-5)   # each within 2e-5 of the oracle
+                assert torch.equal(res[3]["pivot_idx"], first[3]["pivot_idx"]) and torch.equal(res[3]["l1"], first[3]["l1"])
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("norm_kind,smallest", [(1, 1), (2, 0), (2, 1)])
+def test_flow_ranking_variants(oracle, norm_kind, smallest):
+    k, h = gaussian(3, 500, 256, seed=77)
+    rep = compare(oracle, k, h, 20, 444, 6, 90, path=FLOW, norm_kind=norm_kind, smallest=smallest)
+    assert rep.exact >= rep.above_margin and rep.max_abs_sim < 2e-5
+
+
+def test_flow_equal_scores_rank_the_lower_index_first(oracle):
+    """Rows that are copies of each other tie in score: the list above the selection's floor holds every token."""
+    k, h = gaussian(2, 1300, 128, seed=78)
+    k[:, 10:1300] = k[:, 10:11] * 0.5         # all vision rows but the first equal; the first one larger
+    k[:, 10] = k[:, 11] * 2
+    oh, oi, op, dbg = run_gpu(k, h, 10, 1290, 5, 40, path=FLOW)
+    assert np.array_equal(dbg["pivot_idx"], np.tile(np.arange(5, dtype=np.int32), (2, 1)))
+
+
+@pytest.mark.parametrize("shape", [(1, 64, 64, 0, 64, 33, 40), (1, 8300, 64, 0, 8193, 2, 8), (1, 64, 96, 0, 64, 2, 8)],
+                         ids=["33 pivots", "8193 tokens", "d not a multiple of 64"])
+def test_flow_says_what_it_does_not_take(shape):
+    B, S, d, vo, nv, P, Kp = shape
+    k, h = gaussian(B, S, d, seed=79)
+    ctx = dart.Dart(B, S, d, P, Kp)
+    with pytest.raises(dart.DartError) as e:
+        ctx.reduce(h, k, vo, nv, P, Kp, opts=dart.dart_opts(path=FLOW))
+    assert e.value.code == dart.DART_ERR_UNSUPPORTED
+    ctx.close()
+
+
+def test_flow_expired_waits_are_reported_not_hung():
+    """One row's word is never published: the selecting CTA gives up within its limit and says so, every other wait ends
+    too, and the next call on the same context succeeds."""
+    w = W.LLAVA15_B64.with_(B=3)
+    k, h = W.make_batch(w, device="cuda")
+    ctx = dart.Dart(w.B, w.S, w.d, w.n_pivot, w.n_keep)
+    ctx.reduce(h, k, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep,
+               opts=dart.dart_opts(path=FLOW, wait_limit=20000, test_withhold_pivots=1))      # 20 ms limit
+    torch.cuda.synchronize()
+    assert ctx.status() == dart.DART_ERR_TIMEOUT
+    rc, detail = dart.dart_status_detail(ctx.handle)
+    assert rc == dart.DART_OK and detail[0] == 90, detail
+    good = ctx.reduce(h, k, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep, opts=dart.dart_opts(path=FLOW))
+    torch.cuda.synchronize()
+    assert ctx.status() == dart.DART_OK
+    ref = run_gpu(k, h, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep, path=dart.DART_PATH_STAGED, debug=False)
+    assert np.array_equal(good[1].cpu().numpy(), ref[1]) and np.array_equal(W.bits(good[0]), ref[0])
+    ctx.close()
