@@ -77,8 +77,7 @@ enum {
 
 #define DART_PATH_FLOW 7     /* steps 1-3 in one persistent launch that keeps the time between a row's two reads, and with it
                               the bytes that pass between them, small enough for the L2 to serve the second.  Needs
-                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, no text pivots, else
-                              UNSUPPORTED.  The fastest path up to 16 pivots (AUTO takes it). */
+                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, else UNSUPPORTED.  The fastest path up to 16 pivots (AUTO takes it). */
 
 /* dart_opts.pivot_source: where step 2 takes the pivots from when the caller does not name them (pivots_in == NULL) */
 #define DART_PIVOTS_BY_SCORE 0 /* the n_pivot vision tokens of best score (dart_reduce) */

@@ -323,12 +323,15 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int n_vis, int n_ke
                                                          (uint4 *)out_hidden, fs);
 }
 
-// Step 2 with the caller's pivots: checked and copied into the workspace.
-void launch_pivots_given(dart_ctx *ctx, int B, int vis_offset, int n_vis, int P, const dart_opts &o, cudaStream_t st)
+// Step 2 with the caller's pivots: checked and copied into the workspace (with keys: and the text pivots' sums of squares).
+void launch_pivots_given(dart_ctx *ctx, int B, int vis_offset, int n_vis, int P, const dart_opts &o, cudaStream_t st,
+                         const uint4 *keys = nullptr, float *text_ssq = nullptr)
 {
     Prof p(ctx, st, SLOT_PIVOT);
     const int lo = o.text_pivots ? -vis_offset : 0, hi = o.text_pivots ? ctx->S - vis_offset : n_vis;
-    dart::pivots_given_kernel<<<B, 256, (size_t)((hi - lo + 31) / 32) * 4, st>>>(o.pivots_in, lo, hi, P, ctx->pivot_idx, ctx->status);
+    dart::pivots_given_kernel<<<B, 256, (size_t)((hi - lo + 31) / 32) * 4, st>>>(o.pivots_in, lo, hi, P, ctx->pivot_idx, ctx->status,
+                                                                               o.text_pivots ? keys : nullptr, ctx->S, ctx->desc.d / 8, vis_offset,
+                                                                               n_vis, text_ssq);
 }
 
 int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, const int64_t *pos_in, int vis_offset,
@@ -630,9 +633,9 @@ int launch_onepass_kernel(dart_ctx *ctx, int B, const void *src, bool scores_els
 
 
 // ---- flow path -------------------------------------------------------------------------------------
-bool flow_applies(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
+bool flow_applies(const dart_ctx *ctx, int B, int n_vis, int P)
 {
-    return ctx->flow_ok && P <= dart::flow::kMaxP && n_vis <= dart::flow::kMaxVis && !o.text_pivots && (long long)B * n_vis < (1ll << 29);
+    return ctx->flow_ok && P <= dart::flow::kMaxP && n_vis <= dart::flow::kMaxVis && (long long)B * n_vis < (1ll << 29);
 }
 
 // Slices, ring depth, scorer slots and window of a call.  Returns false when the shape does not fit shared memory or the workspace.
@@ -685,7 +688,7 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
 // (4 x 2880 x 4096: 44 against 58 us, 32 x 576 x 4096: 59 against 73, 32 x 2880 x 4096: 186 against 173).
 bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
 {
-    if (!flow_applies(ctx, B, n_vis, P, o)) return false;
+    if (!flow_applies(ctx, B, n_vis, P)) return false;
     const long long bytes = 2ll * ctx->desc.d * n_vis * B;
     if (o.pivots_in ? bytes > 200000000ll : (P > 16 && bytes > 1000000000ll)) return false;
     dart::flow::Params p = {};
@@ -714,7 +717,8 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
     if (rc == DART_OK && ctx->flow_dirty) rc = flow_reset(ctx, st);
     if (rc != DART_OK) return rc;
     ctx->flow_dirty = true;
-    if (p.given) launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
+    if (o.text_pivots) p.text_ssq = ctx->eps; // (the retention's thresholds: written after the flow kernel only)
+    if (p.given) launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st, p.keys, ctx->eps);
     {
         Prof pr(ctx, st, SLOT_FLOW);
         void *args[2] = {&tm, &p};
@@ -956,7 +960,7 @@ int launch_reduce(dart_ctx *ctx, int B, const void *hidden, const void *keys, co
         return launch_pair(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
     }
     if (o.path == DART_PATH_FLOW) {
-        if (!flow_applies(ctx, B, n_vis, P, o) || (o.cosine_on_hidden && keys && keys != hidden)) return DART_ERR_UNSUPPORTED;
+        if (!flow_applies(ctx, B, n_vis, P) || (o.cosine_on_hidden && keys && keys != hidden)) return DART_ERR_UNSUPPORTED;
         return launch_flow(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
     }
     if (o.cosine_on_hidden && keys && keys != hidden)

@@ -94,6 +94,7 @@ struct Params {
     float *l1, *ssq;                    // [B][n_vis], NULL unless the caller wants them
     int32_t *pivot_idx;                 // [B][P]
     int32_t *pv_word;                   // [B][kMaxP] the same, published word by word; kNoPivot on entry, put back by the gather
+    const float *text_ssq;              // [B][P] sums of squares of given pivots that are text tokens
     int *status;
 };
 
@@ -577,7 +578,13 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
             float n0 = 0.f, n1 = 0.f, np = 0.f;
             if (j < p.n_vis) ok = ok && rec_ssq(rec + j, it.b, n0);
             if (j + 1 < p.n_vis) ok = ok && rec_ssq(rec + j + 1, it.b, n1);
-            if (lane < p.P) ok = ok && rec_ssq(rec + sh.pv[seq % kPvRing][lane], it.b, np);
+            if (lane < p.P) {
+                const int pv = sh.pv[seq % kPvRing][lane];
+                if (pv >= 0 && pv < p.n_vis)
+                    ok = ok && rec_ssq(rec + pv, it.b, np);
+                else
+                    np = p.text_ssq[(size_t)it.b * p.P + lane];
+            }
             if (!__all_sync(0xffffffffu, ok)) return;
             n0 = sqrtf(n0), n1 = sqrtf(n1), np = sqrtf(np);
             const float2 *src = reinterpret_cast<const float2 *>(p.part + group * p.nsl * part_item) + lane;

@@ -296,7 +296,8 @@ constexpr int kCheckPivotsGiven = 100; // second status word: which check failed
 // [lo, hi) is the range a pivot may lie in, relative to the vision block: [0, n_vis), or the whole sequence
 // [-vis_offset, S - vis_offset) when text tokens may serve as pivots (Sec. 5.4).
 __global__ void __launch_bounds__(256)
-pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P, int32_t *__restrict__ pivot_idx, int *status)
+pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P, int32_t *__restrict__ pivot_idx, int *status,
+                    const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, float *__restrict__ text_ssq)
 {
     extern __shared__ uint32_t seen[]; // [(hi - lo + 31) / 32]
     const int b = blockIdx.x;
@@ -313,6 +314,27 @@ pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P
             status[2] = b;
             status[3] = t;
         }
+    }
+    if (!keys) return;
+    // sums of squares of the pivots that are text tokens (no scorer reads their rows): a warp per pivot
+    const int lane = threadIdx.x & 31;
+    for (int t = threadIdx.x >> 5; t < P; t += blockDim.x >> 5) {
+        const int c = min(max(pivots_in[(size_t)b * P + t], lo), hi - 1);
+        if (c >= 0 && c < n_vis) continue;
+        const uint4 *row = keys + ((size_t)b * S + vis_offset + c) * (size_t)d8;
+        float q = 0.f;
+        for (int k = lane; k < d8; k += 32) {
+            const uint4 v = __ldg(row + k);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float x = bf16_lo(w[e]), y = bf16_hi(w[e]);
+                q = fmaf(x, x, q);
+                q = fmaf(y, y, q);
+            }
+        }
+        q = warp_sum(q);
+        if (lane == 0) text_ssq[(size_t)b * P + t] = q;
     }
 }
 

@@ -30,7 +30,7 @@ SHAPES = [
 ]
 
 
-@pytest.mark.parametrize("given", [False, True], ids=["by score", "given"])
+@pytest.mark.parametrize("given", [0, 1, 2], ids=["by score", "given", "given, text tokens among them"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 def test_flow_matches_the_oracle(oracle, shape, given):
     B, S, d, vo, nv, P, Kp = shape
@@ -39,7 +39,9 @@ def test_flow_matches_the_oracle(oracle, shape, given):
     opts, piv = dart.dart_opts(path=FLOW), None
     if given:
         g = torch.Generator(device="cuda").manual_seed(5)
-        piv = torch.rand((B, nv), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
+        n, opts.text_pivots = (nv, 0) if given == 1 else (S, 1)
+        piv = torch.rand((B, n), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32)
+        piv = (piv - (vo if given == 2 else 0)).contiguous()
         opts.pivots_in = piv.data_ptr()
     try:
         for tune in (0, 0x1001, 0x10000):   # default; the least window and one slot; one slice where it fits
@@ -53,9 +55,10 @@ def test_flow_matches_the_oracle(oracle, shape, given):
             assert ctx.status() == dart.DART_OK, dart.dart_status_detail(ctx.handle)
             if tune == 0:
                 kb, hb = W.bits(k), W.bits(h)
-                ora = oracle.reduce(hb, kb, vo, nv, P, Kp, pivots_in=None if piv is None else piv.cpu().numpy())
+                ora = oracle.reduce(hb, kb, vo, nv, P, Kp, pivots_in=None if piv is None else piv.cpu().numpy(),
+                                    text_pivots=given == 2)
                 rep = parity.check_batch(ora, kb, hb, vo, nv, P, Kp, _np(res[0]), _np(res[1]), _np(res[2]),
-                                         dbg={n: _np(v) for n, v in res[3].items()}, pivots_given=given)
+                                         dbg={n: _np(v) for n, v in res[3].items()}, pivots_given=given > 0, text_pivots=given == 2)
                 assert rep.exact >= rep.above_margin
                 assert rep.max_rel_l1 < 5e-5 and rep.max_rel_l2 < 5e-5 and rep.max_abs_sim < 2e-5
                 first = res
