@@ -39,6 +39,8 @@ struct dart_ctx {
     int last_cuda;
     int64_t launches;
     size_t bytes;
+    void *ws_base;                 // the workspace's one allocation
+    std::vector<void **> ws_slots; // until it is made: the arrays' pointers
     // workspace (device), indexed with the shapes of the current call
     float *l1, *ssq, *sim, *eps;
     int32_t *pivot_idx, *owner;
@@ -106,14 +108,25 @@ int cuda_fail(dart_ctx *ctx, cudaError_t e)
         if (e__ != cudaSuccess) return cuda_fail((ctx), e__);  \
     } while (0)
 
+// Workspace arrays are parts of ONE allocation: ws_alloc notes an array's size and hands out its place, ws_commit allocates
+// and turns the places into addresses.  (One cudaMalloc per array: creating a context for one sample of 576 tokens took
+// 2.6 ms, now 0.4.)
 template <typename T>
 int ws_alloc(dart_ctx *ctx, T **p, size_t count)
 {
-    size_t bytes = (count * sizeof(T) + 255) / 256 * 256;
-    cudaError_t e = cudaMalloc((void **)p, bytes);
-    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    const size_t bytes = (count * sizeof(T) + 255) / 256 * 256;
+    *p = reinterpret_cast<T *>(ctx->bytes + 256); // not NULL: the array exists from here on
+    ctx->ws_slots.push_back(reinterpret_cast<void **>(p));
     ctx->bytes += bytes;
     return DART_OK;
+}
+
+int ws_commit(dart_ctx *ctx)
+{
+    const cudaError_t e = cudaMalloc(&ctx->ws_base, ctx->bytes);
+    for (void **p : ctx->ws_slots) *p = e == cudaSuccess ? (char *)ctx->ws_base + ((size_t)*p - 256) : nullptr;
+    ctx->ws_slots.clear();
+    return e == cudaSuccess ? DART_OK : cuda_fail(ctx, e);
 }
 
 // Scoped device switch: the library never leaves another device current.
@@ -389,10 +402,13 @@ int fused_setup(dart_ctx *ctx)
     using namespace dart::sweep;
     const dart_desc &D = ctx->desc;
     ctx->fused_ok = false;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, D.device) != cudaSuccess) return DART_ERR_CUDA;
-    ctx->sm_count = prop.multiProcessorCount;
-    if (prop.major != 10 || D.d % kAtomCols != 0 || D.d * 2 > kMaxRowBytes || !prop.cooperativeLaunch)
+    // (single attributes: cudaGetDeviceProperties asks the driver for all of them)
+    int major = 0, coop = 0;
+    if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, D.device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, D.device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, D.device) != cudaSuccess)
+        return DART_ERR_CUDA;
+    if (major != 10 || D.d % kAtomCols != 0 || D.d * 2 > kMaxRowBytes || !coop)
         return DART_OK; // staged path only
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -418,9 +434,7 @@ int fused_setup(dart_ctx *ctx)
             rc = ws_alloc(ctx, &ctx->flow_rec, (size_t)D.B_max * D.S_max);
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->flow_cnt, flow_groups(ctx));
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->flow_pv, (size_t)D.B_max * dart::flow::kMaxP);
-            if (rc == DART_OK) rc = flow_reset(ctx, 0);
             if (rc != DART_OK) return rc;
-            DART_CUDA(ctx, cudaStreamSynchronize(0)); // the first call may use a stream that does not wait for this one
             const int smem = ctx->max_smem_optin - dart::flow::kStaticSmemReserve;
             ctx->flow_ok =
                 cudaFuncSetAttribute(dart::flow::flow_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
@@ -1069,7 +1083,6 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
         if (bytes <= ((size_t)2 << 30)) rc = ws_alloc(ctx, (uint8_t **)&ctx->piv_rows, bytes);
     }
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->status, 64);
-    if (rc == DART_OK && cudaMemset(ctx->status, 0, 256) != cudaSuccess) rc = DART_ERR_CUDA;
     if (rc == DART_OK) {
         cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, desc->device);
         size_t sim_smem = (size_t)dart::kSimPivotChunk * (desc->d / 8) * 16;
@@ -1131,6 +1144,11 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
                               cudaStreamCreateWithFlags(&ctx->s_d2h, cudaStreamNonBlocking) != cudaSuccess))
             rc = DART_ERR_CUDA;
     }
+    if (rc == DART_OK) rc = ws_commit(ctx);
+    if (rc == DART_OK) rc = cudaMemsetAsync(ctx->status, 0, 256, 0) == cudaSuccess ? DART_OK : DART_ERR_CUDA;
+    if (rc == DART_OK && ctx->flow_rec) rc = flow_reset(ctx, 0);
+    // the first call may use a stream that does not wait for the legacy stream
+    if (rc == DART_OK && cudaStreamSynchronize(0) != cudaSuccess) rc = DART_ERR_CUDA;
     if (rc != DART_OK) {
         dart_destroy(ctx);
         return rc;
@@ -1149,35 +1167,8 @@ int dart_destroy(dart_ctx *ctx)
         cudaEventDestroy(e.start);
         cudaEventDestroy(e.stop);
     }
-    cudaFree(ctx->l1);
-    cudaFree(ctx->ssq);
-    cudaFree(ctx->sim);
-    cudaFree(ctx->eps);
-    cudaFree(ctx->pivot_idx);
-    cudaFree(ctx->owner);
-    cudaFree(ctx->keep);
-    cudaFree(ctx->len);
-    cudaFree(ctx->pivot_src);
-    cudaFree(ctx->text_score);
-    cudaFree(ctx->cand);
-    cudaFree(ctx->piv_rows);
-    cudaFree(ctx->status);
-    cudaFree(ctx->counters);
-    cudaFree(ctx->sim_share);
-    cudaFree(ctx->flow_rec);
-    cudaFree(ctx->flow_cnt);
-    cudaFree(ctx->flow_pv);
-    cudaFree(ctx->band);
-    cudaFree(ctx->band_n);
-    cudaFree(ctx->res_cand);
-    cudaFree(ctx->pair_cand);
-    cudaFree(ctx->pair_res);
+    cudaFree(ctx->ws_base);
     for (int k = 0; k < 2; ++k) {
-        cudaFree(ctx->st_hidden[k]);
-        cudaFree(ctx->st_keys[k]);
-        cudaFree(ctx->st_out_hidden[k]);
-        cudaFree(ctx->st_out_idx[k]);
-        cudaFree(ctx->st_out_pos[k]);
         if (ctx->ev_in[k]) cudaEventDestroy(ctx->ev_in[k]);
         if (ctx->ev_run[k]) cudaEventDestroy(ctx->ev_run[k]);
         if (ctx->ev_out[k]) cudaEventDestroy(ctx->ev_out[k]);
