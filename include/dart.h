@@ -93,9 +93,7 @@ enum {
                                   tickets to the lower index.  The same seed gives the same pivots on every run. */
 
 /* dart_opts.retention */
-#define DART_RETAIN_AUTO 0   /* more samples than SMs: candidate bands; else the bands in one launch for up to 8 pivots
-                                and sorted lists for more; where the chosen form's workspace or shared memory does not
-                                fit: another one, else one kernel */
+#define DART_RETAIN_AUTO 0   /* ranked lists; where their workspace or shared memory does not fit: one of the other forms */
 #define DART_RETAIN_SERIAL 1 /* one kernel, one CTA per sample: the pivots' selections one after the other */
 #define DART_RETAIN_LISTS 2  /* two phases: sorted candidate lists for all (sample, pivot) pairs at once, then the pivots'
                                 turns as walks over the lists; needs n_keep - n_pivot <= 4096, else the one-kernel form runs */
@@ -107,6 +105,10 @@ enum {
 #define DART_RETAIN_FUSED 4  /* the bands' two phases in one launch, one CTA per sample (a few warps build the sample's
                                 bands, then the CTA takes the turns): for batches that cannot fill the GPU.  Same limits as
                                 DART_RETAIN_BANDS, else as without it. */
+
+#define DART_RETAIN_RANKED 5 /* one launch, one CTA per (sample, pivot): the lowest dups a pivot could need, ranked; the CTA of a
+                                sample that finishes last takes the pivots' turns.  Needs n_vis <= 16384 and
+                                n_keep - n_pivot <= 4096, else as without it. */
 
 /* dart_opts.rule */
 #define DART_RULE_QUOTAS 0 /* one threshold per pivot: pivot i keeps its q_i not-yet-kept tokens of lowest dup (dart_reduce) */

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "dart_staged.cuh"
+#include "dart_ranked.cuh"
 #include "dart_sweep.cuh"
 #include "dart_onepass.cuh"
 #include "dart_resident.cuh"
@@ -51,6 +52,9 @@ struct dart_ctx {
     unsigned long long *band; // [B_max][P_max][band_stride] unsorted candidate bands of the band retention (NULL: not available)
     int32_t *band_n;          // [B_max][P_max] their lengths
     int band_stride;
+    uint16_t *rank;  // [B_max][...] ranked lists of the retention (NULL: not available)
+    size_t rank_n;   // their entries
+    int *rank_arrived; // [B_max] zero between launches
     uint8_t *keep;
     int *status; // device status word, followed by three words of detail
     int32_t status_detail[11];
@@ -224,39 +228,77 @@ int copy_debug(dart_ctx *ctx, int B, int n_vis, int P, const dart_debug *dbg, cu
 // Steps 4 and 5a.  Two phases (candidate lists for all pivots at once, then the pivots' turns) when the lists fit
 // the workspace and shared memory, else the one-kernel form.
 void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset, int n_vis, int P, int n_keep,
-                      int32_t *out_idx, int64_t *out_pos, const dart_opts &o, cudaStream_t st)
+                      int32_t *out_idx, int64_t *out_pos, const dart_opts &o, const dart_debug *dbg, cudaStream_t st)
 {
     using namespace dart;
     // the tokens shared out beside the pivots: n_keep - P, or up to n_keep when pivots may be text tokens
     const int S = ctx->S, m = o.text_pivots ? n_keep : n_keep - P, mode = o.retention;
+    // per-step outputs only where the caller asks for them
+    uint8_t *keep_out = dbg && dbg->keep ? ctx->keep : nullptr;
+    int32_t *owner_out = dbg && dbg->owner ? ctx->owner : nullptr;
+    float *eps_out = dbg && dbg->eps ? ctx->eps : nullptr;
+    const bool each = o.rule == DART_RULE_UNION; // independent pivots: lists of q_i instead of Q_i
+    RankParams rp = {};
+    size_t rank_smem = 0;
+    // few lists: as many threads per list as help; many: small CTAs, so that one list's barriers are covered by the others
+    const long long rank_rows = (long long)B * P;
+    const int rank_threads = rank_rows <= 2ll * ctx->sm_count ? 512 : rank_rows <= 8ll * ctx->sm_count ? 256 : n_vis > 1024 ? 128 : 64;
+    const int rank_m = each ? (m + P - 1) / P : m;
+    bool can_rank = ctx->rank && o.rule != DART_RULE_GLOBAL && n_vis <= kRankMaxVis && rank_m <= kRankMaxList;
+    if (can_rank) {
+        rp.sample_entries = (size_t)rank_place(P, m / P, m % P, each) + 8;
+        const size_t flags = rank_flag_bytes(n_vis), phase1 = rank_phase1_bytes(n_vis, rank_m, rp.bins = rank_bins(n_vis, rank_threads));
+        // the turns' staging buffers take what the ranking needs anyway, more where that saves rounds and costs no residency
+        size_t avail = phase1 - flags;
+        const size_t all = rp.sample_entries * 2, least = 4 * ((size_t)rank_m + 16);
+        if (all > avail && (long long)B * P <= ctx->sm_count && all + flags <= (size_t)100 << 10) avail = all;
+        if (avail < least) avail = least;
+        rp.stage_entries = (int)(all <= avail ? rp.sample_entries : avail / 4 / 8 * 8);
+        rank_smem = phase1 > flags + avail ? phase1 : flags + avail;
+        can_rank = (size_t)B * rp.sample_entries <= ctx->rank_n && rank_smem <= (size_t)ctx->max_smem_optin - kRankStaticSmem;
+    }
+    auto launch_ranked = [&]() {
+        rp.sim = ctx->sim, rp.pivot_idx = ctx->pivot_idx, rp.lists = ctx->rank, rp.arrived = ctx->rank_arrived, rp.pos_in = pos_in;
+        rp.S = S, rp.vis_offset = vis_offset, rp.n_vis = n_vis, rp.P = P, rp.n_keep = n_keep, rp.m = rank_m, rp.each = each;
+        rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
+        rp.len_out = ctx->len, rp.status = ctx->status;
+        Prof p(ctx, st, SLOT_RETAIN);
+        rank_kernel<<<dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st>>>(rp);
+    };
     if (o.rule == DART_RULE_GLOBAL) { // one threshold for all pivots: a single selection per sample
         Prof p(ctx, st, SLOT_RETAIN);
         retain_global_kernel<<<B, kSelectThreads, retain_global_smem_bytes(n_vis), st>>>(
-            ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, ctx->keep, ctx->owner, ctx->eps,
+            ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out,
             ctx->status);
         return;
     }
-    if (o.rule == DART_RULE_UNION) { // independent pivots: selections, scan of the packed lengths, index lists at their offsets
-        {
+    if (o.rule == DART_RULE_UNION) { // independent pivots: selections, then index lists at their offsets
+        if (can_rank && (mode == DART_RETAIN_AUTO || mode == DART_RETAIN_RANKED)) {
+            launch_ranked();
+        } else {
             Prof p(ctx, st, SLOT_RETAIN);
             retain_union_kernel<<<B, kSelectThreads, retain_union_smem_bytes(n_vis), st>>>(
-                ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, ctx->owner, ctx->eps, ctx->len, ctx->status);
-        }
-        {
-            Prof p(ctx, st, SLOT_RETAIN);
-            cu_seqlens_kernel<<<1, 256, 0, st>>>(ctx->len, B, o.cu_seqlens, ctx->status);
+                ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, owner_out, eps_out, ctx->len, ctx->status);
         }
         Prof p(ctx, st, SLOT_RETAIN);
-        pack_varlen_kernel<<<B, kWalkThreads, retain_union_smem_bytes(n_vis), st>>>(ctx->keep, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
+        pack_varlen_kernel<<<B, kWalkThreads, retain_union_smem_bytes(n_vis), st>>>(ctx->keep, ctx->len, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
                                                                                     out_idx, out_pos, ctx->status);
         return;
     }
-    const int m_pad = next_pow2(m > 1 ? m : 1);
     // bands: a list must hold the m tokens of the exact route and fit one staging round of phase 2
     const int band_cap = ctx->band_stride < kPickStageEntries ? ctx->band_stride : kPickStageEntries;
     const bool can_bands = ctx->band && m > 0 && m <= band_cap && n_vis <= kBandMaxTokens && band_smem_bytes(n_vis, band_cap) <= (size_t)ctx->max_smem_optin - 2048 &&
                            pick_smem_bytes(n_vis, P) <= (size_t)ctx->max_smem_optin - 2048;
-    // Which form: all do the same selections.  One kernel per sample takes B CTAs through P selections each; sorted
+    // AUTO: ranked lists, except for very many short rows, where one warp per row (bands) is ahead of a CTA's barriers (us,
+    // bands / ranked: 256 samples x 32 pivots x 200 tokens 11 / 19, x 576 66 / 69, x 1000 76 / 76; 128 pivots x 576 234 / 289,
+    // x 1500 122 / 133, x 2880 488 / 389; 8 pivots x 576 31 / 26, x 2880 60 / 38; one sample, 8 pivots x 2880: 39 / 21)
+    const bool prefer_bands = B > ctx->sm_count && P >= 32 && n_vis <= 1536 && can_bands;
+    if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && !prefer_bands))) {
+        launch_ranked();
+        return;
+    }
+    const int m_pad = next_pow2(m > 1 ? m : 1);
+    // Without them: all forms do the same selections.  One kernel per sample takes B CTAs through P selections each; sorted
     // lists spread the selections over B * P CTAs, which pays while B CTAs cannot fill the SMs (measured: batch 4-64 up
     // to 4x faster than one kernel); bands need one warp per selection and no sort, which pays once the batch fills the
     // GPU (measured at batch 256: 8 pivots 93 -> 56 us, 32 pivots 0.36 -> 0.16 ms, 128 pivots 1.38 -> 0.49 ms), while for
@@ -275,7 +317,7 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         Prof p(ctx, st, SLOT_RETAIN);
         retain_fused_kernel<<<B, kPickThreads, retain_fused_smem_bytes(n_vis, P, band_cap, band_warps), st>>>(
             ctx->sim, ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos,
-            ctx->keep, ctx->owner, ctx->eps, ctx->status, band_warps);
+            keep_out, owner_out, eps_out, ctx->status, band_warps);
         return;
     }
     const bool bands = can_bands && (mode == DART_RETAIN_BANDS || (mode == DART_RETAIN_AUTO && (B > ctx->sm_count || !can_lists)));
@@ -287,16 +329,16 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         }
         Prof p(ctx, st, SLOT_RETAIN);
         retain_pick_kernel<<<B, kPickThreads, pick_smem_bytes(n_vis, P), st>>>(
-            ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, ctx->keep,
-            ctx->owner, ctx->eps, ctx->status);
+            ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out,
+            owner_out, eps_out, ctx->status);
         return;
     }
     const bool two_phase = can_lists && (mode == DART_RETAIN_LISTS || (mode == DART_RETAIN_AUTO && B <= ctx->sm_count));
     if (!two_phase) {
         Prof p(ctx, st, SLOT_RETAIN);
         retain_kernel<<<B, kSelectThreads, retain_smem_bytes(n_vis, P), st>>>(ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P,
-                                                               n_keep, out_idx, out_pos, ctx->keep, ctx->owner,
-                                                               ctx->eps, ctx->status, retain_cache_rows(n_vis, P));
+                                                               n_keep, out_idx, out_pos, keep_out, owner_out,
+                                                               eps_out, ctx->status, retain_cache_rows(n_vis, P));
         return;
     }
     if (m > 0) {
@@ -311,7 +353,7 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         Prof p(ctx, st, SLOT_RETAIN);
         retain_walk_kernel<<<B, kWalkThreads, walk_smem_bytes(n_vis), st>>>(ctx->sim, ctx->pivot_idx, ctx->cand, ctx->cand_stride, pos_in,
                                                                           S, vis_offset, n_vis, P, n_keep, out_idx, out_pos,
-                                                                          ctx->keep, ctx->owner, ctx->eps, ctx->status);
+                                                                          keep_out, owner_out, eps_out, ctx->status);
     }
 }
 
@@ -378,7 +420,7 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
                                                               ctx->ssq, ctx->sim);
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -579,7 +621,7 @@ int launch_fused(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, 
         else
             sim_sum_kernel<float><<<grid, kSimSumThreads, 0, st>>>(ctx->sim_share, items, p.n_kc, ctx->sim);
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -742,7 +784,7 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         // every CTA waits for scores that the others publish: co-residency is required
         DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3(F::kThreads), args, smem, st));
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st, true);
     DART_CUDA(ctx, cudaGetLastError());
     ctx->flow_dirty = false;
@@ -788,7 +830,7 @@ int launch_resident(dart_ctx *ctx, int B, const void *hidden, const void *keys_i
         int rc = launch_onepass_kernel(ctx, B, p.keys, true, vis_offset, n_vis, P, o, st, split);
         if (rc != DART_OK) return rc;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -831,7 +873,7 @@ int launch_pair(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         DART_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)Q::pair_kernel, dim3(grid), dim3(Q::kThreads), args,
                                                    Q::smem_bytes(P, p.row_bytes, (int)grid, p.n1, p.n2, p.n3), st));
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -845,7 +887,7 @@ int launch_onepass(dart_ctx *ctx, int B, const void *hidden, const void *keys_in
     launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
     int rc = launch_onepass_kernel(ctx, B, keys_in ? keys_in : hidden, false, vis_offset, n_vis, P, o, st);
     if (rc != DART_OK) return rc;
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -895,7 +937,7 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
                                                               ctx->pivot_idx, ctx->ssq, ctx->sim);
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, st);
+    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -1049,6 +1091,7 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
         delete ctx;
         return DART_ERR_CUDA;
     }
+    cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, desc->device);
     const size_t nv = (size_t)desc->B_max * desc->S_max, np = (size_t)desc->B_max * desc->P_max;
     int rc = DART_OK;
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->l1, nv);
@@ -1077,6 +1120,17 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->band_n, np);
         }
     }
+    if (rc == DART_OK) {
+        // ranked lists of the retention: the most any call within the maxima needs; contexts that would need more than 1 GiB go without
+        ctx->rank_n = (size_t)desc->B_max * ((size_t)dart::rank_place(desc->P_max, desc->Kp_max / desc->P_max, desc->Kp_max % desc->P_max, false) + 8);
+        if (ctx->rank_n * sizeof(uint16_t) <= ((size_t)1 << 30)) {
+            rc = ws_alloc(ctx, &ctx->rank, ctx->rank_n);
+            if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->rank_arrived, (size_t)desc->B_max);
+            if (rc == DART_OK && cudaFuncSetAttribute(dart::rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      ctx->max_smem_optin - dart::kRankStaticSmem) != cudaSuccess)
+                rc = DART_ERR_CUDA;
+        }
+    }
     if (rc == DART_OK && desc->P_max > dart::onepass::kGatherMaxP) {
         // compact pivot rows for the one-pass kernel; contexts that would need more than 2 GiB go without (gather4 then)
         const size_t bytes = (size_t)desc->B_max * ((desc->P_max + 15) / 16 * 16) * desc->d * 2;
@@ -1084,7 +1138,6 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
     }
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->status, 64);
     if (rc == DART_OK) {
-        cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, desc->device);
         size_t sim_smem = (size_t)dart::kSimPivotChunk * (desc->d / 8) * 16;
         if (sim_smem > (size_t)ctx->max_smem_optin ||
             (size_t)desc->S_max + 16 + dart::kRetainCacheBytes > (size_t)ctx->max_smem_optin)
@@ -1147,6 +1200,7 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
     if (rc == DART_OK) rc = ws_commit(ctx);
     if (rc == DART_OK) rc = cudaMemsetAsync(ctx->status, 0, 256, 0) == cudaSuccess ? DART_OK : DART_ERR_CUDA;
     if (rc == DART_OK && ctx->flow_rec) rc = flow_reset(ctx, 0);
+    if (rc == DART_OK && ctx->rank && cudaMemsetAsync(ctx->rank_arrived, 0, (size_t)desc->B_max * sizeof(int), 0) != cudaSuccess) rc = DART_ERR_CUDA;
     // the first call may use a stream that does not wait for the legacy stream
     if (rc == DART_OK && cudaStreamSynchronize(0) != cudaSuccess) rc = DART_ERR_CUDA;
     if (rc != DART_OK) {
@@ -1226,7 +1280,7 @@ int dart_reduce_ex(dart_ctx *ctx, const void *hidden, const void *keys, const in
         dart::retain_global_smem_bytes(n_vis) > (size_t)ctx->max_smem_optin - 2048)
         return DART_ERR_UNSUPPORTED; // the sample's duplication values must fit shared memory
     if (o.retention != DART_RETAIN_AUTO && o.retention != DART_RETAIN_SERIAL && o.retention != DART_RETAIN_LISTS &&
-        o.retention != DART_RETAIN_BANDS && o.retention != DART_RETAIN_FUSED)
+        o.retention != DART_RETAIN_BANDS && o.retention != DART_RETAIN_FUSED && o.retention != DART_RETAIN_RANKED)
         return DART_ERR_UNSUPPORTED;
     if ((uintptr_t)pos_in & 7u) return DART_ERR_ALIGN;
     DeviceGuard g(ctx->desc.device);

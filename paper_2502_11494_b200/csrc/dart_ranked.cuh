@@ -1,0 +1,462 @@
+// Steps 4 and 5a from ranked lists, in one launch.
+//
+// Pivot i's picks are among the Q_i = q_0 + ... + q_i smallest (dup, index) pairs of its row (dart_staged.cuh), whatever the
+// other pivots take.  One CTA per (sample, pivot) puts those Q_i into order; the CTA of a sample that finishes last takes the
+// pivots' turns over the ranked lists, in rank order, and writes the packed index list.  What bounded the other forms:
+//   - ordering: a radix select and a sort are some twenty block-wide steps (16 us for 128 lists of 312 out of 2880 values).
+//     Here: a histogram of equal bins over the row's low end, its prefix sums as the bins' places, and every entry
+//     counts the smaller ones among the few that share its bin: eight block-wide steps;
+//   - the turns: a walk 32 entries at a time, one dependent vote after the other (1.4 us per turn).  Here a lane holds eight
+//     consecutive entries (16 bytes), their eight flags are read at once, and four votes over the bits of the lanes' counts
+//     give every lane its rank among 256 entries: 0.45 us per turn.
+// Measured (us, before: the bands or sorted lists): 1 x 2880 tokens, 8 pivots 39 -> 21; 4 x 4608, 32 pivots 70 -> 31; 8 x 1500
+// keeping half 60 -> 20; 256 x 2880, 8 pivots 60 -> 38, 128 pivots 488 -> 389.  Of the 12 us that one sample takes, ranking
+// is 5, the counter and the lists' way to the last CTA 2, the turns 3.5 and the packed list 1.5: a chain of short steps.
+// Rows whose values the bins do not separate (many equal values, a value that is not finite) are ranked by an exact radix
+// select and counting.  The result equals retain_kernel's exactly.
+//
+// With independent pivots (DART_RULE_UNION) the lists are the q_i smallest and the last CTA only merges them.
+#pragma once
+#include "dart_staged.cuh"
+
+namespace dart {
+
+constexpr int kRankMaxThreads = 512;
+constexpr int kRankMaxP = 1024;       // a context's most pivots
+constexpr int kRankMaxVis = 16384;    // the row in shared memory
+constexpr int kRankMaxList = 4096;    // longest list
+constexpr uint32_t kRankMaxBin = 192; // entries of one bin that are ranked by counting
+
+// entries of a list in shared memory: the last bin may hold more than the list needs
+__host__ __device__ inline int rank_list_cap(int m) { return m + kRankMaxBin; }
+// one flag per token and one more that is never free
+__host__ __device__ inline size_t rank_flag_bytes(int n_vis) { return ((size_t)n_vis + 16) / 16 * 16; }
+// bins: a multiple of 4 per thread, about one per one to three tokens
+inline int rank_bins(int n_vis, int threads)
+{
+    int bins = 4 * threads;
+    while (bins < 2048 && 3 * bins < n_vis) bins *= 2;
+    return bins;
+}
+inline size_t rank_phase1_bytes(int n_vis, int m, int bins)
+{
+    return ((size_t)n_vis * 4 + 15) / 16 * 16 + (size_t)bins * 4 + (size_t)rank_list_cap(m) * 8;
+}
+// places of the lists in the sample's part of the workspace, in entries of 16 bits: list i starts at rank_place(i), a multiple of 8
+__host__ __device__ inline int rank_place(int i, int q, int r, bool each)
+{
+    // sum over k < i of (Q_k or q_k), every list rounded up by at most 7
+    const int n = i < r ? i : r;
+    const int sum = each ? i * q + n : q * (i * (i + 1) / 2) + n * (n + 1) / 2 + r * (i - n);
+    return ((sum + 7) & ~7) + 8 * i;
+}
+__host__ __device__ inline int rank_length(int i, int q, int r, bool each) { return each ? q + (i < r ? 1 : 0) : quota_prefix(i, q, r); }
+
+struct RankParams {
+    const float *sim;          // [B][P][n_vis]
+    const int32_t *pivot_idx;  // [B][P]
+    uint16_t *lists;           // [B][sample_entries]
+    size_t sample_entries;
+    int *arrived;              // [B] lists written; zero on entry and on exit
+    const int64_t *pos_in;
+    int S, vis_offset, n_vis, P, n_keep, m; // m: the longest list (n_keep - P, or n_keep when pivots may be text tokens)
+    int each;                  // 1: independent pivots (lists of q_i, merged)
+    int bins;
+    int stage_entries;         // entries of 16 bits per staging buffer of the turns
+    int32_t *out_idx;          // quotas: [B][S_out]; independent pivots: unused
+    int64_t *out_pos;
+    uint8_t *keep_out;         // [B][n_vis]; NULL unless wanted
+    int32_t *owner_out;        // [B][n_vis]; NULL unless wanted
+    float *eps_out;            // [B][P]; NULL unless wanted
+    int32_t *len_out;          // independent pivots: [B] packed length
+    const int *status;
+};
+
+struct RankShared {
+    SelectSmem sel;
+    float red_lo[kRankMaxThreads / 32], red_hi[kRankMaxThreads / 32], red_sum[kRankMaxThreads / 32];
+    uint32_t scan[kRankMaxThreads / 32];
+    int32_t piv[kRankMaxP];
+    uint32_t n_pivots, last_bin, n_band, biggest, n_list, last;
+};
+
+constexpr int kRankStaticSmem = 8192;
+static_assert(sizeof(RankShared) + 64 <= kRankStaticSmem, "static shared memory exceeds its reserve");
+
+// Inclusive sum over the CTA's threads (two barriers)
+__device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *per_warp)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) per_warp[warp] = v;
+    __syncthreads();
+    uint32_t x = lane < nwarp && lane < warp ? per_warp[lane] : 0u;
+    return v + __reduce_add_sync(0xffffffffu, x);
+}
+
+// Phase 1: the list of pivot i of sample b, ranked, into out[0 .. C).  row_s, hist, list: shared memory.
+__device__ __forceinline__ void rank_row(const RankParams &p, const float *__restrict__ row, const int32_t *__restrict__ piv, uint16_t *out,
+                                         int C, float *row_s, uint32_t *hist, unsigned long long *list, RankShared &sh)
+{
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5, n = p.n_vis, n4 = (n + 3) / 4;
+    const float kNotAToken = __uint_as_float(0xffffffffu); // a pivot, or the filler behind the row: a NaN that no arithmetic produces, in no interval
+    const float4 *row4 = reinterpret_cast<const float4 *>(row_s);
+    // smallest and largest value and the mean (pivots included: they only stretch the range)
+    float lo = __int_as_float(0x7f800000), hi = __int_as_float(0xff800000), sum = 0.f;
+#pragma unroll 2
+    for (int j = t; j < n4; j += T) {
+        const float4 f = row4[j];
+        lo = fminf(fminf(lo, f.x), fminf(fminf(f.y, f.z), f.w));
+        hi = fmaxf(fmaxf(hi, f.x), fmaxf(fmaxf(f.y, f.z), f.w));
+        sum += (f.x + f.y) + (f.z + f.w);
+    }
+    lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
+    hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
+    sum = warp_sum(sum);
+    if (lane == 0) sh.red_lo[warp] = lo, sh.red_hi[warp] = hi, sh.red_sum[warp] = sum;
+    __syncthreads();
+    for (int i = t; i < p.P; i += T)
+        if (piv[i] >= 0 && piv[i] < n) row_s[piv[i]] = kNotAToken;
+    if (t < 4 * n4 - n) row_s[n + t] = kNotAToken;
+    lo = lane < nwarp ? sh.red_lo[lane] : lo;
+    hi = lane < nwarp ? sh.red_hi[lane] : hi;
+    sum = warp_sum(lane < nwarp ? sh.red_sum[lane] : 0.f);
+    lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
+    hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
+    // The bins span [min, 2 mean - min]: a list is the row's low end, and a few large dups - the pivot's own cluster - would
+    // otherwise take most of the bins; if the list reaches beyond, again over [min, max].
+    const float mid = 2.0f * (sum / (float)(4 * n4) - lo);
+    float span = mid > 0.0f && mid < hi - lo ? mid : hi - lo;
+    bool exact = !(hi > lo) || !(hi - lo < 3.0e38f);
+    float scale = 0.f;
+    __syncthreads(); // the pivots are marked
+    const int per = p.bins / T; // bins per thread, a multiple of 4
+    for (int pass = 0; !exact; ++pass) {
+        scale = (float)p.bins / span * 0.9999f; // (places stay below the number of bins for values inside the span)
+        if (!(scale < 3.0e38f)) {
+            exact = true;
+            break;
+        }
+        const float top = (float)p.bins;
+#pragma unroll 2
+        for (int j = t; j < n4; j += T) {
+            const float4 v = row4[j];
+            const float x[4] = {(v.x - lo) * scale, (v.y - lo) * scale, (v.z - lo) * scale, (v.w - lo) * scale};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (x[e] < top) atomicAdd(&hist[(int)x[e]], 1u);
+        }
+        __syncthreads();
+        // thread t owns bins [per t, per t + per)
+        uint4 *h4 = reinterpret_cast<uint4 *>(hist) + (size_t)t * (per / 4);
+        uint32_t s = 0;
+        for (int u = 0; u < per / 4; ++u) {
+            const uint4 c = h4[u];
+            s += c.x + c.y + c.z + c.w;
+        }
+        const uint32_t incl = cta_scan(s, sh.scan);
+        uint32_t run = incl - s, big = 0;
+        for (int u = 0; u < per / 4; ++u) {
+            uint4 c = h4[u];
+            uint32_t *cc = reinterpret_cast<uint32_t *>(&c);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t k = cc[e];
+                if (run < (uint32_t)C) { // a bin the list needs
+                    big = max(big, k);
+                    if (run + k >= (uint32_t)C) sh.last_bin = (uint32_t)(per * t + 4 * u + e), sh.n_band = run + k;
+                }
+                cc[e] = run; // the bin's place
+                run += k;
+            }
+            h4[u] = c;
+        }
+        big = __reduce_max_sync(0xffffffffu, big);
+        if (lane == 0 && big > kRankMaxBin) sh.biggest = big;
+        if (t == T - 1) sh.n_list = incl;
+        __syncthreads();
+        if (sh.n_list >= (uint32_t)C) {
+            exact = sh.biggest != 0;
+            break;
+        }
+        if (pass == 1 || !(span < hi - lo)) { // values that are not finite
+            exact = true;
+            break;
+        }
+        span = hi - lo;
+        for (int i = t; i < p.bins; i += T) hist[i] = 0;
+        __syncthreads();
+    }
+    if (!exact) {
+        const int m = (int)sh.n_band;
+        const float edge = (float)((int)sh.last_bin + 1);
+#pragma unroll 2
+        for (int j = t; j < n4; j += T) {
+            const float4 v = row4[j];
+            const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float x = (f[e] - lo) * scale;
+                if (x < edge) list[atomicAdd(&hist[(int)x], 1u)] = ((unsigned long long)order_key(f[e]) << 32) | (uint32_t)(4 * j + e);
+            }
+        }
+        __syncthreads();
+        // hist[x] is now the end of bin x
+        for (int e = t; e < m; e += T) {
+            const unsigned long long x = list[e];
+            const int bin = (int)((order_key_inv((uint32_t)(x >> 32)) - lo) * scale);
+            const int end = (int)hist[bin];
+            int u = bin > 0 ? (int)hist[bin - 1] : 0, r = u;
+            for (; u < end; ++u) r += list[u] < x ? 1 : 0;
+            if (r < C) out[r] = (uint16_t)x;
+        }
+        return;
+    }
+    // the exact route
+    auto keyfn = [&](int j, uint32_t &key) {
+        if (__float_as_uint(row_s[j]) == 0xffffffffu) return false;
+        key = order_key(row_s[j]);
+        return true;
+    };
+    if (t == 0) sh.n_list = 0;
+    uint32_t thr, need_eq, cnt_eq;
+    block_select_threshold(CtaGroup(), keyfn, n, (uint32_t)C, sh.sel, thr, need_eq, cnt_eq);
+    block_select_apply(CtaGroup(), keyfn, n, thr, need_eq, cnt_eq, sh.sel, [&](int j, uint32_t key) {
+        list[atomicAdd(&sh.n_list, 1u)] = ((unsigned long long)key << 32) | (uint32_t)j;
+    });
+    rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (uint16_t)x; });
+}
+
+// Step 5a (as pack_indices; flags are 0 or 1, 16-byte aligned), a contiguous range of flags per warp: two barriers in all instead of two per blockDim.x flags.
+__device__ __forceinline__ void pack_ranges(const uint8_t *keep, int S, int vis_offset, int n_vis, int n_keep, const int64_t *__restrict__ pin,
+                                            int32_t *__restrict__ oi, int64_t *__restrict__ op, uint32_t *per_warp)
+{
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5;
+    const int per = ((n_vis + 31) / 32 + nwarp - 1) / nwarp * 32, j0 = warp * per, j1 = min(n_vis, j0 + per);
+    uint32_t mine = 0;
+    for (int j = j0 + 4 * lane; j < j1; j += 128) { // four flags at a time (the flags end with zeros up to a multiple of 16)
+        uint32_t f = *reinterpret_cast<const uint32_t *>(keep + j);
+        if (j + 4 > j1) f &= (1u << (8 * (j1 - j))) - 1u;
+        mine += __popc(f);
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) per_warp[warp] = mine;
+    for (int s = t; s < vis_offset; s += T) {
+        oi[s] = s;
+        op[s] = pin ? pin[s] : (int64_t)s;
+    }
+    for (int u = t; u < S - vis_offset - n_vis; u += T) {
+        const int s = vis_offset + n_vis + u;
+        oi[vis_offset + n_keep + u] = s;
+        op[vis_offset + n_keep + u] = pin ? pin[s] : (int64_t)s;
+    }
+    __syncthreads();
+    int at = vis_offset + (int)__reduce_add_sync(0xffffffffu, lane < warp ? per_warp[lane] : 0u);
+#pragma unroll 4
+    for (int c = j0; c < j1; c += 32) {
+        const int j = c + lane, s = vis_offset + j;
+        const bool f = j < j1 && keep[j];
+        const uint32_t bal = __ballot_sync(0xffffffffu, f);
+        if (f) {
+            const int k = at + __popc(bal & ((1u << lane) - 1u));
+            oi[k] = s;
+            op[k] = pin ? pin[s] : (int64_t)s;
+        }
+        at += __popc(bal);
+    }
+    __syncthreads();
+}
+
+// One pivot's turn, by a warp: the first `want` free entries of its ranked list L[0 .. M) (shared memory, 16-byte aligned) are
+// taken.  flags[none] is a place that is never free.  No branch depends on an entry: what a lane does not hold or does not take
+// goes to `none` (with a branch per entry a turn took 1.4 us, without 0.45).  kDetail: owners, and the last entry taken is
+// returned to every lane (-1 if none).
+template <bool kDetail>
+__device__ __forceinline__ int take_turn(const uint16_t *L, int M, int want, uint8_t *flags, uint32_t none, int32_t *owner, int i)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    int last = -1;
+    for (int s = 0; s < M && want > 0; s += 256) {
+        const int at = s + 8 * lane;
+        uint4 e = make_uint4(0, 0, 0, 0);
+        if (at < M) e = *reinterpret_cast<const uint4 *>(L + at);
+        const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+        uint32_t j[8], f = 0; // f: which of the lane's entries are free
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            j[k] = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
+            if (at + k >= M) j[k] = none;
+        }
+        uint32_t taken[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) taken[k] = flags[j[k]];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) f |= taken[k] == 0 ? 1u << k : 0u;
+        const int c = __popc(f);
+        int before = 0, total = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t v = __ballot_sync(0xffffffffu, (c >> k) & 1);
+            before += __popc(v & lt) << k;
+            total += __popc(v) << k;
+        }
+        const int may = want - before; // how many of its free entries the lane may take
+        uint32_t g = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const bool take = ((f >> k) & 1u) && __popc(f & ((1u << k) - 1u)) < may;
+            g |= take ? 1u << k : 0u;
+            flags[take ? j[k] : none] = 1;
+        }
+        if (kDetail) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if ((g >> k) & 1u) {
+                    if (owner) owner[j[k]] = i;
+                    last = (int)j[k];
+                }
+            const uint32_t any = __ballot_sync(0xffffffffu, g != 0);
+            last = any ? __shfl_sync(0xffffffffu, last, 31 - __clz(any)) : last;
+        }
+        want -= total;
+        __syncwarp(); // the flags are visible to the next block and the next pivot
+    }
+    return last;
+}
+
+__global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams p)
+{
+    extern __shared__ __align__(16) uint8_t rank_smem[];
+    __shared__ RankShared sh;
+    if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
+    const int t = threadIdx.x, T = blockDim.x, warp = t >> 5, n = p.n_vis;
+    const int i = blockIdx.x, b = blockIdx.y;
+    const int32_t *piv = sh.piv;
+    const float *rows = p.sim + (size_t)b * p.P * n, *row = rows + (size_t)i * n;
+    float *row_s = reinterpret_cast<float *>(rank_smem);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(rank_smem + ((size_t)n * 4 + 15) / 16 * 16);
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(hist + p.bins);
+    if ((n & 3) == 0) // rows start on 16-byte boundaries
+        for (int j = t; j < n / 4; j += T) copy_async<16>(row_s + 4 * j, row + 4 * j);
+    else
+        for (int j = t; j < (n + 3) / 4 * 4; j += T) row_s[j] = __ldcs(row + (j < n ? j : 0)); // (filler: a value of the row)
+    copy_async_commit();
+    for (int k = t; k < p.bins / 4; k += T) reinterpret_cast<uint4 *>(hist)[k] = make_uint4(0, 0, 0, 0);
+    if (t == 0) sh.n_pivots = 0, sh.biggest = 0;
+    __syncthreads();
+    uint32_t mine = 0;
+    for (int k = t; k < p.P; k += T) {
+        const int pv = p.pivot_idx[(size_t)b * p.P + k];
+        sh.piv[k] = pv;
+        mine += pv >= 0 && pv < n ? 1u : 0u;
+    }
+    if (mine) atomicAdd(&sh.n_pivots, mine);
+    copy_async_wait<0>();
+    __syncthreads();
+    const int Pv = (int)sh.n_pivots, q = (p.n_keep - Pv) / p.P, r = (p.n_keep - Pv) % p.P;
+    const bool each = p.each != 0;
+    uint16_t *lists = p.lists + (size_t)b * p.sample_entries;
+    if (q + (i < r ? 1 : 0) > 0) // (else this pivot keeps nothing, and so do all later ones)
+        rank_row(p, row, piv, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), row_s, hist, list, sh);
+    __syncthreads();
+    if (t == 0) { // release: the list; acquire: the other pivots' lists
+        int before;
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(p.arrived + b) : "memory");
+        sh.last = before == p.P - 1;
+        if (before == p.P - 1) p.arrived[b] = 0;
+    }
+    __syncthreads();
+    if (!sh.last) return;
+    // ---- the sample's last CTA: the turns
+    uint8_t *flags = rank_smem;
+    uint16_t *stage = reinterpret_cast<uint16_t *>(rank_smem + rank_flag_bytes(n));
+    int32_t *owner = p.owner_out ? p.owner_out + (size_t)b * n : nullptr;
+    float *eps = p.eps_out ? p.eps_out + (size_t)b * p.P : nullptr;
+    for (int k = t; k < (n + 16) / 16; k += T) reinterpret_cast<uint4 *>(flags)[k] = make_uint4(0, 0, 0, 0);
+    if (owner)
+        for (int j = t; j < n; j += T) owner[j] = -1;
+    __syncthreads();
+    if (t == 0) flags[n] = 1;
+    for (int k = t; k < p.P; k += T)
+        if (piv[k] >= 0 && piv[k] < n) {
+            flags[piv[k]] = 1;
+            if (owner) owner[piv[k]] = p.P + k;
+        }
+    const int n_active = q > 0 ? p.P : r; // pivots with a quota
+    if (eps)
+        for (int k = n_active + t; k < p.P; k += T) eps[k] = __int_as_float(0x7fc00000);
+    if (each) { // independent pivots: the lists are what they keep
+        for (int k = n_active - 1; k >= 0; --k) {
+            const uint16_t *L = lists + rank_place(k, q, r, true);
+            const int M = rank_length(k, q, r, true);
+            for (int e = t; e < M; e += T) {
+                const int j = __ldcg(L + e);
+                flags[j] = 1;
+                if (owner) owner[j] = k; // the first pivot in rank order that took a token owns it: it writes last
+                if (eps && e == M - 1) eps[k] = rows[(size_t)k * n + j];
+            }
+            if (owner) __syncthreads();
+        }
+        if (t == 0) sh.n_list = 0;
+        __syncthreads();
+        uint32_t kept = 0;
+        for (int j = t; j < n; j += T) {
+            const uint8_t f = flags[j] != 0;
+            kept += f;
+            p.keep_out[(size_t)b * n + j] = f;
+        }
+        kept = __reduce_add_sync(0xffffffffu, kept);
+        if ((t & 31) == 0) atomicAdd(&sh.n_list, kept);
+        __syncthreads();
+        if (t == 0) p.len_out[b] = p.S - n + (int)sh.n_list;
+        return;
+    }
+    // rounds: the lists of as many pivots as fit a staging buffer; while warp 0 takes one round's turns the others fetch the next
+    auto round_end = [&](int k0) {
+        if (rank_place(n_active, q, r, false) - rank_place(k0, q, r, false) <= p.stage_entries) return n_active;
+        int k1 = k0;
+        while (k1 < n_active && (k1 == k0 || rank_place(k1 + 1, q, r, false) - rank_place(k0, q, r, false) <= p.stage_entries)) ++k1;
+        return k1;
+    };
+    auto fetch = [&](int k0, int k1, uint16_t *buf, int first, int threads) {
+        const int from = rank_place(k0, q, r, false), words = k1 > k0 ? (rank_place(k1 - 1, q, r, false) + (rank_length(k1 - 1, q, r, false) + 7) / 8 * 8 - from) / 8 : 0;
+        const uint4 *src = reinterpret_cast<const uint4 *>(lists + from);
+        for (int e = first; e < words; e += threads) reinterpret_cast<uint4 *>(buf)[e] = __ldcg(src + e);
+    };
+    int k0 = 0, k1 = round_end(0);
+    fetch(k0, k1, stage, t, T);
+    __syncthreads(); // (and the pivots are flagged)
+    for (int round = 0; k0 < n_active; ++round) {
+        uint16_t *buf = stage + (size_t)(round & 1) * p.stage_entries;
+        const int k2 = round_end(k1);
+        if (warp == 0) {
+            const int from = rank_place(k0, q, r, false);
+            for (int k = k0; k < k1; ++k) {
+                const uint16_t *L = buf + rank_place(k, q, r, false) - from;
+                const int M = rank_length(k, q, r, false), want = q + (k < r ? 1 : 0);
+                int last = -1;
+                if (owner || eps)
+                    last = take_turn<true>(L, M, want, flags, (uint32_t)n, owner, k);
+                else
+                    take_turn<false>(L, M, want, flags, (uint32_t)n, nullptr, k);
+                if (eps && t == 0) eps[k] = last >= 0 ? rows[(size_t)k * n + last] : __int_as_float(0x7fc00000);
+            }
+        } else if (k2 > k1) {
+            fetch(k1, k2, stage + (size_t)((round + 1) & 1) * p.stage_entries, t - 32, T - 32);
+        }
+        __syncthreads();
+        k0 = k1, k1 = k2;
+    }
+    const int S_out = p.S - n + p.n_keep;
+    pack_ranges(flags, p.S, p.vis_offset, n, p.n_keep, p.pos_in ? p.pos_in + (size_t)b * p.S : nullptr, p.out_idx + (size_t)b * S_out,
+                p.out_pos + (size_t)b * S_out, sh.scan);
+    if (p.keep_out)
+        for (int j = t; j < n; j += T) p.keep_out[(size_t)b * n + j] = flags[j] != 0;
+}
+
+} // namespace dart

@@ -1271,9 +1271,9 @@ retain_global_kernel(const float *__restrict__ sim, const int32_t *__restrict__ 
 // Steps 4 and 5a with INDEPENDENT pivots (Eq. 9-10 read literally: R = P u U_i R_i): pivot i takes its q_i
 // non-pivot tokens of lowest dup whatever the other pivots took; a token two pivots take is kept once, so a
 // sample keeps between P and n_keep vision tokens and the packed length depends on the data.  Three launches:
-// the selections (one CTA per sample; writes the keep flags and the sample's packed length), an exclusive
-// scan of the lengths (cu_seqlens, the layout variable-length attention kernels take), and the packed index
-// lists written at the samples' offsets.
+// the selections (writes the keep flags and the sample's packed length; one CTA per sample, or the ranked lists of
+// dart_ranked.cuh), then the packed index lists written at the samples' offsets (cu_seqlens, the layout
+// variable-length attention kernels take).
 // ------------------------------------------------------------------------------------------------
 constexpr int kGatherWarps = 8; // warps per CTA of the gather kernels, one output row each
 inline size_t retain_union_smem_bytes(int n_vis) { return ((size_t)n_vis + 15) / 16 * 16; }
@@ -1345,35 +1345,10 @@ retain_union_kernel(const float *__restrict__ sim, const int32_t *__restrict__ p
     if (threadIdx.x == 0) len_out[b] = S - n_vis + total;
 }
 
-// cu[0] = 0, cu[b + 1] = cu[b] + len[b]: one CTA, chunks of blockDim.x lengths with a running carry
-__global__ void __launch_bounds__(256) cu_seqlens_kernel(const int32_t *__restrict__ len, int B, int32_t *__restrict__ cu,
-                                                         const int *__restrict__ status)
-{
-    __shared__ int32_t buf[256];
-    __shared__ int32_t carry;
-    if (*status != 0) return;
-    if (threadIdx.x == 0) carry = 0, cu[0] = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < B; b0 += blockDim.x) {
-        const int b = b0 + threadIdx.x;
-        buf[threadIdx.x] = b < B ? len[b] : 0;
-        __syncthreads();
-        for (int o = 1; o < (int)blockDim.x; o <<= 1) { // inclusive scan
-            const int32_t v = threadIdx.x >= (unsigned)o ? buf[threadIdx.x - o] : 0;
-            __syncthreads();
-            buf[threadIdx.x] += v;
-            __syncthreads();
-        }
-        if (b < B) cu[b + 1] = carry + buf[threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry += buf[threadIdx.x];
-        __syncthreads();
-    }
-}
-
-// The packed index list and position ids of every sample at its offset cu[b].
+// cu_seqlens, and the packed index list and position ids of every sample at its offset.  Every CTA adds up the lengths before
+// its sample's (a scan kernel of its own took 4 us).
 __global__ void __launch_bounds__(kWalkThreads)
-pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restrict__ cu, const int64_t *__restrict__ pos_in, int S,
+pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restrict__ len, int32_t *__restrict__ cu, const int64_t *__restrict__ pos_in, int S,
                    int vis_offset, int n_vis, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
                    const int *__restrict__ status)
 {
@@ -1383,7 +1358,19 @@ pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restric
     const int b = blockIdx.x;
     for (int j = threadIdx.x; j < n_vis; j += blockDim.x) keep[j] = keep_in[(size_t)b * n_vis + j];
     __syncthreads();
-    const int start = cu[b], kept = cu[b + 1] - start - (S - n_vis);
+    int before = 0;
+    for (int k = threadIdx.x; k < b; k += blockDim.x) before += len[k];
+    before = __reduce_add_sync(0xffffffffu, before);
+    if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = (uint32_t)before;
+    __syncthreads();
+    int start = 0;
+    for (int w = 0; w < kWalkThreads / 32; ++w) start += (int)warp_tot[w];
+    __syncthreads();
+    const int kept = len[b] - (S - n_vis);
+    if (threadIdx.x == 0) {
+        if (b == 0) cu[0] = 0;
+        cu[b + 1] = start + len[b];
+    }
     pack_indices(keep, S, vis_offset, n_vis, kept, pos_in ? pos_in + (size_t)b * S : nullptr, out_idx + start, out_pos + start,
                  warp_tot);
 }

@@ -21,6 +21,7 @@ DART_FLAG_HOST_STAGING = 1
 DART_PATH_AUTO, DART_PATH_STAGED, DART_PATH_FUSED, DART_PATH_TWO_PASS, DART_PATH_RESIDENT, DART_PATH_SPLIT, DART_PATH_PAIRED = 0, 1, 2, 3, 4, 5, 6
 DART_PATH_FLOW = 7
 DART_RETAIN_AUTO, DART_RETAIN_SERIAL, DART_RETAIN_LISTS, DART_RETAIN_BANDS, DART_RETAIN_FUSED = 0, 1, 2, 3, 4
+DART_RETAIN_RANKED = 5
 DART_RULE_QUOTAS, DART_RULE_GLOBAL, DART_RULE_UNION = 0, 1, 2
 DART_PIVOTS_BY_SCORE, DART_PIVOTS_MIXED, DART_PIVOTS_RANDOM = 0, 1, 2
 

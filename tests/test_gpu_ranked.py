@@ -1,0 +1,53 @@
+"""The retention from ranked lists against the one-kernel form, bit for bit, through the C ABI (needs a B200)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2502_11494_b200 import dart  # noqa: E402
+from test_gpu_parity import BAND_CASES, RETENTION_SHAPES, _band_inputs, run_gpu  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+CASES = BAND_CASES + [("gaussian", s) for s in RETENTION_SHAPES] + [
+    # (kind, (B, S, d, vis_offset, n_vis, P, Kp))
+    ("gaussian", (1, 300, 64, 1, 257, 1, 257)),           # one block of 256 entries and one entry more, one pivot
+    ("gaussian", (40, 700, 64, 40, 576, 8, 520)),         # 256 threads per list; 90 % kept: the bins reach the row's upper end
+    ("gaussian", (200, 300, 64, 40, 255, 8, 100)),        # 128 threads per list
+    ("gaussian", (1, 16400, 64, 3, 16384, 2, 4098)),      # the longest row and the longest lists
+    ("gaussian", (1, 3000, 64, 0, 2880, 1000, 2000)),     # 1000 pivots: several rounds of staging
+    ("equal tokens", (3, 1500, 64, 10, 1402, 32, 1402)),
+]
+
+
+@pytest.mark.parametrize("kind,shape", CASES, ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
+def test_ranked_lists_make_the_same_selections(kind, shape):
+    B, S, d, vo, nv, P, Kp = shape
+    k, h = _band_inputs(kind, B, S, d, vo, nv, P, seed=17 + sum(shape))
+    a = run_gpu(k, h, vo, nv, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
+    b = run_gpu(k, h, vo, nv, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED)
+    c = run_gpu(k, h, vo, nv, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED, debug=False)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], c[:3]))      # without the per-step outputs
+    assert all(np.array_equal(a[3][n], b[3][n], equal_nan=(n == "eps")) for n in a[3])
+
+
+@pytest.mark.parametrize("kind,shape", [("gaussian", (3, 333, 264, 17, 301, 7, 60)), ("equal tokens", (2, 700, 64, 10, 640, 16, 200)),
+                                        ("gaussian", (260, 130, 64, 5, 100, 3, 90)), ("gaussian", (2, 3000, 64, 0, 2880, 128, 640))],
+                         ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
+def test_ranked_lists_with_independent_pivots(kind, shape):
+    B, S, d, vo, nv, P, Kp = shape
+    k, h = _band_inputs(kind, B, S, d, vo, nv, P, seed=19 + sum(shape))
+    got = []
+    for retention in (dart.DART_RETAIN_SERIAL, dart.DART_RETAIN_RANKED):
+        cu = torch.zeros(B + 1, dtype=torch.int32, device="cuda")
+        ctx = dart.Dart(B, S, d, P, Kp)
+        oh, oi, op, dbg = ctx.reduce(h, k, vo, nv, P, Kp, debug=True, opts=dart.dart_opts(
+            path=dart.DART_PATH_STAGED, retention=retention, rule=dart.DART_RULE_UNION, cu_seqlens=cu.data_ptr()))
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        ctx.close()
+        n = int(cu[-1])
+        got.append([oh.view(-1, d)[:n].view(torch.int16), oi.view(-1)[:n], op.view(-1)[:n], cu, dbg["keep"], dbg["owner"],
+                    dbg["eps"].view(torch.int32)])
+    assert all(torch.equal(x, y) for x, y in zip(*got))
