@@ -705,6 +705,9 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     const size_t limit = (size_t)ctx->max_smem_optin - F::kStaticSmemReserve - 1024;
     p.n_atoms = ctx->n_atoms, p.n_rg = (n_vis + F::kRows - 1) / F::kRows;
     double best = 0;
+    // two rows to a chunk where they fill it: a task's fixed costs are paid per chunk
+    p.rows_task = 2 * (ctx->desc.d / 8) == F::kChunkUnits ? 2 : 1;
+    p.n_chunk = p.rows_task == 2 ? 1 : (ctx->desc.d / 8 + F::kChunkUnits - 1) / F::kChunkUnits;
     p.nsl = 0;
     for (int nsl = 1; nsl <= F::kMaxSlices && nsl <= p.n_atoms && nsl <= p.n_stream; nsl *= 2) {
         const int na = (p.n_atoms + nsl - 1) / nsl;

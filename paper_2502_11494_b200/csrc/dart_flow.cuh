@@ -19,7 +19,7 @@
 // slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
 //
-// Per CTA (704 threads, one CTA per SM, cooperative launch):
+// Per CTA (736 threads, one CTA per SM, cooperative launch):
 //   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
 //   warps 4-7    second pass: mma.sync.m16n8k16 (16 rows each; P <= 32 leaves the tensor pipe idle whatever the form, and
 //                64-row items do not fill the 128 rows of a tcgen05.mma)
@@ -27,6 +27,7 @@
 //   warps 9-12   combine: count the item, and if it is its row group's last, add up the slices and write the similarities
 //   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
 //   warp 21      watcher: how far the pivots of the batch have got, for the scorers' window
+//   warp 22      feeder: the scorers' rows into their slots
 // Every wait is bounded in time; on expiry the kernel records DART_ERR_TIMEOUT in the status word, lets the copies in flight
 // land and exits normally.
 #pragma once
@@ -56,8 +57,10 @@ constexpr int kProdWarp = 8;
 constexpr int kCombWarp0 = 9, kCombWarps = 4; // (an item is counted 2-3 us after its shares were written: two warps held the others up)
 constexpr int kScoreWarp0 = kCombWarp0 + kCombWarps, kScoreWarps = 8;
 constexpr int kWatchWarp = kScoreWarp0 + kScoreWarps;
-constexpr int kThreads = 32 * (kWatchWarp + 1);
-constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane and chunk of a row
+constexpr int kFeedWarp = kWatchWarp + 1;
+constexpr int kThreads = 32 * (kFeedWarp + 1);
+constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane and chunk
+constexpr int kChunkUnits = 32 * kChunk;
 constexpr uint32_t kChunkBytes = kChunk * 512; // 4 KB: half a row of 4096 columns
 constexpr int kMaxSlots = 6;               // chunks of a row on their way per scorer
 constexpr int kSel = 512;                  // threads of a selector CTA that select
@@ -80,6 +83,7 @@ struct Params {
     int B, S, vis_offset, n_vis, P, d8; // d8: row width in 16-byte units
     int n_atoms, n_rg, nsl, na_max;     // atoms per row; row groups per sample; column slices; atoms of the widest slice
     int n_st, n_slot;                   // ring depth; chunks on their way per scorer
+    int rows_task, n_chunk;             // scoring: rows per task (2: two rows to a chunk); chunks per task
     int n_stream;                       // CTAs that stream; the others select
     int given;                          // the pivots are in pivot_idx already
     int norm_kind, smallest, withhold;
@@ -100,7 +104,7 @@ struct Params {
 
 struct Shared {
     unsigned long long full[kMaxStages], empty[kMaxStages];
-    unsigned long long chunk_full[kScoreWarps][kMaxSlots];
+    unsigned long long chunk_full[kScoreWarps][kMaxSlots], chunk_empty[kScoreWarps][kMaxSlots];
     unsigned long long piv_full[2], piv_empty[2];
     unsigned long long mail_full[kCombWarps][kMail], mail_empty[kCombWarps][kMail];
     uint32_t group_best[32];          // selectors: best keys of groups of 16 threads
@@ -188,105 +192,147 @@ struct Items {
     }
 };
 
-// |x| and x^2 of a chunk of kChunk x 16 bytes
-__device__ __forceinline__ void add_chunk(const uint4 (&v)[kChunk], unsigned long long (&s)[2], unsigned long long (&q)[2])
-{
-#pragma unroll
-    for (int u = 0; u < kChunk; ++u) {
-        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const uint32_t a = w[e] & 0x7fff7fffu; // both signs cleared: neither sum looks at them
-            unsigned long long x;
-            asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(a << 16), "r"(a & 0xffff0000u));
-            add2(s[e & 1], x);
-            fma2(q[e & 1], x);
-        }
+// The scoring tasks of one scorer (warp w of SM c): of the batch's tasks - p.rows_task rows of one sample, one row where rows are
+// wider than half a chunk - every (8 n_stream)-th, sample-major.  The feeder and the scorer walk the same list.
+struct Tasks {
+    int b, t;       // sample, task within it
+    int db, dt, T, B;
+    __device__ Tasks(const Params &p, int w)
+    {
+        T = (p.n_vis + p.rows_task - 1) / p.rows_task, B = p.B;
+        const int first = w * p.n_stream + (int)blockIdx.x, step = p.n_stream * kScoreWarps;
+        b = first / T, t = first - b * T;
+        db = step / T, dt = step - db * T;
     }
-}
+    __device__ __forceinline__ bool valid() const { return b < B; }
+    __device__ __forceinline__ void next()
+    {
+        b += db, t += dt;
+        if (t >= T) t -= T, ++b;
+    }
+};
 
-// The scorers: warp w of SM c takes the batch's rows w * n_stream + c, + 8 * n_stream, ...  Every warp has p.n_slot slots of
-// shared memory for chunks of a row (4 KB each) and refills a slot itself as soon as it has read it.  (Straight into registers,
-// with three chunks' loads written ahead of the sums, the rows arrived at 2.5 TB/s: the loads did not stay ahead.)
-__device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
+// Feeder: lane w keeps scorer w's p.n_slot slots (4 KB chunks of rows) on their way, as far as the window allows.  A warp of its
+// own: a bulk copy takes its thread some 500 cycles to issue (with every scorer refilling its own slots a row of 8 KB took
+// 4000 cycles, and the scorers bound the whole path).
+__device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
 {
-    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) - kScoreWarp0;
-    const int total = p.B * p.n_vis, stride = p.n_stream * kScoreWarps;
-    const int nc = (p.d8 + kChunk * 32 - 1) / (kChunk * 32); // chunks per row
+    const int w = threadIdx.x & 31;
     unsigned long long policy;
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
-    slot0 += (uint32_t)(w * p.n_slot) * kChunkBytes;
-    int r = w * p.n_stream + (int)blockIdx.x, c = 0; // the chunk that is added up next
-    int rq = r, cq = 0;                               // the chunk that is requested next
-    int n_way = 0, in = 0, out = 0;                   // chunks on their way; the slot requested next, read next
-    uint32_t phase = 0;
-    auto allowed = [&](int row) { return row - sh.pos < p.window; };
-    auto wait_allowed = [&](int row) {
-        const long long t0 = clock64();
-        for (uint32_t it = 0;; ++it) {
-            if (allowed(row)) return true;
-            __nanosleep(40);
-            if ((it & 15u) == 15u) {
-                if (ctl.aborted()) return false;
-                if ((unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
-                    if (lane == 0) ctl.give_up(kWaitWindow, row);
-                    return false;
+    const int nc = p.n_chunk;
+    Tasks it(p, w < kScoreWarps ? w : 0);
+    bool more = w < kScoreWarps && it.valid();
+    int c = 0, in = 0;
+    uint32_t phase = 1;
+    long long issued = 0, since = clock64();
+    for (uint32_t spin = 0; __any_sync(0xffffffffu, more);) {
+        bool go = false;
+        if (more) {
+            const int row = it.b * p.n_vis + it.t * p.rows_task;
+            go = (c > 0 || row - sh.pos < p.window) && sweep::mbar_test(smem_u32(&sh.chunk_empty[w][in]), phase);
+            if (go) {
+                const int j = it.t * p.rows_task, rows = min(p.rows_task, p.n_vis - j);
+                const int from = c * kChunkUnits, n = p.rows_task > 1 ? rows * p.d8 : min(kChunkUnits, p.d8 - from);
+                const uint32_t bar = smem_u32(&sh.chunk_full[w][in]);
+                mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
+                sweep::bulk_load(slot0 + (uint32_t)(w * p.n_slot + in) * kChunkBytes,
+                                 p.keys + ((size_t)it.b * p.S + p.vis_offset + j) * (size_t)p.d8 + from, (uint32_t)n * 16u, bar, policy);
+                ++issued;
+                if (++in == p.n_slot) in = 0, phase ^= 1u;
+                if (++c == nc) {
+                    c = 0;
+                    it.next();
+                    more = it.valid();
                 }
             }
         }
-    };
-    // Asks for chunks while there are free slots and their rows are within the window.  (It must not wait for the window: the
-    // rows on their way may be what moves it.)
-    auto refill = [&]() {
-        while (n_way < p.n_slot && rq < total && (cq > 0 || __all_sync(0xffffffffu, allowed(rq)))) {
-            if (lane == 0) {
-                const int b = rq / p.n_vis, j = rq - b * p.n_vis, n = min(kChunk * 32, p.d8 - cq * kChunk * 32);
-                const uint4 *src = p.keys + ((size_t)b * p.S + p.vis_offset + j) * (size_t)p.d8 + cq * kChunk * 32;
-                const uint32_t bar = smem_u32(&sh.chunk_full[w][in]);
-                mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
-                sweep::bulk_load(slot0 + (uint32_t)in * kChunkBytes, src, (uint32_t)n * 16u, bar, policy);
-            }
-            ++n_way;
-            if (++in == p.n_slot) in = 0;
-            if (++cq == nc) cq = 0, rq += stride;
-        }
-    };
-    unsigned long long s[2] = {0ull, 0ull}, q[2] = {0ull, 0ull};
-    bool ok = true;
-    while (r < total) {
-        refill();
-        if (n_way == 0) {
-            ok = __all_sync(0xffffffffu, wait_allowed(rq));
-            if (!ok) break;
+        if (__any_sync(0xffffffffu, go)) {
+            since = clock64();
             continue;
         }
-        ok = ctl.wait_bar(smem_u32(&sh.chunk_full[w][out]), phase, kWaitChunk, r);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        const int n = p.d8 - c * kChunk * 32;
-        uint4 v[kChunk];
-#pragma unroll
-        for (int u = 0; u < kChunk; ++u)
-            v[u] = u * 32 + lane < n ? sweep::lds128(slot0 + (uint32_t)out * kChunkBytes + (uint32_t)(u * 32 + lane) * 16u) : make_uint4(0, 0, 0, 0);
-        add_chunk(v, s, q);
-        __syncwarp(); // the slot has been read
-        --n_way;
-        if (++out == p.n_slot) out = 0, phase ^= 1u;
-        if (++c == nc) {
-            const float l1 = warp_sum(sum2(s[0]) + sum2(s[1])), ssq = warp_sum(sum2(q[0]) + sum2(q[1]));
-            if (lane == 0 && !(p.withhold && r == 0)) {
-                st_rec(p.rec + r, ((unsigned long long)__float_as_uint(ssq) << 32) | __float_as_uint(l1));
-                if (p.l1) p.l1[r] = l1, p.ssq[r] = ssq;
+        __nanosleep(20);
+        if ((++spin & 31u) == 0u) {
+            bool dead = ctl.aborted();
+            if (!dead && (unsigned long long)(clock64() - since) > ctl.limit_cycles) {
+                if (w == 0) ctl.give_up(kWaitWindow, it.b);
+                dead = true;
             }
-            s[0] = s[1] = q[0] = q[1] = 0ull;
-            c = 0, r += stride;
+            if (__any_sync(0xffffffffu, dead)) break;
         }
     }
-    if (!ok && lane == 0) // let the copies on their way land before the CTA may exit
-        for (; n_way > 0; --n_way) {
-            ctl.wait_landed(smem_u32(&sh.chunk_full[w][out]), phase);
+    // the CTA must not exit while a copy is on its way, whatever became of the scorers
+    __syncwarp();
+    for (long long i = issued > p.n_slot ? issued - p.n_slot : 0; i < issued; ++i)
+        ctl.wait_landed(smem_u32(&sh.chunk_full[w][i % p.n_slot]), (uint32_t)((i / p.n_slot) & 1));
+}
+
+// The scorers.  A lane adds up the two halves of a chunk apart: they are two rows' (rows_task = 2) or the same row's.
+__device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
+{
+    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) - kScoreWarp0;
+    slot0 += (uint32_t)(w * p.n_slot) * kChunkBytes + (uint32_t)lane * 16u;
+    int out = 0;
+    uint32_t phase = 0;
+    for (Tasks it(p, w); it.valid(); it.next()) {
+        unsigned long long s[2] = {0ull, 0ull}, q[2] = {0ull, 0ull}; // |x| and x^2, by half of the chunk
+        const int j = it.t * p.rows_task, rows = min(p.rows_task, p.n_vis - j);
+        int left = rows * p.d8 - lane; // 16-byte pieces from this lane's first on
+        for (int c = 0; c < p.n_chunk; ++c, left -= kChunkUnits) {
+            const bool ok = ctl.wait_bar(smem_u32(&sh.chunk_full[w][out]), phase, kWaitChunk, it.b);
+            if (!__all_sync(0xffffffffu, ok)) return;
+            uint4 v[kChunk];
+#pragma unroll
+            for (int u = 0; u < kChunk; ++u) {
+                v[u] = sweep::lds128(slot0 + (uint32_t)out * kChunkBytes + (uint32_t)u * 512u);
+                if (u * 32 >= left) v[u] = make_uint4(0, 0, 0, 0); // (what a slot holds beyond the row is left from another one)
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh.chunk_empty[w][out])); // (the values are in registers)
             if (++out == p.n_slot) out = 0, phase ^= 1u;
+#pragma unroll
+            for (int u = 0; u < kChunk; ++u) {
+                const uint32_t x4[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t a = x4[e] & 0x7fff7fffu; // both signs cleared: neither sum looks at them
+                    unsigned long long x;
+                    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(a << 16), "r"(a & 0xffff0000u));
+                    add2(s[u / (kChunk / 2)], x);
+                    fma2(q[u / (kChunk / 2)], x);
+                }
+            }
         }
+        float s0 = sum2(s[0]), q0 = sum2(q[0]), s1 = sum2(s[1]), q1 = sum2(q[1]);
+        const size_t r = (size_t)it.b * p.n_vis + j;
+        float l1, ssq;
+        int row = 0;
+        if (p.rows_task == 1) {
+            // two sums over the warp: the halves of the warp exchange one each, then every half adds up its own
+            s0 += s1, q0 += q1;
+            float x = lane < 16 ? s0 : q0;
+            x += __shfl_xor_sync(0xffffffffu, lane < 16 ? q0 : s0, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            l1 = x, ssq = __shfl_xor_sync(0xffffffffu, x, 16);
+        } else {
+            // four sums: rows apart by the halves of the warp, then |x| and x^2 by quarters
+            const bool up = lane >= 16, odd = (lane & 8) != 0;
+            float a = up ? s1 : s0, b = up ? q1 : q0;
+            a += __shfl_xor_sync(0xffffffffu, up ? s0 : s1, 16);
+            b += __shfl_xor_sync(0xffffffffu, up ? q0 : q1, 16);
+            float x = odd ? b : a;
+            x += __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            l1 = x, ssq = __shfl_xor_sync(0xffffffffu, x, 8);
+            row = lane >> 4;
+        }
+        if ((lane & 15) == 0 && (lane == 0 || p.rows_task == 2) && row < rows && !(p.withhold && r + row == 0)) {
+            st_rec(p.rec + r + row, ((unsigned long long)__float_as_uint(ssq) << 32) | __float_as_uint(l1));
+            if (p.l1) p.l1[r + row] = l1, p.ssq[r + row] = ssq;
+        }
+    }
 }
 
 // The selectors (CTAs that do nothing else): sample k, k + n_selectors, ... of the batch each.  512 threads read the sample's
@@ -529,7 +575,7 @@ __device__ __forceinline__ void produce(const Params &p, const Ctl &ctl, Shared 
             ++issued;
         }
     }
-    if ((!ok || ctl.aborted()) && lane == 0) // let the copies already issued land before the CTA may exit
+    if (lane == 0) // the CTA must not exit while a copy is on its way, whatever became of the multipliers
         for (long long i = issued > p.n_st ? issued - p.n_st : 0; i < issued; ++i)
             ctl.wait_landed(smem_u32(&sh.full[i % p.n_st]), (uint32_t)((i / p.n_st) & 1));
 }
@@ -641,7 +687,7 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
             mbar_init(smem_u32(&sh.empty[s]), kMulWarps);
         }
         for (int w = 0; w < kScoreWarps; ++w)
-            for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&sh.chunk_full[w][s]), 1);
+            for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&sh.chunk_full[w][s]), 1), mbar_init(smem_u32(&sh.chunk_empty[w][s]), 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&sh.piv_full[s]), kPivWarps * 32);
             mbar_init(smem_u32(&sh.piv_empty[s]), kMulWarps);
@@ -658,6 +704,8 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
     __syncthreads();
     if ((int)blockIdx.x >= p.n_stream) {
         if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, skey, list);
+    } else if (warp == kFeedWarp) {
+        feed(p, ctl, sh, slot0);
     } else if (warp == kWatchWarp) {
         watch(p, ctl, sh);
     } else if (warp >= kScoreWarp0) {
