@@ -347,27 +347,37 @@ __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, S
         bool dead = false;
         uint32_t best = 0; // larger = better
         for (int j0 = t; j0 < p.n_vis && !dead; j0 += kSel * kPoll) {
-            uint32_t v[kPoll];
-#pragma unroll
-            for (int u = 0; u < kPoll; ++u) v[u] = j0 + u * kSel < p.n_vis ? ld_word(rec + 2 * (j0 + u * kSel)) : 0u;
+            // all words that are still missing are asked for together (one after the other, a thread that had started early
+            // paid a round trip for each of its six)
+            uint32_t v[kPoll], miss = 0;
 #pragma unroll
             for (int u = 0; u < kPoll; ++u) {
-                const int j = j0 + u * kSel;
-                for (uint32_t spin = 0; v[u] == kNoWord && !dead; ++spin) { // not published yet
-                    __nanosleep(32);
-                    v[u] = ld_word(rec + 2 * j);
-                    if ((spin & 63u) == 63u) {
-                        dead = ctl.aborted();
-                        if (!dead && (unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
-                            ctl.give_up(kWaitRec, b);
-                            dead = true;
-                        }
+                v[u] = 0;
+                if (j0 + u * kSel < p.n_vis) miss |= 1u << u;
+            }
+            const uint32_t mine = miss;
+            for (uint32_t spin = 1; miss && !dead; ++spin) {
+#pragma unroll
+                for (int u = 0; u < kPoll; ++u)
+                    if ((miss >> u) & 1u) v[u] = ld_word(rec + 2 * (j0 + u * kSel));
+#pragma unroll
+                for (int u = 0; u < kPoll; ++u)
+                    if (v[u] != kNoWord) miss &= ~(1u << u);
+                if (miss) __nanosleep(32);
+                if ((spin & 63u) == 0u) {
+                    dead = ctl.aborted();
+                    if (!dead && (unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                        ctl.give_up(kWaitRec, b);
+                        dead = true;
                     }
                 }
+            }
+#pragma unroll
+            for (int u = 0; u < kPoll; ++u) {
                 uint32_t k = order_key(__uint_as_float(v[u]));
                 if (p.smallest) k = ~k;
-                if (j < p.n_vis) {
-                    skey[j] = k;
+                if ((mine >> u) & 1u) {
+                    skey[j0 + u * kSel] = k;
                     best = max(best, k);
                 }
             }
@@ -479,38 +489,54 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
         }
         if (p.given && w == 0 && lane == 0) sh.pos = it.b * p.n_vis + it.rg * kRows;
         const uint32_t piv = piv0 + (uint32_t)((seq & 1) * 8 * NT) * p.pitch + b_lane;
-        float acc[NT][2][4];
+        constexpr int kChains = NT == 1 ? 4 : 2; // independent sums per pivot tile
+        float acc[NT][kChains][4];
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int h = 0; h < kChains; ++h)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[n][h][e] = 0.f;
         for (int a = 0; a < it.na; a += kAps) {
             const bool ok = ctl.wait_bar(smem_u32(&sh.full[ring.stage]), ring.phase, kWaitStage, it.b);
             if (!__all_sync(0xffffffffu, ok)) return;
-            // one atom: all its fragments are asked for before the first is multiplied
-            auto atom = [&](int h) {
-                const uint32_t tile = ring0 + (uint32_t)ring.stage * kStageBytes + (uint32_t)h * kAtomBytes + a_row;
-                const uint32_t pb = piv + (uint32_t)(a + h) * 128u;
-                uint32_t af[4][4];
+            // All fragments of the stage (of an atom, with more pivots) are asked for before the first is multiplied, and the
+            // stage is handed back before that too.
+            const uint32_t tile0 = ring0 + (uint32_t)ring.stage * kStageBytes + a_row, pb0 = piv + (uint32_t)a * 128u;
+            const bool two = a + 1 < it.na;
+            constexpr int kTogether = NT == 1 ? 2 : 1; // atoms
 #pragma unroll
-                for (int u = 0; u < 4; ++u) ldmatrix4(tile + ((((uint32_t)(2 * u) + (uint32_t)(lane >> 4)) ^ a_sw) << 4), af[u]);
+            for (int h0 = 0; h0 < kAps; h0 += kTogether) {
+                uint32_t af[kTogether][4][4], bf[kTogether][NT][2][4];
 #pragma unroll
-                for (int n = 0; n < NT; ++n) {
-                    uint32_t b0[4], b1[4];
-                    ldmatrix4(pb + (uint32_t)n * 8u * p.pitch, b0);
-                    ldmatrix4(pb + (uint32_t)n * 8u * p.pitch + 64u, b1);
-                    mma_bf16(acc[n][0], af[0], b0[0], b0[1]);
-                    mma_bf16(acc[n][1], af[1], b0[2], b0[3]);
-                    mma_bf16(acc[n][0], af[2], b1[0], b1[1]);
-                    mma_bf16(acc[n][1], af[3], b1[2], b1[3]);
+                for (int h = 0; h < kTogether; ++h) {
+                    // (an atom that is not there: the first one again, its products are left out)
+                    const uint32_t tile = tile0 + (two ? (uint32_t)(h0 + h) * kAtomBytes : 0u), pb = pb0 + (two ? (uint32_t)(h0 + h) * 128u : 0u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) ldmatrix4(tile + ((((uint32_t)(2 * u) + (uint32_t)(lane >> 4)) ^ a_sw) << 4), af[h][u]);
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) {
+                        ldmatrix4(pb + (uint32_t)n * 8u * p.pitch, bf[h][n][0]);
+                        ldmatrix4(pb + (uint32_t)n * 8u * p.pitch + 64u, bf[h][n][1]);
+                    }
                 }
-            };
-            atom(0);
-            if (a + 1 < it.na) atom(1);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh.empty[ring.stage]));
+                if (h0 + kTogether == kAps) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&sh.empty[ring.stage]));
+                }
+#pragma unroll
+                for (int h = 0; h < kTogether; ++h) {
+                    if (h0 + h > 0 && !two) break;
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) {
+                        float (&c0)[4] = acc[n][kChains > 2 ? 2 * h : 0], (&c1)[4] = acc[n][kChains > 2 ? 2 * h + 1 : 1];
+                        mma_bf16(c0, af[h][0], bf[h][n][0][0], bf[h][n][0][1]);
+                        mma_bf16(c1, af[h][1], bf[h][n][0][2], bf[h][n][0][3]);
+                        mma_bf16(c0, af[h][2], bf[h][n][1][0], bf[h][n][1][1]);
+                        mma_bf16(c1, af[h][3], bf[h][n][1][2], bf[h][n][1][3]);
+                    }
+                }
+            }
             ring.advance();
         }
         // the slice's share of the dot products: 8 consecutive rows of a pivot per 32 bytes
@@ -520,8 +546,10 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 float *o = dst + (size_t)(8 * n + 2 * (lane & 3) + e) * kRows;
-                __stcg(o, acc[n][0][e] + acc[n][1][e]);
-                __stcg(o + 8, acc[n][0][2 + e] + acc[n][1][2 + e]);
+                float v0 = acc[n][0][e] + acc[n][1][e], v1 = acc[n][0][2 + e] + acc[n][1][2 + e];
+                if (kChains > 2) v0 += acc[n][kChains - 2][e] + acc[n][kChains - 1][e], v1 += acc[n][kChains - 2][2 + e] + acc[n][kChains - 1][2 + e];
+                __stcg(o, v0);
+                __stcg(o + 8, v1);
             }
         const int c = k % kCombWarps, slot = k / kCombWarps % kMail;
         const bool ok = ctl.wait_bar(smem_u32(&sh.mail_empty[c][slot]), ((uint32_t)(k / kCombWarps / kMail) & 1u) ^ 1u, kWaitMailFree, it.b);
