@@ -554,7 +554,8 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
         const int c = k % kCombWarps, slot = k / kCombWarps % kMail;
         const bool ok = ctl.wait_bar(smem_u32(&sh.mail_empty[c][slot]), ((uint32_t)(k / kCombWarps / kMail) & 1u) ^ 1u, kWaitMailFree, it.b);
         if (!__all_sync(0xffffffffu, ok)) return;
-        if (lane == 0) mbar_arrive(smem_u32(&sh.mail_full[c][slot])); // release: the warp's stores are ordered before it
+        __syncwarp(); // the lanes' stores are ordered before lane 0's release
+        if (lane == 0) mbar_arrive(smem_u32(&sh.mail_full[c][slot]));
     }
     if (p.given && w == 0 && lane == 0) sh.pos = 0x3fffffff; // nothing holds the scorers back any more
 }

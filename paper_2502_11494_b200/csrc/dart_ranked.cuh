@@ -77,7 +77,7 @@ struct RankShared {
     float red_lo[kRankMaxThreads / 32], red_hi[kRankMaxThreads / 32], red_sum[kRankMaxThreads / 32];
     uint32_t scan[kRankMaxThreads / 32];
     int32_t piv[kRankMaxP];
-    uint32_t n_pivots, last_bin, n_band, biggest, n_list, last;
+    uint32_t n_pivots, last_bin, n_band, biggest, n_list, n_exact, last;
 };
 
 constexpr int kRankStaticSmem = 8192;
@@ -222,11 +222,12 @@ __device__ __forceinline__ void rank_row(const RankParams &p, const float *__res
         key = order_key(row_s[j]);
         return true;
     };
-    if (t == 0) sh.n_list = 0;
+    if (t == 0) sh.n_exact = 0; // (not n_list: other threads may still be reading it; the selection below synchronises)
     uint32_t thr, need_eq, cnt_eq;
     block_select_threshold(CtaGroup(), keyfn, n, (uint32_t)C, sh.sel, thr, need_eq, cnt_eq);
     block_select_apply(CtaGroup(), keyfn, n, thr, need_eq, cnt_eq, sh.sel, [&](int j, uint32_t key) {
-        list[atomicAdd(&sh.n_list, 1u)] = ((unsigned long long)key << 32) | (uint32_t)j;
+        const uint32_t slot = atomicAdd(&sh.n_exact, 1u);
+        if (slot < (uint32_t)C) list[slot] = ((unsigned long long)key << 32) | (uint32_t)j;
     });
     rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (uint16_t)x; });
 }
@@ -290,7 +291,7 @@ __device__ __forceinline__ int take_turn(const uint16_t *L, int M, int want, uin
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             j[k] = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
-            if (at + k >= M) j[k] = none;
+            j[k] = at + k >= M ? none : min(j[k], none);
         }
         uint32_t taken[8];
 #pragma unroll
