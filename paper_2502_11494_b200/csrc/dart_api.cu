@@ -176,6 +176,20 @@ struct Prof {
     }
 };
 
+// Launch behind the kernel before it on the stream, which may still be running (see wait_for_previous): every kernel that is
+// launched this way waits before it reads or writes anything that another one touches.
+template <typename... KArgs, typename... Args>
+void launch_next(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid, cfg.blockDim = dim3(threads), cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    cfg.attrs = &attr, cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...); // (an error is found by the call's cudaGetLastError)
+}
+
 bool overlaps(const void *a, size_t na, const void *b, size_t nb)
 {
     if (!a || !b) return false;
@@ -263,12 +277,11 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
         rp.len_out = ctx->len, rp.status = ctx->status;
         Prof p(ctx, st, SLOT_RETAIN);
-        rank_kernel<<<dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st>>>(rp);
+        launch_next(rank_kernel, dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
     };
     if (o.rule == DART_RULE_GLOBAL) { // one threshold for all pivots: a single selection per sample
         Prof p(ctx, st, SLOT_RETAIN);
-        retain_global_kernel<<<B, kSelectThreads, retain_global_smem_bytes(n_vis), st>>>(
-            ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out,
+        launch_next(retain_global_kernel, dim3(B), kSelectThreads, retain_global_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out,
             ctx->status);
         return;
     }
@@ -277,11 +290,10 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
             launch_ranked();
         } else {
             Prof p(ctx, st, SLOT_RETAIN);
-            retain_union_kernel<<<B, kSelectThreads, retain_union_smem_bytes(n_vis), st>>>(
-                ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, owner_out, eps_out, ctx->len, ctx->status);
+            launch_next(retain_union_kernel, dim3(B), kSelectThreads, retain_union_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, owner_out, eps_out, ctx->len, ctx->status);
         }
         Prof p(ctx, st, SLOT_RETAIN);
-        pack_varlen_kernel<<<B, kWalkThreads, retain_union_smem_bytes(n_vis), st>>>(ctx->keep, ctx->len, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
+        launch_next(pack_varlen_kernel, dim3(B), kWalkThreads, retain_union_smem_bytes(n_vis), st, ctx->keep, ctx->len, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
                                                                                     out_idx, out_pos, ctx->status);
         return;
     }
@@ -324,12 +336,10 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     if (bands) {
         {
             Prof p(ctx, st, SLOT_RETAIN);
-            band_kernel<<<dim3((unsigned)P, (unsigned)B), 32, band_smem_bytes(n_vis, band_cap), st>>>(
-                ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, band_cap, ctx->band, ctx->band_n, ctx->status);
+            launch_next(band_kernel, dim3((unsigned)P, (unsigned)B), 32, band_smem_bytes(n_vis, band_cap), st, ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, band_cap, ctx->band, ctx->band_n, ctx->status);
         }
         Prof p(ctx, st, SLOT_RETAIN);
-        retain_pick_kernel<<<B, kPickThreads, pick_smem_bytes(n_vis, P), st>>>(
-            ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out,
+        launch_next(retain_pick_kernel, dim3(B), kPickThreads, pick_smem_bytes(n_vis, P), st, ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out,
             owner_out, eps_out, ctx->status);
         return;
     }
@@ -358,7 +368,7 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
 }
 
 // Step 5b.  With independent pivots the rows are packed at the samples' offsets (cu_seqlens) instead of B equal blocks.
-void launch_gather(dart_ctx *ctx, int B, const void *hidden, int n_vis, int n_keep, const int32_t *out_idx, void *out_hidden,
+void launch_gather(dart_ctx *ctx, int B, const void *hidden, int vis_offset, int n_vis, int n_keep, const int32_t *out_idx, void *out_hidden,
                    const dart_opts &o, cudaStream_t st, bool flow = false)
 {
     using namespace dart;
@@ -371,11 +381,11 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int n_vis, int n_ke
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
     if (o.rule == DART_RULE_UNION)
-        gather_varlen_kernel<<<grid, kGatherWarps * 32, 0, st>>>((const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
+        launch_next(gather_varlen_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
                                                                 ctx->status, (uint4 *)out_hidden, fs);
     else
-        gather_kernel<<<grid, kGatherWarps * 32, 0, st>>>((const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
-                                                         (uint4 *)out_hidden, fs);
+        launch_next(gather_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
+                                                         (uint4 *)out_hidden, fs, vis_offset, n_keep);
 }
 
 // Step 2 with the caller's pivots: checked and copied into the workspace (with keys: and the text pivots' sums of squares).
@@ -384,8 +394,8 @@ void launch_pivots_given(dart_ctx *ctx, int B, int vis_offset, int n_vis, int P,
 {
     Prof p(ctx, st, SLOT_PIVOT);
     const int lo = o.text_pivots ? -vis_offset : 0, hi = o.text_pivots ? ctx->S - vis_offset : n_vis;
-    dart::pivots_given_kernel<<<B, 256, (size_t)((hi - lo + 31) / 32) * 4, st>>>(o.pivots_in, lo, hi, P, ctx->pivot_idx, ctx->status,
-                                                                               o.text_pivots ? keys : nullptr, ctx->S, ctx->desc.d / 8, vis_offset,
+    launch_next(dart::pivots_given_kernel, dim3(B), 256, (size_t)((hi - lo + 31) / 32) * 4, st, o.pivots_in, lo, hi, P, ctx->pivot_idx, ctx->status,
+                o.text_pivots ? keys : nullptr, ctx->S, ctx->desc.d / 8, vis_offset,
                                                                                n_vis, text_ssq);
 }
 
@@ -408,7 +418,7 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
         Prof p(ctx, st, SLOT_PIVOT);
         int P_pad = next_pow2(P);
         const bool cached = n_vis <= kPivotCacheMax;
-        pivot_kernel<<<B, kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st>>>(o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P,
+        launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st, o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P,
                                                                                        P_pad, o.pivot_smallest, cached, ctx->pivot_idx);
     }
     {
@@ -421,7 +431,7 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -622,7 +632,7 @@ int launch_fused(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, 
             sim_sum_kernel<float><<<grid, kSimSumThreads, 0, st>>>(ctx->sim_share, items, p.n_kc, ctx->sim);
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -677,13 +687,12 @@ int launch_onepass_kernel(dart_ctx *ctx, int B, const void *src, bool scores_els
     if (p.compact) { // the sample's pivot rows side by side, so that a pivot tile is one box
         Prof pc(ctx, st, SLOT_PIVOT);
         const long long prow = (long long)B * p.N;
-        pivot_rows_kernel<<<(unsigned)((prow + kPivotRowWarps - 1) / kPivotRowWarps), kPivotRowWarps * 32, 0, st>>>(
-            (const uint4 *)src, ctx->pivot_idx, S, ctx->desc.d / 8, vis_offset, n_vis, P, p.N, prow, (uint4 *)ctx->piv_rows);
+        launch_next(pivot_rows_kernel, dim3((unsigned)((prow + kPivotRowWarps - 1) / kPivotRowWarps)), kPivotRowWarps * 32, 0, st, (const uint4 *)src, ctx->pivot_idx, S, ctx->desc.d / 8, vis_offset, n_vis, P, p.N, prow, (uint4 *)ctx->piv_rows);
     }
     Prof pr(ctx, st, SLOT_ONEPASS);
     const long long tasks = (long long)B * ((p.n_sel + p.tg - 1) / p.tg);
     const unsigned grid = (unsigned)(tasks < ctx->sm_count ? tasks : ctx->sm_count); // no CTA waits for another
-    onepass::onepass_kernel<<<grid, onepass::kThreads, onepass::smem_bytes(p.N, p.aps, p.n_st, p.tg), st>>>(tm_tile, tm_keys, tm_row, tm_piv, tm_pair, p);
+    launch_next(onepass::onepass_kernel, dim3(grid), onepass::kThreads, onepass::smem_bytes(p.N, p.aps, p.n_st, p.tg), st, tm_tile, tm_keys, tm_row, tm_piv, tm_pair, p);
     return DART_OK;
 }
 
@@ -788,7 +797,7 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3(F::kThreads), args, smem, st));
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st, true);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st, true);
     DART_CUDA(ctx, cudaGetLastError());
     ctx->flow_dirty = false;
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -834,7 +843,7 @@ int launch_resident(dart_ctx *ctx, int B, const void *hidden, const void *keys_i
         if (rc != DART_OK) return rc;
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -877,7 +886,7 @@ int launch_pair(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
                                                    Q::smem_bytes(P, p.row_bytes, (int)grid, p.n1, p.n2, p.n3), st));
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -891,7 +900,7 @@ int launch_onepass(dart_ctx *ctx, int B, const void *hidden, const void *keys_in
     int rc = launch_onepass_kernel(ctx, B, keys_in ? keys_in : hidden, false, vis_offset, n_vis, P, o, st);
     if (rc != DART_OK) return rc;
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -920,7 +929,7 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
         Prof p(ctx, st, SLOT_PIVOT);
         const int P_pad = next_pow2(P);
         const bool cached = n_vis <= kPivotCacheMax;
-        pivot_kernel<<<B, kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st>>>(o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P, P_pad,
+        launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st, o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P, P_pad,
                                                                                        o.pivot_smallest, cached, ctx->pivot_idx);
     }
     if (tensor_cores) {
@@ -941,7 +950,7 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
-    launch_gather(ctx, B, hidden, n_vis, n_keep, out_idx, out_hidden, o, st);
+    launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
 }
@@ -1452,7 +1461,7 @@ int dart_pivots_static(const void *keys, int B, int S, int d, int vis_offset, in
     score_kernel<<<(unsigned)((rows + kScoreWarps - 1) / kScoreWarps), kScoreWarps * 32, 0, st>>>(
         (const uint4 *)keys, S, d / 8, vis_offset, n_vis, rows, l1, ssq);
     const int P_pad = next_pow2(n_pivot);
-    pivot_kernel<<<B, kSelectThreads, pivot_smem_bytes(n_vis, P_pad, false), st>>>(l1, n_vis, n_pivot, P_pad, 0, 0, pivot_idx);
+    launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, false), st, l1, n_vis, n_pivot, P_pad, 0, 0, pivot_idx);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DART_OK : e == cudaErrorMemoryAllocation ? DART_ERR_NOMEM : DART_ERR_CUDA;
 }
@@ -1469,8 +1478,8 @@ int dart_gather_rows(const void *src, const int32_t *idx, int B, int S, int S_ou
     using namespace dart;
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
-    gather_kernel<<<grid, kGatherWarps * 32, 0, (cudaStream_t)stream>>>((const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
-                                                                       nullptr, (uint4 *)out, FlowState{});
+    launch_next(gather_kernel, dim3(grid), kGatherWarps * 32, 0, (cudaStream_t)stream, (const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
+                                                                       nullptr, (uint4 *)out, FlowState{}, 0, S_out);
     return cudaGetLastError() == cudaSuccess ? DART_OK : DART_ERR_CUDA;
 }
 

@@ -25,6 +25,15 @@ __device__ __forceinline__ void st_stream(uint4 *p, uint4 v)
                  : "memory");
 }
 
+// ---- programmatic dependent launch --------------------------------------------------------------
+// A kernel of this library that is launched behind another one may start while that one still runs: it does what depends on
+// nothing, then waits here until the kernel before it (and with it everything before that) has finished and its writes are
+// visible.  Without the launch attribute both do nothing.  (Between two small kernels this saves the 2-3 us that a launch takes
+// to get going.)
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and lets the next one start as soon as every CTA of this one has called it.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- bf16 pairs ----------------------------------------------------------------------------
 // A 32-bit word holds two bf16 values; each widens to fp32 by placing its 16 bits on top.
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }

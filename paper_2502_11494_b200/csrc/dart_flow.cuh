@@ -700,6 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
+    wait_for_previous();
     if (*p.status != 0) return; // an earlier kernel of this call failed (every CTA sees the same word: nobody waits)
     const uint32_t ring0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t slot0 = ring0 + (uint32_t)p.n_st * kStageBytes;
@@ -741,6 +742,9 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
         score_rows(p, ctl, sh, slot0);
     } else if (warp < kPivWarps) {
         take_pivots<NT>(p, ctl, sh, piv0);
+        // The next kernel may start: every SM is at its last items.  (Let go at the beginning, its CTAs crowded on the SMs that
+        // were through first: 8 x 2880 x 4096, 16 pivots 94 -> 97 us.)
+        let_next_start();
     } else if (warp < kMulWarp0 + kMulWarps) {
         multiply<NT>(p, ctl, sh, ring0, piv0);
     } else if (warp == kProdWarp) {

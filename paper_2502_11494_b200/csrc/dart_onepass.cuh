@@ -151,6 +151,8 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    wait_for_previous();
+    let_next_start();
     const uint32_t tmem_base = sh.tmem_base;
     const uint32_t per_sample = (uint32_t)(p.n_sel + p.tg - 1) / (uint32_t)p.tg;
     const uint32_t total = (uint32_t)p.B * per_sample; // tasks: (sample, first row tile), sample-major

@@ -334,7 +334,6 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
 {
     extern __shared__ __align__(16) uint8_t rank_smem[];
     __shared__ RankShared sh;
-    if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
     const int t = threadIdx.x, T = blockDim.x, warp = t >> 5, n = p.n_vis;
     const int i = blockIdx.x, b = blockIdx.y;
     const int32_t *piv = sh.piv;
@@ -342,13 +341,16 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     float *row_s = reinterpret_cast<float *>(rank_smem);
     uint32_t *hist = reinterpret_cast<uint32_t *>(rank_smem + ((size_t)n * 4 + 15) / 16 * 16);
     unsigned long long *list = reinterpret_cast<unsigned long long *>(hist + p.bins);
+    for (int k = t; k < p.bins / 4; k += T) reinterpret_cast<uint4 *>(hist)[k] = make_uint4(0, 0, 0, 0);
+    if (t == 0) sh.n_pivots = 0, sh.biggest = 0;
+    wait_for_previous();
+    let_next_start();
+    if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
     if ((n & 3) == 0) // rows start on 16-byte boundaries
         for (int j = t; j < n / 4; j += T) copy_async<16>(row_s + 4 * j, row + 4 * j);
     else
         for (int j = t; j < (n + 3) / 4 * 4; j += T) row_s[j] = __ldcs(row + (j < n ? j : 0)); // (filler: a value of the row)
     copy_async_commit();
-    for (int k = t; k < p.bins / 4; k += T) reinterpret_cast<uint4 *>(hist)[k] = make_uint4(0, 0, 0, 0);
-    if (t == 0) sh.n_pivots = 0, sh.biggest = 0;
     __syncthreads();
     uint32_t mine = 0;
     for (int k = t; k < p.P; k += T) {

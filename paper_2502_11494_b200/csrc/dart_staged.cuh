@@ -17,6 +17,8 @@ __global__ void __launch_bounds__(kScoreWarps * 32)
 score_kernel(const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, long long rows_total,
              float *__restrict__ l1, float *__restrict__ ssq)
 {
+    wait_for_previous();
+    let_next_start();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kScoreWarps + (threadIdx.x >> 5);
     if (row >= rows_total) return;
@@ -99,6 +101,8 @@ __global__ void __launch_bounds__(kSelectThreads)
 pivot_kernel(const float *__restrict__ score, int n_vis, int P, int P_pad, int smallest, int cached,
              int32_t *__restrict__ pivot_idx)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ unsigned long long piv_list[]; // [P_pad], then (cached) the sample's keys [n_vis]
     uint32_t *keys = reinterpret_cast<uint32_t *>(piv_list + P_pad);
     __shared__ SelectSmem sel;
@@ -132,6 +136,8 @@ __global__ void __launch_bounds__(kSelectThreads)
 pivot_mixed_kernel(const float *__restrict__ score_vis, const float *__restrict__ score_before, const float *__restrict__ score_after,
                    int S, int vis_offset, int n_vis, int Pv, int Pt, int P_pad, int smallest, int32_t *__restrict__ pivot_idx)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ unsigned long long piv_list[]; // [P_pad]
     __shared__ SelectSmem sel;
     __shared__ uint32_t n_picked;
@@ -172,6 +178,8 @@ __device__ __forceinline__ unsigned long long splitmix64_at(unsigned long long s
 __global__ void __launch_bounds__(kSelectThreads)
 pivot_random_kernel(unsigned long long seed, int b0, int n_vis, int P, int P_pad, int32_t *__restrict__ pivot_idx)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ unsigned long long piv_list[]; // [P_pad]
     __shared__ SelectSmem sel;
     __shared__ uint32_t n_picked;
@@ -199,6 +207,8 @@ __global__ void __launch_bounds__(kSimWarps * 32)
 sim_alu_kernel(const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, int P, int p0,
                const int32_t *__restrict__ pivot_idx, const float *__restrict__ ssq, float *__restrict__ sim)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ uint4 piv_rows[]; // [kSimPivotChunk][d8]
     __shared__ float piv_norm[kSimPivotChunk];
     const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -299,6 +309,8 @@ __global__ void __launch_bounds__(256)
 pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P, int32_t *__restrict__ pivot_idx, int *status,
                     const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, float *__restrict__ text_ssq)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ uint32_t seen[]; // [(hi - lo + 31) / 32]
     const int b = blockIdx.x;
     for (int w = threadIdx.x; w < (hi - lo + 31) / 32; w += blockDim.x) seen[w] = 0;
@@ -348,6 +360,8 @@ __global__ void __launch_bounds__(kPivotRowWarps * 32)
 pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *__restrict__ pivot_idx, int S, int d8, int vis_offset, int n_vis,
                   int P, int N, long long rows_total, uint4 *__restrict__ out)
 {
+    wait_for_previous();
+    let_next_start();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kPivotRowWarps + (threadIdx.x >> 5);
     if (row >= rows_total) return;
@@ -460,6 +474,8 @@ retain_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_i
               uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
               const int *__restrict__ status, int cache_rows)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[]; // [n_vis] flags, then the key cache
     uint32_t *cache = reinterpret_cast<uint32_t *>(keep + ((size_t)n_vis + 15) / 16 * 16); // [cache_rows][n_vis]
     __shared__ SelectSmem sel;
@@ -542,6 +558,8 @@ __global__ void __launch_bounds__(kCandThreads)
 candidates_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, int n_vis, int P, int n_keep,
                   int m_pad, int cand_stride, int32_t *__restrict__ cand, const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t cand_smem[];
     uint32_t *keys = reinterpret_cast<uint32_t *>(cand_smem);                      // [n_vis] order-preserving keys of the row
     uint8_t *is_pivot = cand_smem + ((size_t)n_vis * 4 + 15) / 16 * 16;            // [n_vis]
@@ -606,6 +624,8 @@ retain_walk_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pi
                    int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos, uint8_t *__restrict__ keep_out,
                    int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[]; // [n_vis] flags, then the staged candidate lists
     int32_t *stage = reinterpret_cast<int32_t *>(keep + ((size_t)n_vis + 15) / 16 * 16); // [kWalkStageEntries]
     __shared__ uint32_t warp_tot[kWalkThreads / 32];
@@ -947,6 +967,8 @@ __global__ void __launch_bounds__(32)
 band_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, int n_vis, int P, int n_keep, int stride,
             unsigned long long *__restrict__ band, int32_t *__restrict__ band_n, const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t band_smem[];
     __shared__ BandScratch sc;
     if (*status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
@@ -1150,6 +1172,8 @@ retain_pick_kernel(const int32_t *__restrict__ pivot_idx, const unsigned long lo
                    uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
                    const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[]; // [n_vis] flags, the bands' lengths, two buffers of staged bands
     int32_t *len = reinterpret_cast<int32_t *>(keep + ((size_t)n_vis + 15) / 16 * 16);                                  // [P]
     unsigned long long *stage = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(len) + ((size_t)P * 4 + 15) / 16 * 16); // [2][kPickStageEntries]
@@ -1176,6 +1200,8 @@ retain_fused_kernel(const float *__restrict__ sim, const int32_t *__restrict__ p
                     int P, int n_keep, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos, uint8_t *__restrict__ keep_out,
                     int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *__restrict__ status, int band_warps)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[];
     int32_t *len = reinterpret_cast<int32_t *>(keep + ((size_t)n_vis + 15) / 16 * 16);
     uint8_t *work = reinterpret_cast<uint8_t *>(len) + ((size_t)P * 4 + 15) / 16 * 16;
@@ -1213,6 +1239,8 @@ retain_global_kernel(const float *__restrict__ sim, const int32_t *__restrict__ 
                      uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
                      const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[]; // [n_vis] flags, then the keys
     uint32_t *ukey = reinterpret_cast<uint32_t *>(keep + ((size_t)n_vis + 15) / 16 * 16); // [n_vis]
     __shared__ SelectSmem sel;
@@ -1283,6 +1311,8 @@ retain_union_kernel(const float *__restrict__ sim, const int32_t *__restrict__ p
                     uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
                     int32_t *__restrict__ len_out, const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t flags[]; // [n_vis] 0 free, 1 kept, 2 pivot
     __shared__ SelectSmem sel;
     if (*status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
@@ -1352,6 +1382,8 @@ pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restric
                    int vis_offset, int n_vis, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
                    const int *__restrict__ status)
 {
+    wait_for_previous();
+    let_next_start();
     extern __shared__ __align__(16) uint8_t keep[]; // [n_vis]
     __shared__ uint32_t warp_tot[kWalkThreads / 32];
     if (*status != 0) return;
@@ -1381,6 +1413,8 @@ __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, const int32_t *__restrict__ cu, int B,
                      int S, int d8, long long rows_cap, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs)
 {
+    wait_for_previous();
+    let_next_start();
     fs.put_back();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
@@ -1404,29 +1438,36 @@ gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict
 
 __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, int S, int S_out, int d8,
-              long long rows_total, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs)
+              long long rows_total, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep)
 {
-    fs.put_back();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
-    if (row >= rows_total || (status && *status != 0)) return; // after a failed kernel out_idx is undefined
-    const int b = (int)(row / S_out);
-    const int s = out_idx[row];
-    const uint4 *src = hidden + ((size_t)b * S + s) * (size_t)d8;
-    uint4 *dst = out_hidden + (size_t)row * (size_t)d8;
-    for (int c0 = 0; c0 < d8; c0 += 32 * 8) {
-        uint4 v[8];
+    const int b = (int)(row / S_out), t = (int)(row - (long long)b * S_out);
+    // Text rows stand where they stand whatever the retention decides: they are copied while it still runs.  (It lets this kernel
+    // start once everything before it has finished, and it neither writes the status word nor reads a packed row.)
+    const bool text = t < vis_offset || t >= vis_offset + n_keep;
+    if (!text || row >= rows_total) wait_for_previous();
+    let_next_start();
+    if (row < rows_total && !(status && *status != 0)) { // after a failed kernel out_idx is undefined
+        const int s = !text ? out_idx[row] : t < vis_offset ? t : t + S - S_out;
+        const uint4 *src = hidden + ((size_t)b * S + s) * (size_t)d8;
+        uint4 *dst = out_hidden + (size_t)row * (size_t)d8;
+        for (int c0 = 0; c0 < d8; c0 += 32 * 8) {
+            uint4 v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            int c = c0 + u * 32 + lane;
-            if (c < d8) v[u] = ld_stream(src + c);
-        }
+            for (int u = 0; u < 8; ++u) {
+                int c = c0 + u * 32 + lane;
+                if (c < d8) v[u] = ld_stream(src + c);
+            }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            int c = c0 + u * 32 + lane;
-            if (c < d8) st_stream(dst + c, v[u]);
+            for (int u = 0; u < 8; ++u) {
+                int c = c0 + u * 32 + lane;
+                if (c < d8) st_stream(dst + c, v[u]);
+            }
         }
     }
+    if (text) wait_for_previous();
+    fs.put_back();
 }
 
 // Adds up the column chunks' shares of the similarities (the persistent sweep cuts every row tile into chunks of columns
