@@ -50,6 +50,8 @@ struct Params {
     int compact;                       // pivot tiles come from the compact copy [B][N][d] (tm_piv), not by gather4
     int n_sel;                         // row tiles per sample this launch takes: n_rt, or the streamed tiles of `split`
     TileSplit split;                   // k <= 1: all tiles
+    int norms_known;                   // the rows' sums of squares are in ssq already (a score pass over the same tensor came first, all
+                                       // pivots are vision tokens): no warp adds up norms, and the tiles are read by the tensor cores alone
     int withhold;                      // test hook: the first pivot-norm warp never hands its norms over, so that the bounded waits expire
     unsigned long long wait_ns;
     float *sim;                        // [B][P][n_vis] dup(p_i, x_j)
@@ -128,7 +130,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem_u32(&sh.full[s]), 1);
-            mbar_init(smem_u32(&sh.empty[s]), 1 + kNormWarps + kPivWarps); // the MMAs' commit and every norm warp
+            mbar_init(smem_u32(&sh.empty[s]), p.norms_known ? 1 : 1 + kNormWarps + kPivWarps); // the MMAs' commit and every norm warp
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&sh.tmem_full[a]), 1);
@@ -286,7 +288,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
         Ring ring(p.n_st);
         uint32_t n = 0;
         bool dead = false; // warp-uniform
-        for (uint32_t g = blockIdx.x; !dead && g < total; g += gridDim.x) {
+        for (uint32_t g = blockIdx.x; !p.norms_known && !dead && g < total; g += gridDim.x) {
             int b, rt;
             task(g, b, rt);
             const int rows = tile_rows(rt, 0), rows2 = p.tg > 1 ? tile_rows(rt, 1) : 0;
@@ -333,7 +335,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
         Ring ring(p.n_st);
         uint32_t n = 0;
         bool dead = false; // warp-uniform
-        for (uint32_t g = blockIdx.x; !dead && g < total; g += gridDim.x) {
+        for (uint32_t g = blockIdx.x; !p.norms_known && !dead && g < total; g += gridDim.x) {
             float pq[kMaxN / kPivThreads][2]; // sums of squares only
 #pragma unroll
             for (int k = 0; k < kMaxN / kPivThreads; ++k) pq[k][0] = pq[k][1] = 0.f;
@@ -368,12 +370,30 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
         // ------------------------------------------------------------------ epilogue (warps independent)
         const int quarter = warp & 3;        // TMEM lane quarter this warp may read
         const int row = quarter * 32 + lane; // tile row owned by this thread
+        float piv_norm[kMaxN / 32] = {};     // norms_known: |pivot lane + 32 k| of sample norm_b
+        int norm_b = -1;
         uint32_t n = 0;
         for (uint32_t g = blockIdx.x; g < total; g += gridDim.x) {
             int b, rt;
             task(g, b, rt);
             const uint32_t acc = n & 1u;
-            bool ok = ctl.wait_bar(smem_u32(&sh.norm_full[acc]), (n >> 1) & 1u, kWaitNormFull, g);
+            bool ok = true;
+            float row_ssq[2] = {0.f, 0.f};
+            if (p.norms_known) { // on their way while the task's products are still being summed
+                const float *ssq = p.ssq + (size_t)b * p.n_vis;
+#pragma unroll
+                for (int w = 0; w < 2; ++w)
+                    if (w < p.tg && row < tile_rows(rt, w)) row_ssq[w] = __ldg(ssq + (rt + w) * kTileRows + row);
+                if (b != norm_b) {
+                    norm_b = b;
+#pragma unroll
+                    for (int k = 0; k < kMaxN / 32; ++k)
+                        if (lane + 32 * k < p.P) piv_norm[k] = sqrtf(__ldg(ssq + __ldg(p.pivot_idx + (size_t)b * p.P + lane + 32 * k)));
+                }
+            } else {
+                ok = ctl.wait_bar(smem_u32(&sh.norm_full[acc]), (n >> 1) & 1u, kWaitNormFull, g);
+                if (ok) row_ssq[0] = sh.row_ssq[acc][0][row], row_ssq[1] = sh.row_ssq[acc][1][row];
+            }
             if (ok) ok = ctl.wait_bar(smem_u32(&sh.tmem_full[acc]), (n >> 1) & 1u, kWaitAccumFull1, g);
             if (!__all_sync(0xffffffffu, ok)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -381,19 +401,22 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                 const int rows = tile_rows(rt, w);
                 if (rows == 0) break;
                 const int j = (rt + w) * kTileRows + row;
-                const float nj = sqrtf(sh.row_ssq[acc][w][row]);
+                const float nj = sqrtf(w == 0 ? row_ssq[0] : row_ssq[1]);
                 const uint32_t taddr = tmem_base + acc * (uint32_t)(p.tg * p.N) + (uint32_t)(w * p.N) + ((uint32_t)(quarter * 32) << 16);
                 float *dst = p.sim + (size_t)b * p.P * p.n_vis + j;
-                for (int c0 = 0; c0 < p.P; c0 += 8) {
-                    float v[8];
-                    tmem_ld8(taddr + (uint32_t)c0, v); // warp-collective: rows outside the tile still take part
-                    if (row < rows) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (c0 + e < p.P) { // dup = dot / (|pivot| |row|); a zero norm gives 0; a warp writes 128 contiguous bytes
-                                const float den = sqrtf(sh.piv_ssq[acc][c0 + e]) * nj;
-                                dst[(size_t)(c0 + e) * p.n_vis] = den > 0.f ? v[e] / den : 0.f;
-                            }
+                for (int k = 0; k < kMaxN / 32; ++k) { // 32 pivots at a time: their norms are one lane each
+                    if (32 * k >= p.P) break;
+                    for (int c0 = 32 * k; c0 < min(p.P, 32 * k + 32); c0 += 8) {
+                        float v[8];
+                        tmem_ld8(taddr + (uint32_t)c0, v); // warp-collective: rows outside the tile still take part
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0; a warp writes 128 contiguous bytes
+                            const float np = p.norms_known ? __shfl_sync(0xffffffffu, piv_norm[k], (c0 + e) & 31)
+                                                           : sqrtf(sh.piv_ssq[acc][min(c0 + e, p.P - 1)]);
+                            const float den = np * nj;
+                            if (row < rows && c0 + e < p.P) dst[(size_t)(c0 + e) * p.n_vis] = den > 0.f ? v[e] / den : 0.f;
+                        }
                     }
                 }
             }
@@ -401,7 +424,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(smem_u32(&sh.tmem_empty[acc]));
-                mbar_arrive(smem_u32(&sh.norm_empty[acc]));
+                if (!p.norms_known) mbar_arrive(smem_u32(&sh.norm_empty[acc]));
             }
             ++n;
         }
