@@ -148,7 +148,7 @@ typedef struct {
     int32_t sweep_lag;     /* 0: default; > 0: fused path, extra tasks between a row's two sweeps (tuning) */
     int32_t test_withhold_pivots; /* testing only: nonzero withholds one hand-over inside the kernel that waits (the persistent
                                      sweep never publishes a sample's pivots; the resident sweep's CTAs never count themselves in;
-                                     the one-pass kernel's first pivot-norm warp never hands its norms over; the paired sweeps:
+                                     the one-pass kernel's first norm warp never hands its norms over; the paired sweeps:
                                      1 = the lists are never counted in, 2 = the pivots' norms never reach the epilogue), so that
                                      the bounded waits expire and the call ends with DART_ERR_TIMEOUT in dart_status */
     int32_t retention;     /* DART_RETAIN_*: how step 4 is scheduled (same result either way) */

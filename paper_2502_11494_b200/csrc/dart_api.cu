@@ -45,6 +45,7 @@ struct dart_ctx {
     // workspace (device), indexed with the shapes of the current call
     float *l1, *ssq, *sim, *eps;
     int32_t *pivot_idx, *owner;
+    float *piv_ssq;  // [B_max][P_max] sums of squares of the pivot rows
     void *piv_rows;  // [B_max][P_max rounded to 16][d] bf16: compact copy of the pivot rows (NULL: not available)
     int32_t *len;    // [B_max] packed length of every sample (retention with independent pivots)
     int32_t *cand;   // [B_max][P_max][cand_stride] sorted candidate lists of the two-phase retention (NULL: not available)
@@ -545,7 +546,9 @@ int fused_setup(dart_ctx *ctx)
         }
     }
     // the one-pass kernel for the caller's pivots uses the same tensor maps
-    if (cudaFuncSetAttribute(dart::onepass::onepass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(dart::onepass::onepass_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             ctx->max_smem_optin - dart::onepass::kStaticSmemReserve) != cudaSuccess ||
+        cudaFuncSetAttribute(dart::onepass::onepass_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              ctx->max_smem_optin - dart::onepass::kStaticSmemReserve) != cudaSuccess)
         return DART_ERR_CUDA;
     return DART_OK;
@@ -672,9 +675,9 @@ int launch_onepass_kernel(dart_ctx *ctx, int B, const void *src, bool scores_els
     p.n_st = onepass::ring_depth(p.N, p.aps, ctx->max_smem_optin, p.tg);
     if (p.n_st < 2) return DART_ERR_UNSUPPORTED;
     p.wait_ns = o.wait_limit > 0 ? (unsigned long long)o.wait_limit * 1000ull : 2000000000ull;
-    p.withhold = o.test_withhold_pivots, p.norms_known = norms_known;
+    p.withhold = o.test_withhold_pivots;
     p.sim = ctx->sim, p.l1 = scores_elsewhere ? nullptr : ctx->l1, p.ssq = ctx->ssq, p.pivot_idx = ctx->pivot_idx;
-    p.status = ctx->status;
+    p.piv_ssq = ctx->piv_ssq, p.status = ctx->status;
     CUtensorMap tm_tile, tm_keys, tm_row, tm_piv, tm_pair;
     int rc = encode_2d(ctx, &tm_tile, src, (uint64_t)ctx->desc.d, (uint64_t)B * S, kTileRows);
     if (rc == DART_OK) rc = encode_2d(ctx, &tm_pair, src, (uint64_t)ctx->desc.d, (uint64_t)B * S, 2 * kTileRows);
@@ -684,15 +687,20 @@ int launch_onepass_kernel(dart_ctx *ctx, int B, const void *src, bool scores_els
         rc = p.compact ? encode_2d(ctx, &tm_piv, ctx->piv_rows, (uint64_t)ctx->desc.d, (uint64_t)B * p.N, (uint32_t)p.N)
                        : encode_2d(ctx, &tm_piv, src, (uint64_t)ctx->desc.d, (uint64_t)B * S, 1); // unused
     if (rc != DART_OK) return rc;
-    if (p.compact) { // the sample's pivot rows side by side, so that a pivot tile is one box
+    { // the sample's pivot rows side by side, so that a pivot tile is one box, and their norms
         Prof pc(ctx, st, SLOT_PIVOT);
         const long long prow = (long long)B * p.N;
-        launch_next(pivot_rows_kernel, dim3((unsigned)((prow + kPivotRowWarps - 1) / kPivotRowWarps)), kPivotRowWarps * 32, 0, st, (const uint4 *)src, ctx->pivot_idx, S, ctx->desc.d / 8, vis_offset, n_vis, P, p.N, prow, (uint4 *)ctx->piv_rows);
+        launch_next(pivot_rows_kernel, dim3((unsigned)((prow + kPivotRowWarps - 1) / kPivotRowWarps)), kPivotRowWarps * 32, 0, st, (const uint4 *)src,
+                    ctx->pivot_idx, S, ctx->desc.d / 8, vis_offset, n_vis, P, p.N, prow, (uint4 *)(p.compact ? ctx->piv_rows : nullptr), ctx->piv_ssq);
     }
     Prof pr(ctx, st, SLOT_ONEPASS);
     const long long tasks = (long long)B * ((p.n_sel + p.tg - 1) / p.tg);
     const unsigned grid = (unsigned)(tasks < ctx->sm_count ? tasks : ctx->sm_count); // no CTA waits for another
-    launch_next(onepass::onepass_kernel, dim3(grid), onepass::kThreads, onepass::smem_bytes(p.N, p.aps, p.n_st, p.tg), st, tm_tile, tm_keys, tm_row, tm_piv, tm_pair, p);
+    const size_t smem = onepass::smem_bytes(p.N, p.aps, p.n_st, p.tg);
+    if (norms_known)
+        launch_next(onepass::onepass_kernel<false>, dim3(grid), onepass::kThreadsNormsKnown, smem, st, tm_tile, tm_keys, tm_row, tm_piv, tm_pair, p);
+    else
+        launch_next(onepass::onepass_kernel<true>, dim3(grid), onepass::kThreads, smem, st, tm_tile, tm_keys, tm_row, tm_piv, tm_pair, p);
     return DART_OK;
 }
 
@@ -785,8 +793,8 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
     if (rc == DART_OK && ctx->flow_dirty) rc = flow_reset(ctx, st);
     if (rc != DART_OK) return rc;
     ctx->flow_dirty = true;
-    if (o.text_pivots) p.text_ssq = ctx->eps; // (the retention's thresholds: written after the flow kernel only)
-    if (p.given) launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st, p.keys, ctx->eps);
+    if (o.text_pivots) p.text_ssq = ctx->piv_ssq;
+    if (p.given) launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st, p.keys, ctx->piv_ssq);
     {
         Prof pr(ctx, st, SLOT_FLOW);
         void *args[2] = {&tm, &p};
@@ -897,7 +905,7 @@ int launch_onepass(dart_ctx *ctx, int B, const void *hidden, const void *keys_in
                    const dart_debug *dbg, cudaStream_t st)
 {
     launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
-    int rc = launch_onepass_kernel(ctx, B, keys_in ? keys_in : hidden, false, vis_offset, n_vis, P, o, st);
+    int rc = launch_onepass_kernel(ctx, B, keys_in ? keys_in : hidden, !(dbg && dbg->l1), vis_offset, n_vis, P, o, st); // (L1 scores rank nothing here)
     if (rc != DART_OK) return rc;
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
@@ -933,9 +941,9 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
                                                                                        o.pivot_smallest, cached, ctx->pivot_idx);
     }
     if (tensor_cores) {
-        // the score pass has the rows' sums of squares already, where it read the same tensor and every pivot is one of its rows
+        // the score pass has the rows' sums of squares already, where it read the same tensor
         // (256 x 2880 x 4096, 128 pivots: 1.46 -> 1.09 ms per launch, 32 pivots 1.01 -> 0.98; the test of the norms' hand-over keeps them in the kernel)
-        const bool norms_known = same && !o.text_pivots && !o.test_withhold_pivots;
+        const bool norms_known = same && !o.test_withhold_pivots;
         int rc = launch_onepass_kernel(ctx, B, sim_src, true, vis_offset, n_vis, P, o, st, TileSplit{1, 0}, norms_known);
         if (rc != DART_OK) return rc;
     } else {
@@ -1118,6 +1126,7 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->keep, nv);
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->len, (size_t)desc->B_max);
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->pivot_src, np);
+    if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->piv_ssq, np);
     if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->text_score, 2 * nv);
     if (rc == DART_OK) {
         // candidate lists of the two-phase retention: at most kCandMax entries per pivot; contexts whose maxima

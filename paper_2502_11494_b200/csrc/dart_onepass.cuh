@@ -9,15 +9,16 @@
 // norms and writes dup(p_i, x_j) (Eq. 7).  No CTA depends on another one: tasks (sample, row tile) are
 // dealt out round-robin to a persistent grid of one CTA per SM.
 //
-// Per CTA (384 threads):
+// Per CTA (512 threads; 384 where the norms are known):
 //   warp 0     producer: per 64-column atom one or two 128-row TMA tiles (128-byte swizzle) and the pivot rows - as
 //              ONE box from a compact copy of the sample's pivot rows, or, where the context has no room for that
 //              copy, by tile::gather4 straight from the key tensor (4 rows per op, ~13 ops per us: slower) -
 //              up to four atoms per stage of a ring
 //   warp 1     one thread issues tcgen05.mma; tcgen05.commit releases the stage on the tensor cores' behalf
-//   warps 4-7  norms: thread t owns tile row t and sums its 128 bytes of every atom, in column order whatever
-//              the swizzle did to the chunks, so a row's norm does not depend on where in a tile it was read
-//   warps 2-3  the same for the pivot rows of the stage's pivot tile (thread u: rows u, u + 64, ...)
+//   warps 4-7, 12-15  norms: thread t of a group owns tile row t and sums its 128 bytes of every even (odd) atom, in column
+//              order whatever the swizzle did to the chunks, so a row's norm does not depend on where in a tile it was read.
+//              (One group of warps bounded the kernel: 32 x 2880 x 4096, 8 pivots 155 -> 138 us.)  Behind a score pass over
+//              the same tensor the norms are known and nobody adds them up; the pivots' come from pivot_rows_kernel.
 //   warps 8-11 epilogue: TMEM -> normalised similarities [B][P][n_vis]
 // Every wait is bounded in time; on expiry the kernel records DART_ERR_TIMEOUT in the status word, lets the
 // copies and MMAs in flight finish, frees TMEM and exits normally.  Results are bitwise reproducible.
@@ -29,9 +30,8 @@ namespace onepass {
 
 using namespace sweep; // PTX wrappers, Ctl, Ring, tile constants
 
-constexpr int kThreads = 384;
-constexpr int kNormWarp0 = 4, kNormWarps = 4;
-constexpr int kPivWarp0 = 2, kPivWarps = 2, kPivThreads = kPivWarps * 32;
+constexpr int kThreads = 512, kThreadsNormsKnown = 384; // (warps 2-3 idle; without norms 4-7 too)
+constexpr int kNormWarp0 = 4, kNormWarp1 = 12, kNormWarps = 4; // two groups: even and odd atoms
 constexpr int kEpi0 = 8;          // kEpi0 % 4 == 0: warp w reads TMEM lanes 32 (w % 4) ...
 constexpr int kStages = 10;       // at most
 constexpr int kMaxAtomsPerStage = 4; // a stage holds up to four 64-column atoms: the producer's issue latency (wait, expect,
@@ -39,7 +39,7 @@ constexpr int kMaxAtomsPerStage = 4; // a stage holds up to four 64-column atoms
 constexpr int kGatherMaxP = 0;    // up to this many pivots the pivot rows come by gather4 even when the compact copy exists: none
                                   // (gather4 ops issue at ~13 per us and SM: at 8 pivots 128 of them per row tile cost more than
                                   // the copy; measured per launch, 256 x 2880 tokens, 8 pivots: 1.01 -> 0.95 ms)
-constexpr int kStaticSmemReserve = 8192;
+constexpr int kStaticSmemReserve = 9216;
 enum { kWaitStageFree = 64, kWaitStageMma, kWaitStageNorm, kWaitAccumFree1, kWaitAccumFull1, kWaitNormFree, kWaitNormFull };
 
 struct Params {
@@ -50,12 +50,11 @@ struct Params {
     int compact;                       // pivot tiles come from the compact copy [B][N][d] (tm_piv), not by gather4
     int n_sel;                         // row tiles per sample this launch takes: n_rt, or the streamed tiles of `split`
     TileSplit split;                   // k <= 1: all tiles
-    int norms_known;                   // the rows' sums of squares are in ssq already (a score pass over the same tensor came first, all
-                                       // pivots are vision tokens): no warp adds up norms, and the tiles are read by the tensor cores alone
-    int withhold;                      // test hook: the first pivot-norm warp never hands its norms over, so that the bounded waits expire
+    int withhold;                      // test hook: the first norm warp never hands its norms over, so that the bounded waits expire
     unsigned long long wait_ns;
     float *sim;                        // [B][P][n_vis] dup(p_i, x_j)
-    float *l1, *ssq;                   // [B][n_vis]; l1 may be NULL (the scores come from another tensor)
+    float *l1, *ssq;                   // [B][n_vis]; l1 may be NULL (not wanted); norms known: ssq is read, not written
+    const float *piv_ssq;              // [B][P] the pivots' sums of squares
     const int32_t *pivot_idx;          // [B][P], checked and clamped; outside [0, n_vis): a text row of the sample
     int *status;
 };
@@ -66,8 +65,8 @@ struct Shared {
     unsigned long long mma_drain;
     uint32_t tmem_base;
     int abort_flag;
-    float row_ssq[2][2][kTileRows]; // per accumulator buffer and tile of the task: sum of squares of the tile's rows
-    float piv_ssq[2][kMaxN];     // ... and of the sample's pivot rows
+    float row_ssq[2][2][2][kTileRows]; // per accumulator buffer, norm group and tile of the task: the group's share of the rows' sums
+    float row_l1[2][2][2][kTileRows];  // of squares and of absolute values
 };
 static_assert(sizeof(Shared) + 64 <= kStaticSmemReserve, "static shared memory exceeds its reserve");
 
@@ -86,8 +85,9 @@ __host__ inline int atoms_per_stage(int N, size_t smem_limit, int tg = 1)
 }
 __host__ inline size_t smem_bytes(int N, int aps, int n_st, int tg = 1) { return 1024 + (size_t)n_st * stage_bytes(N, aps, tg); }
 
-// |x| and x^2 of one 128-byte row of a 128B-swizzled tile, added to the four running sums in column order:
+// |x| (where wanted) and x^2 of one 128-byte row of a 128B-swizzled tile, added to the four running sums in column order:
 // logical 16-byte chunk c of row r sits at chunk position c ^ (r & 7)
+template <bool kL1>
 __device__ __forceinline__ void add_row(uint32_t tile, int r, float &a0, float &a1, float &q0, float &q1)
 {
     const uint32_t row = tile + (uint32_t)r * 128u;
@@ -98,15 +98,18 @@ __device__ __forceinline__ void add_row(uint32_t tile, int r, float &a0, float &
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float lo = bf16_lo(w[e]), hi = bf16_hi(w[e]);
-            a0 += fabsf(lo);
-            a1 += fabsf(hi);
+            if (kL1) {
+                a0 += fabsf(lo);
+                a1 += fabsf(hi);
+            }
             q0 = fmaf(lo, lo, q0);
             q1 = fmaf(hi, hi, q1);
         }
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kNorms> // false: the norms are known
+__global__ void __launch_bounds__(kNorms ? kThreads : kThreadsNormsKnown, 1)
 onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constant__ CUtensorMap tm_keys,
                const __grid_constant__ CUtensorMap tm_row, const __grid_constant__ CUtensorMap tm_piv,
                const __grid_constant__ CUtensorMap tm_pair, const Params p)
@@ -130,12 +133,12 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem_u32(&sh.full[s]), 1);
-            mbar_init(smem_u32(&sh.empty[s]), p.norms_known ? 1 : 1 + kNormWarps + kPivWarps); // the MMAs' commit and every norm warp
+            mbar_init(smem_u32(&sh.empty[s]), kNorms ? 1 + 2 * kNormWarps : 1); // the MMAs' commit and every norm warp
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(smem_u32(&sh.tmem_full[a]), 1);
             mbar_init(smem_u32(&sh.tmem_empty[a]), kEpiWarps);
-            mbar_init(smem_u32(&sh.norm_full[a]), kNormWarps + kPivWarps);
+            mbar_init(smem_u32(&sh.norm_full[a]), 2 * kNormWarps);
             mbar_init(smem_u32(&sh.norm_empty[a]), kEpiWarps);
         }
         mbar_init(smem_u32(&sh.mma_drain), 1);
@@ -282,13 +285,14 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                 ctl.wait_landed(smem_u32(&sh.mma_drain), 0);
             }
         }
-    } else if (warp >= kNormWarp0 && warp < kNormWarp0 + kNormWarps) {
-        // ------------------------------------------------------------------ norms of the tile's rows and of the pivot rows
-        const int t = (int)threadIdx.x - kNormWarp0 * 32; // tile row owned by this thread
+    } else if (kNorms && ((warp >= kNormWarp0 && warp < kNormWarp0 + kNormWarps) || (warp >= kNormWarp1 && warp < kNormWarp1 + kNormWarps))) {
+        // ------------------------------------------------------------------ norms of the tiles' rows
+        const int grp = warp >= kNormWarp1 ? 1 : 0;                             // which atoms: even or odd ones
+        const int t = (int)threadIdx.x - (grp ? kNormWarp1 : kNormWarp0) * 32; // tile row owned by this thread
         Ring ring(p.n_st);
         uint32_t n = 0;
         bool dead = false; // warp-uniform
-        for (uint32_t g = blockIdx.x; !p.norms_known && !dead && g < total; g += gridDim.x) {
+        for (uint32_t g = blockIdx.x; !dead && g < total; g += gridDim.x) {
             int b, rt;
             task(g, b, rt);
             const int rows = tile_rows(rt, 0), rows2 = p.tg > 1 ? tile_rows(rt, 1) : 0;
@@ -298,9 +302,17 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                 dead = !ctl.wait_bar(smem_u32(&sh.full[ring.stage]), ring.phase, kWaitStageNorm, g);
                 dead = __any_sync(0xffffffffu, dead);
                 if (dead) break;
-                for (int h = 0; h < min(p.aps, na - a); ++h) { // atoms in column order: the sums do not depend on the staging
-                    if (t < rows) add_row(a_addr(ring.stage, h), t, a0, a1, q0, q1);
-                    if (t < rows2) add_row(a_addr(ring.stage, h, 1), t, c0, c1, r0, r1);
+                const int nh = min(p.aps, na - a);
+                if (p.l1) {
+                    for (int h = (a ^ grp) & 1; h < nh; h += 2) { // atoms in column order: the sums do not depend on the staging
+                        if (t < rows) add_row<true>(a_addr(ring.stage, h), t, a0, a1, q0, q1);
+                        if (t < rows2) add_row<true>(a_addr(ring.stage, h, 1), t, c0, c1, r0, r1);
+                    }
+                } else {
+                    for (int h = (a ^ grp) & 1; h < nh; h += 2) {
+                        if (t < rows) add_row<false>(a_addr(ring.stage, h), t, a0, a1, q0, q1);
+                        if (t < rows2) add_row<false>(a_addr(ring.stage, h, 1), t, c0, c1, r0, r1);
+                    }
                 }
                 __syncwarp(); // the warp's reads of the stage are done
                 if (lane == 0) mbar_arrive(smem_u32(&sh.empty[ring.stage]));
@@ -312,65 +324,19 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
             dead = !ctl.wait_bar(smem_u32(&sh.norm_empty[acc]), ((n >> 1) & 1u) ^ 1u, kWaitNormFree, g);
             dead = __any_sync(0xffffffffu, dead);
             if (dead) break;
-            const float q = q0 + q1, r = r0 + r1;
-            sh.row_ssq[acc][0][t] = t < rows ? q : 0.f;
-            sh.row_ssq[acc][1][t] = t < rows2 ? r : 0.f;
-            if (t < rows) {
-                const size_t o = (size_t)b * p.n_vis + rt * kTileRows + t;
-                if (p.l1) p.l1[o] = a0 + a1;
-                p.ssq[o] = q;
-            }
-            if (t < rows2) {
-                const size_t o = (size_t)b * p.n_vis + (rt + 1) * kTileRows + t;
-                if (p.l1) p.l1[o] = c0 + c1;
-                p.ssq[o] = r;
-            }
+            sh.row_ssq[acc][grp][0][t] = q0 + q1;
+            sh.row_ssq[acc][grp][1][t] = r0 + r1;
+            sh.row_l1[acc][grp][0][t] = a0 + a1;
+            sh.row_l1[acc][grp][1][t] = c0 + c1;
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh.norm_full[acc])); // release: the warp's norms are ordered before it
-            ++n;
-        }
-    } else if (warp >= kPivWarp0 && warp < kPivWarp0 + kPivWarps) {
-        // ------------------------------------------------------------------ norms of the pivot rows that come with every tile
-        const int u = (int)threadIdx.x - kPivWarp0 * 32; // pivot rows u, u + 64, u + 128, u + 192
-        Ring ring(p.n_st);
-        uint32_t n = 0;
-        bool dead = false; // warp-uniform
-        for (uint32_t g = blockIdx.x; !p.norms_known && !dead && g < total; g += gridDim.x) {
-            float pq[kMaxN / kPivThreads][2]; // sums of squares only
-#pragma unroll
-            for (int k = 0; k < kMaxN / kPivThreads; ++k) pq[k][0] = pq[k][1] = 0.f;
-            for (int a = 0; a < na; a += p.aps) {
-                dead = !ctl.wait_bar(smem_u32(&sh.full[ring.stage]), ring.phase, kWaitStageNorm, g);
-                dead = __any_sync(0xffffffffu, dead);
-                if (dead) break;
-                for (int h = 0; h < min(p.aps, na - a); ++h)
-#pragma unroll
-                    for (int k = 0; k < kMaxN / kPivThreads; ++k)
-                        if (u + kPivThreads * k < p.P) {
-                            float x0 = 0.f, x1 = 0.f;
-                            add_row(b_addr(ring.stage, h), u + kPivThreads * k, x0, x1, pq[k][0], pq[k][1]);
-                        }
-                __syncwarp(); // the warp's reads of the stage are done
-                if (lane == 0) mbar_arrive(smem_u32(&sh.empty[ring.stage]));
-                ring.advance();
-            }
-            if (dead) break;
-            const uint32_t acc = n & 1u;
-            dead = !ctl.wait_bar(smem_u32(&sh.norm_empty[acc]), ((n >> 1) & 1u) ^ 1u, kWaitNormFree, g);
-            dead = __any_sync(0xffffffffu, dead);
-            if (dead) break;
-#pragma unroll
-            for (int k = 0; k < kMaxN / kPivThreads; ++k)
-                if (u + kPivThreads * k < p.P) sh.piv_ssq[acc][u + kPivThreads * k] = pq[k][0] + pq[k][1];
-            __syncwarp();
-            if (lane == 0 && !(p.withhold && warp == kPivWarp0)) mbar_arrive(smem_u32(&sh.norm_full[acc]));
+            if (lane == 0 && !(p.withhold && warp == kNormWarp0)) mbar_arrive(smem_u32(&sh.norm_full[acc])); // release: the warp's norms are ordered before it
             ++n;
         }
     } else if (warp >= kEpi0 && warp < kEpi0 + kEpiWarps) {
         // ------------------------------------------------------------------ epilogue (warps independent)
         const int quarter = warp & 3;        // TMEM lane quarter this warp may read
         const int row = quarter * 32 + lane; // tile row owned by this thread
-        float piv_norm[kMaxN / 32] = {};     // norms_known: |pivot lane + 32 k| of sample norm_b
+        float piv_norm[kMaxN / 32] = {};     // |pivot lane + 32 k| of sample norm_b
         int norm_b = -1;
         uint32_t n = 0;
         for (uint32_t g = blockIdx.x; g < total; g += gridDim.x) {
@@ -379,20 +345,27 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
             const uint32_t acc = n & 1u;
             bool ok = true;
             float row_ssq[2] = {0.f, 0.f};
-            if (p.norms_known) { // on their way while the task's products are still being summed
-                const float *ssq = p.ssq + (size_t)b * p.n_vis;
+            if (b != norm_b) { // (on their way while the task's products are still being summed)
+                norm_b = b;
 #pragma unroll
-                for (int w = 0; w < 2; ++w)
-                    if (w < p.tg && row < tile_rows(rt, w)) row_ssq[w] = __ldg(ssq + (rt + w) * kTileRows + row);
-                if (b != norm_b) {
-                    norm_b = b;
-#pragma unroll
-                    for (int k = 0; k < kMaxN / 32; ++k)
-                        if (lane + 32 * k < p.P) piv_norm[k] = sqrtf(__ldg(ssq + __ldg(p.pivot_idx + (size_t)b * p.P + lane + 32 * k)));
-                }
-            } else {
+                for (int k = 0; k < kMaxN / 32; ++k)
+                    if (lane + 32 * k < p.P) piv_norm[k] = sqrtf(__ldg(p.piv_ssq + (size_t)b * p.P + lane + 32 * k));
+            }
+            if (kNorms) {
                 ok = ctl.wait_bar(smem_u32(&sh.norm_full[acc]), (n >> 1) & 1u, kWaitNormFull, g);
-                if (ok) row_ssq[0] = sh.row_ssq[acc][0][row], row_ssq[1] = sh.row_ssq[acc][1][row];
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok)
+                    for (int w = 0; w < p.tg; ++w) {
+                        row_ssq[w] = sh.row_ssq[acc][0][w][row] + sh.row_ssq[acc][1][w][row];
+                        if (row < tile_rows(rt, w)) {
+                            const size_t o = (size_t)b * p.n_vis + (rt + w) * kTileRows + row;
+                            if (p.l1) p.l1[o] = sh.row_l1[acc][0][w][row] + sh.row_l1[acc][1][w][row];
+                            p.ssq[o] = row_ssq[w];
+                        }
+                    }
+            } else {
+                for (int w = 0; w < p.tg; ++w)
+                    if (row < tile_rows(rt, w)) row_ssq[w] = __ldg(p.ssq + (size_t)b * p.n_vis + (rt + w) * kTileRows + row);
             }
             if (ok) ok = ctl.wait_bar(smem_u32(&sh.tmem_full[acc]), (n >> 1) & 1u, kWaitAccumFull1, g);
             if (!__all_sync(0xffffffffu, ok)) break;
@@ -412,9 +385,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                         tmem_ld8(taddr + (uint32_t)c0, v); // warp-collective: rows outside the tile still take part
 #pragma unroll
                         for (int e = 0; e < 8; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0; a warp writes 128 contiguous bytes
-                            const float np = p.norms_known ? __shfl_sync(0xffffffffu, piv_norm[k], (c0 + e) & 31)
-                                                           : sqrtf(sh.piv_ssq[acc][min(c0 + e, p.P - 1)]);
-                            const float den = np * nj;
+                            const float den = __shfl_sync(0xffffffffu, piv_norm[k], (c0 + e) & 31) * nj;
                             if (row < rows && c0 + e < p.P) dst[(size_t)(c0 + e) * p.n_vis] = den > 0.f ? v[e] / den : 0.f;
                         }
                     }
@@ -424,7 +395,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(smem_u32(&sh.tmem_empty[acc]));
-                if (!p.norms_known) mbar_arrive(smem_u32(&sh.norm_empty[acc]));
+                if (kNorms) mbar_arrive(smem_u32(&sh.norm_empty[acc]));
             }
             ++n;
         }

@@ -352,13 +352,13 @@ pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P
 
 // ------------------------------------------------------------------------------------------------
 // Compact copy of every sample's pivot rows, [B][N][d8] with N >= P rows per sample (rows P.. are zero), so that a
-// tensor-core kernel can fetch a sample's pivot tile as one box.  One warp per row.
+// tensor-core kernel can fetch a sample's pivot tile as one box, and their sums of squares.  One warp per row; out may be NULL.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPivotRowWarps = 8;
 
 __global__ void __launch_bounds__(kPivotRowWarps * 32)
 pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *__restrict__ pivot_idx, int S, int d8, int vis_offset, int n_vis,
-                  int P, int N, long long rows_total, uint4 *__restrict__ out)
+                  int P, int N, long long rows_total, uint4 *__restrict__ out, float *__restrict__ piv_ssq)
 {
     wait_for_previous();
     let_next_start();
@@ -366,14 +366,29 @@ pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *__restrict__ pi
     const long long row = (long long)blockIdx.x * kPivotRowWarps + (threadIdx.x >> 5);
     if (row >= rows_total) return;
     const int b = (int)(row / N), i = (int)(row % N);
-    uint4 *dst = out + (size_t)row * d8;
+    uint4 *dst = out ? out + (size_t)row * d8 : nullptr;
     if (i >= P) {
-        for (int c = lane; c < d8; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
+        if (dst)
+            for (int c = lane; c < d8; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
         return;
     }
     const int pv = min(max(pivot_idx[(size_t)b * P + i], -vis_offset), S - vis_offset - 1); // any row of the sample
     const uint4 *src = keys + ((size_t)b * S + vis_offset + pv) * (size_t)d8;
-    for (int c = lane; c < d8; c += 32) dst[c] = __ldg(src + c);
+    float q0 = 0.f, q1 = 0.f;
+#pragma unroll 4
+    for (int c = lane; c < d8; c += 32) {
+        const uint4 v = __ldg(src + c);
+        if (dst) dst[c] = v;
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float lo = bf16_lo(w[e]), hi = bf16_hi(w[e]);
+            q0 = fmaf(lo, lo, q0);
+            q1 = fmaf(hi, hi, q1);
+        }
+    }
+    q0 = warp_sum(q0 + q1);
+    if (lane == 0) piv_ssq[(size_t)b * P + i] = q0;
 }
 
 // ------------------------------------------------------------------------------------------------
