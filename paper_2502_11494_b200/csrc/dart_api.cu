@@ -757,16 +757,18 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
 }
 
 // Whether AUTO takes the flow path.  Pivots by score: up to 16 pivots it is the fastest path at every size measured, from one
-// sample of 130 tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.40 against 1.85 ms of
-// the sweep, 16 pivots 1.48 against 1.87).  Up to 32 pivots its multiplying warps bound it on large batches (256 x 2880 x
-// 4096: 2.05 against 1.91 ms of two passes; 32 x 2880 x 4096: 290 against 328 us).  Given pivots: it reads every row into an
-// SM twice where the one-pass kernel reads it once, but needs no launches before it and spreads a few samples over all SMs
-// (4 x 2880 x 4096: 44 against 58 us, 32 x 576 x 4096: 59 against 73, 32 x 2880 x 4096: 186 against 173).
+// sample of 130 tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.25 against 1.85 ms of
+// the sweep, 16 pivots 1.30 against 1.87).  Up to 32 pivots its multiplying warps bound it on larger batches (whole calls, us, flow
+// / two passes: 8 x 2880 x 4096 128 / 132, 16 x 2880 x 4096 203 / 213, 256 x 500 x 2048 353 / 330, 256 x 2880 x 4096 2443 / 2246).
+// Given pivots: it reads every row into an SM twice where the one-pass kernel reads it once, but spreads fewer row tiles than SMs
+// over all of them (whole calls, us, flow / one pass: 4 x 2880 x 4096 53 / 57, 16 x 576 x 4096 52 / 59, 8 x 2880 x 4096 79 / 74,
+// 64 x 300 x 2048 57 / 55; 32 pivots, 8 x 1500 x 3072: 77 / 66).
 bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
 {
     if (!flow_applies(ctx, B, n_vis, P)) return false;
     const long long bytes = 2ll * ctx->desc.d * n_vis * B;
-    if (o.pivots_in ? bytes > 200000000ll : (P > 16 && bytes > 1000000000ll)) return false;
+    const long long row_tiles = (long long)B * ((n_vis + dart::sweep::kTileRows - 1) / dart::sweep::kTileRows);
+    if (o.pivots_in ? (row_tiles >= ctx->sm_count || P > 16) : (P > 16 && bytes > 300000000ll)) return false;
     dart::flow::Params p = {};
     return flow_config(ctx, B, n_vis, P, o, p);
 }
@@ -802,7 +804,7 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         size_t smem = 1024 + (size_t)p.n_st * F::kStageBytes + (size_t)F::kScoreWarps * p.n_slot * F::kChunkBytes + F::pivot_bytes(NT, p.na_max);
         if (smem < F::selector_bytes(n_vis)) smem = F::selector_bytes(n_vis);
         // every CTA waits for scores that the others publish: co-residency is required
-        DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3(F::kThreads), args, smem, st));
+        DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3((unsigned)F::threads(NT)), args, smem, st));
     }
     launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st, true);

@@ -19,7 +19,7 @@
 // slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
 //
-// Per CTA (736 threads, one CTA per SM, cooperative launch):
+// Per CTA (736 or 864 threads, one CTA per SM, cooperative launch):
 //   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
 //   warps 4-7    second pass: mma.sync.m16n8k16 (16 rows each; P <= 32 leaves the tensor pipe idle whatever the form, and
 //                64-row items do not fill the 128 rows of a tcgen05.mma)
@@ -28,6 +28,7 @@
 //   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
 //   warp 21      watcher: how far the pivots of the batch have got, for the scorers' window
 //   warp 22      feeder: the scorers' rows into their slots
+//   warps 23-26  with more than 16 pivots: second pass for the second half of the pivots
 // Every wait is bounded in time; on expiry the kernel records DART_ERR_TIMEOUT in the status word, lets the copies in flight
 // land and exits normally.
 #pragma once
@@ -52,13 +53,15 @@ constexpr int kAps = 2;                    // atoms per ring stage
 constexpr int kStageBytes = kAps * kAtomBytes;
 constexpr int kMaxStages = 13;
 constexpr int kPivWarps = 4;
-constexpr int kMulWarp0 = 4, kMulWarps = 4;
+constexpr int kMulWarp0 = 4, kMulWarps = 4; // 16 rows each; with more than 16 pivots a second group of four takes half of the pivots
 constexpr int kProdWarp = 8;
 constexpr int kCombWarp0 = 9, kCombWarps = 4; // (an item is counted 2-3 us after its shares were written: two warps held the others up)
 constexpr int kScoreWarp0 = kCombWarp0 + kCombWarps, kScoreWarps = 8;
 constexpr int kWatchWarp = kScoreWarp0 + kScoreWarps;
 constexpr int kFeedWarp = kWatchWarp + 1;
-constexpr int kThreads = 32 * (kFeedWarp + 1);
+constexpr int kMulWarp1 = kFeedWarp + 1;
+__host__ __device__ constexpr int mul_groups(int NT) { return NT > 2 ? 2 : 1; }
+__host__ __device__ constexpr int threads(int NT) { return 32 * (kMulWarp1 + (mul_groups(NT) - 1) * kMulWarps); }
 constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane and chunk
 constexpr int kChunkUnits = 32 * kChunk;
 constexpr uint32_t kChunkBytes = kChunk * 512; // 4 KB: half a row of 4096 columns
@@ -468,15 +471,18 @@ __device__ __forceinline__ void take_pivots(const Params &p, const Ctl &ctl, Sha
     }
 }
 
-// Second pass: 16 rows of the item per warp, all columns of the slice.
-template <int NT>
-__device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared &sh, uint32_t ring0, uint32_t piv0)
+// Second pass: 16 rows of the item per warp, all columns of the slice, NT of the sample's NTall tiles of 8 pivots (from tile n0 on).
+// (32 pivots: one group 2.48, two groups 2.07 ms at 256 x 2880 x 4096: a dependent product returns after some 130 cycles, and a
+// warp had 16 per atom to wait for.  16 pivots: one group 1.30, two 1.76 ms: a second group reads the rows from shared memory a
+// second time, and that is what bounds the kernel then: every key byte is written there twice and read twice.)
+template <int NT, int NTall>
+__device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared &sh, uint32_t ring0, uint32_t piv0, int w, int n0)
 {
-    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) - kMulWarp0;
+    const int lane = threadIdx.x & 31;
     const int row = 16 * w + (lane & 15);                     // tile row whose 16 bytes this lane addresses for ldmatrix
     const uint32_t a_row = (uint32_t)row * 128u, a_sw = (uint32_t)(row & 7);
     const uint32_t b_lane = (uint32_t)(lane & 7) * p.pitch + (uint32_t)(lane >> 3) * 16u;
-    const size_t part_item = (size_t)8 * NT * kRows;
+    const size_t part_item = (size_t)8 * NTall * kRows;
     Ring ring(p.n_st);
     int seq = -1, last_b = -1, k = 0;
     for (Items it(p); it.valid(); it.next(), ++k) {
@@ -487,8 +493,8 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
             const bool ok = ctl.wait_bar(smem_u32(&sh.piv_full[seq & 1]), (uint32_t)(seq >> 1) & 1u, kWaitPiv, it.b);
             if (!__all_sync(0xffffffffu, ok)) return;
         }
-        if (p.given && w == 0 && lane == 0) sh.pos = it.b * p.n_vis + it.rg * kRows;
-        const uint32_t piv = piv0 + (uint32_t)((seq & 1) * 8 * NT) * p.pitch + b_lane;
+        if (p.given && w == 0 && n0 == 0 && lane == 0) sh.pos = it.b * p.n_vis + it.rg * kRows;
+        const uint32_t piv = piv0 + (uint32_t)((seq & 1) * 8 * NTall + 8 * n0) * p.pitch + b_lane;
         constexpr int kChains = NT == 1 ? 4 : 2; // independent sums per pivot tile
         float acc[NT][kChains][4];
 #pragma unroll
@@ -540,7 +546,7 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
             ring.advance();
         }
         // the slice's share of the dot products: 8 consecutive rows of a pivot per 32 bytes
-        float *dst = p.part + (((size_t)it.b * p.n_rg + it.rg) * p.nsl + it.sl) * part_item + 16 * w + (lane >> 2);
+        float *dst = p.part + (((size_t)it.b * p.n_rg + it.rg) * p.nsl + it.sl) * part_item + (size_t)8 * n0 * kRows + 16 * w + (lane >> 2);
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -557,23 +563,30 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
         __syncwarp(); // the lanes' stores are ordered before lane 0's release
         if (lane == 0) mbar_arrive(smem_u32(&sh.mail_full[c][slot]));
     }
-    if (p.given && w == 0 && lane == 0) sh.pos = 0x3fffffff; // nothing holds the scorers back any more
+    if (p.given && w == 0 && n0 == 0 && lane == 0) sh.pos = 0x3fffffff; // nothing holds the scorers back any more
 }
 
 // Watcher: how far the batch's pivots have got, for the scorers.  (Held back by the second pass of their own SM instead, the
-// scorers of an SM with one item more than the others delayed everybody's pivots: 8 us between the first and the last SM.)
+// scorers of an SM with one item more than the others delayed everybody's pivots: 8 us between the first and the last SM.)  It
+// looks at 32 samples at a time: one after the other, a load's 0.45 us per sample held batches of short ones back.
 __device__ __forceinline__ void watch(const Params &p, const Ctl &ctl, Shared &sh)
 {
-    if ((threadIdx.x & 31) != 0 || p.given) return;
+    if (p.given) return;
+    const int lane = threadIdx.x & 31;
     long long last = clock64();
-    for (int b = 0; b < p.B; ++b) {
-        const int32_t *word = p.pv_word + (size_t)b * kMaxP;
-        for (uint32_t spin = 0; (int32_t)ld_word(word) == kNoPivot; ++spin) {
+    for (int b = 0; b < p.B;) {
+        const bool there = b + lane >= p.B || (int32_t)ld_word(p.pv_word + (size_t)(b + lane) * kMaxP) != kNoPivot;
+        const uint32_t missing = ~__ballot_sync(0xffffffffu, there);
+        const int n = missing ? __ffs(missing) - 1 : 32; // samples in a row from b on whose pivots are known
+        if (n > 0) {
+            b += n;
+            if (lane == 0) sh.pos = min(b, p.B) * p.n_vis;
+            last = clock64();
+        } else {
             __nanosleep(32);
-            if ((spin & 31u) == 31u && (ctl.aborted() || (unsigned long long)(clock64() - last) > ctl.limit_cycles)) return; // (the scorers report it)
+            const bool dead = ctl.aborted() || (unsigned long long)(clock64() - last) > ctl.limit_cycles;
+            if (__any_sync(0xffffffffu, dead)) return; // (the scorers' feeder reports it)
         }
-        sh.pos = (b + 1) * p.n_vis;
-        last = clock64();
     }
 }
 
@@ -696,7 +709,7 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant__ CUtensorMap tm, const Params p)
+__global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_constant__ CUtensorMap tm, const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
@@ -714,17 +727,17 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(smem_u32(&sh.full[s]), 1);
-            mbar_init(smem_u32(&sh.empty[s]), kMulWarps);
+            mbar_init(smem_u32(&sh.empty[s]), mul_groups(NT) * kMulWarps);
         }
         for (int w = 0; w < kScoreWarps; ++w)
             for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&sh.chunk_full[w][s]), 1), mbar_init(smem_u32(&sh.chunk_empty[w][s]), 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&sh.piv_full[s]), kPivWarps * 32);
-            mbar_init(smem_u32(&sh.piv_empty[s]), kMulWarps);
+            mbar_init(smem_u32(&sh.piv_empty[s]), mul_groups(NT) * kMulWarps);
         }
         for (int c = 0; c < kCombWarps; ++c)
             for (int s = 0; s < kMail; ++s) {
-                mbar_init(smem_u32(&sh.mail_full[c][s]), kMulWarps);
+                mbar_init(smem_u32(&sh.mail_full[c][s]), mul_groups(NT) * kMulWarps);
                 mbar_init(smem_u32(&sh.mail_empty[c][s]), 1);
             }
         sh.abort_flag = 0;
@@ -734,6 +747,8 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
     __syncthreads();
     if ((int)blockIdx.x >= p.n_stream) {
         if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, skey, list);
+    } else if (warp >= kMulWarp1) {
+        multiply<NT / mul_groups(NT), NT>(p, ctl, sh, ring0, piv0, warp - kMulWarp1, NT / mul_groups(NT));
     } else if (warp == kFeedWarp) {
         feed(p, ctl, sh, slot0);
     } else if (warp == kWatchWarp) {
@@ -746,7 +761,7 @@ __global__ void __launch_bounds__(kThreads, 1) flow_kernel(const __grid_constant
         // were through first: 8 x 2880 x 4096, 16 pivots 94 -> 97 us.)
         let_next_start();
     } else if (warp < kMulWarp0 + kMulWarps) {
-        multiply<NT>(p, ctl, sh, ring0, piv0);
+        multiply<NT / mul_groups(NT), NT>(p, ctl, sh, ring0, piv0, warp - kMulWarp0, 0);
     } else if (warp == kProdWarp) {
         produce(p, ctl, sh, ring0, &tm);
     } else {
