@@ -718,6 +718,7 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     const long long row_bytes = (long long)ctx->desc.d * 2, sample = row_bytes * n_vis, MB = 1ll << 20;
     const int NT = flow_tiles(P), want_nsl = (o.tune >> 16) & 31, want_slot = (o.tune >> 12) & 7;
     p.given = o.pivots_in != nullptr;
+    p.sel_threads = F::sel_threads(n_vis);
     p.n_stream = ctx->sm_count - (p.given ? 0 : F::selectors(sample));
     const size_t limit = (size_t)ctx->max_smem_optin - F::kStaticSmemReserve - 1024;
     p.n_atoms = ctx->n_atoms, p.n_rg = (n_vis + F::kRows - 1) / F::kRows;

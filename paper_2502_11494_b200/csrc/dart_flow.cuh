@@ -66,7 +66,8 @@ constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane a
 constexpr int kChunkUnits = 32 * kChunk;
 constexpr uint32_t kChunkBytes = kChunk * 512; // 4 KB: half a row of 4096 columns
 constexpr int kMaxSlots = 6;               // chunks of a row on their way per scorer
-constexpr int kSel = 512;                  // threads of a selector CTA that select
+constexpr int kSel = 512, kSelGroups = 4;  // threads of a selector CTA that select; at most so many groups of them
+__host__ inline int sel_threads(int n_vis) { return n_vis > 1024 ? kSel : kSel / kSelGroups; }
 constexpr int kPoll = 6;                   // words per selecting thread on their way at once: 3072 tokens
 constexpr int kMail = 2;                   // items on their way to each combine warp
 constexpr int kPvRing = 16;                // pivot lists kept for the combine warps: 2 pivot buffers + 8 items on their way, and slack
@@ -79,8 +80,9 @@ constexpr uint32_t kNoWord = ~0u;
 constexpr unsigned long long kNoRec = ~0ull; // a row's word before it is published (no sums produce it)
 enum { kWaitRec = 90, kWaitPivots, kWaitPivFree, kWaitPiv, kWaitStage, kWaitStageFree, kWaitMailFree, kWaitMail, kWaitCombRec,
        kWaitWindow, kWaitChunk = 101 }; // (100 is taken by the check of given pivots)
-// Selector CTAs: a selection takes about 3 us, a sample streams at about 6 MB per us.
-__host__ inline int selectors(long long sample_bytes) { return sample_bytes >= (4 << 20) ? 4 : sample_bytes >= (2 << 20) ? 8 : 16; }
+// Selector CTAs: a selection takes about 3 us, a sample streams at about 6 MB per us.  (256 samples of 1 to 4 MB: 8 or 16 CTAs for
+// them 360 and 237 us, 6 and 8 CTAs 356 and 229; 2 and 3 are no better and cost large samples 1 %.)
+__host__ inline int selectors(long long sample_bytes) { return sample_bytes >= (4 << 20) ? 4 : sample_bytes >= (1 << 20) ? 6 : 8; }
 
 struct Params {
     int B, S, vis_offset, n_vis, P, d8; // d8: row width in 16-byte units
@@ -88,6 +90,7 @@ struct Params {
     int n_st, n_slot;                   // ring depth; chunks on their way per scorer
     int rows_task, n_chunk;             // scoring: rows per task (2: two rows to a chunk); chunks per task
     int n_stream;                       // CTAs that stream; the others select
+    int sel_threads;                    // threads per selection
     int given;                          // the pivots are in pivot_idx already
     int norm_kind, smallest, withhold;
     int window;                         // rows the scorers may be ahead of `pos` (>= n_vis)
@@ -110,8 +113,8 @@ struct Shared {
     unsigned long long chunk_full[kScoreWarps][kMaxSlots], chunk_empty[kScoreWarps][kMaxSlots];
     unsigned long long piv_full[2], piv_empty[2];
     unsigned long long mail_full[kCombWarps][kMail], mail_empty[kCombWarps][kMail];
-    uint32_t group_best[32];          // selectors: best keys of groups of 16 threads
-    uint32_t n_list;
+    uint32_t set_best[kSelGroups][32]; // selectors: best keys of sets of threads
+    uint32_t n_list[kSelGroups];
     int32_t pv[kPvRing][kMaxP];       // pivots of the samples on their way, by the SM's own count of samples
     int abort_flag;
     volatile int pos;                 // rows (of the batch) whose samples have their pivots; given pivots: rows the second pass is through with
@@ -120,7 +123,7 @@ static_assert(sizeof(Shared) + 64 <= kStaticSmemReserve, "static shared memory e
 
 // shared memory of the two pivot buffers; of a selector (the list takes every token: with many equal scores many are at the floor)
 __host__ inline size_t pivot_bytes(int NT, int na_max) { return (size_t)2 * 8 * NT * ((size_t)na_max * 128 + 16); }
-__host__ inline size_t selector_bytes(int n_vis) { return (size_t)n_vis * 12; }
+__host__ inline size_t selector_bytes(int n_vis) { return (size_t)n_vis * 12 * (kSel / sel_threads(n_vis)); }
 
 __device__ __forceinline__ unsigned long long ld_rec(const unsigned long long *p)
 {
@@ -338,31 +341,43 @@ __device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shar
     }
 }
 
-// The selectors (CTAs that do nothing else): sample k, k + n_selectors, ... of the batch each.  512 threads read the sample's
-// words as they appear; the P-th best of 32 groups' best keys is a floor that few keys pass; those are ranked by counting.
-__device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, Shared &sh, uint32_t *skey, unsigned long long *list)
+// The selectors (CTAs that do nothing else).  p.sel_threads threads (512, or four groups of 128 side by side for short samples,
+// which come faster than one group takes them) read a sample's words as they appear; the P-th best of 32 sets' best keys is a
+// floor that few keys pass; those are ranked by counting.
+__device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, Shared &sh, uint8_t *smem)
 {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    auto any = [](bool x) { return sweep::group_any<1, kSel>(x); };
-    for (int b = (int)blockIdx.x - p.n_stream; b < p.B; b += (int)gridDim.x - p.n_stream) {
+    const int T = p.sel_threads, grp = (int)threadIdx.x / T, n_grp = kSel / T;
+    const int t = (int)threadIdx.x - grp * T, lane = t & 31;
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(smem) + (size_t)grp * p.n_vis;
+    uint32_t *skey = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(smem) + (size_t)n_grp * p.n_vis) + (size_t)grp * p.n_vis;
+    auto any = [&](bool x) { // OR over the group; doubles as its barrier
+        uint32_t r;
+        asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\nbar.red.or.pred p, %2, %3, q;\nselp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(r)
+                     : "r"((uint32_t)x), "r"(1 + grp), "r"(T)
+                     : "memory");
+        return r != 0;
+    };
+    const int n_sel = ((int)gridDim.x - p.n_stream) * n_grp;
+    for (int b = ((int)blockIdx.x - p.n_stream) * n_grp + grp; b < p.B; b += n_sel) {
         const uint32_t *rec = reinterpret_cast<const uint32_t *>(p.rec + (size_t)b * p.n_vis) + (p.norm_kind == 2 ? 1 : 0);
         const long long t0 = clock64();
         bool dead = false;
         uint32_t best = 0; // larger = better
-        for (int j0 = t; j0 < p.n_vis && !dead; j0 += kSel * kPoll) {
+        for (int j0 = t; j0 < p.n_vis && !dead; j0 += T * kPoll) {
             // all words that are still missing are asked for together (one after the other, a thread that had started early
             // paid a round trip for each of its six)
             uint32_t v[kPoll], miss = 0;
 #pragma unroll
             for (int u = 0; u < kPoll; ++u) {
                 v[u] = 0;
-                if (j0 + u * kSel < p.n_vis) miss |= 1u << u;
+                if (j0 + u * T < p.n_vis) miss |= 1u << u;
             }
             const uint32_t mine = miss;
             for (uint32_t spin = 1; miss && !dead; ++spin) {
 #pragma unroll
                 for (int u = 0; u < kPoll; ++u)
-                    if ((miss >> u) & 1u) v[u] = ld_word(rec + 2 * (j0 + u * kSel));
+                    if ((miss >> u) & 1u) v[u] = ld_word(rec + 2 * (j0 + u * T));
 #pragma unroll
                 for (int u = 0; u < kPoll; ++u)
                     if (v[u] != kNoWord) miss &= ~(1u << u);
@@ -380,35 +395,34 @@ __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, S
                 uint32_t k = order_key(__uint_as_float(v[u]));
                 if (p.smallest) k = ~k;
                 if ((mine >> u) & 1u) {
-                    skey[j0 + u * kSel] = k;
+                    skey[j0 + u * T] = k;
                     best = max(best, k);
                 }
             }
         }
-        uint32_t g = best; // best of 16 lanes
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
-        if ((lane & 15) == 0) sh.group_best[2 * warp + (lane >> 4)] = g;
-        if (t == 0) sh.n_list = 0;
+        uint32_t g = best; // best of a set of T / 32 lanes
+        for (int o = T / 64; o > 0; o >>= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+        if ((t & (T / 32 - 1)) == 0) sh.set_best[grp][t / (T / 32)] = g;
+        if (t == 0) sh.n_list[grp] = 0;
         if (any(dead)) return;
-        // the floor: the P-th best of the 32 groups' best keys
-        const uint32_t x = sh.group_best[lane];
+        // the floor: the P-th best of the 32 sets' best keys
+        const uint32_t x = sh.set_best[grp][lane];
         int gt = 0, ge = 0;
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
             const uint32_t y = __shfl_sync(0xffffffffu, x, u);
             gt += y > x, ge += y >= x;
         }
-        const uint32_t here = __ballot_sync(0xffffffffu, gt < p.P && ge >= p.P); // (samples of fewer tokens than groups: empty groups hold 0)
+        const uint32_t here = __ballot_sync(0xffffffffu, gt < p.P && ge >= p.P); // (samples of fewer tokens than sets: empty sets hold 0)
         const uint32_t fl = __shfl_sync(0xffffffffu, x, __ffs(here) - 1);
         if (best >= fl)
-            for (int j = t; j < p.n_vis; j += kSel) {
+            for (int j = t; j < p.n_vis; j += T) {
                 const uint32_t k = skey[j];
-                if (k >= fl) list[atomicAdd(&sh.n_list, 1u)] = ((unsigned long long)k << 32) | (0xffffffffu - (uint32_t)j); // equal scores: lower index first
+                if (k >= fl) list[atomicAdd(&sh.n_list[grp], 1u)] = ((unsigned long long)k << 32) | (0xffffffffu - (uint32_t)j); // equal scores: lower index first
             }
         any(false);
-        const int m = (int)sh.n_list;
-        for (int e = t; e < m; e += kSel) {
+        const int m = (int)sh.n_list[grp];
+        for (int e = t; e < m; e += T) {
             const unsigned long long mine = list[e];
             int r = 0;
             for (int u = 0; u < m; ++u) r += list[u] > mine ? 1 : 0;
@@ -718,8 +732,6 @@ __global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_const
     const uint32_t ring0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t slot0 = ring0 + (uint32_t)p.n_st * kStageBytes;
     const uint32_t piv0 = slot0 + (uint32_t)(kScoreWarps * p.n_slot) * kChunkBytes;
-    unsigned long long *list = reinterpret_cast<unsigned long long *>(smem_raw); // (selectors have no ring)
-    uint32_t *skey = reinterpret_cast<uint32_t *>(list + p.n_vis);
     const int warp = threadIdx.x >> 5;
     // whoever waits for something nearest to what is missing has the shortest limit, so that it is the one that reports it
     const unsigned long long limit = 2ull * p.wait_ns; // ns -> cycles at the highest SM clock: never shorter than asked
@@ -746,7 +758,7 @@ __global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_const
     }
     __syncthreads();
     if ((int)blockIdx.x >= p.n_stream) {
-        if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, skey, list);
+        if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, smem_raw); // (selectors have no ring)
     } else if (warp >= kMulWarp1) {
         multiply<NT / mul_groups(NT), NT>(p, ctl, sh, ring0, piv0, warp - kMulWarp1, NT / mul_groups(NT));
     } else if (warp == kFeedWarp) {
