@@ -255,17 +255,21 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     const bool each = o.rule == DART_RULE_UNION; // independent pivots: lists of q_i instead of Q_i
     RankParams rp = {};
     size_t rank_smem = 0;
-    // few lists: as many threads per list as help; many: small CTAs, so that one list's barriers are covered by the others
+    // few lists: as many threads per list as help; many: small CTAs, so that one list's barriers are covered by the others (24 values
+    // per thread: 256 x 2880, 128 pivots with 256 threads per list 490 us, with 128 389)
     const long long rank_rows = (long long)B * P;
-    const int rank_threads = rank_rows <= 2ll * ctx->sm_count ? 512 : rank_rows <= 8ll * ctx->sm_count ? 256 : n_vis > 1024 ? 128 : 64;
+    int rank_threads = rank_rows <= 2ll * ctx->sm_count ? 512 : rank_rows <= 8ll * ctx->sm_count ? 256 : n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
+    while (rank_threads < kRankMaxThreads && 32 * rank_threads < n_vis) rank_threads *= 2; // the row has to fit the registers
     const int rank_m = each ? (m + P - 1) / P : m;
     bool can_rank = ctx->rank && o.rule != DART_RULE_GLOBAL && n_vis <= kRankMaxVis && rank_m <= kRankMaxList;
     if (can_rank) {
         rp.sample_entries = (size_t)rank_place(P, m / P, m % P, each) + 8;
-        const size_t flags = rank_flag_bytes(n_vis), phase1 = rank_phase1_bytes(n_vis, rank_m, rp.bins = rank_bins(n_vis, rank_threads));
+        const size_t flags = rank_flag_bytes(n_vis), phase1 = rank_phase1_bytes(n_vis, rank_m, rank_threads);
         // the turns' staging buffers take what the ranking needs anyway, more where that saves rounds and costs no residency
-        size_t avail = phase1 - flags;
-        const size_t all = rp.sample_entries * 2, least = 4 * ((size_t)rank_m + 16);
+        size_t avail = phase1 > flags ? phase1 - flags : 0;
+        const size_t all = rp.sample_entries * 2, room = (size_t)14336 * rank_threads / 128; // (the registers leave 28 KB per 128 threads)
+        if (avail + flags < room) avail = room - flags < all ? room - flags : all;
+        const size_t least = 4 * ((size_t)rank_m + 16);
         if (all > avail && (long long)B * P <= ctx->sm_count && all + flags <= (size_t)100 << 10) avail = all;
         if (avail < least) avail = least;
         rp.stage_entries = (int)(all <= avail ? rp.sample_entries : avail / 4 / 8 * 8);
@@ -278,7 +282,8 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
         rp.len_out = ctx->len, rp.status = ctx->status;
         Prof p(ctx, st, SLOT_RETAIN);
-        launch_next(rank_kernel, dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
+        const int regs = rank_regs(n_vis, rank_threads);
+        launch_next(regs == 2 ? rank_kernel<2> : regs == 4 ? rank_kernel<4> : regs == 6 ? rank_kernel<6> : rank_kernel<8>, dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
     };
     if (o.rule == DART_RULE_GLOBAL) { // one threshold for all pivots: a single selection per sample
         Prof p(ctx, st, SLOT_RETAIN);
@@ -1153,8 +1158,11 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
         if (ctx->rank_n * sizeof(uint16_t) <= ((size_t)1 << 30)) {
             rc = ws_alloc(ctx, &ctx->rank, ctx->rank_n);
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->rank_arrived, (size_t)desc->B_max);
-            if (rc == DART_OK && cudaFuncSetAttribute(dart::rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      ctx->max_smem_optin - dart::kRankStaticSmem) != cudaSuccess)
+            const int smem = ctx->max_smem_optin - dart::kRankStaticSmem;
+            if (rc == DART_OK && (cudaFuncSetAttribute(dart::rank_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                                  cudaFuncSetAttribute(dart::rank_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                                  cudaFuncSetAttribute(dart::rank_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                                  cudaFuncSetAttribute(dart::rank_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess))
                 rc = DART_ERR_CUDA;
         }
     }

@@ -4,14 +4,19 @@
 // other pivots take.  One CTA per (sample, pivot) puts those Q_i into order; the CTA of a sample that finishes last takes the
 // pivots' turns over the ranked lists, in rank order, and writes the packed index list.  What bounded the other forms:
 //   - ordering: a radix select and a sort are some twenty block-wide steps (16 us for 128 lists of 312 out of 2880 values).
-//     Here: a histogram of equal bins over the row's low end, its prefix sums as the bins' places, and every entry
-//     counts the smaller ones among the few that share its bin: eight block-wide steps;
+//     Here: the row stays in registers; a threshold guessed from its smallest value and its mean lets through a few more
+//     entries than the list needs (counted, and guessed again until it does: 1 to 3 counts); those alone go into a histogram of
+//     equal bins, its prefix sums are the bins' places, and every entry counts the smaller ones among the few that share its bin.
+//     (With the row in shared memory, two passes over all of it and bins over [min, 2 mean - min] one sample took 1 to 4 us more;
+//     a queue of the entries below the threshold, so that only they meet the atomics, was no faster at 32768 rows (402 us for
+//     389) and slower where half of a row is kept: 190 for 146.)
 //   - the turns: a walk 32 entries at a time, one dependent vote after the other (1.4 us per turn).  Here a lane holds eight
 //     consecutive entries (16 bytes), their eight flags are read at once, and four votes over the bits of the lanes' counts
 //     give every lane its rank among 256 entries: 0.45 us per turn.
-// Measured (us, before: the bands or sorted lists): 1 x 2880 tokens, 8 pivots 39 -> 21; 4 x 4608, 32 pivots 70 -> 31; 8 x 1500
-// keeping half 60 -> 20; 256 x 2880, 8 pivots 60 -> 38, 128 pivots 488 -> 389.  Of the 12 us that one sample takes, ranking
-// is 5, the counter and the lists' way to the last CTA 2, the turns 3.5 and the packed list 1.5: a chain of short steps.
+// Measured (us, before: the bands or sorted lists): 1 x 2880 tokens, 8 pivots 39 -> 19; 4 x 4608, 32 pivots 70 -> 29; 8 x 1500
+// keeping half 60 -> 18; 256 x 2880, 8 pivots 60 -> 38, 128 pivots 488 -> 389.  Of the last, reading the rows is 80 (at the
+// memory's rate it would be 57), minimum and mean 25, the counts 30, the atomics' two passes 100, the places 40; what remains is
+// the last samples' turns.  For one sample all of it is a chain of short steps.
 // Rows whose values the bins do not separate (many equal values, a value that is not finite) are ranked by an exact radix
 // select and counting.  The result equals retain_kernel's exactly.
 //
@@ -23,24 +28,19 @@ namespace dart {
 
 constexpr int kRankMaxThreads = 512;
 constexpr int kRankMaxP = 1024;       // a context's most pivots
-constexpr int kRankMaxVis = 16384;    // the row in shared memory
+constexpr int kRankMaxVis = 16384;    // 512 threads x 8 x 4 values in registers
 constexpr int kRankMaxList = 4096;    // longest list
 constexpr uint32_t kRankMaxBin = 192; // entries of one bin that are ranked by counting
+constexpr int kRankTries = 10;        // guesses at the threshold
 
-// entries of a list in shared memory: the last bin may hold more than the list needs
-__host__ __device__ inline int rank_list_cap(int m) { return m + kRankMaxBin; }
 // one flag per token and one more that is never free
 __host__ __device__ inline size_t rank_flag_bytes(int n_vis) { return ((size_t)n_vis + 16) / 16 * 16; }
-// bins: a multiple of 4 per thread, about one per one to three tokens
-inline int rank_bins(int n_vis, int threads)
+// values per thread in registers: 4 R
+inline int rank_regs(int n_vis, int threads) { return n_vis <= 8 * threads ? 2 : n_vis <= 16 * threads ? 4 : n_vis <= 24 * threads ? 6 : 8; }
+// shared memory of the ranking: the entries of the bins a list needs, 4 bins per thread, one bit per token
+inline size_t rank_phase1_bytes(int n_vis, int m, int threads)
 {
-    int bins = 4 * threads;
-    while (bins < 2048 && 3 * bins < n_vis) bins *= 2;
-    return bins;
-}
-inline size_t rank_phase1_bytes(int n_vis, int m, int bins)
-{
-    return ((size_t)n_vis * 4 + 15) / 16 * 16 + (size_t)bins * 4 + (size_t)rank_list_cap(m) * 8;
+    return ((size_t)m + kRankMaxBin + 1) / 2 * 16 + (size_t)threads * 16 + ((size_t)n_vis + 127) / 128 * 16;
 }
 // places of the lists in the sample's part of the workspace, in entries of 16 bits: list i starts at rank_place(i), a multiple of 8
 __host__ __device__ inline int rank_place(int i, int q, int r, bool each)
@@ -61,7 +61,6 @@ struct RankParams {
     const int64_t *pos_in;
     int S, vis_offset, n_vis, P, n_keep, m; // m: the longest list (n_keep - P, or n_keep when pivots may be text tokens)
     int each;                  // 1: independent pivots (lists of q_i, merged)
-    int bins;
     int stage_entries;         // entries of 16 bits per staging buffer of the turns
     int32_t *out_idx;          // quotas: [B][S_out]; independent pivots: unused
     int64_t *out_pos;
@@ -77,7 +76,7 @@ struct RankShared {
     float red_lo[kRankMaxThreads / 32], red_hi[kRankMaxThreads / 32], red_sum[kRankMaxThreads / 32];
     uint32_t scan[kRankMaxThreads / 32];
     int32_t piv[kRankMaxP];
-    uint32_t n_pivots, last_bin, n_band, biggest, n_list, n_exact, last;
+    uint32_t n_pivots, biggest, n_list, n_below[kRankTries], last;
 };
 
 constexpr int kRankStaticSmem = 8192;
@@ -98,135 +97,114 @@ __device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *per_warp)
     return v + __reduce_add_sync(0xffffffffu, x);
 }
 
-// Phase 1: the list of pivot i of sample b, ranked, into out[0 .. C).  row_s, hist, list: shared memory.
-__device__ __forceinline__ void rank_row(const RankParams &p, const float *__restrict__ row, const int32_t *__restrict__ piv, uint16_t *out,
-                                         int C, float *row_s, uint32_t *hist, unsigned long long *list, RankShared &sh)
+// Phase 1: the list of pivot i of sample b, ranked, into out[0 .. C).  v: the thread's values (tokens 4 (T k + t) ...), pivots and
+// what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per pivot): shared memory.
+constexpr uint32_t kNotAToken = 0xffffffffu; // a NaN that no arithmetic produces: below no threshold
+template <int R>
+__device__ __forceinline__ void rank_row(const float *__restrict__ row, const uint32_t *skip, const float4 (&v)[R], int n, uint16_t *out, int C,
+                                         unsigned long long *list, uint32_t *hist, RankShared &sh)
 {
-    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5, n = p.n_vis, n4 = (n + 3) / 4;
-    const float kNotAToken = __uint_as_float(0xffffffffu); // a pivot, or the filler behind the row: a NaN that no arithmetic produces, in no interval
-    const float4 *row4 = reinterpret_cast<const float4 *>(row_s);
-    // smallest and largest value and the mean (pivots included: they only stretch the range)
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5;
+    // smallest and largest value and the mean (a NaN is passed over)
     float lo = __int_as_float(0x7f800000), hi = __int_as_float(0xff800000), sum = 0.f;
-#pragma unroll 2
-    for (int j = t; j < n4; j += T) {
-        const float4 f = row4[j];
-        lo = fminf(fminf(lo, f.x), fminf(fminf(f.y, f.z), f.w));
-        hi = fmaxf(fmaxf(hi, f.x), fmaxf(fmaxf(f.y, f.z), f.w));
-        sum += (f.x + f.y) + (f.z + f.w);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) lo = fminf(lo, f[e]), hi = fmaxf(hi, f[e]), sum += f[e] == f[e] ? f[e] : 0.f;
     }
     lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
     hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
     sum = warp_sum(sum);
     if (lane == 0) sh.red_lo[warp] = lo, sh.red_hi[warp] = hi, sh.red_sum[warp] = sum;
     __syncthreads();
-    for (int i = t; i < p.P; i += T)
-        if (piv[i] >= 0 && piv[i] < n) row_s[piv[i]] = kNotAToken;
-    if (t < 4 * n4 - n) row_s[n + t] = kNotAToken;
     lo = lane < nwarp ? sh.red_lo[lane] : lo;
     hi = lane < nwarp ? sh.red_hi[lane] : hi;
     sum = warp_sum(lane < nwarp ? sh.red_sum[lane] : 0.f);
     lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
     hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
-    // The bins span [min, 2 mean - min]: a list is the row's low end, and a few large dups - the pivot's own cluster - would
-    // otherwise take most of the bins; if the list reaches beyond, again over [min, max].
-    const float mid = 2.0f * (sum / (float)(4 * n4) - lo);
-    float span = mid > 0.0f && mid < hi - lo ? mid : hi - lo;
-    bool exact = !(hi > lo) || !(hi - lo < 3.0e38f);
-    float scale = 0.f;
-    __syncthreads(); // the pivots are marked
-    const int per = p.bins / T; // bins per thread, a multiple of 4
-    for (int pass = 0; !exact; ++pass) {
-        scale = (float)p.bins / span * 0.9999f; // (places stay below the number of bins for values inside the span)
-        if (!(scale < 3.0e38f)) {
-            exact = true;
-            break;
-        }
-        const float top = (float)p.bins;
-#pragma unroll 2
-        for (int j = t; j < n4; j += T) {
-            const float4 v = row4[j];
-            const float x[4] = {(v.x - lo) * scale, (v.y - lo) * scale, (v.z - lo) * scale, (v.w - lo) * scale};
+    // The first threshold: normal values whose smallest is at its expected place; the quantile by Tukey's approximation
+    // 4.91 (u^0.14 - (1 - u)^0.14).  The next ones move on by what the count says.  Only the number of guesses depends on it.
+    auto quantile = [](float u) { return 4.91f * (__powf(u, 0.14f) - __powf(1.0f - u, 0.14f)); };
+    const float inv_n = 1.0f / (float)n, least = -quantile(0.5f * inv_n), wanted = quantile(fminf((1.3f * (float)C + 40.f) * inv_n, 0.97f));
+    const float mid = sum * inv_n - lo;
+    float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f;
+    bool exact = !(hi > lo) || !(hi - lo < 3.0e38f) || !(mid > 0.0f);
+    int m = 0;
+    reinterpret_cast<uint4 *>(hist)[t] = make_uint4(0, 0, 0, 0);
+    for (int guess = 0; !exact; ++guess) {
+        top = lo + part * mid;
+        if (!(top < hi)) top = hi;
+        uint32_t c = 0;
+#pragma unroll
+        for (int k = 0; k < R; ++k) c += (v[k].x <= top) + (v[k].y <= top) + (v[k].z <= top) + (v[k].w <= top);
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) atomicAdd(&sh.n_below[guess], c);
+        __syncthreads();
+        m = (int)sh.n_below[guess];
+        if (m >= C && m <= 3 * C + 256) break;
+        exact = guess + 1 == kRankTries || (m < C && top == hi);
+        (m < C ? few : many) = part;
+        part += (wanted - quantile(fminf(((float)m + 0.5f) * inv_n, 0.97f))) / least;
+        if (many > 0.f && !(part > 0.9f * few + 0.1f * many && part < 0.1f * few + 0.9f * many)) part = 0.5f * (few + many);
+    }
+    // bins: the low bits of 2^23 + (x - lo) scale, never below 0 or above 4 T - 1
+    const float scale = ((float)(4 * T) - 1.0f) / (top - lo);
+    if (!exact && scale < 3.0e38f) {
+        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(x - lo, scale, 8388608.0f)) - 0x4b000000u); };
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (x[e] < top) atomicAdd(&hist[(int)x[e]], 1u);
+                if (f[e] <= top) atomicAdd(&hist[bin_of(f[e])], 1u);
         }
         __syncthreads();
-        // thread t owns bins [per t, per t + per)
-        uint4 *h4 = reinterpret_cast<uint4 *>(hist) + (size_t)t * (per / 4);
-        uint32_t s = 0;
-        for (int u = 0; u < per / 4; ++u) {
-            const uint4 c = h4[u];
-            s += c.x + c.y + c.z + c.w;
-        }
-        const uint32_t incl = cta_scan(s, sh.scan);
-        uint32_t run = incl - s, big = 0;
-        for (int u = 0; u < per / 4; ++u) {
-            uint4 c = h4[u];
-            uint32_t *cc = reinterpret_cast<uint32_t *>(&c);
+        uint4 *h4 = reinterpret_cast<uint4 *>(hist) + t; // thread t owns bins 4 t ... 4 t + 3
+        const uint4 c = *h4;
+        const uint32_t incl = cta_scan(c.x + c.y + c.z + c.w, sh.scan);
+        uint4 at; // the bins' places
+        at.x = incl - (c.x + c.y + c.z + c.w), at.y = at.x + c.x, at.z = at.y + c.y, at.w = at.z + c.z;
+        *h4 = at;
+        const uint32_t big = max(max(at.x < (uint32_t)C ? c.x : 0u, at.y < (uint32_t)C ? c.y : 0u), max(at.z < (uint32_t)C ? c.z : 0u, at.w < (uint32_t)C ? c.w : 0u));
+        if (__reduce_max_sync(0xffffffffu, big) > kRankMaxBin && lane == 0) sh.biggest = 1;
+        __syncthreads();
+        if (sh.biggest == 0) {
+            // entries behind the bin that completes the list have no place in it
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t k = cc[e];
-                if (run < (uint32_t)C) { // a bin the list needs
-                    big = max(big, k);
-                    if (run + k >= (uint32_t)C) sh.last_bin = (uint32_t)(per * t + 4 * u + e), sh.n_band = run + k;
-                }
-                cc[e] = run; // the bin's place
-                run += k;
-            }
-            h4[u] = c;
-        }
-        big = __reduce_max_sync(0xffffffffu, big);
-        if (lane == 0 && big > kRankMaxBin) sh.biggest = big;
-        if (t == T - 1) sh.n_list = incl;
-        __syncthreads();
-        if (sh.n_list >= (uint32_t)C) {
-            exact = sh.biggest != 0;
-            break;
-        }
-        if (pass == 1 || !(span < hi - lo)) { // values that are not finite
-            exact = true;
-            break;
-        }
-        span = hi - lo;
-        for (int i = t; i < p.bins; i += T) hist[i] = 0;
-        __syncthreads();
-    }
-    if (!exact) {
-        const int m = (int)sh.n_band;
-        const float edge = (float)((int)sh.last_bin + 1);
-#pragma unroll 2
-        for (int j = t; j < n4; j += T) {
-            const float4 v = row4[j];
-            const float f[4] = {v.x, v.y, v.z, v.w};
+            for (int k = 0; k < R; ++k) {
+                const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float x = (f[e] - lo) * scale;
-                if (x < edge) list[atomicAdd(&hist[(int)x], 1u)] = ((unsigned long long)order_key(f[e]) << 32) | (uint32_t)(4 * j + e);
+                for (int e = 0; e < 4; ++e)
+                    if (f[e] <= top) {
+                        const uint32_t place = atomicAdd(&hist[bin_of(f[e])], 1u);
+                        if (place < (uint32_t)C + kRankMaxBin) list[place] = ((unsigned long long)order_key(f[e]) << 32) | (uint32_t)(4 * (T * k + t) + e);
+                    }
             }
+            __syncthreads();
+            // hist[b] is now the end of bin b
+            for (int e = t; e < min(m, C + (int)kRankMaxBin); e += T) {
+                const unsigned long long x = list[e];
+                const int bin = bin_of(order_key_inv((uint32_t)(x >> 32)));
+                int k = bin > 0 ? (int)hist[bin - 1] : 0, r = k;
+                if (k >= C) continue;
+                for (const int end = (int)hist[bin]; k < end; ++k) r += list[k] < x ? 1 : 0;
+                if (r < C) out[r] = (uint16_t)x;
+            }
+            return;
         }
-        __syncthreads();
-        // hist[x] is now the end of bin x
-        for (int e = t; e < m; e += T) {
-            const unsigned long long x = list[e];
-            const int bin = (int)((order_key_inv((uint32_t)(x >> 32)) - lo) * scale);
-            const int end = (int)hist[bin];
-            int u = bin > 0 ? (int)hist[bin - 1] : 0, r = u;
-            for (; u < end; ++u) r += list[u] < x ? 1 : 0;
-            if (r < C) out[r] = (uint16_t)x;
-        }
-        return;
     }
-    // the exact route
+    // the exact route: many equal values, or one that is not finite
     auto keyfn = [&](int j, uint32_t &key) {
-        if (__float_as_uint(row_s[j]) == 0xffffffffu) return false;
-        key = order_key(row_s[j]);
+        if ((skip[j >> 5] >> (j & 31)) & 1u) return false;
+        key = order_key(row[j]);
         return true;
     };
-    if (t == 0) sh.n_exact = 0; // (not n_list: other threads may still be reading it; the selection below synchronises)
+    if (t == 0) sh.n_list = 0;
     uint32_t thr, need_eq, cnt_eq;
     block_select_threshold(CtaGroup(), keyfn, n, (uint32_t)C, sh.sel, thr, need_eq, cnt_eq);
     block_select_apply(CtaGroup(), keyfn, n, thr, need_eq, cnt_eq, sh.sel, [&](int j, uint32_t key) {
-        const uint32_t slot = atomicAdd(&sh.n_exact, 1u);
+        const uint32_t slot = atomicAdd(&sh.n_list, 1u);
         if (slot < (uint32_t)C) list[slot] = ((unsigned long long)key << 32) | (uint32_t)j;
     });
     rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (uint16_t)x; });
@@ -330,6 +308,7 @@ __device__ __forceinline__ int take_turn(const uint16_t *L, int M, int want, uin
     return last;
 }
 
+template <int R>
 __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams p)
 {
     extern __shared__ __align__(16) uint8_t rank_smem[];
@@ -338,34 +317,59 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     const int i = blockIdx.x, b = blockIdx.y;
     const int32_t *piv = sh.piv;
     const float *rows = p.sim + (size_t)b * p.P * n, *row = rows + (size_t)i * n;
-    float *row_s = reinterpret_cast<float *>(rank_smem);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(rank_smem + ((size_t)n * 4 + 15) / 16 * 16);
-    unsigned long long *list = reinterpret_cast<unsigned long long *>(hist + p.bins);
-    for (int k = t; k < p.bins / 4; k += T) reinterpret_cast<uint4 *>(hist)[k] = make_uint4(0, 0, 0, 0);
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(rank_smem);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(list + (p.m + kRankMaxBin + 1) / 2 * 2), *skip = hist + 4 * T;
+    for (int k = t; k < (n + 31) / 32; k += T) skip[k] = 0;
+    if (t < kRankTries) sh.n_below[t] = 0;
     if (t == 0) sh.n_pivots = 0, sh.biggest = 0;
+    __syncthreads();
     wait_for_previous();
     let_next_start();
     if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
-    if ((n & 3) == 0) // rows start on 16-byte boundaries
-        for (int j = t; j < n / 4; j += T) copy_async<16>(row_s + 4 * j, row + 4 * j);
-    else
-        for (int j = t; j < (n + 3) / 4 * 4; j += T) row_s[j] = __ldcs(row + (j < n ? j : 0)); // (filler: a value of the row)
-    copy_async_commit();
-    __syncthreads();
+    float4 v[R];
+    const float none = __uint_as_float(kNotAToken);
+    if ((n & 3) == 0) { // rows start on 16-byte boundaries
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int j = 4 * (T * k + t);
+            v[k] = j < n ? __ldg(reinterpret_cast<const float4 *>(row + j)) : make_float4(none, none, none, none);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int j = 4 * (T * k + t);
+            v[k].x = j < n ? __ldg(row + j) : none;
+            v[k].y = j + 1 < n ? __ldg(row + j + 1) : none;
+            v[k].z = j + 2 < n ? __ldg(row + j + 2) : none;
+            v[k].w = j + 3 < n ? __ldg(row + j + 3) : none;
+        }
+    }
     uint32_t mine = 0;
     for (int k = t; k < p.P; k += T) {
         const int pv = p.pivot_idx[(size_t)b * p.P + k];
         sh.piv[k] = pv;
-        mine += pv >= 0 && pv < n ? 1u : 0u;
+        if (pv >= 0 && pv < n) {
+            atomicOr(&skip[pv >> 5], 1u << (pv & 31));
+            ++mine;
+        }
     }
     if (mine) atomicAdd(&sh.n_pivots, mine);
-    copy_async_wait<0>();
     __syncthreads();
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const int j = 4 * (T * k + t);
+        if (j >= n) break;
+        const uint32_t x = skip[j >> 5] >> (j & 31);
+        if (x & 1u) v[k].x = none;
+        if (x & 2u) v[k].y = none;
+        if (x & 4u) v[k].z = none;
+        if (x & 8u) v[k].w = none;
+    }
     const int Pv = (int)sh.n_pivots, q = (p.n_keep - Pv) / p.P, r = (p.n_keep - Pv) % p.P;
     const bool each = p.each != 0;
     uint16_t *lists = p.lists + (size_t)b * p.sample_entries;
     if (q + (i < r ? 1 : 0) > 0) // (else this pivot keeps nothing, and so do all later ones)
-        rank_row(p, row, piv, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), row_s, hist, list, sh);
+        rank_row<R>(row, skip, v, n, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
     __syncthreads();
     if (t == 0) { // release: the list; acquire: the other pivots' lists
         int before;

@@ -17,6 +17,11 @@ CASES = BAND_CASES + [("gaussian", s) for s in RETENTION_SHAPES] + [
     ("gaussian", (1, 16400, 64, 3, 16384, 2, 4098)),      # the longest row and the longest lists
     ("gaussian", (1, 3000, 64, 0, 2880, 1000, 2000)),     # 1000 pivots: several rounds of staging
     ("equal tokens", (3, 1500, 64, 10, 1402, 32, 1402)),
+    # values per thread: 8, 16, 24 and 32, rows of one quarter more or less, with 64, 128 and 256 threads per list
+    ("gaussian", (150, 600, 64, 3, 512, 8, 60)), ("gaussian", (150, 600, 64, 3, 513, 8, 60)),
+    ("gaussian", (150, 2100, 64, 3, 2048, 8, 300)), ("gaussian", (150, 2100, 64, 3, 2049, 8, 1900)),
+    ("gaussian", (150, 3200, 64, 3, 3072, 8, 9)), ("gaussian", (150, 3200, 64, 3, 3075, 8, 700)),
+    ("gaussian", (150, 4200, 64, 3, 4097, 8, 600)), ("gaussian", (150, 6200, 64, 3, 6146, 8, 600)),
 ]
 
 
