@@ -394,6 +394,22 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int vis_offset, int
                                                          (uint4 *)out_hidden, fs, vis_offset, n_keep);
 }
 
+// Pivots from scores.  Rows of more values than the registers of one CTA hold: radix select, from shared memory where `cached`
+// allows it (the kernel's limit for dynamic shared memory has been raised) and it fits.
+void launch_pivots(const float *score, int B, int n_vis, int P, int smallest, bool cached, int32_t *pivot_idx, cudaStream_t st)
+{
+    using namespace dart;
+    if (n_vis <= kRankMaxVis) {
+        const int threads = n_vis <= 2048 ? 256 : 512, regs = rank_regs(n_vis, threads);
+        launch_next(regs == 2 ? pivot_rank_kernel<2> : regs == 4 ? pivot_rank_kernel<4> : regs == 6 ? pivot_rank_kernel<6> : pivot_rank_kernel<8>, dim3(B), threads,
+                    rank_phase1_bytes(n_vis, P, threads), st, score, n_vis, P, smallest, pivot_idx);
+        return;
+    }
+    const int P_pad = next_pow2(P);
+    cached = cached && n_vis <= kPivotCacheMax;
+    launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st, score, n_vis, P, P_pad, smallest, cached, pivot_idx);
+}
+
 // Step 2 with the caller's pivots: checked and copied into the workspace (with keys: and the text pivots' sums of squares).
 void launch_pivots_given(dart_ctx *ctx, int B, int vis_offset, int n_vis, int P, const dart_opts &o, cudaStream_t st,
                          const uint4 *keys = nullptr, float *text_ssq = nullptr)
@@ -422,10 +438,7 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
         launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
     } else {
         Prof p(ctx, st, SLOT_PIVOT);
-        int P_pad = next_pow2(P);
-        const bool cached = n_vis <= kPivotCacheMax;
-        launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st, o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P,
-                                                                                       P_pad, o.pivot_smallest, cached, ctx->pivot_idx);
+        launch_pivots(o.norm_kind == 2 ? ctx->ssq : ctx->l1, B, n_vis, P, o.pivot_smallest, true, ctx->pivot_idx, st);
     }
     {
         Prof p(ctx, st, SLOT_SIM);
@@ -943,10 +956,7 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
         launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
     } else {
         Prof p(ctx, st, SLOT_PIVOT);
-        const int P_pad = next_pow2(P);
-        const bool cached = n_vis <= kPivotCacheMax;
-        launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, cached), st, o.norm_kind == 2 ? ctx->ssq : ctx->l1, n_vis, P, P_pad,
-                                                                                       o.pivot_smallest, cached, ctx->pivot_idx);
+        launch_pivots(o.norm_kind == 2 ? ctx->ssq : ctx->l1, B, n_vis, P, o.pivot_smallest, true, ctx->pivot_idx, st);
     }
     if (tensor_cores) {
         // the score pass has the rows' sums of squares already, where it read the same tensor
@@ -1483,8 +1493,7 @@ int dart_pivots_static(const void *keys, int B, int S, int d, int vis_offset, in
     float *l1 = scratch, *ssq = scratch + DART_STATIC_MAX_ROWS;
     score_kernel<<<(unsigned)((rows + kScoreWarps - 1) / kScoreWarps), kScoreWarps * 32, 0, st>>>(
         (const uint4 *)keys, S, d / 8, vis_offset, n_vis, rows, l1, ssq);
-    const int P_pad = next_pow2(n_pivot);
-    launch_next(pivot_kernel, dim3(B), kSelectThreads, pivot_smem_bytes(n_vis, P_pad, false), st, l1, n_vis, n_pivot, P_pad, 0, 0, pivot_idx);
+    launch_pivots(l1, B, n_vis, n_pivot, 0, false, pivot_idx, st);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DART_OK : e == cudaErrorMemoryAllocation ? DART_ERR_NOMEM : DART_ERR_CUDA;
 }

@@ -97,43 +97,91 @@ __device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *per_warp)
     return v + __reduce_add_sync(0xffffffffu, x);
 }
 
-// Phase 1: the list of pivot i of sample b, ranked, into out[0 .. C).  v: the thread's values (tokens 4 (T k + t) ...), pivots and
-// what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per pivot): shared memory.
 constexpr uint32_t kNotAToken = 0xffffffffu; // a NaN that no arithmetic produces: below no threshold
+
+// A row's values into registers, sign: 0, or the sign bit to have their negatives
 template <int R>
-__device__ __forceinline__ void rank_row(const float *__restrict__ row, const uint32_t *skip, const float4 (&v)[R], int n, uint16_t *out, int C,
+__device__ __forceinline__ void load_row(const float *__restrict__ row, int n, uint32_t sign, float4 (&v)[R])
+{
+    const int t = threadIdx.x, T = blockDim.x;
+    const float none = __uint_as_float(kNotAToken);
+    auto value = [&](float x) { return __uint_as_float(__float_as_uint(x) ^ sign); };
+    if (((uintptr_t)row & 15u) == 0 && (n & 3) == 0) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int j = 4 * (T * k + t);
+            if (j < n) {
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(row + j));
+                v[k] = make_float4(value(f.x), value(f.y), value(f.z), value(f.w));
+            } else {
+                v[k] = make_float4(none, none, none, none);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int j = 4 * (T * k + t);
+            v[k].x = j < n ? value(__ldg(row + j)) : none;
+            v[k].y = j + 1 < n ? value(__ldg(row + j + 1)) : none;
+            v[k].z = j + 2 < n ? value(__ldg(row + j + 2)) : none;
+            v[k].w = j + 3 < n ? value(__ldg(row + j + 3)) : none;
+        }
+    }
+}
+
+// The C smallest (value, index) pairs of a row, ranked, into out[0 .. C).  v: the thread's values (tokens 4 (T k + t) ...), tokens
+// that do not take part and what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per token that does not
+// take part): shared memory.  flip: 0, or all ones if v holds the row's values with the opposite sign.
+template <int R, bool kOutliers, typename Out>
+__device__ __forceinline__ void rank_row(const float *__restrict__ row, uint32_t flip, const uint32_t *skip, const float4 (&v)[R], int n, Out *out, int C,
                                          unsigned long long *list, uint32_t *hist, RankShared &sh)
 {
     const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5;
-    // smallest and largest value and the mean (a NaN is passed over)
+    // smallest and largest value, and the mean (NaN if a token's value is)
     float lo = __int_as_float(0x7f800000), hi = __int_as_float(0xff800000), sum = 0.f;
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) lo = fminf(lo, f[e]), hi = fmaxf(hi, f[e]), sum += f[e] == f[e] ? f[e] : 0.f;
+        for (int e = 0; e < 4; ++e) lo = fminf(lo, f[e]), hi = fmaxf(hi, f[e]), sum += __float_as_uint(f[e]) != kNotAToken ? f[e] : 0.f;
     }
     lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
     hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
     sum = warp_sum(sum);
     if (lane == 0) sh.red_lo[warp] = lo, sh.red_hi[warp] = hi, sh.red_sum[warp] = sum;
     __syncthreads();
-    lo = lane < nwarp ? sh.red_lo[lane] : lo;
+    lo = lane < nwarp ? sh.red_lo[lane] : __int_as_float(0x7f800000);
     hi = lane < nwarp ? sh.red_hi[lane] : hi;
-    sum = warp_sum(lane < nwarp ? sh.red_sum[lane] : 0.f);
-    lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
-    hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
+    sum = lane < nwarp ? sh.red_sum[lane] : 0.f;
     // The first threshold: normal values whose smallest is at its expected place; the quantile by Tukey's approximation
     // 4.91 (u^0.14 - (1 - u)^0.14).  The next ones move on by what the count says.  Only the number of guesses depends on it.
+    float low, mid; // the minimum and the mean above it
+    int n_of = n;   // of how many values
+    if constexpr (kOutliers) {
+        // ... of the warp with the largest minimum: over all values a few outliers (a sample's largest norms) move them by more than
+        // the others' spread, and 6 to 9 guesses were needed instead of 1 or 2.
+        int n_warp = 0; // values of warp `lane`
+#pragma unroll
+        for (int k = 0; k < R; ++k) n_warp += min(max(n - 4 * (T * k + 32 * lane), 0), 128);
+        const uint32_t high = lo < __int_as_float(0x7f800000) ? order_key(lo) : 0u;
+        const int from = __ffs((int)__ballot_sync(0xffffffffu, high == __reduce_max_sync(0xffffffffu, high))) - 1;
+        low = __shfl_sync(0xffffffffu, lo, from), mid = __shfl_sync(0xffffffffu, sum / (float)n_warp, from) - low;
+        n_of = __shfl_sync(0xffffffffu, n_warp, from);
+        if (__any_sync(0xffffffffu, sum != sum)) mid = __uint_as_float(kNotAToken);
+        lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
+    } else {
+        low = lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(lo)));
+        mid = warp_sum(sum) / (float)n - low;
+    }
+    hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
     auto quantile = [](float u) { return 4.91f * (__powf(u, 0.14f) - __powf(1.0f - u, 0.14f)); };
-    const float inv_n = 1.0f / (float)n, least = -quantile(0.5f * inv_n), wanted = quantile(fminf((1.3f * (float)C + 40.f) * inv_n, 0.97f));
-    const float mid = sum * inv_n - lo;
+    const float inv_n = 1.0f / (float)n, least = -quantile(fminf(0.5f / (float)n_of, 0.25f)), wanted = quantile(fminf((1.3f * (float)C + 40.f) * inv_n, 0.97f));
     float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f;
-    bool exact = !(hi > lo) || !(hi - lo < 3.0e38f) || !(mid > 0.0f);
+    bool has_few = false, has_many = false, exact = !(hi > lo) || !(hi - lo < 3.0e38f) || !(mid > 0.0f);
     int m = 0;
     reinterpret_cast<uint4 *>(hist)[t] = make_uint4(0, 0, 0, 0);
     for (int guess = 0; !exact; ++guess) {
-        top = lo + part * mid;
+        top = low + part * mid;
         if (!(top < hi)) top = hi;
         uint32_t c = 0;
 #pragma unroll
@@ -145,13 +193,14 @@ __device__ __forceinline__ void rank_row(const float *__restrict__ row, const ui
         if (m >= C && m <= 3 * C + 256) break;
         exact = guess + 1 == kRankTries || (m < C && top == hi);
         (m < C ? few : many) = part;
+        (m < C ? has_few : has_many) = true;
         part += (wanted - quantile(fminf(((float)m + 0.5f) * inv_n, 0.97f))) / least;
-        if (many > 0.f && !(part > 0.9f * few + 0.1f * many && part < 0.1f * few + 0.9f * many)) part = 0.5f * (few + many);
+        if (has_few && has_many && !(part > 0.9f * few + 0.1f * many && part < 0.1f * few + 0.9f * many)) part = 0.5f * (few + many);
     }
-    // bins: the low bits of 2^23 + (x - lo) scale, never below 0 or above 4 T - 1
-    const float scale = ((float)(4 * T) - 1.0f) / (top - lo);
+    // bins: the low bits of 2^23 + (x - base) scale, never below 0 or above 4 T - 1; outliers go to the first one
+    const float base = kOutliers && low - lo > top - low && top > low ? low : lo, scale = ((float)(4 * T) - 1.0f) / (top - base);
     if (!exact && scale < 3.0e38f) {
-        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(x - lo, scale, 8388608.0f)) - 0x4b000000u); };
+        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(kOutliers ? fmaxf(x - base, 0.f) : x - base, scale, 8388608.0f)) - 0x4b000000u); };
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
@@ -189,7 +238,7 @@ __device__ __forceinline__ void rank_row(const float *__restrict__ row, const ui
                 int k = bin > 0 ? (int)hist[bin - 1] : 0, r = k;
                 if (k >= C) continue;
                 for (const int end = (int)hist[bin]; k < end; ++k) r += list[k] < x ? 1 : 0;
-                if (r < C) out[r] = (uint16_t)x;
+                if (r < C) out[r] = (Out)(uint32_t)x;
             }
             return;
         }
@@ -197,7 +246,7 @@ __device__ __forceinline__ void rank_row(const float *__restrict__ row, const ui
     // the exact route: many equal values, or one that is not finite
     auto keyfn = [&](int j, uint32_t &key) {
         if ((skip[j >> 5] >> (j & 31)) & 1u) return false;
-        key = order_key(row[j]);
+        key = order_key(row[j]) ^ flip; // (the key of -x is the complement of that of x)
         return true;
     };
     if (t == 0) sh.n_list = 0;
@@ -207,7 +256,7 @@ __device__ __forceinline__ void rank_row(const float *__restrict__ row, const ui
         const uint32_t slot = atomicAdd(&sh.n_list, 1u);
         if (slot < (uint32_t)C) list[slot] = ((unsigned long long)key << 32) | (uint32_t)j;
     });
-    rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (uint16_t)x; });
+    rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (Out)(uint32_t)x; });
 }
 
 // Step 5a (as pack_indices; flags are 0 or 1, 16-byte aligned), a contiguous range of flags per warp: two barriers in all instead of two per blockDim.x flags.
@@ -327,23 +376,8 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     let_next_start();
     if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
     float4 v[R];
+    load_row<R>(row, n, 0u, v);
     const float none = __uint_as_float(kNotAToken);
-    if ((n & 3) == 0) { // rows start on 16-byte boundaries
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int j = 4 * (T * k + t);
-            v[k] = j < n ? __ldg(reinterpret_cast<const float4 *>(row + j)) : make_float4(none, none, none, none);
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int j = 4 * (T * k + t);
-            v[k].x = j < n ? __ldg(row + j) : none;
-            v[k].y = j + 1 < n ? __ldg(row + j + 1) : none;
-            v[k].z = j + 2 < n ? __ldg(row + j + 2) : none;
-            v[k].w = j + 3 < n ? __ldg(row + j + 3) : none;
-        }
-    }
     uint32_t mine = 0;
     for (int k = t; k < p.P; k += T) {
         const int pv = p.pivot_idx[(size_t)b * p.P + k];
@@ -369,7 +403,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     const bool each = p.each != 0;
     uint16_t *lists = p.lists + (size_t)b * p.sample_entries;
     if (q + (i < r ? 1 : 0) > 0) // (else this pivot keeps nothing, and so do all later ones)
-        rank_row<R>(row, skip, v, n, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
+        rank_row<R, false>(row, 0u, skip, v, n, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
     __syncthreads();
     if (t == 0) { // release: the list; acquire: the other pivots' lists
         int before;
@@ -464,6 +498,30 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
                 p.out_pos + (size_t)b * S_out, sh.scan);
     if (p.keep_out)
         for (int j = t; j < n; j += T) p.keep_out[(size_t)b * n + j] = flags[j] != 0;
+}
+
+// Steps 1 and 2's selection, pivots from scores: the P best tokens of a sample in order of (score, index), one CTA per sample, the
+// ranking above over the scores or, where the largest are best, their negatives.  A radix select and a sort
+// (pivot_kernel) are some twenty block-wide steps.  Measured (us, with the copy of the pivots' rows, which starts behind it): 1 x 2880
+// tokens, 128 pivots 26 -> 18; 16 x 1000, 64 pivots 21 -> 17; 256 x 2880, 32 pivots 30 -> 22; 140 x 2880, 128 pivots 36 -> 28.
+template <int R>
+__global__ void __launch_bounds__(kRankMaxThreads) pivot_rank_kernel(const float *__restrict__ score, int n, int P, int smallest, int32_t *__restrict__ pivot_idx)
+{
+    extern __shared__ __align__(16) uint8_t rank_smem[];
+    __shared__ RankShared sh;
+    const int t = threadIdx.x, T = blockDim.x;
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(rank_smem);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(list + (P + kRankMaxBin + 1) / 2 * 2), *skip = hist + 4 * T;
+    for (int k = t; k < (n + 31) / 32; k += T) skip[k] = 0;
+    if (t < kRankTries) sh.n_below[t] = 0;
+    if (t == 0) sh.biggest = 0;
+    __syncthreads();
+    wait_for_previous();
+    let_next_start();
+    const float *row = score + (size_t)blockIdx.x * n;
+    float4 v[R];
+    load_row<R>(row, n, smallest ? 0u : 0x80000000u, v);
+    rank_row<R, true>(row, smallest ? 0u : 0xffffffffu, skip, v, n, pivot_idx + (size_t)blockIdx.x * P, P, list, hist, sh);
 }
 
 } // namespace dart

@@ -56,3 +56,25 @@ def test_ranked_lists_with_independent_pivots(kind, shape):
         got.append([oh.view(-1, d)[:n].view(torch.int16), oi.view(-1)[:n], op.view(-1)[:n], cu, dbg["keep"], dbg["owner"],
                     dbg["eps"].view(torch.int32)])
     assert all(torch.equal(x, y) for x, y in zip(*got))
+
+
+@pytest.mark.parametrize("n,P", [(1, 1), (5, 5), (2048, 8), (2049, 100), (4096, 1024), (4097, 33), (8195, 7), (12289, 1000), (16384, 1), (16385, 40)])
+@pytest.mark.parametrize("values", ["distinct", "few", "equal", "one infinite"])
+def test_ranked_pivots(n, P, values):
+    """Scores that are exact in any order of summation (sums of 64 small whole numbers): a stable sort is the answer."""
+    B, vo = 3, 2
+    g = torch.Generator(device="cuda").manual_seed(n + P)
+    keys = torch.randint(-127, 128, (B, n + 5, 64), generator=g, device="cuda").bfloat16()
+    if values == "few":
+        keys[:, :, 2:] = 1
+        keys[:, :, :2] %= 5
+    elif values == "equal":
+        keys[:] = 3
+    elif values == "one infinite":
+        keys[:, vo + n // 2, 5] = float("inf")
+    got = torch.full((B, P), -1, dtype=torch.int32, device="cuda")
+    assert dart.dart_pivots_static(keys.data_ptr(), B, n + 5, 64, vo, n, P, got.data_ptr(), 0, None) == dart.DART_OK
+    torch.cuda.synchronize()
+    score = keys[:, vo:vo + n].float().abs().sum(-1)
+    want = torch.sort(score, dim=1, descending=True, stable=True).indices[:, :P]
+    assert torch.equal(got.long(), want)
