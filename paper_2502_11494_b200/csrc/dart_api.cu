@@ -282,8 +282,8 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
         rp.len_out = ctx->len, rp.status = ctx->status;
         Prof p(ctx, st, SLOT_RETAIN);
-        const int regs = rank_regs(n_vis, rank_threads);
-        launch_next(regs == 2 ? rank_kernel<2> : regs == 4 ? rank_kernel<4> : regs == 6 ? rank_kernel<6> : rank_kernel<8>, dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
+        const int groups = each || owner_out || eps_out ? 0 : rank_turn_groups(rank_m, rank_m / P);
+        launch_next(rank_kernel_of(rank_regs(n_vis, rank_threads), groups), dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
     };
     if (o.rule == DART_RULE_GLOBAL) { // one threshold for all pivots: a single selection per sample
         Prof p(ctx, st, SLOT_RETAIN);
@@ -1169,11 +1169,9 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
             rc = ws_alloc(ctx, &ctx->rank, ctx->rank_n);
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->rank_arrived, (size_t)desc->B_max);
             const int smem = ctx->max_smem_optin - dart::kRankStaticSmem;
-            if (rc == DART_OK && (cudaFuncSetAttribute(dart::rank_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-                                  cudaFuncSetAttribute(dart::rank_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-                                  cudaFuncSetAttribute(dart::rank_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-                                  cudaFuncSetAttribute(dart::rank_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess))
-                rc = DART_ERR_CUDA;
+            for (int regs = 2; rc == DART_OK && regs <= 8; regs += 2)
+                for (int groups : {0, 1, 2, 4})
+                    if (cudaFuncSetAttribute(dart::rank_kernel_of(regs, groups), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) rc = DART_ERR_CUDA;
         }
     }
     if (rc == DART_OK && desc->P_max > dart::onepass::kGatherMaxP) {

@@ -357,7 +357,60 @@ __device__ __forceinline__ int take_turn(const uint16_t *L, int M, int want, uin
     return last;
 }
 
-template <int R>
+// The same for short lists: 32 kGroups entries at a time, an entry of each group per lane, so that a group takes one vote; the first
+// entries of the next list (or of this one) are on their way while this turn's flags are read.
+template <int kGroups>
+__device__ __forceinline__ void turn_entries(const uint16_t *L, int M, int s, uint32_t none, uint32_t (&j)[kGroups])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < kGroups; ++k) {
+        const int at = s + 32 * k + lane;
+        const uint32_t e = L[min(at, M - 1)];
+        j[k] = at < M ? min(e, none) : none;
+    }
+}
+template <int kGroups>
+__device__ __forceinline__ void take_short_turns(const uint16_t *buf, int k0, int k1, int q, int r, uint8_t *flags, uint32_t none)
+{
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+    const int from = rank_place(k0, q, r, false);
+    const uint16_t *L = buf;
+    int M = rank_length(k0, q, r, false);
+    uint32_t j[kGroups];
+    turn_entries<kGroups>(L, M, 0, none, j);
+    for (int i = k0; i < k1; ++i) {
+        const int i2 = i + 1 < k1 ? i + 1 : i, M2 = rank_length(i2, q, r, false);
+        const uint16_t *L2 = buf + rank_place(i2, q, r, false) - from;
+        int want = q + (i < r ? 1 : 0);
+        for (int s = 0;;) {
+            uint32_t taken[kGroups], next[kGroups];
+#pragma unroll
+            for (int k = 0; k < kGroups; ++k) taken[k] = flags[j[k]];
+            s += 32 * kGroups;
+            const bool more = s < M;
+            turn_entries<kGroups>(more ? L : L2, more ? M : M2, more ? s : 0, none, next);
+            int before = 0;
+#pragma unroll
+            for (int k = 0; k < kGroups; ++k) {
+                const uint32_t free = __ballot_sync(0xffffffffu, taken[k] == 0);
+                if (taken[k] == 0 && before + __popc(free & lt) < want) flags[j[k]] = 1;
+                before += __popc(free);
+            }
+            want -= before;
+            __syncwarp(); // the flags are visible to the next block and the next pivot
+            const bool done = want <= 0 || !more;
+            if (done && more) turn_entries<kGroups>(L2, M2, 0, none, next);
+#pragma unroll
+            for (int k = 0; k < kGroups; ++k) j[k] = next[k];
+            if (done) break;
+        }
+        L = L2, M = M2;
+    }
+}
+
+// kGroups: 0, or the groups of take_short_turns (then neither owners nor a pivot's last dup are wanted, nor `each`)
+template <int R, int kGroups>
 __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams p)
 {
     extern __shared__ __align__(16) uint8_t rank_smem[];
@@ -400,7 +453,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
         if (x & 8u) v[k].w = none;
     }
     const int Pv = (int)sh.n_pivots, q = (p.n_keep - Pv) / p.P, r = (p.n_keep - Pv) % p.P;
-    const bool each = p.each != 0;
+    const bool each = kGroups == 0 && p.each != 0;
     uint16_t *lists = p.lists + (size_t)b * p.sample_entries;
     if (q + (i < r ? 1 : 0) > 0) // (else this pivot keeps nothing, and so do all later ones)
         rank_row<R, false>(row, 0u, skip, v, n, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
@@ -416,8 +469,8 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     // ---- the sample's last CTA: the turns
     uint8_t *flags = rank_smem;
     uint16_t *stage = reinterpret_cast<uint16_t *>(rank_smem + rank_flag_bytes(n));
-    int32_t *owner = p.owner_out ? p.owner_out + (size_t)b * n : nullptr;
-    float *eps = p.eps_out ? p.eps_out + (size_t)b * p.P : nullptr;
+    int32_t *owner = kGroups == 0 && p.owner_out ? p.owner_out + (size_t)b * n : nullptr;
+    float *eps = kGroups == 0 && p.eps_out ? p.eps_out + (size_t)b * p.P : nullptr;
     for (int k = t; k < (n + 16) / 16; k += T) reinterpret_cast<uint4 *>(flags)[k] = make_uint4(0, 0, 0, 0);
     if (owner)
         for (int j = t; j < n; j += T) owner[j] = -1;
@@ -477,15 +530,19 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
         const int k2 = round_end(k1);
         if (warp == 0) {
             const int from = rank_place(k0, q, r, false);
-            for (int k = k0; k < k1; ++k) {
-                const uint16_t *L = buf + rank_place(k, q, r, false) - from;
-                const int M = rank_length(k, q, r, false), want = q + (k < r ? 1 : 0);
-                int last = -1;
-                if (owner || eps)
-                    last = take_turn<true>(L, M, want, flags, (uint32_t)n, owner, k);
-                else
-                    take_turn<false>(L, M, want, flags, (uint32_t)n, nullptr, k);
-                if (eps && t == 0) eps[k] = last >= 0 ? rows[(size_t)k * n + last] : __int_as_float(0x7fc00000);
+            if constexpr (kGroups > 0) {
+                take_short_turns<kGroups>(buf, k0, k1, q, r, flags, (uint32_t)n);
+            } else {
+                for (int k = k0; k < k1; ++k) {
+                    const uint16_t *L = buf + rank_place(k, q, r, false) - from;
+                    const int M = rank_length(k, q, r, false), want = q + (k < r ? 1 : 0);
+                    int last = -1;
+                    if (owner || eps)
+                        last = take_turn<true>(L, M, want, flags, (uint32_t)n, owner, k);
+                    else
+                        take_turn<false>(L, M, want, flags, (uint32_t)n, nullptr, k);
+                    if (eps && t == 0) eps[k] = last >= 0 ? rows[(size_t)k * n + last] : __int_as_float(0x7fc00000);
+                }
             }
         } else if (k2 > k1) {
             fetch(k1, k2, stage + (size_t)((round + 1) & 1) * p.stage_entries, t - 32, T - 32);
@@ -499,6 +556,22 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     if (p.keep_out)
         for (int j = t; j < n; j += T) p.keep_out[(size_t)b * n + j] = flags[j] != 0;
 }
+
+// The form for rows of n_vis values; m: the longest list, q: the quota.  Turns by the longest list and the quota (us for the whole
+// retention, 256 entries at a time / as here): 128 pivots keeping 4 each of lists up to 512 60 / 46, 100 pivots keeping 2 of up
+// to 200 48 / 29, 100 keeping 7 of up to 700 57 / 54, 32 keeping 9 of up to 288 26 / 23; but 36 of up to 1168 33.2 / 35.4, 8 keeping 149 of up to 1192 19 / 21.
+// (Kernels of their own: with all four in one the small cases took 1 to 2 us more, for code that is fetched and not used.)
+using RankKernel = void (*)(RankParams);
+template <int R>
+inline RankKernel rank_kernel_of(int groups)
+{
+    return groups == 0 ? rank_kernel<R, 0> : groups == 1 ? rank_kernel<R, 1> : groups == 2 ? rank_kernel<R, 2> : rank_kernel<R, 4>;
+}
+inline RankKernel rank_kernel_of(int regs, int groups)
+{
+    return regs == 2 ? rank_kernel_of<2>(groups) : regs == 4 ? rank_kernel_of<4>(groups) : regs == 6 ? rank_kernel_of<6>(groups) : rank_kernel_of<8>(groups);
+}
+inline int rank_turn_groups(int m, int q) { return q <= 3 ? 1 : q <= 8 ? 2 : m <= 640 ? 4 : 0; }
 
 // Steps 1 and 2's selection, pivots from scores: the P best tokens of a sample in order of (score, index), one CTA per sample, the
 // ranking above over the scores or, where the largest are best, their negatives.  A radix select and a sort

@@ -78,3 +78,13 @@ def test_ranked_pivots(n, P, values):
     score = keys[:, vo:vo + n].float().abs().sum(-1)
     want = torch.sort(score, dim=1, descending=True, stable=True).indices[:, :P]
     assert torch.equal(got.long(), want)
+
+
+@pytest.mark.parametrize("P,m", [(3, 3), (32, 33), (100, 200), (128, 511), (100, 639), (100, 641), (8, 72), (9, 640), (9, 641), (33, 640), (1, 31), (1, 33), (2, 640)])
+@pytest.mark.parametrize("kind", ["gaussian", "same pivots"])
+def test_turns_over_lists_of_every_length(kind, P, m):
+    """Quotas and lists on both sides of the rule's lines; pivots that rank the tokens alike make every turn walk past the others' picks."""
+    k, h = _band_inputs(kind, 3, 900, 64, 20, 850, P, seed=P + m)
+    a = run_gpu(k, h, 20, 850, P, P + m, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
+    b = run_gpu(k, h, 20, 850, P, P + m, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED, debug=False)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
