@@ -311,7 +311,9 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     // bands / ranked: 256 samples x 32 pivots x 200 tokens 11 / 19, x 576 66 / 69, x 1000 76 / 76; 128 pivots x 576 234 / 289,
     // x 1500 122 / 133, x 2880 488 / 389; 8 pivots x 576 31 / 26, x 2880 60 / 38; one sample, 8 pivots x 2880: 39 / 21)
     const bool prefer_bands = B > ctx->sm_count && P >= 32 && n_vis <= 1536 && can_bands;
-    if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && !prefer_bands))) {
+    // Pivots alone are kept: there is no list, and the sorted lists' second kernel is all there is to run (1 x 200, 32 pivots 11 -> 7 us;
+    // 256 x 1000, 128 pivots 58 -> 9, 33 thousand CTAs that only count themselves).
+    if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && !prefer_bands && m > 0))) {
         launch_ranked();
         return;
     }
@@ -349,7 +351,7 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
             owner_out, eps_out, ctx->status);
         return;
     }
-    const bool two_phase = can_lists && (mode == DART_RETAIN_LISTS || (mode == DART_RETAIN_AUTO && B <= ctx->sm_count));
+    const bool two_phase = can_lists && (mode == DART_RETAIN_LISTS || (mode == DART_RETAIN_AUTO && (B <= ctx->sm_count || m == 0)));
     if (!two_phase) {
         Prof p(ctx, st, SLOT_RETAIN);
         retain_kernel<<<B, kSelectThreads, retain_smem_bytes(n_vis, P), st>>>(ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P,

@@ -88,3 +88,12 @@ def test_turns_over_lists_of_every_length(kind, P, m):
     a = run_gpu(k, h, 20, 850, P, P + m, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
     b = run_gpu(k, h, 20, 850, P, P + m, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED, debug=False)
     assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+
+
+@pytest.mark.parametrize("B", [1, 150])
+def test_only_the_pivots_are_kept(B):
+    k, h = _band_inputs("gaussian", B, 400, 64, 20, 350, 40, seed=B)
+    a = run_gpu(k, h, 20, 350, 40, 40, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
+    b = run_gpu(k, h, 20, 350, 40, 40, path=dart.DART_PATH_STAGED)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+    assert all(np.array_equal(a[3][n], b[3][n], equal_nan=(n == "eps")) for n in a[3])
