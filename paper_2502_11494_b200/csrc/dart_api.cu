@@ -307,13 +307,12 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     const int band_cap = ctx->band_stride < kPickStageEntries ? ctx->band_stride : kPickStageEntries;
     const bool can_bands = ctx->band && m > 0 && m <= band_cap && n_vis <= kBandMaxTokens && band_smem_bytes(n_vis, band_cap) <= (size_t)ctx->max_smem_optin - 2048 &&
                            pick_smem_bytes(n_vis, P) <= (size_t)ctx->max_smem_optin - 2048;
-    // AUTO: ranked lists, except for very many short rows, where one warp per row (bands) is ahead of a CTA's barriers (us,
-    // bands / ranked: 256 samples x 32 pivots x 200 tokens 11 / 19, x 576 66 / 69, x 1000 76 / 76; 128 pivots x 576 234 / 289,
-    // x 1500 122 / 133, x 2880 488 / 389; 8 pivots x 576 31 / 26, x 2880 60 / 38; one sample, 8 pivots x 2880: 39 / 21)
-    const bool prefer_bands = B > ctx->sm_count && P >= 32 && n_vis <= 1536 && can_bands;
+    // AUTO: ranked lists wherever they fit (us, bands / ranked: 256 samples x 32 pivots x 200 tokens keeping 60 58 / 37, x 576 66 / 46,
+    // x 1000 73 / 51; 128 pivots x 576 keeping 300 220 / 181, x 1000 keeping 500 279 / 219, x 1500 keeping 166 122 / 123, keeping 700
+    // 355 / 287, x 2880 410 / 354; 8 pivots x 576 31 / 21, x 2880 58 / 38; one sample, 8 pivots x 2880: 39 / 17)
     // Pivots alone are kept: there is no list, and the sorted lists' second kernel is all there is to run (1 x 200, 32 pivots 11 -> 7 us;
     // 256 x 1000, 128 pivots 58 -> 9, 33 thousand CTAs that only count themselves).
-    if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && !prefer_bands && m > 0))) {
+    if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && m > 0))) {
         launch_ranked();
         return;
     }
@@ -784,12 +783,16 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
 // Given pivots: it reads every row into an SM twice where the one-pass kernel reads it once, but spreads fewer row tiles than SMs
 // over all of them (whole calls, us, flow / one pass: 4 x 2880 x 4096 53 / 57, 16 x 576 x 4096 52 / 59, 8 x 2880 x 4096 79 / 74,
 // 64 x 300 x 2048 57 / 55; 32 pivots, 8 x 1500 x 3072: 77 / 66).
+// 17 to 32 pivots by score on large batches: two passes are ahead where their tiles are full (whole calls, us, flow / two passes:
+// 200 x 700 x 3072 565 / 493, 100 x 1100 x 4096 467 / 447, 200 x 400 x 4096 421 / 404), the flow path where the pairs of 128-row tiles
+// hold half as many rows again (250 x 300 x 4096 424 / 458, 256 x 260 418 / 445, 256 x 150 298 / 311).
 bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
 {
     if (!flow_applies(ctx, B, n_vis, P)) return false;
     const long long bytes = 2ll * ctx->desc.d * n_vis * B;
     const long long row_tiles = (long long)B * ((n_vis + dart::sweep::kTileRows - 1) / dart::sweep::kTileRows);
-    if (o.pivots_in ? (row_tiles >= ctx->sm_count || P > 16) : (P > 16 && bytes > 300000000ll)) return false;
+    const int padded = (n_vis + 255) / 256 * 256; // rows of the one-pass kernel's pairs of tiles
+    if (o.pivots_in ? (row_tiles >= ctx->sm_count || P > 16) : (P > 16 && bytes > 300000000ll && 2 * padded < 3 * n_vis)) return false;
     dart::flow::Params p = {};
     return flow_config(ctx, B, n_vis, P, o, p);
 }
@@ -1072,19 +1075,15 @@ int launch_reduce(dart_ctx *ctx, int B, const void *hidden, const void *keys, co
     // sample 80 us against 103 us, four samples 96 against 107, eight samples 118 against 113).
     if (o.path == DART_PATH_AUTO && B <= 4 && resident_applies(ctx, n_vis, P) && !o.pivots_in)
         return launch_resident(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
-    // AUTO prefers the three launches below to the persistent sweep in two cases.  (1) Samples with more vision tokens
-    // than the sweep's shared-memory score buffer holds: it then selects from global memory and stalls (measured at
-    // 4608 tokens, batch 4: 253 us against 111 us).  (2) 32 pivots or more: the sweep fetches pivot tiles four rows per
-    // TMA op, the one-pass kernel as one box from a compact copy (batch 256: 32 pivots 2.83 -> 2.71 ms, 128 pivots
-    // 6.15 -> 4.65 ms; below that the two are within 1 % of each other at batch 256).  (3) Between half a 128-row tile
-    // and two tiles per SM: the persistent sweep has nothing to overlap a sample's pivot dependency with (measured, us per
-    // step: 8 samples of 2880 tokens 178 -> 165, 12 samples 218 -> 201, 16 samples of 576 tokens 115 -> 104; with fewer
-    // tiles still, the two extra launches cost more: 8 samples of 576 tokens 84 -> 95).
+    // AUTO prefers the launches below to the persistent sweep: with the row tiles' sums of squares from the score pass and the pivots'
+    // rows in one compact copy they read the keys twice at close to the memory's rate (measured, us per call, sweep / two passes:
+    // 64 x 2880 x 4096, 20 pivots 712 / 645, 31 pivots 774 / 659; 256 x 576, 24 pivots 811 / 630; 100 x 1000 x 2048 262 / 242; 17 x 2880
+    // 256 / 230).  Without the copy (a context that has no room for it) the sweep stays where it was measured ahead: samples whose
+    // scores fit its shared memory, fewer than half a 128-row tile or more than two tiles per SM.
     const long long row_tiles = (long long)B * ((n_vis + dart::sweep::kTileRows - 1) / dart::sweep::kTileRows);
     const bool two_pass = o.path == DART_PATH_TWO_PASS ||
                           (o.path == DART_PATH_AUTO && fused_applies(ctx, P) && !o.pivots_in &&
-                           (n_vis > dart::sweep::kSelMax || (P >= 32 && ctx->piv_rows) ||
-                            (2 * row_tiles >= ctx->sm_count && row_tiles < 2ll * ctx->sm_count)));
+                           (n_vis > dart::sweep::kSelMax || ctx->piv_rows || (2 * row_tiles >= ctx->sm_count && row_tiles < 2ll * ctx->sm_count)));
     if (two_pass) {
         if (!fused_applies(ctx, P)) return DART_ERR_UNSUPPORTED;
         const void *k = keys ? keys : hidden;
