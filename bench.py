@@ -40,7 +40,7 @@ def parse():
     ap.add_argument("--keep", type=int, default=None)
     ap.add_argument("--batch", type=int, default=None, help="override the workload's batch size")
     ap.add_argument("--sweep", action="store_true", help="also time every (pivots, keep) cell of the sweep")
-    ap.add_argument("--path", type=int, default=0, help="0 auto, 1 staged, 2 fused (persistent sweep), 3 two passes (score pass + one tensor-core pass), 4 resident sweep, 5 split (resident for a share of the tiles, second read for the rest)")
+    ap.add_argument("--path", type=int, default=0, help="0 auto, 1 staged, 2 fused (persistent sweep), 3 two passes (score pass + one tensor-core pass), 4 resident sweep, 5 split (resident for a share of the tiles, second read for the rest), 6 paired sweeps, 7 flow")
     ap.add_argument("--tune", type=int, default=0, help="path 6: 16 * n1 + n2 ring depths")
     ap.add_argument("--split", type=int, default=0, help="path 5: k keeps tiles with index %% k == 0 on the chip, -k all others")
     ap.add_argument("--lag", type=int, default=0, help="fused path: extra tasks between a row's two sweeps")
@@ -81,6 +81,7 @@ def kernel_bytes_per_launch(name, w, B):
         "sweep": keys,                       # fused scores + pivots + similarities: the keys count once
         "onepass": keys,                     # the caller's pivots: scores + similarities from one pass
         "resident": keys,                    # scores + pivots + similarities, rows held on the chip: one read
+        "flow": keys,                        # flow path: the second read of a row is meant to come from the L2
         "pair": keys,                        # paired sweeps: the second read of a row is meant to come from the L2
         "gather": 2 * (2 * w.d * w.S_out) * B,
         "pivot": 4 * w.n_vis * B,
@@ -92,6 +93,7 @@ def kernel_bytes_per_launch(name, w, B):
 # on the sweep workload at batch 32; traffic is proportional to the batch (every sample is read and written
 # independently), so a launch over B samples moves B times this.
 NCU_TRAFFIC_PER_SAMPLE = {("sweep", 2880, 4096, 8): (1.508338e9 + 8.540928e6) / 32,
+                          ("flow", 2880, 4096, 8): (770.742272e6 + 15.713024e6) / 32,
                           ("onepass", 2880, 4096, 8): (759.286272e6 + 5.440000e6) / 32,
                           ("resident", 2880, 4096, 8): (755.073536e6 + 6.136064e6) / 32}
 

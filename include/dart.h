@@ -54,7 +54,7 @@ enum {
 #define DART_PATH_STAGED 1 /* one kernel per step of the method, every intermediate in the workspace */
 #define DART_PATH_FUSED 2  /* persistent sweep kernel (scores, pivots and similarities in one launch; with the caller's
                               pivots: scores and similarities from one pass over the keys); needs d % 64 == 0 and
-                              n_pivot <= 256, else UNSUPPORTED.  AUTO picks it when it applies. */
+                              n_pivot <= 256, else UNSUPPORTED. */
 #define DART_PATH_TWO_PASS 3 /* two launches instead of the persistent sweep: a plain score pass, pivot selection, then
                               scores' sums of squares and similarities from one tensor-core pass; same limits as FUSED.
                               Reads the keys twice like FUSED but has no waits between CTAs: faster for small batches. */
@@ -62,9 +62,9 @@ enum {
 #define DART_PATH_RESIDENT 4 /* steps 1-3 from ONE read of the keys: every sample is spread over all SMs and stays in their
                               shared and tensor memory until its pivots are known.  Needs n_pivot <= 8, d % 64 == 0,
                               d <= 4096, n_vis <= 32 rows per SM (and the pivots chosen by score, one tensor for
-                              steps 1-3), else UNSUPPORTED.  The fastest path for a few samples (AUTO takes it up to
-                              four); at half the speed of FUSED on the large batched workloads, where the wait for a
-                              sample's pivots is longer than the samples that fit the chip can cover. */
+                              steps 1-3), else UNSUPPORTED.  Faster than FUSED for up to four samples; at half
+                              its speed on the large batched workloads, where the wait for a sample's pivots is longer
+                              than the samples that fit the chip can cover. */
 
 #define DART_PATH_SPLIT 5    /* RESIDENT for a share of every sample's 128-row tiles, one tensor-core pass (as in TWO_PASS)
                               for the others once the pivots are known: the rows that stay on the chip are read once, the
@@ -77,7 +77,8 @@ enum {
 
 #define DART_PATH_FLOW 7     /* steps 1-3 in one persistent launch that keeps the time between a row's two reads, and with it
                               the bytes that pass between them, small enough for the L2 to serve the second.  Needs
-                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, else UNSUPPORTED.  The fastest path up to 16 pivots (AUTO takes it). */
+                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, else UNSUPPORTED.  The fastest path up
+                              to 16 pivots, and up to 32 on small batches (AUTO takes it there). */
 
 /* dart_opts.pivot_source: where step 2 takes the pivots from when the caller does not name them (pivots_in == NULL) */
 #define DART_PIVOTS_BY_SCORE 0 /* the n_pivot vision tokens of best score (dart_reduce) */
