@@ -1070,11 +1070,6 @@ int launch_reduce(dart_ctx *ctx, int B, const void *hidden, const void *keys, co
                                dbg, fused, st);
     if (o.path == DART_PATH_AUTO && flow_preferred(ctx, B, n_vis, P, o))
         return launch_flow(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
-    // AUTO takes the resident sweep for up to four samples: nothing has to be hidden behind other samples there, and
-    // rows that stay on the chip save the second read and most of the sweep's waits (measured, 576 tokens: one
-    // sample 80 us against 103 us, four samples 96 against 107, eight samples 118 against 113).
-    if (o.path == DART_PATH_AUTO && B <= 4 && resident_applies(ctx, n_vis, P) && !o.pivots_in)
-        return launch_resident(ctx, B, hidden, keys, pos_in, vis_offset, n_vis, P, n_keep, out_hidden, out_idx, out_pos, o, dbg, st);
     // AUTO prefers the launches below to the persistent sweep: with the row tiles' sums of squares from the score pass and the pivots'
     // rows in one compact copy they read the keys twice at close to the memory's rate (measured, us per call, sweep / two passes:
     // 64 x 2880 x 4096, 20 pivots 712 / 645, 31 pivots 774 / 659; 256 x 576, 24 pivots 811 / 630; 100 x 1000 x 2048 262 / 242; 17 x 2880

@@ -541,7 +541,7 @@ retain_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_i
 }
 
 // ------------------------------------------------------------------------------------------------
-// Steps 4 and 5a in two phases (the default; retain_kernel above is the plain one-kernel form).
+// Steps 4 and 5a in two phases (retain_kernel above is the plain one-kernel form).
 //
 // Pivot i keeps its q_i not-yet-kept tokens of lowest dup (Eq. 9-10, rank order).  Before its turn at
 // most Q_{i-1} = q_0 + ... + q_{i-1} non-pivot tokens have been kept, so its picks are among the
