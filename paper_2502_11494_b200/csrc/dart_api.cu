@@ -19,6 +19,7 @@ namespace {
 
 constexpr int kSweepChunks = 8;     // column chunks per row tile of the persistent sweep's second pass
 constexpr int kSweepChunkMaxP = 16; // ... for up to this many pivots
+constexpr int kMaxGridY = 65535;    // CUDA's limit for a grid's second dimension
 
 enum Slot { SLOT_SCORE = 0, SLOT_PIVOT, SLOT_SIM, SLOT_RETAIN, SLOT_GATHER, SLOT_SWEEP, SLOT_ONEPASS, SLOT_RESIDENT, SLOT_PAIR, SLOT_FLOW, SLOT_COUNT };
 const char *const kSlotNames[SLOT_COUNT] = {"score", "pivot", "sim", "retain", "gather", "sweep", "onepass", "resident", "pair", "flow"};
@@ -179,8 +180,10 @@ struct Prof {
 
 // Launch behind the kernel before it on the stream, which may still be running (see wait_for_previous): every kernel that is
 // launched this way waits before it reads or writes anything that another one touches.
+// The launch's own result is returned: a kernel that reads indices must not be launched behind one that failed to launch (what a
+// launch leaves unnoticed is found by the call's cudaGetLastError).
 template <typename... KArgs, typename... Args>
-void launch_next(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args)
+cudaError_t launch_next(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args)
 {
     cudaLaunchAttribute attr = {};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -188,7 +191,16 @@ void launch_next(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t s
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid, cfg.blockDim = dim3(threads), cfg.dynamicSmemBytes = smem, cfg.stream = st;
     cfg.attrs = &attr, cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...); // (an error is found by the call's cudaGetLastError)
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Launch behind everything before it on the stream.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_alone(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid, cfg.blockDim = dim3(threads), cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
 bool overlaps(const void *a, size_t na, const void *b, size_t nb)
@@ -242,7 +254,7 @@ int copy_debug(dart_ctx *ctx, int B, int n_vis, int P, const dart_debug *dbg, cu
 
 // Steps 4 and 5a.  Two phases (candidate lists for all pivots at once, then the pivots' turns) when the lists fit
 // the workspace and shared memory, else the one-kernel form.
-void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset, int n_vis, int P, int n_keep,
+int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset, int n_vis, int P, int n_keep,
                       int32_t *out_idx, int64_t *out_pos, const dart_opts &o, const dart_debug *dbg, cudaStream_t st)
 {
     using namespace dart;
@@ -261,7 +273,9 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     int rank_threads = rank_rows <= 2ll * ctx->sm_count ? 512 : rank_rows <= 8ll * ctx->sm_count ? 256 : n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
     while (rank_threads < kRankMaxThreads && 32 * rank_threads < n_vis) rank_threads *= 2; // the row has to fit the registers
     const int rank_m = each ? (m + P - 1) / P : m;
-    bool can_rank = ctx->rank && o.rule != DART_RULE_GLOBAL && n_vis <= kRankMaxVis && rank_m <= kRankMaxList;
+    // the forms with a CTA per (sample, pivot) count the samples in the grid's second dimension
+    const bool grid_fits = B <= kMaxGridY;
+    bool can_rank = ctx->rank && grid_fits && o.rule != DART_RULE_GLOBAL && n_vis <= kRankMaxVis && rank_m <= kRankMaxList;
     if (can_rank) {
         rp.sample_entries = (size_t)rank_place(P, m / P, m % P, each) + 8;
         const size_t flags = rank_flag_bytes(n_vis), phase1 = rank_phase1_bytes(n_vis, rank_m, rank_threads);
@@ -276,36 +290,36 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
         rank_smem = phase1 > flags + avail ? phase1 : flags + avail;
         can_rank = (size_t)B * rp.sample_entries <= ctx->rank_n && rank_smem <= (size_t)ctx->max_smem_optin - kRankStaticSmem;
     }
-    auto launch_ranked = [&]() {
+    auto launch_ranked = [&]() -> cudaError_t {
         rp.sim = ctx->sim, rp.pivot_idx = ctx->pivot_idx, rp.lists = ctx->rank, rp.arrived = ctx->rank_arrived, rp.pos_in = pos_in;
         rp.S = S, rp.vis_offset = vis_offset, rp.n_vis = n_vis, rp.P = P, rp.n_keep = n_keep, rp.m = rank_m, rp.each = each;
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
         rp.len_out = ctx->len, rp.status = ctx->status;
         Prof p(ctx, st, SLOT_RETAIN);
         const int groups = each || owner_out || eps_out ? 0 : rank_turn_groups(rank_m, rank_m / P);
-        launch_next(rank_kernel_of(rank_regs(n_vis, rank_threads), groups), dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
+        return launch_next(rank_kernel_of(rank_regs(n_vis, rank_threads), groups), dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
     };
     if (o.rule == DART_RULE_GLOBAL) { // one threshold for all pivots: a single selection per sample
         Prof p(ctx, st, SLOT_RETAIN);
-        launch_next(retain_global_kernel, dim3(B), kSelectThreads, retain_global_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out,
-            ctx->status);
-        return;
+        DART_CUDA(ctx, launch_next(retain_global_kernel, dim3(B), kSelectThreads, retain_global_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out,
+            ctx->status));
+        return DART_OK;
     }
     if (o.rule == DART_RULE_UNION) { // independent pivots: selections, then index lists at their offsets
         if (can_rank && (mode == DART_RETAIN_AUTO || mode == DART_RETAIN_RANKED)) {
-            launch_ranked();
+            DART_CUDA(ctx, launch_ranked());
         } else {
             Prof p(ctx, st, SLOT_RETAIN);
-            launch_next(retain_union_kernel, dim3(B), kSelectThreads, retain_union_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, owner_out, eps_out, ctx->len, ctx->status);
+            DART_CUDA(ctx, launch_next(retain_union_kernel, dim3(B), kSelectThreads, retain_union_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, S, n_vis, P, n_keep, ctx->keep, owner_out, eps_out, ctx->len, ctx->status));
         }
         Prof p(ctx, st, SLOT_RETAIN);
-        launch_next(pack_varlen_kernel, dim3(B), kWalkThreads, retain_union_smem_bytes(n_vis), st, ctx->keep, ctx->len, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
-                                                                                    out_idx, out_pos, ctx->status);
-        return;
+        DART_CUDA(ctx, launch_next(pack_varlen_kernel, dim3(B), kWalkThreads, retain_union_smem_bytes(n_vis), st, ctx->keep, ctx->len, o.cu_seqlens, pos_in, S, vis_offset, n_vis,
+                                                                                    out_idx, out_pos, ctx->status));
+        return DART_OK;
     }
     // bands: a list must hold the m tokens of the exact route and fit one staging round of phase 2
     const int band_cap = ctx->band_stride < kPickStageEntries ? ctx->band_stride : kPickStageEntries;
-    const bool can_bands = ctx->band && m > 0 && m <= band_cap && n_vis <= kBandMaxTokens && band_smem_bytes(n_vis, band_cap) <= (size_t)ctx->max_smem_optin - 2048 &&
+    const bool can_bands = ctx->band && grid_fits && m > 0 && m <= band_cap && n_vis <= kBandMaxTokens && band_smem_bytes(n_vis, band_cap) <= (size_t)ctx->max_smem_optin - 2048 &&
                            pick_smem_bytes(n_vis, P) <= (size_t)ctx->max_smem_optin - 2048;
     // AUTO: ranked lists wherever they fit (us, bands / ranked: 256 samples x 32 pivots x 200 tokens keeping 60 58 / 37, x 576 66 / 46,
     // x 1000 73 / 51; 128 pivots x 576 keeping 300 220 / 181, x 1000 keeping 500 279 / 219, x 1500 keeping 166 122 / 123, keeping 700
@@ -313,8 +327,8 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     // Pivots alone are kept: there is no list, and the sorted lists' second kernel is all there is to run (1 x 200, 32 pivots 11 -> 7 us;
     // 256 x 1000, 128 pivots 58 -> 9, 33 thousand CTAs that only count themselves).
     if (can_rank && (mode == DART_RETAIN_RANKED || (mode == DART_RETAIN_AUTO && m > 0))) {
-        launch_ranked();
-        return;
+        DART_CUDA(ctx, launch_ranked());
+        return DART_OK;
     }
     const int m_pad = next_pow2(m > 1 ? m : 1);
     // Without them: all forms do the same selections.  One kernel per sample takes B CTAs through P selections each; sorted
@@ -322,7 +336,7 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     // to 4x faster than one kernel); bands need one warp per selection and no sort, which pays once the batch fills the
     // GPU (measured at batch 256: 8 pivots 93 -> 56 us, 32 pivots 0.36 -> 0.16 ms, 128 pivots 1.38 -> 0.49 ms), while for
     // a few samples their turns, one warp per sample, take longer than the sorted lists' walks.
-    const bool can_lists = ctx->cand && m <= ctx->cand_stride && m <= kCandMax &&
+    const bool can_lists = ctx->cand && grid_fits && m <= ctx->cand_stride && m <= kCandMax &&
                                candidates_smem_bytes(n_vis, m_pad) <= (size_t)ctx->max_smem_optin - 2048 &&
                                walk_smem_bytes(n_vis) <= (size_t)ctx->max_smem_optin - 2048;
     // ... and both phases of the bands in one launch for batches that cannot fill the GPU: as many band-building warps as
@@ -334,44 +348,43 @@ void launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offse
     // band-building warps the lists stay ahead: 16 pivots, 8 samples of 2880 tokens 45 vs 55; 32 pivots, 4 samples 66 vs 123)
     if (can_fused && (mode == DART_RETAIN_FUSED || (mode == DART_RETAIN_AUTO && B <= ctx->sm_count && P <= band_warps))) {
         Prof p(ctx, st, SLOT_RETAIN);
-        retain_fused_kernel<<<B, kPickThreads, retain_fused_smem_bytes(n_vis, P, band_cap, band_warps), st>>>(
+        DART_CUDA(ctx, launch_alone(retain_fused_kernel, dim3(B), kPickThreads, retain_fused_smem_bytes(n_vis, P, band_cap, band_warps), st,
             ctx->sim, ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos,
-            keep_out, owner_out, eps_out, ctx->status, band_warps);
-        return;
+            keep_out, owner_out, eps_out, ctx->status, band_warps));
+        return DART_OK;
     }
     const bool bands = can_bands && (mode == DART_RETAIN_BANDS || (mode == DART_RETAIN_AUTO && (B > ctx->sm_count || !can_lists)));
     if (bands) {
         {
             Prof p(ctx, st, SLOT_RETAIN);
-            launch_next(band_kernel, dim3((unsigned)P, (unsigned)B), 32, band_smem_bytes(n_vis, band_cap), st, ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, band_cap, ctx->band, ctx->band_n, ctx->status);
+            DART_CUDA(ctx, launch_next(band_kernel, dim3((unsigned)P, (unsigned)B), 32, band_smem_bytes(n_vis, band_cap), st, ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, band_cap, ctx->band, ctx->band_n, ctx->status));
         }
         Prof p(ctx, st, SLOT_RETAIN);
-        launch_next(retain_pick_kernel, dim3(B), kPickThreads, pick_smem_bytes(n_vis, P), st, ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out,
-            owner_out, eps_out, ctx->status);
-        return;
+        DART_CUDA(ctx, launch_next(retain_pick_kernel, dim3(B), kPickThreads, pick_smem_bytes(n_vis, P), st, ctx->pivot_idx, ctx->band, ctx->band_n, band_cap, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out,
+            owner_out, eps_out, ctx->status));
+        return DART_OK;
     }
     const bool two_phase = can_lists && (mode == DART_RETAIN_LISTS || (mode == DART_RETAIN_AUTO && (B <= ctx->sm_count || m == 0)));
     if (!two_phase) {
         Prof p(ctx, st, SLOT_RETAIN);
-        retain_kernel<<<B, kSelectThreads, retain_smem_bytes(n_vis, P), st>>>(ctx->sim, ctx->pivot_idx, pos_in, S, vis_offset, n_vis, P,
-                                                               n_keep, out_idx, out_pos, keep_out, owner_out,
-                                                               eps_out, ctx->status, retain_cache_rows(n_vis, P));
-        return;
+        DART_CUDA(ctx, launch_alone(retain_kernel, dim3(B), kSelectThreads, retain_smem_bytes(n_vis, P), st, ctx->sim, ctx->pivot_idx, pos_in, S,
+            vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out, ctx->status, retain_cache_rows(n_vis, P)));
+        return DART_OK;
     }
     if (m > 0) {
         Prof p(ctx, st, SLOT_RETAIN);
         // one CTA per SM at most: big CTAs shorten each selection; more CTAs than SMs: small ones overlap better
         // (measured: 8 x 16 lists 67 -> 54 us with 1024 threads, 64 x 8 lists 36 -> 45 us)
         const int threads = (long long)B * P <= ctx->sm_count ? kCandThreads : 256;
-        candidates_kernel<<<dim3((unsigned)P, (unsigned)B), threads, candidates_smem_bytes(n_vis, m_pad), st>>>(
-            ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, m_pad, ctx->cand_stride, ctx->cand, ctx->status);
+        DART_CUDA(ctx, launch_alone(candidates_kernel, dim3((unsigned)P, (unsigned)B), threads, candidates_smem_bytes(n_vis, m_pad), st,
+            ctx->sim, ctx->pivot_idx, n_vis, P, n_keep, m_pad, ctx->cand_stride, ctx->cand, ctx->status));
     }
     {
         Prof p(ctx, st, SLOT_RETAIN);
-        retain_walk_kernel<<<B, kWalkThreads, walk_smem_bytes(n_vis), st>>>(ctx->sim, ctx->pivot_idx, ctx->cand, ctx->cand_stride, pos_in,
-                                                                          S, vis_offset, n_vis, P, n_keep, out_idx, out_pos,
-                                                                          keep_out, owner_out, eps_out, ctx->status);
+        DART_CUDA(ctx, launch_alone(retain_walk_kernel, dim3(B), kWalkThreads, walk_smem_bytes(n_vis), st, ctx->sim, ctx->pivot_idx, ctx->cand,
+            ctx->cand_stride, pos_in, S, vis_offset, n_vis, P, n_keep, out_idx, out_pos, keep_out, owner_out, eps_out, ctx->status));
     }
+    return DART_OK;
 }
 
 // Step 5b.  With independent pivots the rows are packed at the samples' offsets (cu_seqlens) instead of B equal blocks.
@@ -446,11 +459,12 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
         size_t smem = (size_t)kSimPivotChunk * d8 * 16;
         dim3 grid((n_vis + kSimRowsPerCta - 1) / kSimRowsPerCta, B);
         for (int p0 = 0; p0 < P; p0 += kSimPivotChunk)
-            sim_alu_kernel<<<grid, kSimWarps * 32, smem, st>>>(keys, S, d8, vis_offset, n_vis, P, p0, ctx->pivot_idx,
-                                                              ctx->ssq, ctx->sim);
+            DART_CUDA(ctx, launch_alone(sim_alu_kernel, grid, kSimWarps * 32, smem, st, keys, S, d8, vis_offset, n_vis, P, p0, ctx->pivot_idx,
+                                        ctx->ssq, ctx->sim));
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -653,7 +667,8 @@ int launch_fused(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, 
         else
             sim_sum_kernel<float><<<grid, kSimSumThreads, 0, st>>>(ctx->sim_share, items, p.n_kc, ctx->sim);
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -830,7 +845,11 @@ int launch_flow(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         // every CTA waits for scores that the others publish: co-residency is required
         DART_CUDA(ctx, cudaLaunchCooperativeKernel(fn, dim3((unsigned)ctx->sm_count), dim3((unsigned)F::threads(NT)), args, smem, st));
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) {
+        flow_reset(ctx, st); // the gather that puts the words back is not launched, and a graph captured earlier would find them
+        return kept;
+    }
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st, true);
     DART_CUDA(ctx, cudaGetLastError());
     ctx->flow_dirty = false;
@@ -876,7 +895,8 @@ int launch_resident(dart_ctx *ctx, int B, const void *hidden, const void *keys_i
         int rc = launch_onepass_kernel(ctx, B, p.keys, true, vis_offset, n_vis, P, o, st, split);
         if (rc != DART_OK) return rc;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -919,7 +939,8 @@ int launch_pair(dart_ctx *ctx, int B, const void *hidden, const void *keys_in, c
         DART_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)Q::pair_kernel, dim3(grid), dim3(Q::kThreads), args,
                                                    Q::smem_bytes(P, p.row_bytes, (int)grid, p.n1, p.n2, p.n3), st));
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -933,7 +954,8 @@ int launch_onepass(dart_ctx *ctx, int B, const void *hidden, const void *keys_in
     launch_pivots_given(ctx, B, vis_offset, n_vis, P, o, st);
     int rc = launch_onepass_kernel(ctx, B, keys_in ? keys_in : hidden, !(dbg && dbg->l1), vis_offset, n_vis, P, o, st); // (L1 scores rank nothing here)
     if (rc != DART_OK) return rc;
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);
@@ -979,11 +1001,12 @@ int launch_two_pass(dart_ctx *ctx, int B, const void *hidden, const void *keys, 
         const size_t smem = (size_t)kSimPivotChunk * d8 * 16;
         const dim3 grid((n_vis + kSimRowsPerCta - 1) / kSimRowsPerCta, B);
         for (int p0 = 0; p0 < P; p0 += kSimPivotChunk)
-            sim_alu_kernel<<<grid, kSimWarps * 32, smem, st>>>((const uint4 *)sim_src, S, d8, vis_offset, n_vis, P, p0,
-                                                              ctx->pivot_idx, ctx->ssq, ctx->sim);
+            DART_CUDA(ctx, launch_alone(sim_alu_kernel, grid, kSimWarps * 32, smem, st, (const uint4 *)sim_src, S, d8, vis_offset, n_vis, P, p0,
+                                        ctx->pivot_idx, ctx->ssq, ctx->sim));
         ctx->launches += (P - 1) / kSimPivotChunk;
     }
-    launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    const int kept = launch_retention(ctx, B, pos_in, vis_offset, n_vis, P, n_keep, out_idx, out_pos, o, dbg, st);
+    if (kept != DART_OK) return kept;
     launch_gather(ctx, B, hidden, vis_offset, n_vis, n_keep, out_idx, out_hidden, o, st);
     DART_CUDA(ctx, cudaGetLastError());
     return copy_debug(ctx, B, n_vis, P, dbg, st);

@@ -97,3 +97,28 @@ def test_only_the_pivots_are_kept(B):
     b = run_gpu(k, h, 20, 350, 40, 40, path=dart.DART_PATH_STAGED)
     assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
     assert all(np.array_equal(a[3][n], b[3][n], equal_nan=(n == "eps")) for n in a[3])
+
+
+@pytest.mark.parametrize("rule", [dart.DART_RULE_QUOTAS, dart.DART_RULE_UNION], ids=["quotas", "independent"])
+@pytest.mark.parametrize("retention", range(6))
+def test_more_samples_than_a_grid_has_rows(rule, retention):
+    """65535 is the most a grid's second dimension takes: the forms that count samples there give way to those that do not."""
+    B, S, d, vo, nv, P, Kp = 65537, 20, 64, 2, 16, 2, 6
+    k, _ = _band_inputs("gaussian", B, S, d, vo, nv, P, seed=7)
+    S_out = S - nv + Kp
+    got = []
+    for parts in ([(0, B)], [(0, 40000), (40000, B)]):
+        rows, lengths = [], []
+        ctx = dart.Dart(B, S, d, P, Kp)
+        for lo, hi in parts:
+            cu = torch.zeros(hi - lo + 1, dtype=torch.int32, device="cuda")
+            opts = dart.dart_opts(retention=retention, rule=rule, cu_seqlens=cu.data_ptr() if rule == dart.DART_RULE_UNION else None)
+            oh, oi, op = ctx.reduce(k[lo:hi], None, vo, nv, P, Kp, opts=opts)
+            torch.cuda.synchronize()
+            assert ctx.status() == dart.DART_OK
+            n = int(cu[-1]) if rule == dart.DART_RULE_UNION else (hi - lo) * S_out
+            rows.append((oh.view(-1, d)[:n].view(torch.int16), oi.view(-1)[:n], op.view(-1)[:n]))
+            lengths.append(cu.diff())
+        ctx.close()
+        got.append([torch.cat(x) for x in zip(*rows)] + [torch.cat(lengths)])
+    assert all(torch.equal(x, y) for x, y in zip(*got))
