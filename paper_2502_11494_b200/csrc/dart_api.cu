@@ -404,7 +404,7 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int vis_offset, int
         launch_next(gather_varlen_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
                                                                 ctx->status, (uint4 *)out_hidden, fs);
     else
-        launch_next(gather_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
+        launch_next(gather_kernel<false>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
                                                          (uint4 *)out_hidden, fs, vis_offset, n_keep);
 }
 
@@ -1527,7 +1527,7 @@ int dart_gather_rows(const void *src, const int32_t *idx, int B, int S, int S_ou
     using namespace dart;
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
-    launch_next(gather_kernel, dim3(grid), kGatherWarps * 32, 0, (cudaStream_t)stream, (const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
+    launch_next(gather_kernel<true>, dim3(grid), kGatherWarps * 32, 0, (cudaStream_t)stream, (const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
                                                                        nullptr, (uint4 *)out, FlowState{}, 0, S_out);
     return cudaGetLastError() == cudaSuccess ? DART_OK : DART_ERR_CUDA;
 }

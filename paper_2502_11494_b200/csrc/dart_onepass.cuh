@@ -189,7 +189,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int i = min(4 * (lane + 32 * k) + e, p.P - 1); // ranks beyond P repeat the last pivot
-                        my_piv[k][e] = b * p.S + min(max(p.vis_offset + __ldg(p.pivot_idx + (size_t)b * p.P + i), 0), p.S - 1); // any row of the sample
+                        my_piv[k][e] = b * p.S + min(max(p.vis_offset + __ldcg(p.pivot_idx + (size_t)b * p.P + i), 0), p.S - 1); // any row of the sample
                     }
                 cur_b = b;
             }
@@ -349,7 +349,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                 norm_b = b;
 #pragma unroll
                 for (int k = 0; k < kMaxN / 32; ++k)
-                    if (lane + 32 * k < p.P) piv_norm[k] = sqrtf(__ldg(p.piv_ssq + (size_t)b * p.P + lane + 32 * k));
+                    if (lane + 32 * k < p.P) piv_norm[k] = sqrtf(__ldcg(p.piv_ssq + (size_t)b * p.P + lane + 32 * k));
             }
             if (kNorms) {
                 ok = ctl.wait_bar(smem_u32(&sh.norm_full[acc]), (n >> 1) & 1u, kWaitNormFull, g);
@@ -365,7 +365,7 @@ onepass_kernel(const __grid_constant__ CUtensorMap tm_tile, const __grid_constan
                     }
             } else {
                 for (int w = 0; w < p.tg; ++w)
-                    if (row < tile_rows(rt, w)) row_ssq[w] = __ldg(p.ssq + (size_t)b * p.n_vis + (rt + w) * kTileRows + row);
+                    if (row < tile_rows(rt, w)) row_ssq[w] = __ldcg(p.ssq + (size_t)b * p.n_vis + (rt + w) * kTileRows + row);
             }
             if (ok) ok = ctl.wait_bar(smem_u32(&sh.tmem_full[acc]), (n >> 1) & 1u, kWaitAccumFull1, g);
             if (!__all_sync(0xffffffffu, ok)) break;

@@ -101,7 +101,7 @@ constexpr uint32_t kNotAToken = 0xffffffffu; // a NaN that no arithmetic produce
 
 // A row's values into registers, sign: 0, or the sign bit to have their negatives
 template <int R>
-__device__ __forceinline__ void load_row(const float *__restrict__ row, int n, uint32_t sign, float4 (&v)[R])
+__device__ __forceinline__ void load_row(const float *row, int n, uint32_t sign, float4 (&v)[R])
 {
     const int t = threadIdx.x, T = blockDim.x;
     const float none = __uint_as_float(kNotAToken);
@@ -111,7 +111,7 @@ __device__ __forceinline__ void load_row(const float *__restrict__ row, int n, u
         for (int k = 0; k < R; ++k) {
             const int j = 4 * (T * k + t);
             if (j < n) {
-                const float4 f = __ldg(reinterpret_cast<const float4 *>(row + j));
+                const float4 f = *reinterpret_cast<const float4 *>(row + j);
                 v[k] = make_float4(value(f.x), value(f.y), value(f.z), value(f.w));
             } else {
                 v[k] = make_float4(none, none, none, none);
@@ -121,10 +121,10 @@ __device__ __forceinline__ void load_row(const float *__restrict__ row, int n, u
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const int j = 4 * (T * k + t);
-            v[k].x = j < n ? value(__ldg(row + j)) : none;
-            v[k].y = j + 1 < n ? value(__ldg(row + j + 1)) : none;
-            v[k].z = j + 2 < n ? value(__ldg(row + j + 2)) : none;
-            v[k].w = j + 3 < n ? value(__ldg(row + j + 3)) : none;
+            v[k].x = j < n ? value(row[j]) : none;
+            v[k].y = j + 1 < n ? value(row[j + 1]) : none;
+            v[k].z = j + 2 < n ? value(row[j + 2]) : none;
+            v[k].w = j + 3 < n ? value(row[j + 3]) : none;
         }
     }
 }
@@ -133,7 +133,7 @@ __device__ __forceinline__ void load_row(const float *__restrict__ row, int n, u
 // that do not take part and what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per token that does not
 // take part): shared memory.  flip: 0, or all ones if v holds the row's values with the opposite sign.
 template <int R, bool kOutliers, typename Out>
-__device__ __forceinline__ void rank_row(const float *__restrict__ row, uint32_t flip, const uint32_t *skip, const float4 (&v)[R], int n, Out *out, int C,
+__device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const uint32_t *skip, const float4 (&v)[R], int n, Out *out, int C,
                                          unsigned long long *list, uint32_t *hist, RankShared &sh)
 {
     const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5;
@@ -578,7 +578,7 @@ inline int rank_turn_groups(int m, int q) { return q <= 3 ? 1 : q <= 8 ? 2 : m <
 // (pivot_kernel) are some twenty block-wide steps.  Measured (us, with the copy of the pivots' rows, which starts behind it): 1 x 2880
 // tokens, 128 pivots 26 -> 18; 16 x 1000, 64 pivots 21 -> 17; 256 x 2880, 32 pivots 30 -> 22; 140 x 2880, 128 pivots 36 -> 28.
 template <int R>
-__global__ void __launch_bounds__(kRankMaxThreads) pivot_rank_kernel(const float *__restrict__ score, int n, int P, int smallest, int32_t *__restrict__ pivot_idx)
+__global__ void __launch_bounds__(kRankMaxThreads) pivot_rank_kernel(const float *score, int n, int P, int smallest, int32_t *__restrict__ pivot_idx)
 {
     extern __shared__ __align__(16) uint8_t rank_smem[];
     __shared__ RankShared sh;

@@ -98,7 +98,7 @@ __device__ __forceinline__ void cta_smallest_k(KeyFn keyfn, int n, int k, int k_
 }
 
 __global__ void __launch_bounds__(kSelectThreads)
-pivot_kernel(const float *__restrict__ score, int n_vis, int P, int P_pad, int smallest, int cached,
+pivot_kernel(const float *score, int n_vis, int P, int P_pad, int smallest, int cached,
              int32_t *__restrict__ pivot_idx)
 {
     wait_for_previous();
@@ -133,7 +133,7 @@ pivot_kernel(const float *__restrict__ score, int n_vis, int P, int P_pad, int s
 // as indices relative to the vision block (a text token before it is negative, one after it >= n_vis).
 //   score_vis [B][n_vis]; score_before [B][vis_offset]; score_after [B][S - vis_offset - n_vis]
 __global__ void __launch_bounds__(kSelectThreads)
-pivot_mixed_kernel(const float *__restrict__ score_vis, const float *__restrict__ score_before, const float *__restrict__ score_after,
+pivot_mixed_kernel(const float *score_vis, const float *score_before, const float *score_after,
                    int S, int vis_offset, int n_vis, int Pv, int Pt, int P_pad, int smallest, int32_t *__restrict__ pivot_idx)
 {
     wait_for_previous();
@@ -205,7 +205,7 @@ constexpr int kSimRowsPerCta = 64;
 
 __global__ void __launch_bounds__(kSimWarps * 32)
 sim_alu_kernel(const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, int P, int p0,
-               const int32_t *__restrict__ pivot_idx, const float *__restrict__ ssq, float *__restrict__ sim)
+               const int32_t *pivot_idx, const float *ssq, float *__restrict__ sim)
 {
     wait_for_previous();
     let_next_start();
@@ -217,7 +217,7 @@ sim_alu_kernel(const uint4 *__restrict__ keys, int S, int d8, int vis_offset, in
     // a pivot outside [0, n_vis) is a text token of the same sample (checked and clamped to the sample by step 2)
     for (int i = threadIdx.x; i < kSimPivotChunk * d8; i += blockDim.x) {
         int p = i / d8, c = i - p * d8;
-        piv_rows[i] = (p < np) ? __ldg(base + (long long)pivot_idx[(size_t)b * P + p0 + p] * d8 + c)
+        piv_rows[i] = (p < np) ? base[(long long)pivot_idx[(size_t)b * P + p0 + p] * d8 + c]
                                : make_uint4(0, 0, 0, 0);
     }
     __syncthreads();
@@ -306,8 +306,8 @@ constexpr int kCheckPivotsGiven = 100; // second status word: which check failed
 // [lo, hi) is the range a pivot may lie in, relative to the vision block: [0, n_vis), or the whole sequence
 // [-vis_offset, S - vis_offset) when text tokens may serve as pivots (Sec. 5.4).
 __global__ void __launch_bounds__(256)
-pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P, int32_t *__restrict__ pivot_idx, int *status,
-                    const uint4 *__restrict__ keys, int S, int d8, int vis_offset, int n_vis, float *__restrict__ text_ssq)
+pivots_given_kernel(const int32_t *pivots_in, int lo, int hi, int P, int32_t *__restrict__ pivot_idx, int *status,
+                    const uint4 *keys, int S, int d8, int vis_offset, int n_vis, float *__restrict__ text_ssq)
 {
     wait_for_previous();
     let_next_start();
@@ -336,7 +336,7 @@ pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P
         const uint4 *row = keys + ((size_t)b * S + vis_offset + c) * (size_t)d8;
         float q = 0.f;
         for (int k = lane; k < d8; k += 32) {
-            const uint4 v = __ldg(row + k);
+            const uint4 v = row[k];
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -357,7 +357,7 @@ pivots_given_kernel(const int32_t *__restrict__ pivots_in, int lo, int hi, int P
 constexpr int kPivotRowWarps = 8;
 
 __global__ void __launch_bounds__(kPivotRowWarps * 32)
-pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *__restrict__ pivot_idx, int S, int d8, int vis_offset, int n_vis,
+pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *pivot_idx, int S, int d8, int vis_offset, int n_vis,
                   int P, int N, long long rows_total, uint4 *__restrict__ out, float *__restrict__ piv_ssq)
 {
     wait_for_previous();
@@ -377,7 +377,7 @@ pivot_rows_kernel(const uint4 *__restrict__ keys, const int32_t *__restrict__ pi
     float q0 = 0.f, q1 = 0.f;
 #pragma unroll 4
     for (int c = lane; c < d8; c += 32) {
-        const uint4 v = __ldg(src + c);
+        const uint4 v = src[c];
         if (dst) dst[c] = v;
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -483,11 +483,11 @@ inline size_t retain_smem_bytes(int n_vis, int P)
 }
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSelectThreads)
-retain_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, const int64_t *__restrict__ pos_in,
+retain_kernel(const float *sim, const int32_t *pivot_idx, const int64_t *__restrict__ pos_in,
               int S, int vis_offset, int n_vis, int P, int n_keep,
               int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
               uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
-              const int *__restrict__ status, int cache_rows)
+              const int *status, int cache_rows)
 {
     wait_for_previous();
     let_next_start();
@@ -570,8 +570,8 @@ inline size_t candidates_smem_bytes(int n_vis, int m_pad)
 inline size_t walk_smem_bytes(int n_vis) { return ((size_t)n_vis + 15) / 16 * 16 + (size_t)kWalkStageEntries * 4; }
 
 __global__ void __launch_bounds__(kCandThreads)
-candidates_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, int n_vis, int P, int n_keep,
-                  int m_pad, int cand_stride, int32_t *__restrict__ cand, const int *__restrict__ status)
+candidates_kernel(const float *sim, const int32_t *pivot_idx, int n_vis, int P, int n_keep,
+                  int m_pad, int cand_stride, int32_t *__restrict__ cand, const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -634,10 +634,10 @@ candidates_kernel(const float *__restrict__ sim, const int32_t *__restrict__ piv
 }
 
 __global__ void __launch_bounds__(kWalkThreads)
-retain_walk_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, const int32_t *__restrict__ cand,
+retain_walk_kernel(const float *sim, const int32_t *pivot_idx, const int32_t *cand,
                    int cand_stride, const int64_t *__restrict__ pos_in, int S, int vis_offset, int n_vis, int P, int n_keep,
                    int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos, uint8_t *__restrict__ keep_out,
-                   int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *__restrict__ status)
+                   int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -979,8 +979,8 @@ __device__ void band_of_row(const float *__restrict__ row, const int32_t *__rest
 }
 
 __global__ void __launch_bounds__(32)
-band_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, int n_vis, int P, int n_keep, int stride,
-            unsigned long long *__restrict__ band, int32_t *__restrict__ band_n, const int *__restrict__ status)
+band_kernel(const float *sim, const int32_t *pivot_idx, int n_vis, int P, int n_keep, int stride,
+            unsigned long long *__restrict__ band, int32_t *__restrict__ band_n, const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -1181,11 +1181,11 @@ __device__ void pick_sample(const int b, const int32_t *__restrict__ pivot_idx, 
 }
 
 __global__ void __launch_bounds__(kPickThreads)
-retain_pick_kernel(const int32_t *__restrict__ pivot_idx, const unsigned long long *__restrict__ band,
-                   const int32_t *__restrict__ band_n, int stride, const int64_t *__restrict__ pos_in, int S, int vis_offset,
+retain_pick_kernel(const int32_t *pivot_idx, const unsigned long long *band,
+                   const int32_t *band_n, int stride, const int64_t *__restrict__ pos_in, int S, int vis_offset,
                    int n_vis, int P, int n_keep, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
                    uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
-                   const int *__restrict__ status)
+                   const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -1210,10 +1210,10 @@ inline size_t retain_fused_smem_bytes(int n_vis, int P, int stride, int band_war
     return ((size_t)n_vis + 15) / 16 * 16 + ((size_t)P * 4 + 15) / 16 * 16 + (phase1 > phase2 ? phase1 : phase2);
 }
 __global__ void __launch_bounds__(kPickThreads)
-retain_fused_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, unsigned long long *__restrict__ band,
+retain_fused_kernel(const float *sim, const int32_t *pivot_idx, unsigned long long *__restrict__ band,
                     int32_t *__restrict__ band_n, int stride, const int64_t *__restrict__ pos_in, int S, int vis_offset, int n_vis,
                     int P, int n_keep, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos, uint8_t *__restrict__ keep_out,
-                    int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *__restrict__ status, int band_warps)
+                    int32_t *__restrict__ owner_out, float *__restrict__ eps_out, const int *status, int band_warps)
 {
     wait_for_previous();
     let_next_start();
@@ -1248,11 +1248,11 @@ retain_fused_kernel(const float *__restrict__ sim, const int32_t *__restrict__ p
 inline size_t retain_global_smem_bytes(int n_vis) { return ((size_t)n_vis + 15) / 16 * 16 + (size_t)n_vis * 4; }
 
 __global__ void __launch_bounds__(kSelectThreads)
-retain_global_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, const int64_t *__restrict__ pos_in,
+retain_global_kernel(const float *sim, const int32_t *pivot_idx, const int64_t *__restrict__ pos_in,
                      int S, int vis_offset, int n_vis, int P, int n_keep,
                      int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
                      uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
-                     const int *__restrict__ status)
+                     const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -1322,9 +1322,9 @@ constexpr int kGatherWarps = 8; // warps per CTA of the gather kernels, one outp
 inline size_t retain_union_smem_bytes(int n_vis) { return ((size_t)n_vis + 15) / 16 * 16; }
 
 __global__ void __launch_bounds__(kSelectThreads)
-retain_union_kernel(const float *__restrict__ sim, const int32_t *__restrict__ pivot_idx, int S, int n_vis, int P, int n_keep,
+retain_union_kernel(const float *sim, const int32_t *pivot_idx, int S, int n_vis, int P, int n_keep,
                     uint8_t *__restrict__ keep_out, int32_t *__restrict__ owner_out, float *__restrict__ eps_out,
-                    int32_t *__restrict__ len_out, const int *__restrict__ status)
+                    int32_t *__restrict__ len_out, const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -1393,9 +1393,9 @@ retain_union_kernel(const float *__restrict__ sim, const int32_t *__restrict__ p
 // cu_seqlens, and the packed index list and position ids of every sample at its offset.  Every CTA adds up the lengths before
 // its sample's (a scan kernel of its own took 4 us).
 __global__ void __launch_bounds__(kWalkThreads)
-pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restrict__ len, int32_t *__restrict__ cu, const int64_t *__restrict__ pos_in, int S,
+pack_varlen_kernel(const uint8_t *keep_in, const int32_t *len, int32_t *__restrict__ cu, const int64_t *__restrict__ pos_in, int S,
                    int vis_offset, int n_vis, int32_t *__restrict__ out_idx, int64_t *__restrict__ out_pos,
-                   const int *__restrict__ status)
+                   const int *status)
 {
     wait_for_previous();
     let_next_start();
@@ -1425,8 +1425,8 @@ pack_varlen_kernel(const uint8_t *__restrict__ keep_in, const int32_t *__restric
 // Step 5b for packed rows of variable length: output row t belongs to the sample b with cu[b] <= t < cu[b + 1].
 // One warp per output row (as gather_kernel); rows at and beyond cu[B] do not exist.
 __global__ void __launch_bounds__(kGatherWarps * 32)
-gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, const int32_t *__restrict__ cu, int B,
-                     int S, int d8, long long rows_cap, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs)
+gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, const int32_t *cu, int B,
+                     int S, int d8, long long rows_cap, const int *status, uint4 *__restrict__ out_hidden, FlowState fs)
 {
     wait_for_previous();
     let_next_start();
@@ -1451,9 +1451,11 @@ gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict
 // 128-bit loads and streaming stores, 8 loads in flight per lane.
 // ------------------------------------------------------------------------------------------------
 
+// kFirst: launched behind whatever the caller's stream runs (no call of the library before it): its rows are read coherently
+template <bool kFirst>
 __global__ void __launch_bounds__(kGatherWarps * 32)
-gather_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_idx, int S, int S_out, int d8,
-              long long rows_total, const int *__restrict__ status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep)
+gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, int S_out, int d8,
+              long long rows_total, const int *status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep)
 {
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
@@ -1472,7 +1474,7 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 int c = c0 + u * 32 + lane;
-                if (c < d8) v[u] = ld_stream(src + c);
+                if (c < d8) v[u] = ld_stream<kFirst>(src + c);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -1489,7 +1491,7 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ out_
 // so that all SMs re-read a sample at the same time): sim[i] = share[0][i] + share[1][i] + ... in this fixed order.
 constexpr int kSimSumThreads = 256;
 template <typename V>
-__global__ void __launch_bounds__(kSimSumThreads) sim_sum_kernel(const V *__restrict__ share, long long n, int n_kc, V *__restrict__ sim)
+__global__ void __launch_bounds__(kSimSumThreads) sim_sum_kernel(const V *share, long long n, int n_kc, V *__restrict__ sim)
 {
     for (long long i = (long long)blockIdx.x * kSimSumThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kSimSumThreads) {
         V a = __ldcs(share + i);
