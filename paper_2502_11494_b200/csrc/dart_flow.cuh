@@ -68,6 +68,9 @@ constexpr uint32_t kChunkBytes = kChunk * 512; // 4 KB: half a row of 4096 colum
 constexpr int kMaxSlots = 6;               // chunks of a row on their way per scorer
 constexpr int kSel = 512, kSelGroups = 4;  // threads of a selector CTA that select; at most so many groups of them
 __host__ inline int sel_threads(int n_vis) { return n_vis > 1024 ? kSel : kSel / kSelGroups; }
+// Longest list that a group of T threads ranks by counting: 3 x 384 or 2 x 640 steps a thread, about what a radix select takes
+// (64 x 576 tokens, whole call: lists of 288 111 us, of 576 227, radix select 143; 8 x 2880: lists of 720 108, radix select 101).
+__host__ __device__ constexpr int sel_list(int T) { return T == kSel ? 640 : 384; }
 constexpr int kPoll = 6;                   // words per selecting thread on their way at once: 3072 tokens
 constexpr int kMail = 2;                   // items on their way to each combine warp
 constexpr int kPvRing = 16;                // pivot lists kept for the combine warps: 2 pivot buffers + 8 items on their way, and slack
@@ -121,9 +124,21 @@ struct Shared {
 };
 static_assert(sizeof(Shared) + 64 <= kStaticSmemReserve, "static shared memory exceeds its reserve");
 
-// shared memory of the two pivot buffers; of a selector (the list takes every token: with many equal scores many are at the floor)
+// shared memory of the two pivot buffers; of a selector: every group's list, histogram and keys
 __host__ inline size_t pivot_bytes(int NT, int na_max) { return (size_t)2 * 8 * NT * ((size_t)na_max * 128 + 16); }
-__host__ inline size_t selector_bytes(int n_vis) { return (size_t)n_vis * 12 * (kSel / sel_threads(n_vis)); }
+__host__ inline size_t selector_bytes(int n_vis)
+{
+    const int T = sel_threads(n_vis);
+    return ((size_t)sel_list(T) * 8 + sizeof(SelectSmem) + (size_t)n_vis * 4) * (kSel / T);
+}
+
+// `size` threads of a selector CTA, with a named barrier
+struct SelGroup {
+    int t, T, barrier;
+    __device__ __forceinline__ int tid() const { return t; }
+    __device__ __forceinline__ int size() const { return T; }
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(barrier), "r"(T) : "memory"); }
+};
 
 __device__ __forceinline__ unsigned long long ld_rec(const unsigned long long *p)
 {
@@ -341,15 +356,32 @@ __device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shar
     }
 }
 
+// The P largest of n keys, equal ones by index, into list[0 .. P), in no order (not inlined: the code that every selection runs stays together)
+__device__ __noinline__ void radix_best(SelGroup group, const uint32_t *skey, int n, int P, SelectSmem &sel, unsigned long long *list, uint32_t *n_list)
+{
+    auto keyfn = [&](int j, uint32_t &key) {
+        key = ~skey[j];
+        return true;
+    };
+    uint32_t thr, need_eq, cnt_eq;
+    block_select_threshold(group, keyfn, n, (uint32_t)P, sel, thr, need_eq, cnt_eq);
+    block_select_apply(group, keyfn, n, thr, need_eq, cnt_eq, sel, [&](int j, uint32_t key) {
+        list[atomicAdd(n_list, 1u)] = ((unsigned long long)~key << 32) | (0xffffffffu - (uint32_t)j);
+    });
+}
+
 // The selectors (CTAs that do nothing else).  p.sel_threads threads (512, or four groups of 128 side by side for short samples,
 // which come faster than one group takes them) read a sample's words as they appear; the P-th best of 32 sets' best keys is a
-// floor that few keys pass; those are ranked by counting.
+// floor that few keys pass; those are ranked by counting.  Where many pass (equal scores: blank patches, padding) a radix select
+// finds the P best first, since counting is quadratic (equal rows, pivots alone kept, whole calls, us, counting / so: 64 x 576 227 / 143,
+// 8 x 2880 547 / 103, 32 x 2880 1954 / 303, 2 x 8192 1824 / 61).
 __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, Shared &sh, uint8_t *smem)
 {
-    const int T = p.sel_threads, grp = (int)threadIdx.x / T, n_grp = kSel / T;
+    const int T = p.sel_threads, grp = (int)threadIdx.x / T, n_grp = kSel / T, most = sel_list(T);
     const int t = (int)threadIdx.x - grp * T, lane = t & 31;
-    unsigned long long *list = reinterpret_cast<unsigned long long *>(smem) + (size_t)grp * p.n_vis;
-    uint32_t *skey = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(smem) + (size_t)n_grp * p.n_vis) + (size_t)grp * p.n_vis;
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(smem) + grp * most;
+    SelectSmem &sel = reinterpret_cast<SelectSmem *>(smem + n_grp * most * 8)[grp];
+    uint32_t *skey = reinterpret_cast<uint32_t *>(smem + n_grp * (most * 8 + sizeof(SelectSmem))) + (size_t)grp * p.n_vis;
     auto any = [&](bool x) { // OR over the group; doubles as its barrier
         uint32_t r;
         asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\nbar.red.or.pred p, %2, %3, q;\nselp.u32 %0, 1, 0, p;\n}"
@@ -418,10 +450,19 @@ __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, S
         if (best >= fl)
             for (int j = t; j < p.n_vis; j += T) {
                 const uint32_t k = skey[j];
-                if (k >= fl) list[atomicAdd(&sh.n_list[grp], 1u)] = ((unsigned long long)k << 32) | (0xffffffffu - (uint32_t)j); // equal scores: lower index first
+                if (k >= fl) {
+                    const uint32_t slot = atomicAdd(&sh.n_list[grp], 1u);
+                    if (slot < (uint32_t)most) list[slot] = ((unsigned long long)k << 32) | (0xffffffffu - (uint32_t)j); // equal scores: lower index first
+                }
             }
         any(false);
-        const int m = (int)sh.n_list[grp];
+        int m = (int)sh.n_list[grp];
+        if (m > most) {
+            any(false); // everybody has read the count
+            if (t == 0) sh.n_list[grp] = 0;
+            radix_best(SelGroup{t, T, 1 + grp}, skey, p.n_vis, p.P, sel, list, &sh.n_list[grp]);
+            m = p.P;
+        }
         for (int e = t; e < m; e += T) {
             const unsigned long long mine = list[e];
             int r = 0;

@@ -85,6 +85,42 @@ def test_flow_equal_scores_rank_the_lower_index_first(oracle):
     assert np.array_equal(dbg["pivot_idx"], np.tile(np.arange(5, dtype=np.int32), (2, 1)))
 
 
+@pytest.mark.parametrize("n_vis", [128, 384, 385, 640, 641, 1024, 1025, 8192])
+@pytest.mark.parametrize("P", [1, 5, 32])
+@pytest.mark.parametrize("values", ["equal", "four values", "half at the top"])
+def test_flow_many_equal_scores(values, P, n_vis):
+    """More tokens at the selection's floor than its list holds (384 entries up to 1024 tokens, 640 beyond).  Scores are sums of 64
+    small whole numbers, exact in any order: a stable sort is the answer, in time that does not grow with the square of the ties."""
+    B, vo = 5, 3
+    g = torch.Generator(device="cuda").manual_seed(n_vis + P)
+    keys = torch.randint(-9, 10, (B, n_vis + 5, 64), generator=g, device="cuda").bfloat16()
+    if values == "equal":
+        keys[:] = 3
+    elif values == "four values":
+        keys[:] = keys[:, :1].abs() + torch.randint(1, 5, (B, n_vis + 5, 1), generator=g, device="cuda")
+    else:
+        keys[:, vo + n_vis // 2:vo + n_vis] = 9
+    score = keys[:, vo:vo + n_vis].float().abs().sum(-1)
+    ctx = dart.Dart(B, n_vis + 5, 64, P, P)
+    for smallest in (0, 1):
+        dbg = ctx.reduce(keys, None, vo, n_vis, P, P, debug=True, opts=dart.dart_opts(path=FLOW, pivot_smallest=smallest))[3]
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        want = torch.sort(score, dim=1, descending=not smallest, stable=True).indices[:, :P]
+        assert torch.equal(dbg["pivot_idx"].long(), want)
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times = {}
+    for path in (FLOW, dart.DART_PATH_STAGED):       # the staged path selects by radix passes whatever the scores
+        start.record()
+        for _ in range(10):
+            ctx.reduce(keys, None, vo, n_vis, P, P, opts=dart.dart_opts(path=path))
+        end.record()
+        torch.cuda.synchronize()
+        times[path] = start.elapsed_time(end)
+    assert times[FLOW] < 3 * times[dart.DART_PATH_STAGED], times   # quadratic: 20 times as long at 8192 equal scores
+    ctx.close()
+
+
 @pytest.mark.parametrize("shape", [(1, 64, 64, 0, 64, 33, 40), (1, 8300, 64, 0, 8193, 2, 8), (1, 64, 96, 0, 64, 2, 8)],
                          ids=["33 pivots", "8193 tokens", "d not a multiple of 64"])
 def test_flow_says_what_it_does_not_take(shape):
