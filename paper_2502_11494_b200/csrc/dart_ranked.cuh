@@ -17,8 +17,11 @@
 // keeping half 60 -> 18; 256 x 2880, 8 pivots 60 -> 38, 128 pivots 488 -> 389.  Of the last, reading the rows is 80 (at the
 // memory's rate it would be 57), minimum and mean 25, the counts 30, the atomics' two passes 100, the places 40; what remains is
 // the last samples' turns.  For one sample all of it is a chain of short steps.
+// A list of nearly all tokens cannot wait for a guess that lets all of them through: the few above the threshold share the last bin
+// (8 x 2880 keeping everything, 8 pivots 237 us -> 27; 256 x 576 125 -> 31).
 // Rows whose values the bins do not separate (many equal values, a value that is not finite) are ranked by an exact radix
-// select and counting.  The result equals retain_kernel's exactly.
+// select, then by counting or, as that grows with the square of the length, a sort (8 x 2880 equal rows, 8 pivots, keeping half
+// 82 us -> 50, everything 238 -> 70; 256 x 1000, 64 pivots, half 533 -> 470).  The result equals retain_kernel's exactly.
 //
 // With independent pivots (DART_RULE_UNION) the lists are the q_i smallest and the last CTA only merges them.
 #pragma once
@@ -32,6 +35,7 @@ constexpr int kRankMaxVis = 16384;    // 512 threads x 8 x 4 values in registers
 constexpr int kRankMaxList = 4096;    // longest list
 constexpr uint32_t kRankMaxBin = 192; // entries of one bin that are ranked by counting
 constexpr int kRankTries = 10;        // guesses at the threshold
+constexpr int kRankMaxCount = 1000;   // steps per thread up to which the exact route orders a list by counting (their number grows with the square)
 
 // one flag per token and one more that is never free
 __host__ __device__ inline size_t rank_flag_bytes(int n_vis) { return ((size_t)n_vis + 16) / 16 * 16; }
@@ -97,6 +101,33 @@ __device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *per_warp)
     return v + __reduce_add_sync(0xffffffffu, x);
 }
 
+// n distinct entries of `list` in ascending order: a bitonic sort of any length (every comparison puts the smaller entry at the
+// lower place, so that what is missing up to a power of two would never move).
+__device__ __forceinline__ void cta_sort(unsigned long long *list, int n)
+{
+    auto order = [&](int i, int l) {
+        if (l >= n) return;
+        const unsigned long long x = list[i], y = list[l];
+        if (x > y) list[i] = y, list[l] = x;
+    };
+    __syncthreads();
+    for (int k = 1; k < n; k <<= 1) { // sorted runs of k to runs of 2 k
+        const int pairs = (n + 2 * k - 1) / (2 * k) * k;
+        for (int e = threadIdx.x; e < pairs; e += blockDim.x) {
+            const int at = e & (k - 1), run = 2 * (e - at);
+            order(run + at, run + 2 * k - 1 - at);
+        }
+        __syncthreads();
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int e = threadIdx.x; e < pairs; e += blockDim.x) {
+                const int i = 2 * e - (e & (j - 1));
+                order(i, i + j);
+            }
+            __syncthreads();
+        }
+    }
+}
+
 constexpr uint32_t kNotAToken = 0xffffffffu; // a NaN that no arithmetic produces: below no threshold
 
 // A row's values into registers, sign: 0, or the sign bit to have their negatives
@@ -129,11 +160,11 @@ __device__ __forceinline__ void load_row(const float *row, int n, uint32_t sign,
     }
 }
 
-// The C smallest (value, index) pairs of a row, ranked, into out[0 .. C).  v: the thread's values (tokens 4 (T k + t) ...), tokens
-// that do not take part and what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per token that does not
+// The C smallest (value, index) pairs of a row of which n_in tokens take part, ranked, into out[0 .. C).  v: the thread's values (tokens
+// 4 (T k + t) ...), tokens that do not take part and what lies behind the row as kNotAToken; list, hist (4 T words), skip (a bit per token that does not
 // take part): shared memory.  flip: 0, or all ones if v holds the row's values with the opposite sign.
 template <int R, bool kOutliers, typename Out>
-__device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const uint32_t *skip, const float4 (&v)[R], int n, Out *out, int C,
+__device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const uint32_t *skip, const float4 (&v)[R], int n, int n_in, Out *out, int C,
                                          unsigned long long *list, uint32_t *hist, RankShared &sh)
 {
     const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = T >> 5;
@@ -176,13 +207,14 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
     hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
     auto quantile = [](float u) { return 4.91f * (__powf(u, 0.14f) - __powf(1.0f - u, 0.14f)); };
     const float inv_n = 1.0f / (float)n, least = -quantile(fminf(0.5f / (float)n_of, 0.25f)), wanted = quantile(fminf((1.3f * (float)C + 40.f) * inv_n, 0.97f));
-    float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f;
+    float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f, cut;
     bool has_few = false, has_many = false, exact = !(hi > lo) || !(hi - lo < 3.0e38f) || !(mid > 0.0f);
     int m = 0;
     reinterpret_cast<uint4 *>(hist)[t] = make_uint4(0, 0, 0, 0);
     for (int guess = 0; !exact; ++guess) {
         top = low + part * mid;
         if (!(top < hi)) top = hi;
+        cut = top;
         uint32_t c = 0;
 #pragma unroll
         for (int k = 0; k < R; ++k) c += (v[k].x <= top) + (v[k].y <= top) + (v[k].z <= top) + (v[k].w <= top);
@@ -191,22 +223,27 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
         __syncthreads();
         m = (int)sh.n_below[guess];
         if (m >= C && m <= 3 * C + 256) break;
+        if (m < C && n_in - m <= (int)kRankMaxBin / 4 * 3) { // the list takes nearly all tokens: what lies above goes to the last bin
+            m = n_in, cut = hi;
+            break;
+        }
         exact = guess + 1 == kRankTries || (m < C && top == hi);
         (m < C ? few : many) = part;
         (m < C ? has_few : has_many) = true;
         part += (wanted - quantile(fminf(((float)m + 0.5f) * inv_n, 0.97f))) / least;
         if (has_few && has_many && !(part > 0.9f * few + 0.1f * many && part < 0.1f * few + 0.9f * many)) part = 0.5f * (few + many);
     }
-    // bins: the low bits of 2^23 + (x - base) scale, never below 0 or above 4 T - 1; outliers go to the first one
+    // bins of the values up to `cut`: the low bits of 2^23 + (x - base) scale, never below 0 or above 4 T - 1; outliers go to the first
+    // one, what lies above the threshold to the last
     const float base = kOutliers && low - lo > top - low && top > low ? low : lo, scale = ((float)(4 * T) - 1.0f) / (top - base);
     if (!exact && scale < 3.0e38f) {
-        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(kOutliers ? fmaxf(x - base, 0.f) : x - base, scale, 8388608.0f)) - 0x4b000000u); };
+        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(kOutliers ? fmaxf(fminf(x, top) - base, 0.f) : fminf(x, top) - base, scale, 8388608.0f)) - 0x4b000000u); };
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (f[e] <= top) atomicAdd(&hist[bin_of(f[e])], 1u);
+                if (f[e] <= cut) atomicAdd(&hist[bin_of(f[e])], 1u);
         }
         __syncthreads();
         uint4 *h4 = reinterpret_cast<uint4 *>(hist) + t; // thread t owns bins 4 t ... 4 t + 3
@@ -225,7 +262,7 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
                 const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (f[e] <= top) {
+                    if (f[e] <= cut) {
                         const uint32_t place = atomicAdd(&hist[bin_of(f[e])], 1u);
                         if (place < (uint32_t)C + kRankMaxBin) list[place] = ((unsigned long long)order_key(f[e]) << 32) | (uint32_t)(4 * (T * k + t) + e);
                     }
@@ -250,13 +287,29 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
         return true;
     };
     if (t == 0) sh.n_list = 0;
-    uint32_t thr, need_eq, cnt_eq;
-    block_select_threshold(CtaGroup(), keyfn, n, (uint32_t)C, sh.sel, thr, need_eq, cnt_eq);
-    block_select_apply(CtaGroup(), keyfn, n, thr, need_eq, cnt_eq, sh.sel, [&](int j, uint32_t key) {
-        const uint32_t slot = atomicAdd(&sh.n_list, 1u);
-        if (slot < (uint32_t)C) list[slot] = ((unsigned long long)key << 32) | (uint32_t)j;
-    });
-    rank_sort(list, C, [&](int r, unsigned long long x) { out[r] = (Out)(uint32_t)x; });
+    auto put = [&](int j, uint32_t key) { list[atomicAdd(&sh.n_list, 1u)] = ((unsigned long long)key << 32) | (uint32_t)j; };
+    int held = C; // entries of the list
+    if (n_in <= C + (int)kRankMaxBin) { // it has room for all tokens
+        held = n_in;
+        __syncthreads();
+        for (int j = t; j < n; j += T) {
+            uint32_t key;
+            if (keyfn(j, key)) put(j, key);
+        }
+        __syncthreads();
+    } else {
+        uint32_t thr, need_eq, cnt_eq;
+        block_select_threshold(CtaGroup(), keyfn, n, (uint32_t)C, sh.sel, thr, need_eq, cnt_eq);
+        block_select_apply(CtaGroup(), keyfn, n, thr, need_eq, cnt_eq, sh.sel, put);
+    }
+    if ((held + T - 1) / T * held <= kRankMaxCount) {
+        rank_sort(list, held, [&](int r, unsigned long long x) {
+            if (r < C) out[r] = (Out)(uint32_t)x;
+        });
+    } else {
+        cta_sort(list, held);
+        for (int e = t; e < C; e += T) out[e] = (Out)(uint32_t)list[e];
+    }
 }
 
 // Step 5a (as pack_indices; flags are 0 or 1, 16-byte aligned), a contiguous range of flags per warp: two barriers in all instead of two per blockDim.x flags.
@@ -456,7 +509,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     const bool each = kGroups == 0 && p.each != 0;
     uint16_t *lists = p.lists + (size_t)b * p.sample_entries;
     if (q + (i < r ? 1 : 0) > 0) // (else this pivot keeps nothing, and so do all later ones)
-        rank_row<R, false>(row, 0u, skip, v, n, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
+        rank_row<R, false>(row, 0u, skip, v, n, n - Pv, lists + rank_place(i, q, r, each), rank_length(i, q, r, each), list, hist, sh);
     __syncthreads();
     if (t == 0) { // release: the list; acquire: the other pivots' lists
         int before;
@@ -594,7 +647,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) pivot_rank_kernel(const float
     const float *row = score + (size_t)blockIdx.x * n;
     float4 v[R];
     load_row<R>(row, n, smallest ? 0u : 0x80000000u, v);
-    rank_row<R, true>(row, smallest ? 0u : 0xffffffffu, skip, v, n, pivot_idx + (size_t)blockIdx.x * P, P, list, hist, sh);
+    rank_row<R, true>(row, smallest ? 0u : 0xffffffffu, skip, v, n, n, pivot_idx + (size_t)blockIdx.x * P, P, list, hist, sh);
 }
 
 } // namespace dart

@@ -122,3 +122,31 @@ def test_more_samples_than_a_grid_has_rows(rule, retention):
         ctx.close()
         got.append([torch.cat(x) for x in zip(*rows)] + [torch.cat(lengths)])
     assert all(torch.equal(x, y) for x, y in zip(*got))
+
+
+@pytest.mark.parametrize("kind", ["gaussian", "equal tokens"])
+@pytest.mark.parametrize("n,less", [(576, 0), (2880, 0), (2880, 1), (2880, 40), (2881, 100), (2883, 300), (4100, 4), (300, 0)])
+def test_lists_of_nearly_all_tokens(kind, n, less):
+    """The last pivots' lists take nearly every token: what the guessed threshold leaves out goes to the last bin."""
+    B, S, d, vo, P, Kp = 9, n + 9, 64, 4, 8, n - less
+    k, h = _band_inputs(kind, B, S, d, vo, n, P, seed=n + less)
+    a = run_gpu(k, h, vo, n, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
+    b = run_gpu(k, h, vo, n, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+    assert all(np.array_equal(a[3][m], b[3][m], equal_nan=(m == "eps")) for m in a[3])
+
+
+@pytest.mark.parametrize("kind", ["gaussian", "equal tokens"])
+def test_keeping_everything_takes_no_longer_than_the_other_forms(kind):
+    """AUTO with n_keep == n_vis (it took 4 times as long as the bands while the last lists were ordered by counting)."""
+    B, n, P = 32, 2880, 8
+    k, h = _band_inputs(kind, B, n, 64, 0, n, P, seed=3)
+    ctx = dart.Dart(B, n, 64, P, n)
+    dart.dart_profile_enable(ctx.handle, True)
+    ms = {}
+    for retention in (dart.DART_RETAIN_AUTO, dart.DART_RETAIN_BANDS, dart.DART_RETAIN_AUTO, dart.DART_RETAIN_BANDS):
+        for _ in range(5):
+            ctx.reduce(h, k, 0, n, P, n, opts=dart.dart_opts(path=dart.DART_PATH_STAGED, retention=retention))
+        ms[retention] = dart.dart_profile_read(ctx.handle)[1]["retain"][0]
+    ctx.close()
+    assert ms[dart.DART_RETAIN_AUTO] < 2 * ms[dart.DART_RETAIN_BANDS], ms
