@@ -128,15 +128,18 @@ __device__ __forceinline__ void cta_sort(unsigned long long *list, int n)
     }
 }
 
-constexpr uint32_t kNotAToken = 0xffffffffu; // a NaN that no arithmetic produces: below no threshold
+// A NaN that no arithmetic produces (its NaN is 0x7fffffff): below no threshold.  The row's values are results of arithmetic, and so
+// are their negatives (flipping the sign bit of a NaN would give this one): one NaN makes their sum a NaN, and the row takes the
+// exact route.
+constexpr uint32_t kNotAToken = 0xffffffffu;
 
-// A row's values into registers, sign: 0, or the sign bit to have their negatives
-template <int R>
-__device__ __forceinline__ void load_row(const float *row, int n, uint32_t sign, float4 (&v)[R])
+// A row's values into registers, or (kNegate) minus them if sign is -1
+template <bool kNegate, int R>
+__device__ __forceinline__ void load_row(const float *row, int n, float sign, float4 (&v)[R])
 {
     const int t = threadIdx.x, T = blockDim.x;
     const float none = __uint_as_float(kNotAToken);
-    auto value = [&](float x) { return __uint_as_float(__float_as_uint(x) ^ sign); };
+    auto value = [&](float x) { return kNegate ? fmaf(x, sign, 0.0f) : x; };
     if (((uintptr_t)row & 15u) == 0 && (n & 3) == 0) {
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -482,7 +485,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
     let_next_start();
     if (*p.status != 0) return; // an earlier kernel of this call failed: its outputs are undefined
     float4 v[R];
-    load_row<R>(row, n, 0u, v);
+    load_row<false>(row, n, 1.0f, v);
     const float none = __uint_as_float(kNotAToken);
     uint32_t mine = 0;
     for (int k = t; k < p.P; k += T) {
@@ -646,7 +649,7 @@ __global__ void __launch_bounds__(kRankMaxThreads) pivot_rank_kernel(const float
     let_next_start();
     const float *row = score + (size_t)blockIdx.x * n;
     float4 v[R];
-    load_row<R>(row, n, smallest ? 0u : 0x80000000u, v);
+    load_row<true>(row, n, smallest ? 1.0f : -1.0f, v);
     rank_row<R, true>(row, smallest ? 0u : 0xffffffffu, skip, v, n, n, pivot_idx + (size_t)blockIdx.x * P, P, list, hist, sh);
 }
 

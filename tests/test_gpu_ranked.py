@@ -150,3 +150,37 @@ def test_keeping_everything_takes_no_longer_than_the_other_forms(kind):
         ms[retention] = dart.dart_profile_read(ctx.handle)[1]["retain"][0]
     ctx.close()
     assert ms[dart.DART_RETAIN_AUTO] < 2 * ms[dart.DART_RETAIN_BANDS], ms
+
+
+@pytest.mark.parametrize("n,P", [(5, 5), (576, 8), (576, 575), (1000, 1000), (2049, 100), (4096, 33), (16384, 3), (16385, 3)])
+@pytest.mark.parametrize("n_nan", [1, 3])
+def test_scores_that_are_not_numbers_rank_last(n, P, n_nan):
+    """Inputs are meant to be finite; a score that is not a number comes behind all that are, whatever the sample's length."""
+    B, vo = 2, 2
+    g = torch.Generator(device="cuda").manual_seed(n + P)
+    keys = torch.randint(-127, 128, (B, n + 5, 64), generator=g, device="cuda").bfloat16()
+    for i in range(n_nan):
+        keys[:, vo + (n - 1) * (i + 1) // n_nan, 7 * i] = float("nan") * (-1) ** i
+    score = keys[:, vo:vo + n].float().abs().sum(-1).nan_to_num(nan=-1.0)
+    want = torch.sort(score, dim=1, descending=True, stable=True).indices[:, :P]
+    got = torch.full((B, P), -1, dtype=torch.int32, device="cuda")
+    assert dart.dart_pivots_static(keys.data_ptr(), B, n + 5, 64, vo, n, P, got.data_ptr(), 0, None) == dart.DART_OK
+    torch.cuda.synchronize()
+    assert torch.equal(got.long(), want)
+    if P <= 32 and n <= 8192:
+        ctx = dart.Dart(B, n + 5, 64, P, P)
+        dbg = ctx.reduce(keys, None, vo, n, P, P, debug=True, opts=dart.dart_opts(path=dart.DART_PATH_FLOW))[3]
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK and torch.equal(dbg["pivot_idx"].long(), want)
+        ctx.close()
+
+
+def test_similarities_that_are_not_numbers():
+    k, h = _band_inputs("gaussian", 3, 900, 64, 20, 850, 9, seed=4)
+    k[0, 30, 3] = float("inf")      # a pivot (its score is the largest): its own similarities are 0 / inf or inf / inf
+    k[1, 40:60] = float("inf")
+    k[2, 500, 9] = float("nan")
+    a = run_gpu(k, h, 20, 850, 9, 300, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL)
+    b = run_gpu(k, h, 20, 850, 9, 300, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+    assert np.array_equal(a[3]["keep"], b[3]["keep"]) and np.array_equal(a[3]["owner"], b[3]["owner"])
