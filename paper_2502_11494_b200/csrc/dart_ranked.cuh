@@ -17,8 +17,8 @@
 // keeping half 60 -> 18; 256 x 2880, 8 pivots 60 -> 38, 128 pivots 488 -> 389.  Of the last, reading the rows is 80 (at the
 // memory's rate it would be 57), minimum and mean 25, the counts 30, the atomics' two passes 100, the places 40; what remains is
 // the last samples' turns.  For one sample all of it is a chain of short steps.
-// A list of nearly all tokens cannot wait for a guess that lets all of them through: the few above the threshold share the last bin
-// (8 x 2880 keeping everything, 8 pivots 237 us -> 27; 256 x 576 125 -> 31).
+// A list of nearly all tokens cannot wait for a guess that lets all of them through: once few are left the bins reach to the largest
+// value (8 x 2880 keeping everything, 8 pivots 237 us -> 27; 256 x 576 125 -> 31).
 // Rows whose values the bins do not separate (many equal values, a value that is not finite) are ranked by an exact radix
 // select, then by counting or, as that grows with the square of the length, a sort (8 x 2880 equal rows, 8 pivots, keeping half
 // 82 us -> 50, everything 238 -> 70; 256 x 1000, 64 pivots, half 533 -> 470).  The result equals retain_kernel's exactly.
@@ -35,6 +35,7 @@ constexpr int kRankMaxVis = 16384;    // 512 threads x 8 x 4 values in registers
 constexpr int kRankMaxList = 4096;    // longest list
 constexpr uint32_t kRankMaxBin = 192; // entries of one bin that are ranked by counting
 constexpr int kRankTries = 10;        // guesses at the threshold
+constexpr int kRankMaxRest = 144;     // tokens beyond a threshold that a list of nearly all takes along
 constexpr int kRankMaxCount = 1000;   // steps per thread up to which the exact route orders a list by counting (their number grows with the square)
 
 // one flag per token and one more that is never free
@@ -210,14 +211,13 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
     hi = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(hi)));
     auto quantile = [](float u) { return 4.91f * (__powf(u, 0.14f) - __powf(1.0f - u, 0.14f)); };
     const float inv_n = 1.0f / (float)n, least = -quantile(fminf(0.5f / (float)n_of, 0.25f)), wanted = quantile(fminf((1.3f * (float)C + 40.f) * inv_n, 0.97f));
-    float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f, cut;
+    float part = 1.0f + wanted / least, few = 0.f, many = 0.f, top = 0.f;
     bool has_few = false, has_many = false, exact = !(hi > lo) || !(hi - lo < 3.0e38f) || !(mid > 0.0f);
     int m = 0;
     reinterpret_cast<uint4 *>(hist)[t] = make_uint4(0, 0, 0, 0);
     for (int guess = 0; !exact; ++guess) {
         top = low + part * mid;
         if (!(top < hi)) top = hi;
-        cut = top;
         uint32_t c = 0;
 #pragma unroll
         for (int k = 0; k < R; ++k) c += (v[k].x <= top) + (v[k].y <= top) + (v[k].z <= top) + (v[k].w <= top);
@@ -226,8 +226,8 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
         __syncthreads();
         m = (int)sh.n_below[guess];
         if (m >= C && m <= 3 * C + 256) break;
-        if (m < C && n_in - m <= (int)kRankMaxBin / 4 * 3) { // the list takes nearly all tokens: what lies above goes to the last bin
-            m = n_in, cut = hi;
+        if (m < C && n_in - m <= kRankMaxRest) { // the list takes nearly all tokens: let all of them through
+            m = n_in, top = hi;
             break;
         }
         exact = guess + 1 == kRankTries || (m < C && top == hi);
@@ -236,17 +236,16 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
         part += (wanted - quantile(fminf(((float)m + 0.5f) * inv_n, 0.97f))) / least;
         if (has_few && has_many && !(part > 0.9f * few + 0.1f * many && part < 0.1f * few + 0.9f * many)) part = 0.5f * (few + many);
     }
-    // bins of the values up to `cut`: the low bits of 2^23 + (x - base) scale, never below 0 or above 4 T - 1; outliers go to the first
-    // one, what lies above the threshold to the last
+    // bins: the low bits of 2^23 + (x - base) scale, never below 0 or above 4 T - 1; outliers go to the first one
     const float base = kOutliers && low - lo > top - low && top > low ? low : lo, scale = ((float)(4 * T) - 1.0f) / (top - base);
     if (!exact && scale < 3.0e38f) {
-        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(kOutliers ? fmaxf(fminf(x, top) - base, 0.f) : fminf(x, top) - base, scale, 8388608.0f)) - 0x4b000000u); };
+        auto bin_of = [&](float x) { return (int)(__float_as_uint(fmaf(kOutliers ? fmaxf(x - base, 0.f) : x - base, scale, 8388608.0f)) - 0x4b000000u); };
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (f[e] <= cut) atomicAdd(&hist[bin_of(f[e])], 1u);
+                if (f[e] <= top) atomicAdd(&hist[bin_of(f[e])], 1u);
         }
         __syncthreads();
         uint4 *h4 = reinterpret_cast<uint4 *>(hist) + t; // thread t owns bins 4 t ... 4 t + 3
@@ -265,7 +264,7 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
                 const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (f[e] <= cut) {
+                    if (f[e] <= top) {
                         const uint32_t place = atomicAdd(&hist[bin_of(f[e])], 1u);
                         if (place < (uint32_t)C + kRankMaxBin) list[place] = ((unsigned long long)order_key(f[e]) << 32) | (uint32_t)(4 * (T * k + t) + e);
                     }
