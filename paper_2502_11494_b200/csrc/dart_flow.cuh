@@ -356,9 +356,13 @@ __device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shar
     }
 }
 
-// The P largest of n keys, equal ones by index, into list[0 .. P), in no order (not inlined: the code that every selection runs stays together)
-__device__ __noinline__ void radix_best(SelGroup group, const uint32_t *skey, int n, int P, SelectSmem &sel, unsigned long long *list, uint32_t *n_list)
+// The end of a selection where many keys pass the floor: the P best by radix select, ranked and published.  (Not inlined, and with a
+// publication of its own, so that the code of every other selection stays together: 256 x 2880 1741 us as a branch in it, 1732 so.)
+__device__ __noinline__ void select_among_many(const SelGroup group, const uint32_t *skey, int n, int P, SelectSmem &sel, unsigned long long *list, uint32_t *n_list,
+                                               int32_t *pv_word, int32_t *pivot_idx)
 {
+    group.sync(); // everybody has read the list's length
+    if (group.t == 0) *n_list = 0;
     auto keyfn = [&](int j, uint32_t &key) {
         key = ~skey[j];
         return true;
@@ -366,8 +370,16 @@ __device__ __noinline__ void radix_best(SelGroup group, const uint32_t *skey, in
     uint32_t thr, need_eq, cnt_eq;
     block_select_threshold(group, keyfn, n, (uint32_t)P, sel, thr, need_eq, cnt_eq);
     block_select_apply(group, keyfn, n, thr, need_eq, cnt_eq, sel, [&](int j, uint32_t key) {
-        list[atomicAdd(n_list, 1u)] = ((unsigned long long)~key << 32) | (0xffffffffu - (uint32_t)j);
+        list[atomicAdd(n_list, 1u)] = ((unsigned long long)key << 32) | (uint32_t)j;
     });
+    if (group.t < P) { // P <= 32
+        const unsigned long long mine = list[group.t];
+        int r = 0;
+        for (int u = 0; u < P; ++u) r += list[u] < mine ? 1 : 0;
+        st_word(pv_word + r, (int32_t)(uint32_t)mine);
+        pivot_idx[r] = (int32_t)(uint32_t)mine;
+    }
+    group.sync(); // the list may be filled again
 }
 
 // The selectors (CTAs that do nothing else).  p.sel_threads threads (512, or four groups of 128 side by side for short samples,
@@ -456,12 +468,10 @@ __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, S
                 }
             }
         any(false);
-        int m = (int)sh.n_list[grp];
+        const int m = (int)sh.n_list[grp];
         if (m > most) {
-            any(false); // everybody has read the count
-            if (t == 0) sh.n_list[grp] = 0;
-            radix_best(SelGroup{t, T, 1 + grp}, skey, p.n_vis, p.P, sel, list, &sh.n_list[grp]);
-            m = p.P;
+            select_among_many(SelGroup{t, T, 1 + grp}, skey, p.n_vis, p.P, sel, list, &sh.n_list[grp], p.pv_word + (size_t)b * kMaxP, p.pivot_idx + (size_t)b * p.P);
+            continue;
         }
         for (int e = t; e < m; e += T) {
             const unsigned long long mine = list[e];
