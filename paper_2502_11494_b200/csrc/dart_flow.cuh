@@ -476,6 +476,7 @@ __device__ __forceinline__ void select_pivots(const Params &p, const Ctl &ctl, S
         for (int e = t; e < m; e += T) {
             const unsigned long long mine = list[e];
             int r = 0;
+#pragma unroll 8 // (left to the compiler: 4 x 117 x 4096, 31 pivots 45 or 53 us, 25 x 925 x 6144 187 or 208, as it happens to choose)
             for (int u = 0; u < m; ++u) r += list[u] > mine ? 1 : 0;
             if (r < p.P) {
                 const int32_t pv = (int32_t)(0xffffffffu - (uint32_t)mine);
