@@ -791,23 +791,36 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     return true;
 }
 
-// Whether AUTO takes the flow path.  Pivots by score: up to 16 pivots it is the fastest path at every size measured, from one
-// sample of 130 tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.25 against 1.85 ms of
-// the sweep, 16 pivots 1.30 against 1.87).  Up to 32 pivots its multiplying warps bound it on larger batches (whole calls, us, flow
-// / two passes: 8 x 2880 x 4096 128 / 132, 16 x 2880 x 4096 203 / 213, 256 x 500 x 2048 353 / 330, 256 x 2880 x 4096 2443 / 2246).
+// Whether AUTO takes the flow path.
+// Pivots by score, up to 16: for rows of 1024 columns and more it is the fastest path at every size measured, from one sample of 130
+// tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.25 against 1.85 ms of the sweep, 16 pivots
+// 1.30 against 1.87).  Narrower rows have two passes up to 1.5 times as fast on large batches (256 x 2880 x 64, 8 pivots; 64 x 2880 x
+// 512 1.24 times): nobody's hidden states are that narrow, and there is no line for them.
+// 17 to 32 pivots by score: its multiplying warps bound it, and every row takes as many products as for 32.  Over 1100 shapes of 64
+// to 7000 tokens and 1 to 250 samples (whole calls, us, flow / two passes: 2 x 576 x 4096 41 / 58, 8 x 1000 x 4096 70 / 81, 8 x 1500 84 / 91, but 8 x 2880 x 4096 126 / 115, 4 x 4608 115 / 98, 32 x 1000 156 / 144, 128 x 700 x 3072
+// 294 / 264) the two meet at about 12 thousand rows from 3072 columns on and 8 thousand of 2048 (8 x 1000 x 2048 56 / 58, 8 x 1500 64 / 63);
+// with 1024 columns it is ahead from one to eight thousand rows (16 x 200 35 / 35; 2 x 200 41 / 32, 32 x 2880 133 / 124; up to 24 pivots
+// and 1400 tokens longer: 108 x 522, 18 pivots 90 / 98), with fewer nowhere.
+// Beyond that the flow path is ahead where the pairs of 128-row tiles hold half as many rows again (250 x 300 x 4096 352 / 369, 250 x
+// 100 182 / 202; not with 5120 columns: 254 / 234).  A context without the compact copy of the pivots' rows has slower passes: there
+// the line stays where it was measured against the sweep.
 // Given pivots: it reads every row into an SM twice where the one-pass kernel reads it once, but spreads fewer row tiles than SMs
 // over all of them (whole calls, us, flow / one pass: 4 x 2880 x 4096 53 / 57, 16 x 576 x 4096 52 / 59, 8 x 2880 x 4096 79 / 74,
 // 64 x 300 x 2048 57 / 55; 32 pivots, 8 x 1500 x 3072: 77 / 66).
-// 17 to 32 pivots by score on large batches: two passes are ahead where their tiles are full (whole calls, us, flow / two passes:
-// 200 x 700 x 3072 565 / 493, 100 x 1100 x 4096 467 / 447, 200 x 400 x 4096 421 / 404), the flow path where the pairs of 128-row tiles
-// hold half as many rows again (250 x 300 x 4096 424 / 458, 256 x 260 418 / 445, 256 x 150 298 / 311).
 bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &o)
 {
     if (!flow_applies(ctx, B, n_vis, P)) return false;
-    const long long bytes = 2ll * ctx->desc.d * n_vis * B;
+    const long long rows = (long long)B * n_vis, d = ctx->desc.d;
     const long long row_tiles = (long long)B * ((n_vis + dart::sweep::kTileRows - 1) / dart::sweep::kTileRows);
-    const int padded = (n_vis + 255) / 256 * 256; // rows of the one-pass kernel's pairs of tiles
-    if (o.pivots_in ? (row_tiles >= ctx->sm_count || P > 16) : (P > 16 && bytes > 300000000ll && 2 * padded < 3 * n_vis)) return false;
+    if (o.pivots_in) {
+        if (row_tiles >= ctx->sm_count || P > 16) return false;
+    } else if (P > 16 && fused_applies(ctx, P)) { // (rows too wide for the other tensor-core kernels: nothing else is near it)
+        const int padded = (n_vis + 255) / 256 * 256; // rows of the one-pass kernel's pairs of tiles
+        const long long most = d >= 2048 ? (4 * d < 12000 ? 4 * d : 12000) : P <= 24 && n_vis <= 1400 ? 60000 : 8000, least = d >= 2048 ? 1 : 1000;
+        const bool few = ctx->piv_rows ? d >= 1024 && rows <= most && rows >= least : rows * d * 2 <= 300000000ll;
+        const bool ragged = d >= 1024 && d <= 4608 && rows >= 1000 && 2 * padded >= 3 * n_vis;
+        if (!few && !ragged) return false;
+    }
     dart::flow::Params p = {};
     return flow_config(ctx, B, n_vis, P, o, p);
 }

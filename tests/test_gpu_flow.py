@@ -69,6 +69,33 @@ def test_flow_matches_the_oracle(oracle, shape, given):
         ctx.close()
 
 
+@pytest.mark.parametrize("B,n,d,P,flow", [
+    (2, 300, 960, 8, True), (2, 300, 960, 17, False),          # up to 16 pivots always; rows of fewer than 1024 columns never
+    (3, 333, 1024, 17, False), (2, 500, 1024, 32, True),       # 1000 rows and more of 1024 columns
+    (8, 1000, 1024, 25, True), (9, 1000, 1024, 25, False),     # ... up to 8000
+    (60, 1000, 1024, 24, True), (9, 1401, 1024, 17, False),    # ... up to 60000 with up to 24 pivots and 1400 tokens
+    (8, 1024, 2048, 32, True), (9, 1000, 2048, 32, False),     # 4 rows per column
+    (12, 1000, 3072, 20, True), (13, 1000, 3072, 20, False), (4, 3000, 5120, 32, True),   # up to 12000
+    (1, 100, 4096, 24, True), (50, 300, 2048, 24, True), (50, 400, 2048, 24, False),      # pairs of tiles half empty
+    (50, 300, 5120, 24, False), (20, 700, 8192, 17, True),     # rows too wide for the other tensor-core kernels
+], ids=lambda v: str(v))
+def test_which_path_auto_takes_for_17_to_32_pivots(B, n, d, P, flow):
+    """Both sides of every line of the rule; keys whose sums are exact in any order, so that the other paths give the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(B + n + d)
+    k = torch.randint(-15, 16, (B, n + 9, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
+    outs = []
+    for path in (dart.DART_PATH_AUTO, dart.DART_PATH_STAGED):
+        ctx = dart.Dart(B, n + 9, d, P, P + 40)
+        dart.dart_profile_enable(ctx.handle, True)
+        outs.append(ctx.reduce(k, None, 4, n, P, P + 40, opts=dart.dart_opts(path=path)))
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        launched = {name for name, (_, c) in dart.dart_profile_read(ctx.handle)[1].items() if c}
+        assert ("flow" in launched) == (flow and path == dart.DART_PATH_AUTO), launched
+        ctx.close()
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
 @pytest.mark.parametrize("norm_kind,smallest", [(1, 1), (2, 0), (2, 1)])
 def test_flow_ranking_variants(oracle, norm_kind, smallest):
     k, h = gaussian(3, 500, 256, seed=77)
