@@ -55,9 +55,9 @@ enum {
 #define DART_PATH_FUSED 2  /* persistent sweep kernel (scores, pivots and similarities in one launch; with the caller's
                               pivots: scores and similarities from one pass over the keys); needs d % 64 == 0 and
                               n_pivot <= 256, else UNSUPPORTED. */
-#define DART_PATH_TWO_PASS 3 /* two launches instead of the persistent sweep: a plain score pass, pivot selection, then
-                              scores' sums of squares and similarities from one tensor-core pass; same limits as FUSED.
-                              Reads the keys twice like FUSED but has no waits between CTAs: faster for small batches. */
+#define DART_PATH_TWO_PASS 3 /* launches without waits between CTAs instead of the persistent sweep: a plain score pass, pivot
+                              selection, then the similarities from one tensor-core pass; same limits as FUSED.  AUTO takes it
+                              from 17 pivots on where the flow path is behind it. */
 
 #define DART_PATH_RESIDENT 4 /* steps 1-3 from ONE read of the keys: every sample is spread over all SMs and stays in their
                               shared and tensor memory until its pivots are known.  Needs n_pivot <= 8, d % 64 == 0,
@@ -77,8 +77,10 @@ enum {
 
 #define DART_PATH_FLOW 7     /* steps 1-3 in one persistent launch that keeps the time between a row's two reads, and with it
                               the bytes that pass between them, small enough for the L2 to serve the second.  Needs
-                              n_pivot <= 32, d % 64 == 0, n_vis <= 8192, one tensor for steps 1-3, else UNSUPPORTED.  The fastest path up
-                              to 16 pivots, and up to 32 on small batches (AUTO takes it there). */
+                              n_pivot <= 32, d % 64 == 0, d <= 8192, n_vis <= 8192, one tensor for steps 1-3, and a context whose
+                              maxima leave the slices' shares of the similarities (32 to 256 floats per row, by P_max and d)
+                              within 1 GiB, else UNSUPPORTED.  The fastest path up to 16 pivots for d >= 1024, and
+                              up to 32 on small batches (AUTO takes it there). */
 
 /* dart_opts.pivot_source: where step 2 takes the pivots from when the caller does not name them (pivots_in == NULL) */
 #define DART_PIVOTS_BY_SCORE 0 /* the n_pivot vision tokens of best score (dart_reduce) */

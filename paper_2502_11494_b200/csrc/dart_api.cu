@@ -473,6 +473,14 @@ int launch_staged(dart_ctx *ctx, int B, const void *hidden, const void *keys_in,
 int flow_tiles(int P) { return P <= 8 ? 1 : P <= 16 ? 2 : 4; } // pivot tiles of 8 the flow kernel is compiled for
 size_t flow_groups(const dart_ctx *ctx) { return (size_t)ctx->desc.B_max * ((ctx->desc.S_max + dart::flow::kRows - 1) / dart::flow::kRows); }
 
+// Whether slices of na atoms leave shared memory room for the least rings beside the pivot tiles.
+size_t flow_smem_limit(const dart_ctx *ctx) { return (size_t)ctx->max_smem_optin - dart::flow::kStaticSmemReserve - 1024; }
+bool flow_fits(const dart_ctx *ctx, int NT, int na)
+{
+    namespace F = dart::flow;
+    return F::pivot_bytes(NT, na) + 2 * (size_t)F::kStageBytes + (size_t)F::kScoreWarps * F::kChunkBytes <= flow_smem_limit(ctx);
+}
+
 // The words and counters of the flow path as every call expects to find them.
 int flow_reset(dart_ctx *ctx, cudaStream_t st)
 {
@@ -510,9 +518,14 @@ int fused_setup(dart_ctx *ctx)
     {   // shares of the similarities: the sweep's column chunks for up to 16 pivots, or the flow path's slices (four of them,
         // more for small batches); contexts that would need more than 1 GiB go without
         size_t n = (size_t)kSweepChunks * D.B_max * (D.P_max < kSweepChunkMaxP ? D.P_max : kSweepChunkMaxP) * D.S_max;
-        const size_t one = flow_groups(ctx) * dart::flow::kRows * 8 * flow_tiles(D.P_max < dart::flow::kMaxP ? D.P_max : dart::flow::kMaxP);
+        // (as many slices at least as the widest pivot tile needs to fit shared memory, if that is within the GiB)
+        const int NT = flow_tiles(D.P_max < dart::flow::kMaxP ? D.P_max : dart::flow::kMaxP);
+        const size_t one = flow_groups(ctx) * dart::flow::kRows * 8 * NT, gib = ((size_t)1 << 30) / sizeof(float);
         const size_t small = one * dart::flow::kMaxSlices < ((size_t)8 << 20) ? one * dart::flow::kMaxSlices : ((size_t)8 << 20);
-        ctx->flow_part_n = one * 4 > small ? one * 4 : small;
+        size_t least = 4;
+        while (least < dart::flow::kMaxSlices && !flow_fits(ctx, NT, (ctx->n_atoms + (int)least - 1) / (int)least)) least *= 2;
+        if (one * least > gib) least = 4;
+        ctx->flow_part_n = one * least > small ? one * least : small;
         if (n < ctx->flow_part_n) n = ctx->flow_part_n;
         if (n * sizeof(float) <= ((size_t)1 << 30)) rc = ws_alloc(ctx, &ctx->sim_share, n);
         if (rc != DART_OK) return rc;
@@ -754,7 +767,7 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     p.given = o.pivots_in != nullptr;
     p.sel_threads = F::sel_threads(n_vis);
     p.n_stream = ctx->sm_count - (p.given ? 0 : F::selectors(sample));
-    const size_t limit = (size_t)ctx->max_smem_optin - F::kStaticSmemReserve - 1024;
+    const size_t limit = flow_smem_limit(ctx);
     p.n_atoms = ctx->n_atoms, p.n_rg = (n_vis + F::kRows - 1) / F::kRows;
     double best = 0;
     // two rows to a chunk where they fill it: a task's fixed costs are paid per chunk
@@ -763,7 +776,7 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     p.nsl = 0;
     for (int nsl = 1; nsl <= F::kMaxSlices && nsl <= p.n_atoms && nsl <= p.n_stream; nsl *= 2) {
         const int na = (p.n_atoms + nsl - 1) / nsl;
-        if (F::pivot_bytes(NT, na) + 2 * (size_t)F::kStageBytes + (size_t)F::kScoreWarps * F::kChunkBytes > limit) continue;
+        if (!flow_fits(ctx, NT, na)) continue;
         if (na > F::kMaxItemAtoms && nsl < 4 && !want_nsl) continue; // an item's time is part of what lies between the two reads of a row
         if ((size_t)B * p.n_rg * nsl * 8 * NT * F::kRows > ctx->flow_part_n) continue;
         // the longest queue of items of any SM, in bytes plus what an item costs beside its bytes

@@ -96,6 +96,25 @@ def test_which_path_auto_takes_for_17_to_32_pivots(B, n, d, P, flow):
     assert all(torch.equal(a, b) for a, b in zip(*outs))
 
 
+@pytest.mark.parametrize("P", [17, 32])
+@pytest.mark.parametrize("d", [4608, 4672, 5120, 8192])
+def test_flow_takes_wide_rows_with_many_pivots_in_large_contexts(oracle, d, P):
+    """The widest pivot tiles of the widest rows need eight slices, whose shares the workspace has to hold however large it is."""
+    B, S, vo, nv, Kp = 2, 300, 7, 280, 60
+    k, h = gaussian(B, S, d, seed=d + P)
+    ctx = dart.Dart(600, S, d, P, Kp)     # 3000 row groups
+    try:
+        res = ctx.reduce(h, k, vo, nv, P, Kp, debug=True, opts=dart.dart_opts(path=FLOW))
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+    finally:
+        ctx.close()
+    kb, hb = W.bits(k), W.bits(h)
+    rep = parity.check_batch(oracle.reduce(hb, kb, vo, nv, P, Kp), kb, hb, vo, nv, P, Kp, _np(res[0]), _np(res[1]), _np(res[2]),
+                             dbg={n: _np(v) for n, v in res[3].items()})
+    assert rep.exact >= rep.above_margin and rep.max_abs_sim < 2e-5
+
+
 @pytest.mark.parametrize("norm_kind,smallest", [(1, 1), (2, 0), (2, 1)])
 def test_flow_ranking_variants(oracle, norm_kind, smallest):
     k, h = gaussian(3, 500, 256, seed=77)
