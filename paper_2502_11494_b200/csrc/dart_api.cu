@@ -19,6 +19,7 @@ namespace {
 
 constexpr int kSweepChunks = 8;     // column chunks per row tile of the persistent sweep's second pass
 constexpr int kSweepChunkMaxP = 16; // ... for up to this many pivots
+constexpr int kMaxArrays = 64;      // of a context's workspace (a plain array: nothing in dart_create may throw)
 constexpr int kMaxGridY = 65535;    // CUDA's limit for a grid's second dimension
 
 enum Slot { SLOT_SCORE = 0, SLOT_PIVOT, SLOT_SIM, SLOT_RETAIN, SLOT_GATHER, SLOT_SWEEP, SLOT_ONEPASS, SLOT_RESIDENT, SLOT_PAIR, SLOT_FLOW, SLOT_COUNT };
@@ -42,7 +43,8 @@ struct dart_ctx {
     int64_t launches;
     size_t bytes;
     void *ws_base;                 // the workspace's one allocation
-    std::vector<void **> ws_slots; // until it is made: the arrays' pointers
+    void **ws_slots[kMaxArrays];   // until it is made: the arrays' pointers
+    int ws_n;
     // workspace (device), indexed with the shapes of the current call
     float *l1, *ssq, *sim, *eps;
     int32_t *pivot_idx, *owner;
@@ -121,8 +123,9 @@ template <typename T>
 int ws_alloc(dart_ctx *ctx, T **p, size_t count)
 {
     const size_t bytes = (count * sizeof(T) + 255) / 256 * 256;
+    if (ctx->ws_n == kMaxArrays) return DART_ERR_NOMEM;
     *p = reinterpret_cast<T *>(ctx->bytes + 256); // not NULL: the array exists from here on
-    ctx->ws_slots.push_back(reinterpret_cast<void **>(p));
+    ctx->ws_slots[ctx->ws_n++] = reinterpret_cast<void **>(p);
     ctx->bytes += bytes;
     return DART_OK;
 }
@@ -130,8 +133,8 @@ int ws_alloc(dart_ctx *ctx, T **p, size_t count)
 int ws_commit(dart_ctx *ctx)
 {
     const cudaError_t e = cudaMalloc(&ctx->ws_base, ctx->bytes);
-    for (void **p : ctx->ws_slots) *p = e == cudaSuccess ? (char *)ctx->ws_base + ((size_t)*p - 256) : nullptr;
-    ctx->ws_slots.clear();
+    for (int k = 0; k < ctx->ws_n; ++k) *ctx->ws_slots[k] = e == cudaSuccess ? (char *)ctx->ws_base + ((size_t)*ctx->ws_slots[k] - 256) : nullptr;
+    ctx->ws_n = 0;
     return e == cudaSuccess ? DART_OK : cuda_fail(ctx, e);
 }
 

@@ -99,3 +99,12 @@ def test_product_does_not_import_the_oracle():
                 assert "oracle" not in src.lower() or f == "workloads.py", "%s mentions the oracle" % f
     src = open(os.path.join(pkg, "workloads.py")).read()
     assert "import oracle" not in src and "from oracle" not in src
+
+
+def test_creating_a_context_cannot_throw():
+    """C entries return codes: what dart_create runs allocates host memory by the one new that returns NULL."""
+    src = open(os.path.join(ROOT, "paper_2502_11494_b200", "csrc", "dart_api.cu")).read()
+    bodies = [src.split(head)[1].split("\n}\n")[0] for head in ("int ws_alloc(dart_ctx", "int ws_commit(dart_ctx", "int flow_reset(dart_ctx", "int fused_setup(dart_ctx", "int dart_create(dart_ctx")]
+    for body in bodies:
+        code = re.sub(r"//[^\n]*", "", body).replace("new (std::nothrow) dart_ctx()", "")
+        assert not re.search(r"push_back|resize|reserve|\bnew\b|std::(vector|string|map)", code), body[:80]
