@@ -107,6 +107,7 @@ namespace {
 int cuda_fail(dart_ctx *ctx, cudaError_t e)
 {
     if (ctx) ctx->last_cuda = (int)e;
+    cudaGetLastError(); // reported here: the next call that looks for launch errors must not find it again
     return e == cudaErrorMemoryAllocation ? DART_ERR_NOMEM : DART_ERR_CUDA;
 }
 

@@ -526,3 +526,16 @@ def test_the_call_can_be_captured_in_a_cuda_graph(B):
         assert all(torch.equal(a, b) for a, b in zip(out, ref))
     finally:
         ctx.close()
+
+
+def test_a_failed_allocation_is_reported_once():
+    """A context too large for the device is refused; calls on other contexts afterwards do not find its error."""
+    k, h = gaussian(2, 300, 64, seed=3)
+    ctx = dart.Dart(2, 300, 64, 4, 40)
+    rc, other = dart.dart_create(4096, 65536, 64, 1024, 4096)    # similarities alone: 1 TiB
+    assert rc == dart.DART_ERR_NOMEM and not other
+    for path in (dart.DART_PATH_AUTO, dart.DART_PATH_STAGED):
+        ctx.reduce(h, k, 10, 280, 4, 40, opts=dart.dart_opts(path=path))
+    torch.cuda.synchronize()
+    assert ctx.status() == dart.DART_OK
+    ctx.close()
