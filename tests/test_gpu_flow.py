@@ -27,6 +27,8 @@ SHAPES = [
     (1, 9000, 192, 5, 4097, 32, 500),     # a last row group of one row
     (3, 80, 8192, 2, 70, 12, 30),         # the widest rows
     (300, 40, 64, 1, 33, 4, 9),           # more samples than SMs
+    (3, 400, 1024, 5, 301, 7, 60),        # two rows to a scoring task, the last task of one row
+    (2, 9, 1024, 3, 1, 1, 1), (3, 80, 1024, 2, 65, 20, 40), (5, 300, 1024, 9, 128, 16, 30),
 ]
 
 
@@ -196,4 +198,88 @@ def test_flow_expired_waits_are_reported_not_hung():
     assert ctx.status() == dart.DART_OK
     ref = run_gpu(k, h, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep, path=dart.DART_PATH_STAGED, debug=False)
     assert np.array_equal(good[1].cpu().numpy(), ref[1]) and np.array_equal(W.bits(good[0]), ref[0])
+    ctx.close()
+
+
+def _calls(seed, n):
+    """A mixed bag of calls within the maxima (6, 900, 256, 32, 700): batch sizes, lengths, pivots, paths, rules."""
+    rng = np.random.default_rng(seed)
+    for i in range(n):
+        nv = int(rng.choice([rng.integers(1, 70), rng.integers(64, 800)]))
+        P = int(rng.integers(1, min(nv, 32) + 1))
+        path = int(rng.choice([FLOW, FLOW, FLOW, dart.DART_PATH_AUTO, dart.DART_PATH_TWO_PASS, dart.DART_PATH_FUSED, dart.DART_PATH_STAGED]))
+        yield dict(B=int(rng.integers(1, 7)), vo=int(rng.integers(0, 50)), nv=nv, after=int(rng.integers(0, 50)), P=P,
+                   Kp=int(rng.integers(P, min(nv, 700) + 1)), path=path, given=bool(rng.integers(0, 3) == 0), union=bool(rng.integers(0, 4) == 0),
+                   retention=int(rng.choice([dart.DART_RETAIN_AUTO, dart.DART_RETAIN_RANKED])), seed=1000 * seed + i)
+
+
+def _inputs(c, d):
+    k, h = gaussian(c["B"], c["vo"] + c["nv"] + c["after"], d, seed=c["seed"])
+    g = torch.Generator(device="cuda").manual_seed(c["seed"])
+    piv = torch.rand((c["B"], c["nv"]), generator=g, device="cuda").topk(c["P"], dim=1).indices.to(torch.int32).contiguous()
+    S_out = c["vo"] + c["after"] + c["Kp"]
+    out = (torch.zeros((c["B"], S_out, d), dtype=torch.bfloat16, device="cuda"), torch.zeros((c["B"], S_out), dtype=torch.int32, device="cuda"),
+           torch.zeros((c["B"], S_out), dtype=torch.int64, device="cuda"))
+    cu = torch.zeros(c["B"] + 1, dtype=torch.int32, device="cuda")
+    opts = dart.dart_opts(path=c["path"], retention=c["retention"], pivots_in=piv.data_ptr() if c["given"] else None,
+                          rule=dart.DART_RULE_UNION if c["union"] else dart.DART_RULE_QUOTAS, cu_seqlens=cu.data_ptr() if c["union"] else None)
+    return dict(k=k, h=h, piv=piv, out=out, cu=cu, opts=opts)
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_one_context_through_changing_calls(seed):
+    """The words and counters that a call leaves behind are the next call's, whatever its tensors, batch, length, pivots and path:
+    forty different calls on one context, nothing between them, against a context of its own for each."""
+    d, calls = 256, list(_calls(seed, 40))
+    bags = [_inputs(c, d) for c in calls]
+    shared = dart.Dart(6, 900, d, 32, 700)
+    torch.cuda.synchronize()
+    for c, x in zip(calls, bags):
+        shared.reduce(x["h"], x["k"], c["vo"], c["nv"], c["P"], c["Kp"], out=x["out"], opts=x["opts"])
+    torch.cuda.synchronize()
+    assert shared.status() == dart.DART_OK, dart.dart_status_detail(shared.handle)
+    shared.close()
+    for c, x in zip(calls, bags):
+        y = _inputs(c, d)
+        ctx = dart.Dart(c["B"], c["vo"] + c["nv"] + c["after"], d, c["P"], c["Kp"])
+        ctx.reduce(x["h"], x["k"], c["vo"], c["nv"], c["P"], c["Kp"], out=y["out"], opts=y["opts"])
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        ctx.close()
+        n = int(y["cu"][-1]) if c["union"] else None      # rows beyond the packed ones are not written
+        assert torch.equal(x["cu"], y["cu"]), c
+        for a, b in zip(x["out"], y["out"]):
+            a, b = (a.view(-1, d) if a.dim() == 3 else a.view(-1), b.view(-1, d) if b.dim() == 3 else b.view(-1))
+            assert torch.equal(a[:n], b[:n]), c
+
+
+def test_a_graph_replays_on_new_contents_between_other_calls():
+    """A captured call reads what its input buffers hold when it is replayed, and finds its words as it expects them after eager
+    calls of other shapes on the same context."""
+    d, s, g = 256, torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    c = dict(B=5, vo=7, nv=600, after=30, P=8, Kp=90, path=FLOW, given=False, union=False, retention=0, seed=1)
+    others = list(_calls(77, 6))
+    x = _inputs(c, d)
+    ctx = dart.Dart(6, 900, d, 32, 700)
+    with torch.cuda.stream(s):
+        ctx.reduce(x["h"], x["k"], c["vo"], c["nv"], c["P"], c["Kp"], out=x["out"], opts=x["opts"], stream=s)
+        s.synchronize()
+        g.capture_begin()
+        ctx.reduce(x["h"], x["k"], c["vo"], c["nv"], c["P"], c["Kp"], out=x["out"], opts=x["opts"], stream=s)
+        g.capture_end()
+        for i, o in enumerate(others):
+            y = _inputs(dict(o, union=False), d)
+            ctx.reduce(y["h"], y["k"], o["vo"], o["nv"], o["P"], o["Kp"], out=y["out"], opts=y["opts"], stream=s)
+            fresh = _inputs(dict(c, seed=100 + i), d)
+            x["k"].copy_(fresh["k"])
+            x["h"].copy_(fresh["h"])
+            g.replay()
+            s.synchronize()
+            assert ctx.status() == dart.DART_OK
+            got = [t.clone() for t in x["out"]]
+            own = dart.Dart(c["B"], 637, d, 8, 90)
+            own.reduce(fresh["h"], fresh["k"], c["vo"], c["nv"], c["P"], c["Kp"], out=fresh["out"], opts=fresh["opts"], stream=s)
+            s.synchronize()
+            own.close()
+            assert all(torch.equal(a, b) for a, b in zip(got, fresh["out"]))
     ctx.close()

@@ -503,7 +503,7 @@ def test_profile_slots_cover_every_launch():
 @pytest.mark.parametrize("B", [1, 6])
 def test_the_call_can_be_captured_in_a_cuda_graph(B):
     """All work goes to the caller's stream and nothing synchronises the host: a captured call replays with the
-    same outputs (one sample takes the resident sweep, six the persistent one; both launch cooperatively)."""
+    same outputs (the flow kernel launches cooperatively, the kernels behind it as programmatic dependents)."""
     w = W.LLAVA15_B64.with_(B=B)
     k, h = W.make_batch(w, device="cuda")
     ctx = dart.Dart(w.B, w.S, w.d, w.n_pivot, w.n_keep)
