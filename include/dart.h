@@ -188,8 +188,8 @@ typedef struct {
     int32_t tune;          /* 0 = defaults.  DART_PATH_PAIRED: 256 * n1 + 16 * n2 + n3 = depths of the three shared-memory rings.
                               DART_PATH_FUSED: >= 2 cuts the second pass of a row tile into eight column chunks (one task each)
                               and keeps the first pass within `tune` steps of the second (low 12 bits).  One-pass kernel:
-                              bit 0x1000 = one row tile per task, bit 0x2000 = two where they fit (default: two when every
-                              CTA gets at least two tasks).  DART_PATH_FLOW: low 8 bits = how many MB of rows the scores may be ahead of
+                              bit 0x1000 = one row tile per task, bit 0x2000 = two where they fit (default: two where that
+                              shortens the longest queue of any CTA).  DART_PATH_FLOW: low 8 bits = how many MB of rows the scores may be ahead of
                               the pivots, bits 12-14 = chunks of a row on their way per scoring warp, bits 16-20 = column
                               slices (1, 2, 4, 8 or 16).  All of them tuning options: same results. */
 } dart_opts;

@@ -256,8 +256,9 @@ int copy_debug(dart_ctx *ctx, int B, int n_vis, int P, const dart_debug *dbg, cu
     return DART_OK;
 }
 
-// Steps 4 and 5a.  Two phases (candidate lists for all pivots at once, then the pivots' turns) when the lists fit
-// the workspace and shared memory, else the one-kernel form.
+// Steps 4 and 5a.  Ranked lists wherever their workspace, their limits and the grid take the call (rows of up to 16384 tokens, lists
+// of up to 4096); the older forms below serve what is left - longer rows and lists, contexts without the lists, calls that keep
+// the pivots alone - and by option.
 int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset, int n_vis, int P, int n_keep,
                       int32_t *out_idx, int64_t *out_pos, const dart_opts &o, const dart_debug *dbg, cudaStream_t st)
 {
@@ -325,7 +326,8 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     const int band_cap = ctx->band_stride < kPickStageEntries ? ctx->band_stride : kPickStageEntries;
     const bool can_bands = ctx->band && grid_fits && m > 0 && m <= band_cap && n_vis <= kBandMaxTokens && band_smem_bytes(n_vis, band_cap) <= (size_t)ctx->max_smem_optin - 2048 &&
                            pick_smem_bytes(n_vis, P) <= (size_t)ctx->max_smem_optin - 2048;
-    // AUTO: ranked lists wherever they fit (us, bands / ranked: 256 samples x 32 pivots x 200 tokens keeping 60 58 / 37, x 576 66 / 46,
+    // AUTO: ranked lists wherever they fit (over 23 batches of many lists, keeping 40 % to everything, the bands are ahead only around 1000
+    // tokens with 32 or 64 pivots from 70 % on, by 3 to 17 %; us, bands / ranked: 256 samples x 32 pivots x 200 tokens keeping 60 58 / 37, x 576 66 / 46,
     // x 1000 73 / 51; 128 pivots x 576 keeping 300 220 / 181, x 1000 keeping 500 279 / 219, x 1500 keeping 166 122 / 123, keeping 700
     // 355 / 287, x 2880 410 / 354; 8 pivots x 576 31 / 21, x 2880 58 / 38; one sample, 8 pivots x 2880: 39 / 17)
     // Pivots alone are kept: there is no list, and the sorted lists' second kernel is all there is to run (1 x 200, 32 pivots 11 -> 7 us;
@@ -798,8 +800,10 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     p.n_st = (int)(n_st > (size_t)F::kMaxStages ? (size_t)F::kMaxStages : n_st);
     // The scorers' lead over the last sample whose pivots are known, in bytes of rows: enough to keep them busy while a
     // sample's last rows, its selection and its pivots' publication take their time (36 MB), but no more than the L2 keeps for
-    // the second read.  Measured at 256 x 2880 x 4096, us per launch: 32 MB 1557, 52 MB 1519, 60 MB 1395, 64 MB 1498, 72 MB
-    // 1593, 128 MB 2070 (both reads from HBM); at 64 x 4096 x 4096: 64 MB 579, 72 MB 552, 80 MB 605.
+    // the second read.  us per launch, 8 pivots, by MB (the rule's in brackets): 256 x 2880 x 4096 44: 1665, 52: 1300, [59: 1256], 72:
+    // 1263, 96: 1529; 16 pivots 52: 1361, [59: 1352], 60: 1321, 72: 1372; 64 x 4096 x 4096 56: 518, [68: 477], 80: 480, 96: 558; 100 x
+    // 6000 x 4096 64: 1352, [72: 1200], 80: 1133, 96: 1309; 256 x 2880 x 2048 36: 718, [47: 679], 72: 674, 96: 773.  Short samples do not
+    // mind: 256 x 576 x 4096 272 to 273 from 44 to 80 MB, 250 x 1000 x 3072 423 to 426 from 44 to 128.
     long long window = sample + 36 * MB < 72 * MB ? sample + 36 * MB : 72 * MB;
     if (window < sample + 20 * MB) window = sample + 20 * MB;
     if (o.tune & 0xff) window = (long long)(o.tune & 0xff) * MB > sample ? (long long)(o.tune & 0xff) * MB : sample;

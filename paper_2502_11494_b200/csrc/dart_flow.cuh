@@ -19,10 +19,14 @@
 // slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
 //
+// What bounds it: no unit.  16 x 2880 x 4096, 8 pivots (99 us): DRAM 49 % of its peak, L2 40 %, L2 to SM 25 % (8.5 TB/s: every key byte crosses
+// twice), shared-memory wavefronts 32 %, issue slots 46 %, tensor pipe 6 %; the warps wait for values on their way (long scoreboard 4.3
+// of 11.4 cycles per instruction) - the distance between a row's two reads, start and tail.
+//
 // Per CTA (736 or 864 threads, one CTA per SM, cooperative launch):
 //   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
-//   warps 4-7    second pass: mma.sync.m16n8k16 (16 rows each; P <= 32 leaves the tensor pipe idle whatever the form, and
-//                64-row items do not fill the 128 rows of a tcgen05.mma)
+//   warps 4-7    second pass: mma.sync.m16n8k16, 16 rows each (the tensor pipe is 6 % busy; what the form costs is that every warp
+//                reads the pivot tile from shared memory again, which a tcgen05.mma of 64 rows would do once)
 //   warp 8       producer: TMA tiles of 64 rows x 64 columns (128-byte swizzle), two per ring stage
 //   warps 9-12   combine: count the item, and if it is its row group's last, add up the slices and write the similarities
 //   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
@@ -540,7 +544,7 @@ __device__ __forceinline__ void take_pivots(const Params &p, const Ctl &ctl, Sha
 // Second pass: 16 rows of the item per warp, all columns of the slice, NT of the sample's NTall tiles of 8 pivots (from tile n0 on).
 // (32 pivots: one group 2.48, two groups 2.07 ms at 256 x 2880 x 4096: a dependent product returns after some 130 cycles, and a
 // warp had 16 per atom to wait for.  16 pivots: one group 1.30, two 1.76 ms: a second group reads the rows from shared memory a
-// second time, and that is what bounds the kernel then: every key byte is written there twice and read twice.)
+// second time.)
 template <int NT, int NTall>
 __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared &sh, uint32_t ring0, uint32_t piv0, int w, int n0)
 {
