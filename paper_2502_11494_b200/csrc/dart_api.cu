@@ -815,8 +815,9 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
 // Whether AUTO takes the flow path.
 // Pivots by score, up to 16: for rows of 1024 columns and more it is the fastest path at every size measured, from one sample of 130
 // tokens (21 us against 23 us of the resident sweep) to 256 x 2880 x 4096 (8 pivots 1.25 against 1.85 ms of the sweep, 16 pivots
-// 1.30 against 1.87).  Narrower rows have two passes up to 1.5 times as fast on large batches (256 x 2880 x 64, 8 pivots; 64 x 2880 x
-// 512 1.24 times): nobody's hidden states are that narrow, and there is no line for them.
+// 1.30 against 1.87).  Narrower rows take a scorer or a selector no less time than wide ones, and two passes are ahead from about 64 rows per
+// column on (whole calls, us, flow / two passes: 32 x 1025 x 512 1.02 times as long, 64 x 1025 1.09, 64 x 5000 288 / 227, 150 x 5000 x 256
+// 630 / 421, 64 x 576 x 256 1.10, 32 x 576 1.01, 150 x 5000 x 768 665 / 562, 32 x 1500 1.01).
 // 17 to 32 pivots by score: its multiplying warps bound it, and every row takes as many products as for 32.  Over 1100 shapes of 64
 // to 7000 tokens and 1 to 250 samples (whole calls, us, flow / two passes: 2 x 576 x 4096 41 / 58, 8 x 1000 x 4096 70 / 81, 8 x 1500 84 / 91, but 8 x 2880 x 4096 126 / 115, 4 x 4608 115 / 98, 32 x 1000 156 / 144, 128 x 700 x 3072
 // 294 / 264) the two meet at about 12 thousand rows from 3072 columns on and 8 thousand of 2048 (8 x 1000 x 2048 56 / 58, 8 x 1500 64 / 63);
@@ -835,7 +836,9 @@ bool flow_preferred(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opt
     const long long row_tiles = (long long)B * ((n_vis + dart::sweep::kTileRows - 1) / dart::sweep::kTileRows);
     if (o.pivots_in) {
         if (row_tiles >= ctx->sm_count || P > 16) return false;
-    } else if (P > 16 && fused_applies(ctx, P)) { // (rows too wide for the other tensor-core kernels: nothing else is near it)
+    } else if (P <= 16) {
+        if (d < 1024 && rows > 64 * d && fused_applies(ctx, P) && ctx->piv_rows) return false;
+    } else if (fused_applies(ctx, P)) { // (rows too wide for the other tensor-core kernels: nothing else is near it)
         const int padded = (n_vis + 255) / 256 * 256; // rows of the one-pass kernel's pairs of tiles
         const long long most = d >= 2048 ? (4 * d < 12000 ? 4 * d : 12000) : P <= 24 && n_vis <= 1400 ? 60000 : 8000, least = d >= 2048 ? 1 : 1000;
         const bool few = ctx->piv_rows ? d >= 1024 && rows <= most && rows >= least : rows * d * 2 <= 300000000ll;

@@ -72,7 +72,9 @@ def test_flow_matches_the_oracle(oracle, shape, given):
 
 
 @pytest.mark.parametrize("B,n,d,P,flow", [
-    (2, 300, 960, 8, True), (2, 300, 960, 17, False),          # up to 16 pivots always; rows of fewer than 1024 columns never
+    (2, 300, 960, 8, True), (2, 300, 960, 17, False),          # rows of fewer than 1024 columns: never, up to 16 pivots
+    (16, 2048, 512, 16, True), (5, 6554, 512, 16, False),      # ... up to 64 rows per column
+    (5, 819, 64, 1, True), (5, 820, 64, 1, False), (40, 1700, 1024, 16, True),
     (3, 333, 1024, 17, False), (2, 500, 1024, 32, True),       # 1000 rows and more of 1024 columns
     (8, 1000, 1024, 25, True), (9, 1000, 1024, 25, False),     # ... up to 8000
     (60, 1000, 1024, 24, True), (9, 1401, 1024, 17, False),    # ... up to 60000 with up to 24 pivots and 1400 tokens
@@ -81,7 +83,7 @@ def test_flow_matches_the_oracle(oracle, shape, given):
     (1, 100, 4096, 24, True), (50, 300, 2048, 24, True), (50, 400, 2048, 24, False),      # pairs of tiles half empty
     (50, 300, 5120, 24, False), (20, 700, 8192, 17, True),     # rows too wide for the other tensor-core kernels
 ], ids=lambda v: str(v))
-def test_which_path_auto_takes_for_17_to_32_pivots(B, n, d, P, flow):
+def test_which_path_auto_takes(B, n, d, P, flow):
     """Both sides of every line of the rule; keys whose sums are exact in any order, so that the other paths give the same bits."""
     g = torch.Generator(device="cuda").manual_seed(B + n + d)
     k = torch.randint(-15, 16, (B, n + 9, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
