@@ -93,6 +93,7 @@ struct FlowState {
     long long n_rec, n_cnt, n_pv;
     __device__ __forceinline__ void put_back() const
     {
+        if (!rec) return; // (another path's call: the three loops alone took a fifth of a copy of narrow rows)
         const long long n = (long long)gridDim.x * blockDim.x, t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
         for (long long i = t; i < n_rec; i += n) rec[i] = ~0ull;
         for (long long i = t; i < n_cnt; i += n) cnt[i] = 0;
