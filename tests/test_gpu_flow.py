@@ -159,15 +159,15 @@ def test_flow_many_equal_scores(values, P, n_vis):
         want = torch.sort(score, dim=1, descending=not smallest, stable=True).indices[:, :P]
         assert torch.equal(dbg["pivot_idx"].long(), want)
     start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    times = {}
-    for path in (FLOW, dart.DART_PATH_STAGED):       # the staged path selects by radix passes whatever the scores
+    times = {FLOW: [], dart.DART_PATH_STAGED: []}    # the staged path selects by radix passes whatever the scores
+    for path in list(times) * 5:                      # (the best of five: the host may pause between launches)
         start.record()
-        for _ in range(10):
+        for _ in range(4):
             ctx.reduce(keys, None, vo, n_vis, P, P, opts=dart.dart_opts(path=path))
         end.record()
         torch.cuda.synchronize()
-        times[path] = start.elapsed_time(end)
-    assert times[FLOW] < 3 * times[dart.DART_PATH_STAGED], times   # quadratic: 20 times as long at 8192 equal scores
+        times[path].append(start.elapsed_time(end))
+    assert min(times[FLOW]) < 3 * min(times[dart.DART_PATH_STAGED]), times   # quadratic: 20 times as long at 8192 equal scores
     ctx.close()
 
 
