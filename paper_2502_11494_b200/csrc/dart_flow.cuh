@@ -23,7 +23,7 @@
 // twice), shared-memory wavefronts 32 %, issue slots 46 %, tensor pipe 6 %; the warps wait for values on their way (long scoreboard 4.3
 // of 11.4 cycles per instruction) - the distance between a row's two reads, start and tail.
 //
-// Per CTA (736 or 864 threads, one CTA per SM, cooperative launch):
+// Per CTA (768 or 896 threads, one CTA per SM, cooperative launch):
 //   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
 //   warps 4-7    second pass: mma.sync.m16n8k16, 16 rows each (the tensor pipe is 6 % busy; what the form costs is that every warp
 //                reads the pivot tile from shared memory again, which a tcgen05.mma of 64 rows would do once)
@@ -31,8 +31,8 @@
 //   warps 9-12   combine: count the item, and if it is its row group's last, add up the slices and write the similarities
 //   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
 //   warp 21      watcher: how far the pivots of the batch have got, for the scorers' window
-//   warp 22      feeder: the scorers' rows into their slots
-//   warps 23-26  with more than 16 pivots: second pass for the second half of the pivots
+//   warps 22-23  feeders: the scorers' rows into their slots
+//   warps 24-27  with more than 16 pivots: second pass for the second half of the pivots
 // Every wait is bounded in time; on expiry the kernel records DART_ERR_TIMEOUT in the status word, lets the copies in flight
 // land and exits normally.
 #pragma once
@@ -63,7 +63,8 @@ constexpr int kCombWarp0 = 9, kCombWarps = 4; // (an item is counted 2-3 us afte
 constexpr int kScoreWarp0 = kCombWarp0 + kCombWarps, kScoreWarps = 8;
 constexpr int kWatchWarp = kScoreWarp0 + kScoreWarps;
 constexpr int kFeedWarp = kWatchWarp + 1;
-constexpr int kMulWarp1 = kFeedWarp + 1;
+constexpr int kFeedWarps = 2;
+constexpr int kMulWarp1 = kFeedWarp + kFeedWarps;
 __host__ __device__ constexpr int mul_groups(int NT) { return NT > 2 ? 2 : 1; }
 __host__ __device__ constexpr int threads(int NT) { return 32 * (kMulWarp1 + (mul_groups(NT) - 1) * kMulWarps); }
 constexpr int kChunk = 8;                  // scorers: 16-byte pieces per lane and chunk
@@ -237,12 +238,14 @@ struct Tasks {
     }
 };
 
-// Feeder: lane w keeps scorer w's p.n_slot slots (4 KB chunks of rows) on their way, as far as the window allows.  A warp of its
+// Feeders: a lane keeps one scorer's p.n_slot slots (4 KB chunks of rows) on their way, as far as the window allows.  Warps of their
 // own: a bulk copy takes its thread some 500 cycles to issue (with every scorer refilling its own slots a row of 8 KB took
-// 4000 cycles, and the scorers bound the whole path).
+// 4000 cycles, and the scorers bound the whole path).  Two: a warp that feeds all eight scorers spends 195 cycles per copy and nothing
+// else 88 % of the time (whole calls, us, one / two: 64 x 576 118 / 115, 8 x 1500 x 3072 60.5 / 59.3, 256 x 2880 1585 / 1535; three 1595, and four,
+// which costs registers, 1645).
 __device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
 {
-    const int w = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, w = ((int)(threadIdx.x >> 5) - kFeedWarp) + kFeedWarps * lane; // this lane's scorer
     unsigned long long policy;
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
     const int nc = p.n_chunk;
@@ -280,7 +283,7 @@ __device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh
         if ((++spin & 31u) == 0u) {
             bool dead = ctl.aborted();
             if (!dead && (unsigned long long)(clock64() - since) > ctl.limit_cycles) {
-                if (w == 0) ctl.give_up(kWaitWindow, it.b);
+                if (lane == 0) ctl.give_up(kWaitWindow, it.b);
                 dead = true;
             }
             if (__any_sync(0xffffffffu, dead)) break;
@@ -817,7 +820,7 @@ __global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_const
         if (threadIdx.x < kSel) select_pivots(p, Ctl{&sh.abort_flag, p.status, limit}, sh, smem_raw); // (selectors have no ring)
     } else if (warp >= kMulWarp1) {
         multiply<NT / mul_groups(NT), NT>(p, ctl, sh, ring0, piv0, warp - kMulWarp1, NT / mul_groups(NT));
-    } else if (warp == kFeedWarp) {
+    } else if (warp >= kFeedWarp) {
         feed(p, ctl, sh, slot0);
     } else if (warp == kWatchWarp) {
         watch(p, ctl, sh);
