@@ -15,8 +15,8 @@
 //     slices) instead of P x d, and the item takes about 2.5 us instead of the 20 us of a 128-row tile of full rows;
 //   - the item's rows are fetched into a ring before the pivots are known;
 //   - the scorers are held back to `window` rows beyond the samples that have their pivots.
-// The slices' shares of a dot product meet in global memory (L2): the SM that finishes a row group last adds them up in
-// slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
+// The slices' shares of a dot product meet in global memory (L2): when a row group's are all there, each of its SMs adds up a part of
+// them in slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
 //
 // What bounds it: no unit.  16 x 2880 x 4096, 8 pivots (99 us): DRAM 49 % of its peak, L2 40 %, L2 to SM 25 % (8.5 TB/s: every key byte crosses
@@ -28,7 +28,7 @@
 //   warps 4-7    second pass: mma.sync.m16n8k16, 16 rows each (the tensor pipe is 6 % busy; what the form costs is that every warp
 //                reads the pivot tile from shared memory again, which a tcgen05.mma of 64 rows would do once)
 //   warp 8       producer: TMA tiles of 64 rows x 64 columns (128-byte swizzle), two per ring stage
-//   warps 9-12   combine: count the item, and if it is its row group's last, add up the slices and write the similarities
+//   warps 9-12   combine: count the item, wait for its row group's other slices, add up a part of the shares and write the similarities
 //   warps 13-20  scorers: sum |x| (the K-norm of the Sec. 3.3 footnote) and sum x^2 (Eq. 7's denominator) of a row
 //   warp 21      watcher: how far the pivots of the batch have got, for the scorers' window
 //   warps 22-23  feeders: the scorers' rows into their slots
@@ -87,7 +87,7 @@ constexpr int32_t kNoPivot = -1;           // a pivot's word before it is publis
 constexpr uint32_t kNoWord = ~0u;
 constexpr unsigned long long kNoRec = ~0ull; // a row's word before it is published (no sums produce it)
 enum { kWaitRec = 90, kWaitPivots, kWaitPivFree, kWaitPiv, kWaitStage, kWaitStageFree, kWaitMailFree, kWaitMail, kWaitCombRec,
-       kWaitWindow, kWaitChunk = 101 }; // (100 is taken by the check of given pivots)
+       kWaitWindow, kWaitChunk = 101, kWaitShares }; // (100 is taken by the check of given pivots)
 // Selector CTAs: a selection takes about 3 us, a sample streams at about 6 MB per us.  (256 samples of 1 to 4 MB: 8 or 16 CTAs for
 // them 360 and 237 us, 6 and 8 CTAs 356 and 229; 2 and 3 are no better and cost large samples 1 %.)
 __host__ inline int selectors(long long sample_bytes) { return sample_bytes >= (4 << 20) ? 4 : sample_bytes >= (1 << 20) ? 6 : 8; }
@@ -695,29 +695,33 @@ __device__ __forceinline__ void produce(const Params &p, const Ctl &ctl, Shared 
             ctl.wait_landed(smem_u32(&sh.full[i % p.n_st]), (uint32_t)((i / p.n_st) & 1));
 }
 
-// Combine: an item is counted once its shares are written; whoever counts a row group's last slice adds the shares up.
-template <int NT>
+// Combine: an item is counted once its shares are written; when all slices of its row group are, each of their SMs adds up one part
+// in NSL of the group's similarities.  So a warp has 16 values per pivot tile to fetch, all at once, whatever the number of slices.
+// (With the SM that counted last adding up the whole group, one sample of 576 tokens in 16 slices took 7 us from count to
+// similarities, now 2.  Whole calls, us: 1 x 576 30.8 -> 26.7, 1 x 2880 39.0 -> 36.7, 16 x 256 36.9 -> 34.9, 64 x 576 115.4 -> 113.5, 8 x 2880
+// with 16 pivots 87.5 -> 84.9.)
+// A warp here waits for the other SMs' shares of its row group, and those for nothing but earlier groups: every SM takes its items
+// in the groups' order.
+template <int NT, int NSL>
 __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared &sh)
 {
+    constexpr int V = NSL >= 4 ? 16 / NSL : 4, H = 16 / NSL / V; // consecutive rows per lane and load; blocks of 32 V values per pivot tile
+    constexpr int NTat = NT == 2 ? 2 : 1;                        // pivot tiles at a time (registers)
     const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - kCombWarp0;
     const size_t part_item = (size_t)8 * NT * kRows;
     int seq = -1, last_b = -1, k = 0;
-    auto rec_ssq = [&](const unsigned long long *rec, int b, float &ssq) { // the word may not be there yet when the pivots were given
-        unsigned long long v = ld_rec(rec);
-        if (v == kNoRec) {
-            const long long t0 = clock64();
-            for (uint32_t spin = 0; (v = ld_rec(rec)) == kNoRec; ++spin) {
-                __nanosleep(100);
-                if ((spin & 15u) == 15u) {
-                    if (ctl.aborted()) return false;
-                    if ((unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
-                        ctl.give_up(kWaitCombRec, b);
-                        return false;
-                    }
+    auto late = [&](const unsigned long long *rec, int b, unsigned long long &v) { // the word may not be there yet when the pivots were given
+        const long long t0 = clock64();
+        for (uint32_t spin = 0; (v = ld_rec(rec)) == kNoRec; ++spin) {
+            __nanosleep(100);
+            if ((spin & 15u) == 15u) {
+                if (ctl.aborted()) return false;
+                if ((unsigned long long)(clock64() - t0) > ctl.limit_cycles) {
+                    ctl.give_up(kWaitCombRec, b);
+                    return false;
                 }
             }
         }
-        ssq = __uint_as_float((uint32_t)(v >> 32));
         return true;
     };
     for (Items it(p); it.valid(); it.next(), ++k) {
@@ -727,51 +731,71 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
         bool ok = ctl.wait_bar(smem_u32(&sh.mail_full[c][slot]), (uint32_t)(k / kCombWarps / kMail) & 1u, kWaitMail, it.b);
         if (!__all_sync(0xffffffffu, ok)) return;
         const size_t group = (size_t)it.b * p.n_rg + it.rg;
-        int before = 0;
-        // release: the item's shares, written by the warps that filled the mailbox; acquire: the other slices' shares
-        if (lane == 0 && p.nsl > 1)
-            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(p.cnt + group) : "memory");
-        before = __shfl_sync(0xffffffffu, before, 0);
-        __syncwarp();
-        if (before == p.nsl - 1) {
-            const int j = it.rg * kRows + 2 * lane; // this lane's rows: j and j + 1
+        // release: the item's shares, written by the warps that filled the mailbox
+        if (NSL > 1 && lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.cnt + group) : "memory");
+        bool waited = NSL == 1;
+        for (int h = 0; h < H; ++h) {
+            const int f = it.sl * (512 / NSL) + (32 * h + lane) * V, i0 = f >> 6, r0 = f & 63; // pivot of a tile and (first) row
+            if (NT == 1 && __all_sync(0xffffffffu, i0 >= p.P)) continue; // none of it is wanted
+            const int j = it.rg * kRows + r0;
             const unsigned long long *rec = p.rec + (size_t)it.b * p.n_vis;
-            float n0 = 0.f, n1 = 0.f, np = 0.f;
-            if (j < p.n_vis) ok = ok && rec_ssq(rec + j, it.b, n0);
-            if (j + 1 < p.n_vis) ok = ok && rec_ssq(rec + j + 1, it.b, n1);
-            if (lane < p.P) {
-                const int pv = sh.pv[seq % kPvRing][lane];
-                if (pv >= 0 && pv < p.n_vis)
-                    ok = ok && rec_ssq(rec + pv, it.b, np);
-                else
-                    np = p.text_ssq[(size_t)it.b * p.P + lane];
+            unsigned long long w[V], wp[NT];
+            int pv[NT];
+#pragma unroll
+            for (int e = 0; e < V; ++e) w[e] = j + e < p.n_vis ? ld_rec(rec + j + e) : 0ull;
+#pragma unroll
+            for (int n = 0; n < NT; ++n) {
+                pv[n] = 8 * n + i0 < p.P ? sh.pv[seq % kPvRing][8 * n + i0] : 0;
+                const bool text = pv[n] < 0 || pv[n] >= p.n_vis;
+                wp[n] = text ? (unsigned long long)__float_as_uint(p.text_ssq[(size_t)it.b * p.P + 8 * n + i0]) << 32 : ld_rec(rec + pv[n]);
             }
-            if (!__all_sync(0xffffffffu, ok)) return;
-            n0 = sqrtf(n0), n1 = sqrtf(n1), np = sqrtf(np);
-            const float2 *src = reinterpret_cast<const float2 *>(p.part + group * p.nsl * part_item) + lane;
-            float *dst = p.sim + (size_t)it.b * p.P * p.n_vis + j;
-            for (int i0 = 0; i0 < p.P; i0 += 4) { // 4 pivots x 4 slices on their way at once
-                float2 v[4];
+            if (!waited) { // acquire: the other slices' shares
+                if (lane == 0) ok = ctl.wait_flag(p.cnt + group, kWaitShares, it.b, NSL);
+                if (!__all_sync(0xffffffffu, ok)) return;
+                waited = true;
+            }
+            const float *src = p.part + group * NSL * part_item + f;
+            float *dst = p.sim + ((size_t)it.b * p.P + i0) * p.n_vis + j;
+            float nr[V];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = make_float2(0.f, 0.f);
-                for (int s0 = 0; s0 < p.nsl; s0 += 4) {
-                    float2 x[4][4];
+            for (int n0 = 0; n0 < NT; n0 += NTat) {
+                float x[NTat][NSL][V];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s)
+                for (int n = 0; n < NTat; ++n)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            x[s][i] = s0 + s < p.nsl ? __ldcg(src + (((size_t)(s0 + s) * part_item + (size_t)(i0 + i) * kRows) >> 1)) : make_float2(0.f, 0.f);
+                    for (int s = 0; s < NSL; ++s) {
+                        const float *at = src + s * part_item + (n0 + n) * 512;
+                        if constexpr (V == 4) {
+                            const float4 y = __ldcg(reinterpret_cast<const float4 *>(at));
+                            x[n][s][0] = y.x, x[n][s][1] = y.y, x[n][s][2] = y.z, x[n][s][3] = y.w;
+                        } else if constexpr (V == 2) {
+                            const float2 y = __ldcg(reinterpret_cast<const float2 *>(at));
+                            x[n][s][0] = y.x, x[n][s][1] = y.y;
+                        } else {
+                            x[n][s][0] = __ldcg(at);
+                        }
+                    }
+                if (n0 == 0) {
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) // in slice order
+                    for (int e = 0; e < V; ++e) {
+                        if (w[e] == kNoRec) ok = ok && late(rec + j + e, it.b, w[e]);
+                        nr[e] = sqrtf(__uint_as_float((uint32_t)(w[e] >> 32)));
+                    }
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) v[i].x += x[s][i].x, v[i].y += x[s][i].y;
+                    for (int n = 0; n < NT; ++n)
+                        if (wp[n] == kNoRec) ok = ok && late(rec + pv[n], it.b, wp[n]);
+                    if (!__all_sync(0xffffffffu, ok)) return;
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float ni = __shfl_sync(0xffffffffu, np, i0 + i), d0 = ni * n0, d1 = ni * n1;
-                    if (i0 + i < p.P) { // dup = dot / (|pivot| |row|); a zero norm gives 0
-                        if (j < p.n_vis) dst[(size_t)(i0 + i) * p.n_vis] = d0 > 0.f ? v[i].x / d0 : 0.f;
-                        if (j + 1 < p.n_vis) dst[(size_t)(i0 + i) * p.n_vis + 1] = d1 > 0.f ? v[i].y / d1 : 0.f;
+                for (int n = 0; n < NTat; ++n) {
+                    const float np = sqrtf(__uint_as_float((uint32_t)(wp[n0 + n] >> 32)));
+#pragma unroll
+                    for (int e = 0; e < V; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0
+                        float a = 0.f;
+#pragma unroll
+                        for (int s = 0; s < NSL; ++s) a += x[n][s][e]; // in slice order
+                        const float den = np * nr[e];
+                        if (8 * (n0 + n) + i0 < p.P && j + e < p.n_vis) dst[(size_t)8 * (n0 + n) * p.n_vis + e] = den > 0.f ? a / den : 0.f;
                     }
                 }
             }
@@ -836,7 +860,13 @@ __global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_const
     } else if (warp == kProdWarp) {
         produce(p, ctl, sh, ring0, &tm);
     } else {
-        combine<NT>(p, ctl, sh);
+        switch (p.nsl) {
+        case 1: combine<NT, 1>(p, ctl, sh); break;
+        case 2: combine<NT, 2>(p, ctl, sh); break;
+        case 4: combine<NT, 4>(p, ctl, sh); break;
+        case 8: combine<NT, 8>(p, ctl, sh); break;
+        default: combine<NT, 16>(p, ctl, sh); break;
+        }
     }
     __syncthreads(); // nobody leaves while a copy may still land in the CTA's shared memory
 }
