@@ -119,6 +119,27 @@ def test_flow_takes_wide_rows_with_many_pivots_in_large_contexts(oracle, d, P):
     assert rep.exact >= rep.above_margin and rep.max_abs_sim < 2e-5
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("P", [1, 5, 8, 13, 16, 31])
+@pytest.mark.parametrize("nsl", [1, 2, 4, 8, 16])
+def test_flow_shares_of_every_number_of_slices(nsl, P, given):
+    """Keys whose sums are exact in any order: the similarities added up from the slices' shares equal the plain kernels' bit for bit."""
+    B, n, d, Kp = 5, 131, 1024, P + 40                # row groups of 64, 64 and 3 rows
+    g = torch.Generator(device="cuda").manual_seed(nsl + P)
+    k = torch.randint(-15, 16, (B, n + 9, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
+    piv = torch.rand((B, n), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
+    outs = []
+    for path in (FLOW, dart.DART_PATH_STAGED):
+        ctx = dart.Dart(B, n + 9, d, P, Kp)
+        o = dart.dart_opts(path=path, tune=nsl << 16 if path == FLOW else 0, pivots_in=piv.data_ptr() if given else None)
+        oh, oi, op, dbg = ctx.reduce(k, None, 4, n, P, Kp, opts=o, debug=True)
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        ctx.close()
+        outs.append((oh.view(torch.int16), oi, op, dbg["sim"]))
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
 @pytest.mark.parametrize("norm_kind,smallest", [(1, 1), (2, 0), (2, 1)])
 def test_flow_ranking_variants(oracle, norm_kind, smallest):
     k, h = gaussian(3, 500, 256, seed=77)
