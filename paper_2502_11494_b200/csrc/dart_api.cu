@@ -272,11 +272,13 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     const bool each = o.rule == DART_RULE_UNION; // independent pivots: lists of q_i instead of Q_i
     RankParams rp = {};
     size_t rank_smem = 0;
-    // few lists: as many threads per list as help; many: small CTAs, so that one list's barriers are covered by the others (24 values
-    // per thread: 256 x 2880, 128 pivots with 256 threads per list 490 us, with 128 389)
+    // few lists: as many threads per list as help - a warp more lengthens every barrier of the chain, a value more every pass over a
+    // thread's own (whole calls, us, 192 / 256 / 384 / 512 threads: 1 x 576 25.9 / 25.9 / 26.3 / 26.7, 1 x 2880 37.0 / 37.0 / 35.2 / 36.8, 4 x 4608 with 32
+    // pivots 98.3 / 96.0 / 93.6 / 94.3); more lists, 192 / 256: 64 x 576 113.5 / 113.8, one after the other 123.0 / 124.0; many: small CTAs, so that
+    // one list's barriers are covered by the others (24 values per thread: 256 x 2880, 128 pivots with 256 threads per list 490 us, with 128 389)
     const long long rank_rows = (long long)B * P;
-    int rank_threads = rank_rows <= 2ll * ctx->sm_count ? 512 : rank_rows <= 8ll * ctx->sm_count ? 256 : n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
-    while (rank_threads < kRankMaxThreads && 32 * rank_threads < n_vis) rank_threads *= 2; // the row has to fit the registers
+    int rank_threads = rank_rows <= 8ll * ctx->sm_count ? n_vis > 1024 && rank_rows <= 2ll * ctx->sm_count ? 384 : 192 : n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
+    if (32 * rank_threads < n_vis) rank_threads = 32 * 256 < n_vis ? kRankMaxThreads : 256; // the row has to fit the registers
     const int rank_m = each ? (m + P - 1) / P : m;
     // the forms with a CTA per (sample, pivot) count the samples in the grid's second dimension
     const bool grid_fits = B <= kMaxGridY;

@@ -37,6 +37,20 @@ def test_ranked_lists_make_the_same_selections(kind, shape):
     assert all(np.array_equal(a[3][n], b[3][n], equal_nan=(n == "eps")) for n in a[3])
 
 
+@pytest.mark.parametrize("shape", [
+    # (B, S, d, vis_offset, n_vis, P, Kp): up to two lists per SM, short rows and long ones; up to eight; rows that take more threads than the rule's
+    (1, 1040, 64, 3, 1024, 8, 90), (1, 1040, 64, 3, 1025, 8, 90), (37, 1600, 64, 3, 1537, 8, 700), (38, 1600, 64, 3, 1536, 8, 700),
+    (148, 600, 64, 3, 576, 8, 300), (149, 600, 64, 3, 576, 8, 300), (1, 6200, 64, 3, 6145, 3, 2000), (40, 6200, 64, 3, 6144, 8, 200), (40, 6200, 64, 3, 6145, 8, 200),
+    (1, 12300, 64, 3, 8193, 2, 100), (1, 12300, 64, 3, 12288, 2, 4000), (1, 12300, 64, 3, 12289, 2, 4000),
+], ids=lambda v: "x".join(map(str, v)))
+def test_ranked_lists_at_the_lines_between_threads_per_list(shape):
+    B, S, d, vo, nv, P, Kp = shape
+    k, h = _band_inputs("gaussian", B, S, d, vo, nv, P, seed=23 + sum(shape))
+    a = run_gpu(k, h, vo, nv, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL, debug=False)
+    b = run_gpu(k, h, vo, nv, P, Kp, path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_RANKED, debug=False)
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+
+
 @pytest.mark.parametrize("kind,shape", [("gaussian", (3, 333, 264, 17, 301, 7, 60)), ("equal tokens", (2, 700, 64, 10, 640, 16, 200)),
                                         ("gaussian", (260, 130, 64, 5, 100, 3, 90)), ("gaussian", (2, 3000, 64, 0, 2880, 128, 640))],
                          ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
