@@ -752,6 +752,7 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
             if (!waited) { // acquire: the other slices' shares
                 if (lane == 0) ok = ctl.wait_flag(p.cnt + group, kWaitShares, it.b, NSL);
                 if (!__all_sync(0xffffffffu, ok)) return;
+                __syncwarp(); // (every lane's loads come after lane 0's)
                 waited = true;
             }
             const float *src = p.part + group * NSL * part_item + f;
@@ -765,15 +766,12 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
 #pragma unroll
                     for (int s = 0; s < NSL; ++s) {
                         const float *at = src + s * part_item + (n0 + n) * 512;
-                        if constexpr (V == 4) {
-                            const float4 y = __ldcg(reinterpret_cast<const float4 *>(at));
-                            x[n][s][0] = y.x, x[n][s][1] = y.y, x[n][s][2] = y.z, x[n][s][3] = y.w;
-                        } else if constexpr (V == 2) {
-                            const float2 y = __ldcg(reinterpret_cast<const float2 *>(at));
-                            x[n][s][0] = y.x, x[n][s][1] = y.y;
-                        } else {
-                            x[n][s][0] = __ldcg(at);
-                        }
+                        if constexpr (V == 4)
+                            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]), "=f"(x[n][s][2]), "=f"(x[n][s][3]) : "l"(at) : "memory");
+                        else if constexpr (V == 2)
+                            asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]) : "l"(at) : "memory");
+                        else
+                            asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(x[n][s][0]) : "l"(at) : "memory");
                     }
                 if (n0 == 0) {
 #pragma unroll
