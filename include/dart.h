@@ -296,8 +296,8 @@ int dart_status(dart_ctx *ctx);
  * sample's lists not all counted in, 50 its pivots not published, 51 their norms not handed over, ...); 64-70 the one-pass
  * kernel's waits (stage not freed, tile not loaded (MMA / norms), accumulator not freed / not filled, norms not taken /
  * not ready); 80-86 the resident sweep's waits (83 = a sample's candidates not all published);
- * 90-99, 101 the flow path's (90 a row's score not published, 91 a sample's pivots, ...); 100 = a failed check of
- * opts->pivots_in),
+ * 90-99, 101, 102 the flow path's (90 a row's score not published, 91 a sample's pivots, ...); 103 a kept row's index not
+ * published to the gather; 100 = a failed check of opts->pivots_in),
  * detail[1] = index of the step in the kernel's schedule (or the sample), detail[2] = CTA; for wait 1 also
  * detail[3] = sample.  For bug reports.
  */

@@ -59,6 +59,8 @@ struct dart_ctx {
     uint16_t *rank;  // [B_max][...] ranked lists of the retention (NULL: not available)
     size_t rank_n;   // their entries
     int *rank_arrived; // [B_max] zero between launches
+    int32_t *row_word; // [B_max][S_max] kept rows as the gather waits for them; all -1 between calls
+    bool row_word_dirty, row_word_used; // as flow_dirty; the call's retention publishes them
     uint8_t *keep;
     int *status; // device status word, followed by three words of detail
     int32_t status_detail[11];
@@ -256,6 +258,12 @@ int copy_debug(dart_ctx *ctx, int B, int n_vis, int P, const dart_debug *dbg, cu
     return DART_OK;
 }
 
+// The words through which the retention hands the kept rows to the gather, as every call expects to find them.
+cudaError_t row_word_reset(dart_ctx *ctx, cudaStream_t st)
+{
+    return cudaMemsetAsync(ctx->row_word, 0xff, (size_t)ctx->desc.B_max * ctx->desc.S_max * sizeof(int32_t), st);
+}
+
 // Steps 4 and 5a.  Ranked lists wherever their workspace, their limits and the grid take the call (rows of up to 16384 tokens, lists
 // of up to 4096); the older forms below serve what is left - longer rows and lists, contexts without the lists, calls that keep
 // the pivots alone - and by option.
@@ -297,11 +305,22 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
         rank_smem = phase1 > flags + avail ? phase1 : flags + avail;
         can_rank = (size_t)B * rp.sample_entries <= ctx->rank_n && rank_smem <= (size_t)ctx->max_smem_optin - kRankStaticSmem;
     }
+    ctx->row_word_used = false;
+    // The gather waits for its rows' words where the SMs hold few of its CTAs beside the turns, which its waiting warps slow down (whole
+    // calls, us, behind the kernel / behind the words: 16 x 256 keeping 56, 182 CTAs 34.9 / 33.0, 4 x 4608 keeping 512, 306 CTAs 93.6 / 92.0; 8 x 1500
+    // keeping 750, 995 CTAs 57.1 / 58.6, 32 x 2880 keeping 320, 1680 CTAs 187.2 / 188.3, 256 x 2880 keeping 640 2947 / 2985).
+    const bool follow = !each && (long long)B * (S - n_vis + n_keep) <= 4ll * kGatherWarps * ctx->sm_count;
     auto launch_ranked = [&]() -> cudaError_t {
+        if (follow && ctx->row_word_dirty) {
+            const cudaError_t e = row_word_reset(ctx, st);
+            if (e != cudaSuccess) return e;
+        }
+        if (follow) ctx->row_word_dirty = true;
         rp.sim = ctx->sim, rp.pivot_idx = ctx->pivot_idx, rp.lists = ctx->rank, rp.arrived = ctx->rank_arrived, rp.pos_in = pos_in;
         rp.S = S, rp.vis_offset = vis_offset, rp.n_vis = n_vis, rp.P = P, rp.n_keep = n_keep, rp.m = rank_m, rp.each = each;
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
         rp.len_out = ctx->len, rp.status = ctx->status;
+        if (follow) rp.row_word = ctx->row_word, ctx->row_word_used = true;
         Prof p(ctx, st, SLOT_RETAIN);
         const int groups = each || owner_out || eps_out ? 0 : rank_turn_groups(rank_m, rank_m / P);
         return launch_next(rank_kernel_of(rank_regs(n_vis, rank_threads), groups), dim3((unsigned)P, (unsigned)B), rank_threads, rank_smem, st, rp);
@@ -408,12 +427,20 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int vis_offset, int
     Prof pr(ctx, st, SLOT_GATHER);
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
+    cudaError_t followed = cudaErrorNotReady;
     if (o.rule == DART_RULE_UNION)
         launch_next(gather_varlen_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
                                                                 ctx->status, (uint4 *)out_hidden, fs);
+    else if (ctx->row_word_used)
+        followed = launch_next(gather_kernel<false, true>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
+                               (uint4 *)out_hidden, fs, vis_offset, n_keep, ctx->row_word, o.wait_limit > 0 ? (unsigned long long)o.wait_limit * 1000ull : 2000000000ull);
     else
         launch_next(gather_kernel<false>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
-                                                         (uint4 *)out_hidden, fs, vis_offset, n_keep);
+                    (uint4 *)out_hidden, fs, vis_offset, n_keep, nullptr, 0ull);
+    if (followed == cudaSuccess)
+        ctx->row_word_dirty = false;
+    else if (ctx->row_word_used)
+        row_word_reset(ctx, st); // (a graph captured earlier would find what rank_kernel publishes)
 }
 
 // Pivots from scores.  Rows of more values than the registers of one CTA hold: radix select, from shared memory where `cached`
@@ -1162,6 +1189,7 @@ int read_status(dart_ctx *ctx)
     DART_CUDA(ctx, cudaMemcpy(word, ctx->status, sizeof word, cudaMemcpyDeviceToHost));
     if (word[0] != 0) {
         for (int k = 0; k < 11; ++k) ctx->status_detail[k] = word[k + 1];
+        if (word[0] == DART_ERR_TIMEOUT) ctx->row_word_dirty = true; // a gather that gave up may have left words behind
         DART_CUDA(ctx, cudaMemset(ctx->status, 0, sizeof word));
     }
     return word[0];
@@ -1226,6 +1254,7 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
         if (ctx->rank_n * sizeof(uint16_t) <= ((size_t)1 << 30)) {
             rc = ws_alloc(ctx, &ctx->rank, ctx->rank_n);
             if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->rank_arrived, (size_t)desc->B_max);
+            if (rc == DART_OK) rc = ws_alloc(ctx, &ctx->row_word, nv);
             const int smem = ctx->max_smem_optin - dart::kRankStaticSmem;
             for (int regs = 2; rc == DART_OK && regs <= 8; regs += 2)
                 for (int groups : {0, 1, 2, 4})
@@ -1302,6 +1331,7 @@ int dart_create(dart_ctx **out, const dart_desc *desc)
     if (rc == DART_OK) rc = cudaMemsetAsync(ctx->status, 0, 256, 0) == cudaSuccess ? DART_OK : DART_ERR_CUDA;
     if (rc == DART_OK && ctx->flow_rec) rc = flow_reset(ctx, 0);
     if (rc == DART_OK && ctx->rank && cudaMemsetAsync(ctx->rank_arrived, 0, (size_t)desc->B_max * sizeof(int), 0) != cudaSuccess) rc = DART_ERR_CUDA;
+    if (rc == DART_OK && ctx->rank && row_word_reset(ctx, 0) != cudaSuccess) rc = DART_ERR_CUDA;
     // the first call may use a stream that does not wait for the legacy stream
     if (rc == DART_OK && cudaStreamSynchronize(0) != cudaSuccess) rc = DART_ERR_CUDA;
     if (rc != DART_OK) {
@@ -1567,7 +1597,7 @@ int dart_gather_rows(const void *src, const int32_t *idx, int B, int S, int S_ou
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
     launch_next(gather_kernel<true>, dim3(grid), kGatherWarps * 32, 0, (cudaStream_t)stream, (const uint4 *)src, idx, S, S_out, row_bytes / 16, orows,
-                                                                       nullptr, (uint4 *)out, FlowState{}, 0, S_out);
+                                                                       nullptr, (uint4 *)out, FlowState{}, 0, S_out, nullptr, 0ull);
     return cudaGetLastError() == cudaSuccess ? DART_OK : DART_ERR_CUDA;
 }
 

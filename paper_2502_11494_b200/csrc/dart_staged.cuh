@@ -1453,10 +1453,17 @@ gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, c
 
 // kFirst: launched behind whatever the caller's stream runs (no call of the library before it): its rows are read coherently, and
 // there are no text rows and nothing to put back (150 x 5700 rows of 512 bytes 258 us with both, 203 without; 256 x 420 of 1 KB 41, 37).
-template <bool kFirst>
+// kFollow: launched behind rank_kernel, which publishes every kept vision row's index as one word (row_word): a warp waits for its own
+// row's word instead of for the whole kernel before it, and then for the index (1 x 576 25.9 -> 24.5 us a call, 5 x 1237 34.1 -> 32.1).
+// It starts once every CTA of rank_kernel has (all of them have let it start), so that none of those waits for room that a waiting warp
+// takes, and that wait is bounded.
+constexpr int kWaitRowWord = 103;   // second status word
+constexpr int kStatusLate = -7;     // DART_ERR_TIMEOUT
+template <bool kFirst, bool kFollow = false>
 __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, int S_out, int d8,
-              long long rows_total, const int *status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep)
+              long long rows_total, int *status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep, int32_t *row_word,
+              unsigned long long wait_ns)
 {
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
@@ -1465,12 +1472,35 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, i
     // Text rows stand where they stand whatever the retention decides: they are copied while it still runs.  (It lets this kernel
     // start once everything before it has finished, and it neither writes the status word nor reads a packed row.)
     const bool text = !kFirst && (t < vis_offset || t >= vis_offset + n_keep);
-    if (!text || row >= rows_total) wait_for_previous();
+    if (!kFollow && (!text || row >= rows_total)) wait_for_previous();
     let_next_start();
     int s = 0, failed = 0; // (both asked for at once: narrow rows are copied in the time of the chain of loads)
     if (row < rows_total) {
-        s = !text ? out_idx[row] : t < vis_offset ? t : t + S - S_out;
-        if (status) failed = *status; // after a failed kernel out_idx is undefined
+        if (kFollow) {
+            s = t < vis_offset ? t : t + S - S_out;
+            failed = *(volatile int *)status; // (of a kernel before rank_kernel, which then publishes nothing)
+            if (!text && failed == 0) {
+                int32_t *word = row_word + row;
+                const long long t0 = clock64();
+                for (uint32_t spin = 1;; ++spin) {
+                    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(s) : "l"(word) : "memory");
+                    if (__any_sync(0xffffffffu, s >= 0)) break;
+                    __nanosleep(40);
+                    const bool late = (spin & 63u) == 0u && (unsigned long long)(clock64() - t0) > 2ull * wait_ns; // ns -> cycles at the highest SM clock
+                    if (__any_sync(0xffffffffu, late)) {
+                        if (lane == 0 && atomicCAS(status, 0, kStatusLate) == 0) status[1] = kWaitRowWord, status[2] = b, status[3] = (int)blockIdx.x;
+                        break;
+                    }
+                }
+                s = __reduce_max_sync(0xffffffffu, s);
+                if (s < 0) failed = kStatusLate;
+                __syncwarp();
+                if (lane == 0) *word = -1;
+            }
+        } else {
+            s = !text ? out_idx[row] : t < vis_offset ? t : t + S - S_out;
+            if (status) failed = *status; // after a failed kernel out_idx is undefined
+        }
     }
     if (row < rows_total && failed == 0) {
         const uint4 *src = hidden + ((size_t)b * S + s) * (size_t)d8;
@@ -1490,7 +1520,7 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, i
         }
     }
     if (!kFirst) {
-        if (text) wait_for_previous();
+        if (kFollow || text) wait_for_previous(); // (what follows this kernel follows the one before it too)
         fs.put_back();
     }
 }

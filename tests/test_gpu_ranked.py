@@ -51,6 +51,44 @@ def test_ranked_lists_at_the_lines_between_threads_per_list(shape):
     assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
 
 
+@pytest.mark.parametrize("kept", [700, 699, 90])
+def test_rows_handed_to_the_gather_word_by_word(kept):
+    """Both sides of the line (4736 packed rows on 148 SMs), one context through several calls, a refused call and a replayed one among them."""
+    B, S, d, vo, nv, P = 4, 1700, 128, 11, 1216, 5                         # 4 x (484 + 700) rows
+    bits = lambda t: t.view(torch.int16) if t.dtype == torch.bfloat16 else t
+    g = torch.Generator(device="cuda").manual_seed(kept)
+    k = torch.randint(-15, 16, (B, S, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
+    h = torch.randn((B, S, d), generator=g, device="cuda").bfloat16()
+    bad = torch.zeros((B, P), dtype=torch.int32, device="cuda")             # the same pivot five times
+    pos = (torch.randperm(B * S, generator=g, device="cuda") + 7).view(B, S).contiguous()
+    ref, ctx = dart.Dart(B, S, d, P, 800), dart.Dart(B, S, d, P, 800)
+    want = ref.reduce(h, k, vo, nv, P, kept, pos_in=pos, opts=dart.dart_opts(path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL))
+    for n in (kept, kept + 1, 0, kept):
+        if n == 0:
+            ctx.reduce(h, k, vo, nv, P, kept, opts=dart.dart_opts(pivots_in=bad.data_ptr()))
+            torch.cuda.synchronize()
+            assert ctx.status() == dart.DART_ERR_CHECK
+        else:
+            got = ctx.reduce(h, k, vo, nv, P, n, pos_in=pos)
+    torch.cuda.synchronize()
+    assert ctx.status() == dart.DART_OK
+    assert all(torch.equal(bits(a), bits(b)) for a, b in zip(want, got))
+    for t in got:
+        t.zero_()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.reduce(h, k, vo, nv, P, kept, pos_in=pos, out=got)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert ctx.status() == dart.DART_OK
+    assert all(torch.equal(bits(a), bits(b)) for a, b in zip(want, got))
+    del graph
+    ctx.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("kind,shape", [("gaussian", (3, 333, 264, 17, 301, 7, 60)), ("equal tokens", (2, 700, 64, 10, 640, 16, 200)),
                                         ("gaussian", (260, 130, 64, 5, 100, 3, 90)), ("gaussian", (2, 3000, 64, 0, 2880, 128, 640))],
                          ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
