@@ -284,10 +284,15 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     // thread's own (whole calls, us, 192 / 256 / 384 / 512 threads: 1 x 576 25.9 / 25.9 / 26.3 / 26.7, 1 x 2880 37.0 / 37.0 / 35.2 / 36.8, 4 x 4608 with 32
     // pivots 98.3 / 96.0 / 93.6 / 94.3); more lists, 192 / 256: 64 x 576 113.5 / 113.8, one after the other 123.0 / 124.0; many: small CTAs, so that
     // one list's barriers are covered by the others (24 values per thread: 256 x 2880, 128 pivots with 256 threads per list 490 us, with 128 389)
+    // Long lists take more threads again (5 x 3466, 8 pivots keeping 1605 59.7 with 384, 57.5 with 512; 17 x 4607, 21 pivots keeping 3474 413 with 192, 409 with 256).
     const long long rank_rows = (long long)B * P;
-    int rank_threads = rank_rows <= 8ll * ctx->sm_count ? n_vis > 1024 && rank_rows <= 2ll * ctx->sm_count ? 384 : 192 : n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
-    if (32 * rank_threads < n_vis) rank_threads = 32 * 256 < n_vis ? kRankMaxThreads : 256; // the row has to fit the registers
     const int rank_m = each ? (m + P - 1) / P : m;
+    int rank_threads = n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
+    if (rank_rows <= 2ll * ctx->sm_count)
+        rank_threads = rank_m > kRankLongList ? 512 : n_vis > 1024 ? 384 : 192;
+    else if (rank_rows <= 8ll * ctx->sm_count)
+        rank_threads = rank_m > kRankLongList ? 256 : 192;
+    if (32 * rank_threads < n_vis) rank_threads = 32 * 256 < n_vis ? kRankMaxThreads : 256; // the row has to fit the registers
     // the forms with a CTA per (sample, pivot) count the samples in the grid's second dimension
     const bool grid_fits = B <= kMaxGridY;
     bool can_rank = ctx->rank && grid_fits && o.rule != DART_RULE_GLOBAL && n_vis <= kRankMaxVis && rank_m <= kRankMaxList;
@@ -307,9 +312,10 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     }
     ctx->row_word_used = false;
     // The gather waits for its rows' words where the SMs hold few of its CTAs beside the turns, which its waiting warps slow down (whole
-    // calls, us, behind the kernel / behind the words: 16 x 256 keeping 56, 182 CTAs 34.9 / 33.0, 4 x 4608 keeping 512, 306 CTAs 93.6 / 92.0; 8 x 1500
+    // calls, us, behind the kernel / behind the words: 16 x 256 keeping 56, 182 CTAs 34.9 / 33.0, 4 x 4608 keeping 512, 306 CTAs 93.6 / 92.0; 5 x 1733 keeping 747,
+    // 530 CTAs 41.1 / 43.4, 8 x 1500
     // keeping 750, 995 CTAs 57.1 / 58.6, 32 x 2880 keeping 320, 1680 CTAs 187.2 / 188.3, 256 x 2880 keeping 640 2947 / 2985).
-    const bool follow = !each && (long long)B * (S - n_vis + n_keep) <= 4ll * kGatherWarps * ctx->sm_count;
+    const bool follow = !each && (long long)B * (S - n_vis + n_keep) <= 5ll * kGatherWarps * ctx->sm_count / 2;
     auto launch_ranked = [&]() -> cudaError_t {
         if (follow && ctx->row_word_dirty) {
             const cudaError_t e = row_word_reset(ctx, st);

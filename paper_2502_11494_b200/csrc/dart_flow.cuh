@@ -766,6 +766,11 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
 #pragma unroll
                     for (int s = 0; s < NSL; ++s) {
                         const float *at = src + s * part_item + (n0 + n) * 512;
+                        if (8 * (n0 + n) + i0 >= p.P) { // not wanted
+#pragma unroll
+                            for (int e = 0; e < V; ++e) x[n][s][e] = 0.f;
+                            continue;
+                        }
                         if constexpr (V == 4)
                             asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]), "=f"(x[n][s][2]), "=f"(x[n][s][3]) : "l"(at) : "memory");
                         else if constexpr (V == 2)

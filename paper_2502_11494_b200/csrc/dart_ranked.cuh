@@ -33,6 +33,7 @@ constexpr int kRankMaxThreads = 512;
 constexpr int kRankMaxP = 1024;       // a context's most pivots
 constexpr int kRankMaxVis = 16384;    // 512 threads x 8 x 4 values in registers
 constexpr int kRankMaxList = 4096;    // longest list
+constexpr int kRankLongList = 1000;   // lists that take more threads
 constexpr uint32_t kRankMaxBin = 192; // entries of one bin that are ranked by counting
 constexpr int kRankTries = 10;        // guesses at the threshold
 constexpr int kRankMaxRest = 144;     // tokens beyond a threshold that a list of nearly all takes along
@@ -316,10 +317,10 @@ __device__ __forceinline__ void rank_row(const float *row, uint32_t flip, const 
 }
 
 // Step 5a's vision tokens (flags are 0 or 1, 16-byte aligned): every thread has up to eight consecutive words of four flags, so that one
-// sum over the CTA places all of them; row_word: the same indices once more, word by word for the gather that is waiting for them.
+// sum over the CTA places all of them - in shared memory first (list, if it has room), so that what is written is written side by side; row_word: the same indices once more, word by word for the gather that is waiting for them.
 // (32 flags of a warp at a time, and the text rows before them, took 1.1 us for 576 tokens and 1.8 for 2880, now 0.8 and 1.0.)
-__device__ __forceinline__ void pack_flags(const uint8_t *keep, int vis_offset, int n_vis, const int64_t *__restrict__ pin, int32_t *__restrict__ oi,
-                                           int64_t *__restrict__ op, int32_t *row_word, uint32_t *per_warp)
+__device__ __forceinline__ void pack_flags(const uint8_t *keep, int vis_offset, int n_vis, int n_keep, const int64_t *__restrict__ pin, int32_t *__restrict__ oi,
+                                           int64_t *__restrict__ op, int32_t *row_word, uint16_t *list, bool listed, uint32_t *per_warp)
 {
     const int words = (n_vis + 3) / 4, per = (words + (int)blockDim.x - 1) / (int)blockDim.x, w0 = (int)threadIdx.x * per;
     auto flags = [&](int w) { // (what lies behind the last token does not count)
@@ -328,14 +329,24 @@ __device__ __forceinline__ void pack_flags(const uint8_t *keep, int vis_offset, 
     };
     uint32_t mine = 0;
     for (int w = w0; w < min(w0 + per, words); ++w) mine += __popc(flags(w));
-    int at = vis_offset + (int)(cta_scan(mine, per_warp) - mine);
+    int at = (int)(cta_scan(mine, per_warp) - mine);
+    auto put = [&](int k, int j) { // kept token number k is token j
+        const int s = vis_offset + j;
+        if (row_word) asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(row_word + vis_offset + k), "r"(s) : "memory");
+        oi[vis_offset + k] = s;
+        op[vis_offset + k] = pin ? pin[s] : (int64_t)s;
+    };
     for (int w = w0; w < min(w0 + per, words); ++w)
         for (uint32_t f = flags(w); f; f &= f - 1u, ++at) {
-            const int s = vis_offset + 4 * w + (__ffs((int)f) - 1) / 8;
-            if (row_word) asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(row_word + at), "r"(s) : "memory");
-            oi[at] = s;
-            op[at] = pin ? pin[s] : (int64_t)s;
+            const int j = 4 * w + (__ffs((int)f) - 1) / 8;
+            if (listed)
+                list[at] = (uint16_t)j;
+            else
+                put(at, j);
         }
+    if (!listed) return;
+    __syncthreads();
+    for (int k = threadIdx.x; k < n_keep; k += blockDim.x) put(k, list[k]);
 }
 // ... and its text rows, by threads first, first + threads ...
 __device__ __forceinline__ void pack_text(int S, int vis_offset, int n_vis, int n_keep, const int64_t *__restrict__ pin, int32_t *__restrict__ oi,
@@ -605,7 +616,9 @@ __global__ void __launch_bounds__(kRankMaxThreads) rank_kernel(const RankParams 
         k0 = k1, k1 = k2;
     }
     if (n_active == 0) pack_text(p.S, p.vis_offset, n, p.n_keep, pin, oi, op, t, T);
-    pack_flags(flags, p.vis_offset, n, pin, oi, op, p.row_word ? p.row_word + (size_t)b * S_out : nullptr, sh.scan);
+    // (the staging buffers, one where all lists fit it, two otherwise, are free again)
+    const int room = p.stage_entries >= (int)p.sample_entries ? p.stage_entries : 2 * p.stage_entries;
+    pack_flags(flags, p.vis_offset, n, p.n_keep, pin, oi, op, p.row_word ? p.row_word + (size_t)b * S_out : nullptr, stage, p.n_keep <= room, sh.scan);
     if (p.keep_out)
         for (int j = t; j < n; j += T) p.keep_out[(size_t)b * n + j] = flags[j] != 0;
 }
