@@ -147,7 +147,8 @@ typedef struct {
     int32_t norm_kind;     /* 0 or 1: L1 row norm (the paper's "K-norm", Sec. 3.3 footnote); 2: Euclidean norm */
     int32_t pivot_smallest; /* 0: pivots = largest scores (Table 1 caption); 1: smallest (ablation variant) */
     int32_t path;          /* DART_PATH_* */
-    int32_t wait_limit;    /* 0: default (2 s); > 0: time limit in microseconds of every bounded device-side wait */
+    int32_t wait_limit;    /* 0: default (2 s); > 0: time limit in microseconds of every bounded device-side wait (a gather whose
+                              rows are not named within it waits for the whole ranking instead, and the call succeeds) */
     int32_t sweep_lag;     /* 0: default; > 0: fused path, extra tasks between a row's two sweeps (tuning) */
     int32_t test_withhold_pivots; /* testing only: nonzero withholds one hand-over inside the kernel that waits (the persistent
                                      sweep never publishes a sample's pivots; the resident sweep's CTAs never count themselves in;
@@ -296,8 +297,8 @@ int dart_status(dart_ctx *ctx);
  * sample's lists not all counted in, 50 its pivots not published, 51 their norms not handed over, ...); 64-70 the one-pass
  * kernel's waits (stage not freed, tile not loaded (MMA / norms), accumulator not freed / not filled, norms not taken /
  * not ready); 80-86 the resident sweep's waits (83 = a sample's candidates not all published);
- * 90-99, 101, 102 the flow path's (90 a row's score not published, 91 a sample's pivots, ...); 103 a kept row's index not
- * published to the gather; 100 = a failed check of opts->pivots_in),
+ * 90-99, 101, 102 the flow path's (90 a row's score not published, 91 a sample's pivots, ...); 100 = a failed check of
+ * opts->pivots_in),
  * detail[1] = index of the step in the kernel's schedule (or the sample), detail[2] = CTA; for wait 1 also
  * detail[3] = sample.  For bug reports.
  */

@@ -60,7 +60,7 @@ struct dart_ctx {
     size_t rank_n;   // their entries
     int *rank_arrived; // [B_max] zero between launches
     int32_t *row_word; // [B_max][S_max] kept rows as the gather waits for them; all -1 between calls
-    bool row_word_dirty, row_word_used; // as flow_dirty; the call's retention publishes them
+    bool row_word_used; // the call's retention publishes them
     uint8_t *keep;
     int *status; // device status word, followed by three words of detail
     int32_t status_detail[11];
@@ -317,11 +317,6 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     // keeping 750, 995 CTAs 57.1 / 58.6, 32 x 2880 keeping 320, 1680 CTAs 187.2 / 188.3, 256 x 2880 keeping 640 2947 / 2985).
     const bool follow = !each && (long long)B * (S - n_vis + n_keep) <= 5ll * kGatherWarps * ctx->sm_count / 2;
     auto launch_ranked = [&]() -> cudaError_t {
-        if (follow && ctx->row_word_dirty) {
-            const cudaError_t e = row_word_reset(ctx, st);
-            if (e != cudaSuccess) return e;
-        }
-        if (follow) ctx->row_word_dirty = true;
         rp.sim = ctx->sim, rp.pivot_idx = ctx->pivot_idx, rp.lists = ctx->rank, rp.arrived = ctx->rank_arrived, rp.pos_in = pos_in;
         rp.S = S, rp.vis_offset = vis_offset, rp.n_vis = n_vis, rp.P = P, rp.n_keep = n_keep, rp.m = rank_m, rp.each = each;
         rp.out_idx = out_idx, rp.out_pos = out_pos, rp.keep_out = each ? ctx->keep : keep_out, rp.owner_out = owner_out, rp.eps_out = eps_out;
@@ -433,20 +428,17 @@ void launch_gather(dart_ctx *ctx, int B, const void *hidden, int vis_offset, int
     Prof pr(ctx, st, SLOT_GATHER);
     const long long orows = (long long)B * S_out;
     const unsigned grid = (unsigned)((orows + kGatherWarps - 1) / kGatherWarps);
-    cudaError_t followed = cudaErrorNotReady;
     if (o.rule == DART_RULE_UNION)
         launch_next(gather_varlen_kernel, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, o.cu_seqlens, B, S, d8, orows,
                                                                 ctx->status, (uint4 *)out_hidden, fs);
-    else if (ctx->row_word_used)
-        followed = launch_next(gather_kernel<false, true>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
-                               (uint4 *)out_hidden, fs, vis_offset, n_keep, ctx->row_word, o.wait_limit > 0 ? (unsigned long long)o.wait_limit * 1000ull : 2000000000ull);
-    else
+    else if (ctx->row_word_used) {
+        if (launch_next(gather_kernel<false, true>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
+                        (uint4 *)out_hidden, fs, vis_offset, n_keep, ctx->row_word,
+                        o.wait_limit > 0 ? (unsigned long long)o.wait_limit * 1000ull : 2000000000ull) != cudaSuccess)
+            row_word_reset(ctx, st); // nobody puts back what rank_kernel publishes
+    } else
         launch_next(gather_kernel<false>, dim3(grid), kGatherWarps * 32, 0, st, (const uint4 *)hidden, out_idx, S, S_out, d8, orows, ctx->status,
                     (uint4 *)out_hidden, fs, vis_offset, n_keep, nullptr, 0ull);
-    if (followed == cudaSuccess)
-        ctx->row_word_dirty = false;
-    else if (ctx->row_word_used)
-        row_word_reset(ctx, st); // (a graph captured earlier would find what rank_kernel publishes)
 }
 
 // Pivots from scores.  Rows of more values than the registers of one CTA hold: radix select, from shared memory where `cached`
@@ -1195,7 +1187,6 @@ int read_status(dart_ctx *ctx)
     DART_CUDA(ctx, cudaMemcpy(word, ctx->status, sizeof word, cudaMemcpyDeviceToHost));
     if (word[0] != 0) {
         for (int k = 0; k < 11; ++k) ctx->status_detail[k] = word[k + 1];
-        if (word[0] == DART_ERR_TIMEOUT) ctx->row_word_dirty = true; // a gather that gave up may have left words behind
         DART_CUDA(ctx, cudaMemset(ctx->status, 0, sizeof word));
     }
     return word[0];

@@ -1455,14 +1455,13 @@ gather_varlen_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, c
 // there are no text rows and nothing to put back (150 x 5700 rows of 512 bytes 258 us with both, 203 without; 256 x 420 of 1 KB 41, 37).
 // kFollow: launched behind rank_kernel, which publishes every kept vision row's index as one word (row_word): a warp waits for its own
 // row's word instead of for the whole kernel before it, and then for the index (1 x 576 25.9 -> 24.5 us a call, 5 x 1237 34.1 -> 32.1).
-// It starts once every CTA of rank_kernel has (all of them have let it start), so that none of those waits for room that a waiting warp
-// takes, and that wait is bounded.
-constexpr int kWaitRowWord = 103;   // second status word
-constexpr int kStatusLate = -7;     // DART_ERR_TIMEOUT
+// It starts once every CTA of rank_kernel has (all of them have let it start, behind their own wait), so that none of those waits for
+// room that a waiting warp takes.  A warp whose word does not come within the limit waits for rank_kernel's end and takes the index from
+// out_idx.  The words are put back behind that end: nothing is published after it, whatever became of the wait.
 template <bool kFirst, bool kFollow = false>
 __global__ void __launch_bounds__(kGatherWarps * 32)
 gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, int S_out, int d8,
-              long long rows_total, int *status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep, int32_t *row_word,
+              long long rows_total, const int *status, uint4 *__restrict__ out_hidden, FlowState fs, int vis_offset, int n_keep, int32_t *row_word,
               unsigned long long wait_ns)
 {
     const int lane = threadIdx.x & 31;
@@ -1478,24 +1477,22 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, i
     if (row < rows_total) {
         if (kFollow) {
             s = t < vis_offset ? t : t + S - S_out;
-            failed = *(volatile int *)status; // (of a kernel before rank_kernel, which then publishes nothing)
+            failed = *(volatile const int *)status; // (of a kernel before rank_kernel, which then publishes nothing)
             if (!text && failed == 0) {
-                int32_t *word = row_word + row;
                 const long long t0 = clock64();
-                for (uint32_t spin = 1;; ++spin) {
-                    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(s) : "l"(word) : "memory");
+                for (;;) {
+                    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(s) : "l"(row_word + row) : "memory");
                     if (__any_sync(0xffffffffu, s >= 0)) break;
+                    const bool late = (unsigned long long)(clock64() - t0) > 2ull * wait_ns; // ns -> cycles at the highest SM clock
+                    if (__any_sync(0xffffffffu, late)) break;
                     __nanosleep(40);
-                    const bool late = (spin & 63u) == 0u && (unsigned long long)(clock64() - t0) > 2ull * wait_ns; // ns -> cycles at the highest SM clock
-                    if (__any_sync(0xffffffffu, late)) {
-                        if (lane == 0 && atomicCAS(status, 0, kStatusLate) == 0) status[1] = kWaitRowWord, status[2] = b, status[3] = (int)blockIdx.x;
-                        break;
-                    }
                 }
                 s = __reduce_max_sync(0xffffffffu, s);
-                if (s < 0) failed = kStatusLate;
-                __syncwarp();
-                if (lane == 0) *word = -1;
+                if (s < 0) {
+                    wait_for_previous();
+                    failed = *(volatile const int *)status;
+                    s = out_idx[row];
+                }
             }
         } else {
             s = !text ? out_idx[row] : t < vis_offset ? t : t + S - S_out;
@@ -1521,6 +1518,7 @@ gather_kernel(const uint4 *__restrict__ hidden, const int32_t *out_idx, int S, i
     }
     if (!kFirst) {
         if (kFollow || text) wait_for_previous(); // (what follows this kernel follows the one before it too)
+        if (kFollow && !text && row < rows_total && lane == 0) row_word[row] = -1;
         fs.put_back();
     }
 }

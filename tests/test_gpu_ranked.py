@@ -89,6 +89,53 @@ def test_rows_handed_to_the_gather_word_by_word(kept):
     ref.close()
 
 
+@pytest.mark.parametrize("captured", ["before", "behind"])
+def test_words_that_come_after_the_limit_are_not_the_next_calls(captured):
+    """A wait for a row's word of a microsecond, which ends before 400 pivots have taken their turns: the rows are copied all the same,
+    and a call on new contents - a graph captured before, replayed, or a call made after one was captured - finds no word of that call's."""
+    B, S, d, vo, nv, P, Kp = 1, 16100, 64, 40, 16000, 400, 2600
+    assert B * (S - nv + Kp) <= 20 * torch.cuda.get_device_properties(0).multi_processor_count  # the gather waits for words
+    bits = lambda t: t.view(torch.int16) if t.dtype == torch.bfloat16 else t
+    g = torch.Generator(device="cuda").manual_seed(5)
+    draw = lambda: (torch.randint(-15, 16, (B, S, d), generator=g, device="cuda", dtype=torch.int8).bfloat16(),
+                    torch.randn((B, S, d), generator=g, device="cuda").bfloat16())
+    plain = dart.dart_opts(path=dart.DART_PATH_STAGED)
+    ref, ctx = dart.Dart(B, S, d, P, Kp), dart.Dart(B, S, d, P, Kp)
+    want = lambda: ref.reduce(h, k, vo, nv, P, Kp, opts=dart.dart_opts(path=dart.DART_PATH_STAGED, retention=dart.DART_RETAIN_SERIAL))
+    same = lambda a, b: all(torch.equal(bits(x), bits(y)) for x, y in zip(a, b))
+    k, h = draw()
+    got = ctx.reduce(h, k, vo, nv, P, Kp, opts=plain)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+
+    def capture():
+        with torch.cuda.graph(graph):
+            ctx.reduce(h, k, vo, nv, P, Kp, out=got, opts=plain)
+
+    if captured == "before":
+        capture()
+    late = ctx.reduce(h, k, vo, nv, P, Kp, opts=dart.dart_opts(path=dart.DART_PATH_STAGED, wait_limit=1))
+    torch.cuda.synchronize()
+    first, right = ctx.status(), same(late, want())
+    if captured == "behind":
+        capture()
+    later = []
+    for _ in range(3):
+        for t, n in zip((k, h), draw()):
+            t.copy_(n)
+        if captured == "before":
+            graph.replay()
+        else:
+            ctx.reduce(h, k, vo, nv, P, Kp, out=got, opts=plain)
+        later.append(same(got, want()))
+        assert ctx.status() == dart.DART_OK
+    assert later == [True] * 3
+    assert first == dart.DART_OK and right
+    del graph
+    ctx.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("kind,shape", [("gaussian", (3, 333, 264, 17, 301, 7, 60)), ("equal tokens", (2, 700, 64, 10, 640, 16, 200)),
                                         ("gaussian", (260, 130, 64, 5, 100, 3, 90)), ("gaussian", (2, 3000, 64, 0, 2880, 128, 640))],
                          ids=lambda v: v if isinstance(v, str) else "x".join(map(str, v)))
