@@ -705,9 +705,8 @@ __device__ __forceinline__ void produce(const Params &p, const Ctl &ctl, Shared 
 template <int NT, int NSL>
 __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared &sh)
 {
-    constexpr int V = NSL >= 4 ? 16 / NSL : 4, H = 16 / NSL / V; // consecutive rows per lane and load; pivots per lane and tile
-    constexpr int NTat = NT == 2 && H == 1 ? 2 : 1;              // pivot tiles at a time (registers)
-    constexpr int W = H == 1 ? NT : NTat;                        // ... whose pivots' norms are asked for at a time: before the wait, or with the shares
+    constexpr int V = NSL >= 4 ? 16 / NSL : 4, H = 16 / NSL / V; // consecutive rows per lane and load; blocks of 32 V values per pivot tile
+    constexpr int NTat = NT == 2 ? 2 : 1;                        // pivot tiles at a time (registers)
     const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - kCombWarp0;
     const size_t part_item = (size_t)8 * NT * kRows;
     int seq = -1, last_b = -1, k = 0;
@@ -734,92 +733,74 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
         const size_t group = (size_t)it.b * p.n_rg + it.rg;
         // release: the item's shares, written by the warps that filled the mailbox
         if (NSL > 1 && lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.cnt + group) : "memory");
-        const int f = it.sl * (512 / NSL) + lane * V, i0 = f >> 6, r0 = f & 63; // this lane's first pivot of a tile (the others: every second one) and first row
-        if (NT > 1 || __any_sync(0xffffffffu, i0 < p.P)) {
+        bool waited = NSL == 1;
+        for (int h = 0; h < H; ++h) {
+            const int f = it.sl * (512 / NSL) + (32 * h + lane) * V, i0 = f >> 6, r0 = f & 63; // pivot of a tile and (first) row
+            if (NT == 1 && __all_sync(0xffffffffu, i0 >= p.P)) continue; // none of it is wanted
             const int j = it.rg * kRows + r0;
             const unsigned long long *rec = p.rec + (size_t)it.b * p.n_vis;
-            unsigned long long w[V];
+            unsigned long long w[V], wp[NT];
+            int pv[NT];
 #pragma unroll
             for (int e = 0; e < V; ++e) w[e] = j + e < p.n_vis ? ld_rec(rec + j + e) : 0ull;
-            unsigned long long wp[W][H];
-            int pv[W][H];
-            auto ask = [&](int n, int at) {
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const int i = 8 * n + 2 * h + i0;
-                    pv[at][h] = i < p.P ? sh.pv[seq % kPvRing][i] : 0;
-                    wp[at][h] = pv[at][h] < 0 || pv[at][h] >= p.n_vis ? (unsigned long long)__float_as_uint(p.text_ssq[(size_t)it.b * p.P + i]) << 32 : ld_rec(rec + pv[at][h]);
-                }
-            };
-            if constexpr (H == 1) {
-#pragma unroll
-                for (int n = 0; n < NT; ++n) ask(n, n);
+            for (int n = 0; n < NT; ++n) {
+                pv[n] = 8 * n + i0 < p.P ? sh.pv[seq % kPvRing][8 * n + i0] : 0;
+                const bool text = pv[n] < 0 || pv[n] >= p.n_vis;
+                wp[n] = text ? (unsigned long long)__float_as_uint(p.text_ssq[(size_t)it.b * p.P + 8 * n + i0]) << 32 : ld_rec(rec + pv[n]);
             }
-            if (NSL > 1) { // acquire: the other slices' shares
+            if (!waited) { // acquire: the other slices' shares
                 if (lane == 0) ok = ctl.wait_flag(p.cnt + group, kWaitShares, it.b, NSL);
                 if (!__all_sync(0xffffffffu, ok)) return;
                 __syncwarp(); // (every lane's loads come after lane 0's)
+                waited = true;
             }
             const float *src = p.part + group * NSL * part_item + f;
             float *dst = p.sim + ((size_t)it.b * p.P + i0) * p.n_vis + j;
             float nr[V];
 #pragma unroll
             for (int n0 = 0; n0 < NT; n0 += NTat) {
-                float x[NTat][H][NSL][V];
+                float x[NTat][NSL][V];
 #pragma unroll
-                for (int n = 0; n < NTat; ++n) {
-                    if constexpr (H > 1) ask(n0 + n, n);
+                for (int n = 0; n < NTat; ++n)
 #pragma unroll
-                    for (int h = 0; h < H; ++h) {
-                        const bool wanted = 8 * (n0 + n) + 2 * h + i0 < p.P;
+                    for (int s = 0; s < NSL; ++s) {
+                        const float *at = src + s * part_item + (n0 + n) * 512;
+                        if (8 * (n0 + n) + i0 >= p.P) { // not wanted
 #pragma unroll
-                        for (int s = 0; s < NSL; ++s) {
-                            const float *at = src + s * part_item + (n0 + n) * 512 + h * 128;
-                            float (&v)[V] = x[n][h][s];
-                            if (!wanted) {
-#pragma unroll
-                                for (int e = 0; e < V; ++e) v[e] = 0.f;
-                            } else if constexpr (V == 4) {
-                                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(at) : "memory");
-                            } else if constexpr (V == 2) {
-                                asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "l"(at) : "memory");
-                            } else {
-                                asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v[0]) : "l"(at) : "memory");
-                            }
+                            for (int e = 0; e < V; ++e) x[n][s][e] = 0.f;
+                            continue;
                         }
+                        if constexpr (V == 4)
+                            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]), "=f"(x[n][s][2]), "=f"(x[n][s][3]) : "l"(at) : "memory");
+                        else if constexpr (V == 2)
+                            asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]) : "l"(at) : "memory");
+                        else
+                            asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(x[n][s][0]) : "l"(at) : "memory");
                     }
-                }
                 if (n0 == 0) {
 #pragma unroll
                     for (int e = 0; e < V; ++e) {
                         if (w[e] == kNoRec) ok = ok && late(rec + j + e, it.b, w[e]);
                         nr[e] = sqrtf(__uint_as_float((uint32_t)(w[e] >> 32)));
                     }
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+                        if (wp[n] == kNoRec) ok = ok && late(rec + pv[n], it.b, wp[n]);
+                    if (!__all_sync(0xffffffffu, ok)) return;
                 }
 #pragma unroll
-                for (int n = 0; n < NTat; ++n)
+                for (int n = 0; n < NTat; ++n) {
+                    const float np = sqrtf(__uint_as_float((uint32_t)(wp[n0 + n] >> 32)));
 #pragma unroll
-                    for (int h = 0; h < H; ++h)
-                    {
-                        const int at = H == 1 ? n0 + n : n;
-                        if (wp[at][h] == kNoRec) ok = ok && late(rec + pv[at][h], it.b, wp[at][h]);
+                    for (int e = 0; e < V; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0
+                        float a = 0.f;
+#pragma unroll
+                        for (int s = 0; s < NSL; ++s) a += x[n][s][e]; // in slice order
+                        const float den = np * nr[e];
+                        if (8 * (n0 + n) + i0 < p.P && j + e < p.n_vis) dst[(size_t)8 * (n0 + n) * p.n_vis + e] = den > 0.f ? a / den : 0.f;
                     }
-                if (!__all_sync(0xffffffffu, ok)) return;
-#pragma unroll
-                for (int n = 0; n < NTat; ++n)
-#pragma unroll
-                    for (int h = 0; h < H; ++h) {
-                        const int i = 8 * (n0 + n) + 2 * h + i0;
-                        const float np = sqrtf(__uint_as_float((uint32_t)(wp[H == 1 ? n0 + n : n][h] >> 32)));
-#pragma unroll
-                        for (int e = 0; e < V; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0
-                            float a = 0.f;
-#pragma unroll
-                            for (int s = 0; s < NSL; ++s) a += x[n][h][s][e]; // in slice order
-                            const float den = np * nr[e];
-                            if (i < p.P && j + e < p.n_vis) dst[(size_t)(i - i0) * p.n_vis + e] = den > 0.f ? a / den : 0.f;
-                        }
-                    }
+                }
             }
         }
         __syncwarp();
