@@ -834,6 +834,13 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     long long window = sample + 36 * MB < 72 * MB ? sample + 36 * MB : 72 * MB;
     if (window < sample + 20 * MB) window = sample + 20 * MB;
     if (o.tune & 0xff) window = (long long)(o.tune & 0xff) * MB > sample ? (long long)(o.tune & 0xff) * MB : sample;
+    // ... and their lead over their own SM's second pass: with two feeders the scorers take what the second pass needs to keep up, and it came
+    // so far behind the pivots that its rows had left the L2 (whole calls, us, without / sample + 44 MB / + 52 / + 60 / + 76: 256 x 2880 x
+    // 4096 1744 / 1686 / 1673 / 1681 / 1688, 16 pivots 1964 / 1830 / 1777 / 1793 / 1810, 200 x 1500 x 5120 877 / 924 / 886 / 880 / 879, 256 x 576 x
+    // 4096 380 / 381 / 373 / 377 / 380; + 48 / + 50 / + 52 elsewhere: 256 x 2880 1671 / 1671 / 1682, 64 x 2880 424 / 425 / 431, 200 x 1500 x 5120
+    // 893 / 888 / 880, 64 x 4096 582 / 581 / 586).  Other windows under this bound change nothing beyond the scatter.
+    const long long lead = (sample + 50 * MB > window ? sample + 50 * MB : window) / row_bytes + 1;
+    p.lead = (int)(lead < (1ll << 29) ? lead : (1ll << 29));
     window = window / row_bytes + 1;
     p.window = (int)(window < (1ll << 29) ? window : (1ll << 29));
     return true;

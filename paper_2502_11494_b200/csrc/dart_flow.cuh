@@ -14,7 +14,7 @@
 //   - a second-pass item is 64 rows x 1/nsl of the columns: an SM's pivot tile is P x d/nsl (16 KB at 8 pivots, d = 4096, 4
 //     slices) instead of P x d, and the item takes about 2.5 us instead of the 20 us of a 128-row tile of full rows;
 //   - the item's rows are fetched into a ring before the pivots are known;
-//   - the scorers are held back to `window` rows beyond the samples that have their pivots.
+//   - the scorers are held back to `window` rows beyond the samples that have their pivots, and to `lead` beyond their SM's second pass.
 // The slices' shares of a dot product meet in global memory (L2): when a row group's are all there, each of its SMs adds up a part of
 // them in slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
@@ -102,6 +102,7 @@ struct Params {
     int given;                          // the pivots are in pivot_idx already
     int norm_kind, smallest, withhold;
     int window;                         // rows the scorers may be ahead of `pos` (>= n_vis)
+    int lead;                           // ... and of their own SM's second pass (>= n_vis: a sample's pivots wait for all of its rows)
     uint32_t pitch;                     // bytes between pivot rows in shared memory
     unsigned long long wait_ns;
     const uint4 *keys;                  // [B][S][d]
@@ -125,6 +126,7 @@ struct Shared {
     uint32_t n_list[kSelGroups];
     int32_t pv[kPvRing][kMaxP];       // pivots of the samples on their way, by the SM's own count of samples
     int abort_flag;
+    volatile int at;                  // first row (of the batch) of the SM's own item in the second pass
     volatile int pos;                 // rows (of the batch) whose samples have their pivots; given pivots: rows the second pass is through with
 };
 static_assert(sizeof(Shared) + 64 <= kStaticSmemReserve, "static shared memory exceeds its reserve");
@@ -241,8 +243,8 @@ struct Tasks {
 // Feeders: a lane keeps one scorer's p.n_slot slots (4 KB chunks of rows) on their way, as far as the window allows.  Warps of their
 // own: a bulk copy takes its thread some 500 cycles to issue (with every scorer refilling its own slots a row of 8 KB took
 // 4000 cycles, and the scorers bound the whole path).  Two: a warp that feeds all eight scorers spends 195 cycles per copy and nothing
-// else 88 % of the time (whole calls, us, one / two: 64 x 576 118 / 115, 8 x 1500 x 3072 60.5 / 59.3, 256 x 2880 1585 / 1535; three 1595, and four,
-// which costs registers, 1645).
+// else 88 % of the time (whole calls, us, one / two: 64 x 576 118 / 115, 8 x 1500 x 3072 60.5 / 59.3, 256 x 1000 x 3072 514 / 494; 256 x 2880 about
+// the same, three there 4 % more than two and four, which costs registers, 7 %).
 __device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh, uint32_t slot0)
 {
     const int lane = threadIdx.x & 31, w = ((int)(threadIdx.x >> 5) - kFeedWarp) + kFeedWarps * lane; // this lane's scorer
@@ -258,7 +260,7 @@ __device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh
         bool go = false;
         if (more) {
             const int row = it.b * p.n_vis + it.t * p.rows_task;
-            go = (c > 0 || row - sh.pos < p.window) && sweep::mbar_test(smem_u32(&sh.chunk_empty[w][in]), phase);
+            go = (c > 0 || (row - sh.pos < p.window && row - sh.at < p.lead)) && sweep::mbar_test(smem_u32(&sh.chunk_empty[w][in]), phase);
             if (go) {
                 const int j = it.t * p.rows_task, rows = min(p.rows_task, p.n_vis - j);
                 const int from = c * kChunkUnits, n = p.rows_task > 1 ? rows * p.d8 : min(kChunkUnits, p.d8 - from);
@@ -559,6 +561,7 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
     Ring ring(p.n_st);
     int seq = -1, last_b = -1, k = 0;
     for (Items it(p); it.valid(); it.next(), ++k) {
+        if (w == 0 && n0 == 0 && lane == 0) sh.at = it.b * p.n_vis + it.rg * kRows;
         if (it.b != last_b) {
             if (seq >= 0 && lane == 0) mbar_arrive(smem_u32(&sh.piv_empty[seq & 1])); // (the warp has converged at the item's end)
             ++seq;
@@ -636,7 +639,10 @@ __device__ __forceinline__ void multiply(const Params &p, const Ctl &ctl, Shared
         __syncwarp(); // the lanes' stores are ordered before lane 0's release
         if (lane == 0) mbar_arrive(smem_u32(&sh.mail_full[c][slot]));
     }
-    if (p.given && w == 0 && n0 == 0 && lane == 0) sh.pos = 0x3fffffff; // nothing holds the scorers back any more
+    if (w == 0 && n0 == 0 && lane == 0) { // nothing holds the scorers back any more
+        sh.at = 0x3fffffff;
+        if (p.given) sh.pos = 0x3fffffff;
+    }
 }
 
 // Watcher: how far the batch's pivots have got, for the scorers.  (Held back by the second pass of their own SM instead, the
@@ -839,7 +845,7 @@ __global__ void __launch_bounds__(threads(NT), 1) flow_kernel(const __grid_const
                 mbar_init(smem_u32(&sh.mail_empty[c][s]), 1);
             }
         sh.abort_flag = 0;
-        sh.pos = 0;
+        sh.pos = sh.at = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();

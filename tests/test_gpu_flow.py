@@ -140,6 +140,28 @@ def test_flow_shares_of_every_number_of_slices(nsl, P, given):
     assert all(torch.equal(a, b) for a, b in zip(*outs))
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("nsl,P,n,B", [(1, 8, 400, 300), (2, 16, 389, 300), (4, 8, 131, 430), (4, 31, 200, 360), (8, 13, 400, 140), (16, 8, 131, 330)])
+def test_flow_many_items_of_every_number_of_slices(nsl, P, n, B, given):
+    """Tens of items and, from four slices on, of samples per SM: the mailboxes, the pivots' ring and the pivot buffers go round several
+    times, and the batch is longer than the scorers' lead over the second pass (as above, bit for bit)."""
+    d, Kp = 1024, P + 20
+    assert B * n * d * 2 > n * d * 2 + (50 << 20)
+    g = torch.Generator(device="cuda").manual_seed(nsl + P)
+    k = torch.randint(-15, 16, (B, n + 3, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
+    piv = torch.rand((B, n), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
+    outs = []
+    for path in (FLOW, dart.DART_PATH_STAGED):
+        ctx = dart.Dart(B, n + 3, d, P, Kp)
+        o = dart.dart_opts(path=path, tune=nsl << 16 if path == FLOW else 0, pivots_in=piv.data_ptr() if given else None)
+        oh, oi, op, dbg = ctx.reduce(k, None, 2, n, P, Kp, opts=o, debug=True)
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        ctx.close()
+        outs.append((oh.view(torch.int16), oi, op, dbg["sim"]))
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
 @pytest.mark.parametrize("norm_kind,smallest", [(1, 1), (2, 0), (2, 1)])
 def test_flow_ranking_variants(oracle, norm_kind, smallest):
     k, h = gaussian(3, 500, 256, seed=77)
