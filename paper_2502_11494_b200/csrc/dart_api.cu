@@ -834,12 +834,20 @@ bool flow_config(const dart_ctx *ctx, int B, int n_vis, int P, const dart_opts &
     long long window = sample + 36 * MB < 72 * MB ? sample + 36 * MB : 72 * MB;
     if (window < sample + 20 * MB) window = sample + 20 * MB;
     if (o.tune & 0xff) window = (long long)(o.tune & 0xff) * MB > sample ? (long long)(o.tune & 0xff) * MB : sample;
-    // ... and their lead over their own SM's second pass: with two feeders the scorers take what the second pass needs to keep up, and it came
-    // so far behind the pivots that its rows had left the L2 (whole calls, us, without / sample + 44 MB / + 52 / + 60 / + 76: 256 x 2880 x
-    // 4096 1744 / 1686 / 1673 / 1681 / 1688, 16 pivots 1964 / 1830 / 1777 / 1793 / 1810, 200 x 1500 x 5120 877 / 924 / 886 / 880 / 879, 256 x 576 x
-    // 4096 380 / 381 / 373 / 377 / 380; + 48 / + 50 / + 52 elsewhere: 256 x 2880 1671 / 1671 / 1682, 64 x 2880 424 / 425 / 431, 200 x 1500 x 5120
-    // 893 / 888 / 880, 64 x 4096 582 / 581 / 586).  Other windows under this bound change nothing beyond the scatter.
-    const long long lead = (sample + 50 * MB > window ? sample + 50 * MB : window) / row_bytes + 1;
+    // ... and, in long batches, their lead over their own SM's second pass: with two feeders the scorers take what the second pass needs to
+    // keep up, and it came so far behind the pivots that its rows had left the L2.  32 MB beyond the sample and the distance between two
+    // items of an SM, by which its place moves (whole calls, us, without / 44 MB beyond the sample with four slices, whose items lie 18 MB
+    // apart / 52 / 60 / 76: 256 x 2880 x 4096 1744 / 1686 / 1673 / 1681 / 1688, 16 pivots 1964 / 1830 / 1777 / 1793 / 1810).  Short batches are
+    // through before that, and there the scorers' time is lost (without / with, by MB of keys: 2880 x 4096 300: 105.0 / 106.7, 500: 152 / 155, 750: 226 /
+    // 223, 1700: 500 / 480; 16 pivots 170 / 172, 258 / 241, 553 / 518; 1000 x 4096 500: 159 / 162, 750: 233 / 237, 1700: 517 / 509; 1500 x 3584, 16
+    // pivots 500: 179 / 182, 750: 261 / 262, 1700: 585 / 565; 2200 x 5120 500: 156 / 158, 750: 230 / 225).
+    long long lead = 1ll << 40;
+    if (sample * B > 640 * MB) {
+        const long long apart = (long long)(p.n_stream / p.nsl) * F::kRows * row_bytes;
+        lead = sample + (apart + 32 * MB > 50 * MB ? apart + 32 * MB : 50 * MB);
+        if (lead < window) lead = window;
+    }
+    lead = lead / row_bytes + 1;
     p.lead = (int)(lead < (1ll << 29) ? lead : (1ll << 29));
     window = window / row_bytes + 1;
     p.window = (int)(window < (1ll << 29) ? window : (1ll << 29));

@@ -258,9 +258,10 @@ __device__ __forceinline__ void feed(const Params &p, const Ctl &ctl, Shared &sh
     long long issued = 0, since = clock64();
     for (uint32_t spin = 0; __any_sync(0xffffffffu, more);) {
         bool go = false;
+        const int far = min(sh.pos + p.window, sh.at + p.lead);
         if (more) {
             const int row = it.b * p.n_vis + it.t * p.rows_task;
-            go = (c > 0 || (row - sh.pos < p.window && row - sh.at < p.lead)) && sweep::mbar_test(smem_u32(&sh.chunk_empty[w][in]), phase);
+            go = (c > 0 || row < far) && sweep::mbar_test(smem_u32(&sh.chunk_empty[w][in]), phase);
             if (go) {
                 const int j = it.t * p.rows_task, rows = min(p.rows_task, p.n_vis - j);
                 const int from = c * kChunkUnits, n = p.rows_task > 1 ? rows * p.d8 : min(kChunkUnits, p.d8 - from);

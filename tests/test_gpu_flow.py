@@ -144,9 +144,29 @@ def test_flow_shares_of_every_number_of_slices(nsl, P, given):
 @pytest.mark.parametrize("nsl,P,n,B", [(1, 8, 400, 300), (2, 16, 389, 300), (4, 8, 131, 430), (4, 31, 200, 360), (8, 13, 400, 140), (16, 8, 131, 330)])
 def test_flow_many_items_of_every_number_of_slices(nsl, P, n, B, given):
     """Tens of items and, from four slices on, of samples per SM: the mailboxes, the pivots' ring and the pivot buffers go round several
-    times, and the batch is longer than the scorers' lead over the second pass (as above, bit for bit)."""
+    times (as above, bit for bit)."""
     d, Kp = 1024, P + 20
-    assert B * n * d * 2 > n * d * 2 + (50 << 20)
+    g = torch.Generator(device="cuda").manual_seed(nsl + P)
+    k = torch.randint(-15, 16, (B, n + 3, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
+    piv = torch.rand((B, n), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
+    outs = []
+    for path in (FLOW, dart.DART_PATH_STAGED):
+        ctx = dart.Dart(B, n + 3, d, P, Kp)
+        o = dart.dart_opts(path=path, tune=nsl << 16 if path == FLOW else 0, pivots_in=piv.data_ptr() if given else None)
+        oh, oi, op, dbg = ctx.reduce(k, None, 2, n, P, Kp, opts=o, debug=True)
+        torch.cuda.synchronize()
+        assert ctx.status() == dart.DART_OK
+        ctx.close()
+        outs.append((oh.view(torch.int16), oi, op, dbg["sim"]))
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("nsl,P,n,B", [(0, 16, 4096, 21), (4, 8, 64, 1300), (8, 3, 1001, 90)])
+def test_flow_scorers_wait_for_the_second_pass(nsl, P, n, B, given):
+    """Batches of more than 640 MB of keys, whose scorers are held back to some 50 MB beyond their SM's second pass."""
+    d, Kp = 4096, P + 20
+    assert B * n * d * 2 > 640 << 20
     g = torch.Generator(device="cuda").manual_seed(nsl + P)
     k = torch.randint(-15, 16, (B, n + 3, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
     piv = torch.rand((B, n), generator=g, device="cuda").topk(P, dim=1).indices.to(torch.int32).contiguous()
