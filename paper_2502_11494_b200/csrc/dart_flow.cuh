@@ -703,17 +703,22 @@ __device__ __forceinline__ void produce(const Params &p, const Ctl &ctl, Shared 
 }
 
 // Combine: an item is counted once its shares are written; when all slices of its row group are, each of their SMs adds up one part
-// in NSL of the group's similarities.  So a warp has 16 values per pivot tile to fetch, all at once, whatever the number of slices.
+// in NSL of the group's similarities.  So from four slices on a lane has 16 values per pivot tile to fetch, all at once.
 // (With the SM that counted last adding up the whole group, one sample of 576 tokens in 16 slices took 7 us from count to
-// similarities, now 2.  Whole calls, us: 1 x 576 30.8 -> 26.7, 1 x 2880 39.0 -> 36.7, 16 x 256 36.9 -> 34.9, 64 x 576 115.4 -> 113.5, 8 x 2880
-// with 16 pivots 87.5 -> 84.9.)
+// similarities, now 2.  Whole calls, us, by number of slices 1 / 2 / 4 / 8 / 16: 16 x 2880 x 1024 51.7 -> 49.3, 54.8 -> 52.4, 63.7 -> 59.4, 94 ->
+// 74, 191 -> 117; 8 x 2880 x 4096 with 16 pivots from two on 108 -> 106, 98.2 -> 93.7, 115 -> 94, 202 -> 113; 4 x 1500 x 2048 with 32 55.4 -> 49.2, 53.4 ->
+// 47.0, 67.6 -> 49.9, 103 -> 55.6.)
 // A warp here waits for the other SMs' shares of its row group, and those for nothing but earlier groups: every SM takes its items
 // in the groups' order.
 template <int NT, int NSL>
 __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared &sh)
 {
     constexpr int V = NSL >= 4 ? 16 / NSL : 4, H = 16 / NSL / V; // consecutive rows per lane and load; blocks of 32 V values per pivot tile
-    constexpr int NTat = NT == 2 ? 2 : 1;                        // pivot tiles at a time (registers)
+    // Blocks at a time: the same rows, every second pivot.  With one slice a block is 4 values of 16, and one after the other their loads are
+    // four rounds (whole calls, us, one / all four: 6 x 4518 x 1024 49.0 / 47.2, 35 x 1072 51.4 / 49.4, 47 x 4329 172.9 / 169.9); two slices 51.9 / 53.4
+    // (16 x 2880 x 1024), two pivot tiles 84.0 / 84.7 (8 x 2880 x 4096, whose own four slices the registers reach).
+    constexpr int U = NSL == 1 && NT == 1 ? H : 1;
+    constexpr int NTat = NT == 2 && U == 1 ? 2 : 1;              // pivot tiles at a time (registers)
     const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - kCombWarp0;
     const size_t part_item = (size_t)8 * NT * kRows;
     int seq = -1, last_b = -1, k = 0;
@@ -741,21 +746,24 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
         // release: the item's shares, written by the warps that filled the mailbox
         if (NSL > 1 && lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.cnt + group) : "memory");
         bool waited = NSL == 1;
-        for (int h = 0; h < H; ++h) {
-            const int f = it.sl * (512 / NSL) + (32 * h + lane) * V, i0 = f >> 6, r0 = f & 63; // pivot of a tile and (first) row
+        for (int h = 0; h < H; h += U) {
+            const int f = it.sl * (512 / NSL) + (32 * h + lane) * V, i0 = f >> 6, r0 = f & 63; // (first) pivot of a tile and (first) row
             if (NT == 1 && __all_sync(0xffffffffu, i0 >= p.P)) continue; // none of it is wanted
             const int j = it.rg * kRows + r0;
             const unsigned long long *rec = p.rec + (size_t)it.b * p.n_vis;
-            unsigned long long w[V], wp[NT];
-            int pv[NT];
+            unsigned long long w[V], wp[NT][U];
+            int pv[NT][U];
 #pragma unroll
             for (int e = 0; e < V; ++e) w[e] = j + e < p.n_vis ? ld_rec(rec + j + e) : 0ull;
 #pragma unroll
-            for (int n = 0; n < NT; ++n) {
-                pv[n] = 8 * n + i0 < p.P ? sh.pv[seq % kPvRing][8 * n + i0] : 0;
-                const bool text = pv[n] < 0 || pv[n] >= p.n_vis;
-                wp[n] = text ? (unsigned long long)__float_as_uint(p.text_ssq[(size_t)it.b * p.P + 8 * n + i0]) << 32 : ld_rec(rec + pv[n]);
-            }
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = 8 * n + 2 * u + i0;
+                    pv[n][u] = i < p.P ? sh.pv[seq % kPvRing][i] : 0;
+                    const bool text = pv[n][u] < 0 || pv[n][u] >= p.n_vis;
+                    wp[n][u] = text ? (unsigned long long)__float_as_uint(p.text_ssq[(size_t)it.b * p.P + i]) << 32 : ld_rec(rec + pv[n][u]);
+                }
             if (!waited) { // acquire: the other slices' shares
                 if (lane == 0) ok = ctl.wait_flag(p.cnt + group, kWaitShares, it.b, NSL);
                 if (!__all_sync(0xffffffffu, ok)) return;
@@ -767,24 +775,27 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
             float nr[V];
 #pragma unroll
             for (int n0 = 0; n0 < NT; n0 += NTat) {
-                float x[NTat][NSL][V];
+                float x[NTat][U][NSL][V];
 #pragma unroll
                 for (int n = 0; n < NTat; ++n)
 #pragma unroll
-                    for (int s = 0; s < NSL; ++s) {
-                        const float *at = src + s * part_item + (n0 + n) * 512;
-                        if (8 * (n0 + n) + i0 >= p.P) { // not wanted
+                    for (int u = 0; u < U; ++u)
 #pragma unroll
-                            for (int e = 0; e < V; ++e) x[n][s][e] = 0.f;
-                            continue;
+                        for (int s = 0; s < NSL; ++s) {
+                            const float *at = src + s * part_item + (n0 + n) * 512 + u * 128;
+                            float (&v)[V] = x[n][u][s];
+                            if (8 * (n0 + n) + 2 * u + i0 >= p.P) { // not wanted
+#pragma unroll
+                                for (int e = 0; e < V; ++e) v[e] = 0.f;
+                                continue;
+                            }
+                            if constexpr (V == 4)
+                                asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(at) : "memory");
+                            else if constexpr (V == 2)
+                                asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "l"(at) : "memory");
+                            else
+                                asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v[0]) : "l"(at) : "memory");
                         }
-                        if constexpr (V == 4)
-                            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]), "=f"(x[n][s][2]), "=f"(x[n][s][3]) : "l"(at) : "memory");
-                        else if constexpr (V == 2)
-                            asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(x[n][s][0]), "=f"(x[n][s][1]) : "l"(at) : "memory");
-                        else
-                            asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(x[n][s][0]) : "l"(at) : "memory");
-                    }
                 if (n0 == 0) {
 #pragma unroll
                     for (int e = 0; e < V; ++e) {
@@ -793,21 +804,26 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
                     }
 #pragma unroll
                     for (int n = 0; n < NT; ++n)
-                        if (wp[n] == kNoRec) ok = ok && late(rec + pv[n], it.b, wp[n]);
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (wp[n][u] == kNoRec) ok = ok && late(rec + pv[n][u], it.b, wp[n][u]);
                     if (!__all_sync(0xffffffffu, ok)) return;
                 }
 #pragma unroll
-                for (int n = 0; n < NTat; ++n) {
-                    const float np = sqrtf(__uint_as_float((uint32_t)(wp[n0 + n] >> 32)));
+                for (int n = 0; n < NTat; ++n)
 #pragma unroll
-                    for (int e = 0; e < V; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0
-                        float a = 0.f;
+                    for (int u = 0; u < U; ++u) {
+                        const float np = sqrtf(__uint_as_float((uint32_t)(wp[n0 + n][u] >> 32)));
 #pragma unroll
-                        for (int s = 0; s < NSL; ++s) a += x[n][s][e]; // in slice order
-                        const float den = np * nr[e];
-                        if (8 * (n0 + n) + i0 < p.P && j + e < p.n_vis) dst[(size_t)8 * (n0 + n) * p.n_vis + e] = den > 0.f ? a / den : 0.f;
+                        for (int e = 0; e < V; ++e) { // dup = dot / (|pivot| |row|); a zero norm gives 0
+                            float a = 0.f;
+#pragma unroll
+                            for (int s = 0; s < NSL; ++s) a += x[n][u][s][e]; // in slice order
+                            const float den = np * nr[e];
+                            if (8 * (n0 + n) + 2 * u + i0 < p.P && j + e < p.n_vis)
+                                dst[(size_t)(8 * (n0 + n) + 2 * u) * p.n_vis + e] = den > 0.f ? a / den : 0.f;
+                        }
                     }
-                }
             }
         }
         __syncwarp();
