@@ -714,10 +714,11 @@ template <int NT, int NSL>
 __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared &sh)
 {
     constexpr int V = NSL >= 4 ? 16 / NSL : 4, H = 16 / NSL / V; // consecutive rows per lane and load; blocks of 32 V values per pivot tile
-    // Blocks at a time: the same rows, every second pivot.  With one slice a block is 4 values of 16, and one after the other their loads are
-    // four rounds (whole calls, us, one / all four: 6 x 4518 x 1024 49.0 / 47.2, 35 x 1072 51.4 / 49.4, 47 x 4329 172.9 / 169.9); two slices 51.9 / 53.4
-    // (16 x 2880 x 1024), two pivot tiles 84.0 / 84.7 (8 x 2880 x 4096, whose own four slices the registers reach).
-    constexpr int U = NSL == 1 && NT == 1 ? H : 1;
+    // Blocks at a time: the same rows, every second pivot.  With one slice and two a lane has several blocks of 4 and 8 values, and one after
+    // the other their loads are four and two rounds (whole calls, us, one at a time / all: 6 x 4518 x 1024 49.0 / 47.2, 35 x 1072 51.4 / 49.4, 47 x
+    // 4329 172.9 / 169.9, 6 x 609 x 2048 30.0 / 28.8, 16 x 256 30.6 / 29.0, 61 x 1643 158.1 / 157.9; 1 pivot, 128 x 570 118.7 / 120.0).  Two pivot tiles
+    // one at a time: 8 x 2880 x 4096 84.0 / 84.7, 39 x 911 x 2048 80.6 / 84.6.
+    constexpr int U = NSL <= 2 && NT == 1 ? H : 1;
     constexpr int NTat = NT == 2 && U == 1 ? 2 : 1;              // pivot tiles at a time (registers)
     const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - kCombWarp0;
     const size_t part_item = (size_t)8 * NT * kRows;
