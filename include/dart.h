@@ -153,8 +153,9 @@ typedef struct {
     int32_t test_withhold_pivots; /* testing only: nonzero withholds one hand-over inside the kernel that waits (the persistent
                                      sweep never publishes a sample's pivots; the resident sweep's CTAs never count themselves in;
                                      the one-pass kernel's first norm warp never hands its norms over; the paired sweeps:
-                                     1 = the lists are never counted in, 2 = the pivots' norms never reach the epilogue), so that
-                                     the bounded waits expire and the call ends with DART_ERR_TIMEOUT in dart_status */
+                                     1 = the lists are never counted in, 2 = the pivots' norms never reach the epilogue; the flow path:
+                                     1 = one row's score is never published, 2 = one item's shares of the similarities are never counted
+                                     in), so that the bounded waits expire and the call ends with DART_ERR_TIMEOUT in dart_status */
     int32_t retention;     /* DART_RETAIN_*: how step 4 is scheduled (same result either way) */
     int32_t rule;          /* DART_RULE_*: which tokens step 4 retains */
     int32_t cosine_on_hidden; /* 0: Eq. 7 on the key rows that are scored (one tensor for steps 1-3).  1: the pivots are still

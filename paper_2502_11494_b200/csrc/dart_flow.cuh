@@ -100,7 +100,8 @@ struct Params {
     int n_stream;                       // CTAs that stream; the others select
     int sel_threads;                    // threads per selection
     int given;                          // the pivots are in pivot_idx already
-    int norm_kind, smallest, withhold;
+    int norm_kind, smallest;
+    int withhold;                       // test hook: 1 = one row's score is never published, 2 = one item's shares are never counted in
     int window;                         // rows the scorers may be ahead of `pos` (>= n_vis)
     int lead;                           // ... and of their own SM's second pass (>= n_vis: a sample's pivots wait for all of its rows)
     uint32_t pitch;                     // bytes between pivot rows in shared memory
@@ -359,7 +360,7 @@ __device__ __forceinline__ void score_rows(const Params &p, const Ctl &ctl, Shar
             l1 = x, ssq = __shfl_xor_sync(0xffffffffu, x, 8);
             row = lane >> 4;
         }
-        if ((lane & 15) == 0 && (lane == 0 || p.rows_task == 2) && row < rows && !(p.withhold && r + row == 0)) {
+        if ((lane & 15) == 0 && (lane == 0 || p.rows_task == 2) && row < rows && !(p.withhold == 1 && r + row == 0)) {
             st_rec(p.rec + r + row, ((unsigned long long)__float_as_uint(ssq) << 32) | __float_as_uint(l1));
             if (p.l1) p.l1[r + row] = l1, p.ssq[r + row] = ssq;
         }
@@ -745,7 +746,7 @@ __device__ __forceinline__ void combine(const Params &p, const Ctl &ctl, Shared 
         if (!__all_sync(0xffffffffu, ok)) return;
         const size_t group = (size_t)it.b * p.n_rg + it.rg;
         // release: the item's shares, written by the warps that filled the mailbox
-        if (NSL > 1 && lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.cnt + group) : "memory");
+        if (NSL > 1 && lane == 0 && !(p.withhold == 2 && group + it.sl == 0)) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.cnt + group) : "memory");
         bool waited = NSL == 1;
         for (int h = 0; h < H; h += U) {
             const int f = it.sl * (512 / NSL) + (32 * h + lane) * V, i0 = f >> 6, r0 = f & 63; // (first) pivot of a tile and (first) row

@@ -246,23 +246,33 @@ def test_flow_says_what_it_does_not_take(shape):
     ctx.close()
 
 
-def test_flow_expired_waits_are_reported_not_hung():
-    """One row's word is never published: the selecting CTA gives up within its limit and says so, every other wait ends
-    too, and the next call on the same context succeeds."""
+@pytest.mark.parametrize("withhold,where", [(1, 90), (2, 102)], ids=["a row's word never published", "an item's shares never counted in"])
+def test_flow_expired_waits_are_reported_not_hung(withhold, where):
+    """The warp that waits for what is withheld gives up within its limit and says so, every other wait ends too, and the next call on
+    the same context succeeds, as does a graph captured before."""
     w = W.LLAVA15_B64.with_(B=3)
     k, h = W.make_batch(w, device="cuda")
+    shape = (w.vis_offset, w.n_vis, w.n_pivot, w.n_keep)
     ctx = dart.Dart(w.B, w.S, w.d, w.n_pivot, w.n_keep)
-    ctx.reduce(h, k, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep,
-               opts=dart.dart_opts(path=FLOW, wait_limit=20000, test_withhold_pivots=1))      # 20 ms limit
+    out = ctx.reduce(h, k, *shape, opts=dart.dart_opts(path=FLOW))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.reduce(h, k, *shape, out=out, opts=dart.dart_opts(path=FLOW))
+    ctx.reduce(h, k, *shape, opts=dart.dart_opts(path=FLOW, wait_limit=20000, test_withhold_pivots=withhold))      # 20 ms limit
     torch.cuda.synchronize()
     assert ctx.status() == dart.DART_ERR_TIMEOUT
     rc, detail = dart.dart_status_detail(ctx.handle)
-    assert rc == dart.DART_OK and detail[0] == 90, detail
-    good = ctx.reduce(h, k, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep, opts=dart.dart_opts(path=FLOW))
+    assert rc == dart.DART_OK and detail[0] == where, detail
+    k, h = k.copy_(k.flip(0)), h.copy_(h.flip(0))
+    graph.replay()
+    good = ctx.reduce(h, k, *shape, opts=dart.dart_opts(path=FLOW))
     torch.cuda.synchronize()
     assert ctx.status() == dart.DART_OK
-    ref = run_gpu(k, h, w.vis_offset, w.n_vis, w.n_pivot, w.n_keep, path=dart.DART_PATH_STAGED, debug=False)
-    assert np.array_equal(good[1].cpu().numpy(), ref[1]) and np.array_equal(W.bits(good[0]), ref[0])
+    ref = run_gpu(k, h, *shape, path=dart.DART_PATH_STAGED, debug=False)
+    for got in (out, good):
+        assert np.array_equal(got[1].cpu().numpy(), ref[1]) and np.array_equal(W.bits(got[0]), ref[0])
+    del graph
     ctx.close()
 
 
