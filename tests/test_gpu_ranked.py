@@ -1,4 +1,6 @@
 """The retention from ranked lists against the one-kernel form, bit for bit, through the C ABI (needs a B200)."""
+import re
+
 import numpy as np
 import pytest
 
@@ -51,10 +53,24 @@ def test_ranked_lists_at_the_lines_between_threads_per_list(shape):
     assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
 
 
-@pytest.mark.parametrize("kept", [256, 255, 90])
-def test_rows_handed_to_the_gather_word_by_word(kept):
-    """Both sides of the line (2960 packed rows on 148 SMs), one context through several calls, a refused call and a replayed one among them."""
-    B, S, d, vo, nv, P = 4, 1700, 128, 11, 1216, 5                         # 4 x (484 + 256) rows
+def _captured(call):
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    graph.enable_debug_mode()
+    with torch.cuda.graph(graph):
+        call()
+    return graph
+
+
+def _waits_for_words(graph, path):
+    graph.debug_dump(str(path))
+    return re.search(r"gather_kernelILb0ELb([01])E", path.read_text()).group(1) == "1"
+
+
+@pytest.mark.parametrize("kept", [257, 256, 255, 90])
+def test_rows_handed_to_the_gather_word_by_word(kept, tmp_path):
+    """Both sides of the line (20 packed rows per SM), one context through several calls, a refused call and a replayed one among them."""
+    B, d, vo, nv, P = 4, 128, 11, 1216, 5
+    S = nv + 5 * torch.cuda.get_device_properties(0).multi_processor_count - 256       # 256 kept: just the line's rows
     bits = lambda t: t.view(torch.int16) if t.dtype == torch.bfloat16 else t
     g = torch.Generator(device="cuda").manual_seed(kept)
     k = torch.randint(-15, 16, (B, S, d), generator=g, device="cuda", dtype=torch.int8).bfloat16()
@@ -76,9 +92,8 @@ def test_rows_handed_to_the_gather_word_by_word(kept):
     for t in got:
         t.zero_()
     torch.cuda.synchronize()
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        ctx.reduce(h, k, vo, nv, P, kept, pos_in=pos, out=got)
+    graph = _captured(lambda: ctx.reduce(h, k, vo, nv, P, kept, pos_in=pos, out=got))
+    assert _waits_for_words(graph, tmp_path / "graph.dot") == (kept <= 256)
     for _ in range(3):
         graph.replay()
     torch.cuda.synchronize()
@@ -90,11 +105,10 @@ def test_rows_handed_to_the_gather_word_by_word(kept):
 
 
 @pytest.mark.parametrize("captured", ["before", "behind"])
-def test_words_that_come_after_the_limit_are_not_the_next_calls(captured):
+def test_words_that_come_after_the_limit_are_not_the_next_calls(captured, tmp_path):
     """A wait for a row's word of a microsecond, which ends before 400 pivots have taken their turns: the rows are copied all the same,
     and a call on new contents - a graph captured before, replayed, or a call made after one was captured - finds no word of that call's."""
     B, S, d, vo, nv, P, Kp = 1, 16100, 64, 40, 16000, 400, 2600
-    assert B * (S - nv + Kp) <= 20 * torch.cuda.get_device_properties(0).multi_processor_count  # the gather waits for words
     bits = lambda t: t.view(torch.int16) if t.dtype == torch.bfloat16 else t
     g = torch.Generator(device="cuda").manual_seed(5)
     draw = lambda: (torch.randint(-15, 16, (B, S, d), generator=g, device="cuda", dtype=torch.int8).bfloat16(),
@@ -106,19 +120,15 @@ def test_words_that_come_after_the_limit_are_not_the_next_calls(captured):
     k, h = draw()
     got = ctx.reduce(h, k, vo, nv, P, Kp, opts=plain)
     torch.cuda.synchronize()
-    graph = torch.cuda.CUDAGraph()
-
-    def capture():
-        with torch.cuda.graph(graph):
-            ctx.reduce(h, k, vo, nv, P, Kp, out=got, opts=plain)
-
+    capture = lambda: _captured(lambda: ctx.reduce(h, k, vo, nv, P, Kp, out=got, opts=plain))
     if captured == "before":
-        capture()
+        graph = capture()
     late = ctx.reduce(h, k, vo, nv, P, Kp, opts=dart.dart_opts(path=dart.DART_PATH_STAGED, wait_limit=1))
     torch.cuda.synchronize()
     first, right = ctx.status(), same(late, want())
     if captured == "behind":
-        capture()
+        graph = capture()
+    assert _waits_for_words(graph, tmp_path / "graph.dot")
     later = []
     for _ in range(3):
         for t, n in zip((k, h), draw()):
