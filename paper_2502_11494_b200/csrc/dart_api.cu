@@ -185,7 +185,9 @@ struct Prof {
 };
 
 // Launch behind the kernel before it on the stream, which may still be running (see wait_for_previous): every kernel that is
-// launched this way waits before it reads or writes anything that another one touches.
+// launched this way waits before it reads or writes anything that another one touches - but for the gather that follows rank_kernel
+// word by word: rank_kernel lets it start behind its own wait, so that all earlier kernels have finished, the words are read and
+// published by relaxed accesses at gpu scope and put back behind the gather's wait, which every one of its warps comes to.
 // The launch's own result is returned: a kernel that reads indices must not be launched behind one that failed to launch (what a
 // launch leaves unnoticed is found by the call's cudaGetLastError).
 template <typename... KArgs, typename... Args>
@@ -281,10 +283,11 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     RankParams rp = {};
     size_t rank_smem = 0;
     // few lists: as many threads per list as help - a warp more lengthens every barrier of the chain, a value more every pass over a
-    // thread's own (whole calls, us, 192 / 256 / 384 / 512 threads: 1 x 576 25.9 / 25.9 / 26.3 / 26.7, 1 x 2880 37.0 / 37.0 / 35.2 / 36.8, 4 x 4608 with 32
-    // pivots 98.3 / 96.0 / 93.6 / 94.3); more lists, 192 / 256: 64 x 576 113.5 / 113.8, one after the other 123.0 / 124.0; many: small CTAs, so that
-    // one list's barriers are covered by the others (24 values per thread: 256 x 2880, 128 pivots with 256 threads per list 490 us, with 128 389)
-    // Long lists take more threads again (5 x 3466, 8 pivots keeping 1605 59.7 with 384, 57.5 with 512; 17 x 4607, 21 pivots keeping 3474 413 with 192, 409 with 256).
+    // thread's own (whole calls, us, 192 / 256 / 384 / 512 threads: 1 x 576 25.9 / 25.9 / 26.3 / 26.7, 1 x 2880 37.0 / 37.0 / 35.2 / 36.8, 4 x
+    // 4608 with 32 pivots 98.3 / 96.0 / 93.6 / 94.3); more lists, 192 / 256: 64 x 576 113.5 / 113.8, independent pivots 123.0 / 124.0; many:
+    // small CTAs, so that one list's barriers are covered by the others (24 values per thread: 256 x 2880, 128 pivots with 256 threads per
+    // list 490 us, with 128 389).  Long lists take more threads again (5 x 3466, 8 pivots keeping 1605 59.7 with 384, 57.5 with 512; 17 x
+    // 4607, 21 pivots keeping 3474 413 with 192, 409 with 256; no others measured).
     const long long rank_rows = (long long)B * P;
     const int rank_m = each ? (m + P - 1) / P : m;
     int rank_threads = n_vis > 4096 ? 256 : n_vis > 1024 ? 128 : 64;
@@ -312,9 +315,9 @@ int launch_retention(dart_ctx *ctx, int B, const int64_t *pos_in, int vis_offset
     }
     ctx->row_word_used = false;
     // The gather waits for its rows' words where the SMs hold few of its CTAs beside the turns, which its waiting warps slow down (whole
-    // calls, us, behind the kernel / behind the words: 16 x 256 keeping 56, 182 CTAs 34.9 / 33.0, 4 x 4608 keeping 512, 306 CTAs 93.6 / 92.0; 5 x 1733 keeping 747,
-    // 530 CTAs 41.1 / 43.4, 8 x 1500
-    // keeping 750, 995 CTAs 57.1 / 58.6, 32 x 2880 keeping 320, 1680 CTAs 187.2 / 188.3, 256 x 2880 keeping 640 2947 / 2985).
+    // calls, us, by CTAs, behind the kernel / behind the words: 80 30.5 / 30.1, 95 38.9 / 37.4, 182 34.9 / 33.0, 195 53.2 / 52.4, 230 32.5 / 31.5, 265
+    // 43.1 / 42.9, 306 93.6 / 92.0, 360 38.9 / 37.0; above the line of 370 both ways: 430 36.6 / 34.9, 480 41.6 / 39.7, 530 41.1 / 43.4, 600
+    // 30.2 / 30.4, 698 115.7 / 110.8, 995 57.1 / 58.6, 1680 187.2 / 188.3, 256 x 2880 keeping 640 2947 / 2985).
     const bool follow = !each && (long long)B * (S - n_vis + n_keep) <= 5ll * kGatherWarps * ctx->sm_count / 2;
     auto launch_ranked = [&]() -> cudaError_t {
         rp.sim = ctx->sim, rp.pivot_idx = ctx->pivot_idx, rp.lists = ctx->rank, rp.arrived = ctx->rank_arrived, rp.pos_in = pos_in;

@@ -14,18 +14,19 @@
 //   - a second-pass item is 64 rows x 1/nsl of the columns: an SM's pivot tile is P x d/nsl (16 KB at 8 pivots, d = 4096, 4
 //     slices) instead of P x d, and the item takes about 2.5 us instead of the 20 us of a 128-row tile of full rows;
 //   - the item's rows are fetched into a ring before the pivots are known;
-//   - the scorers are held back to `window` rows beyond the samples that have their pivots, and to `lead` beyond their SM's second pass.
+//   - the scorers are held back to `window` rows beyond the samples that have their pivots and, in long batches, to `lead` beyond
+//     their SM's second pass.
 // The slices' shares of a dot product meet in global memory (L2): when a row group's are all there, each of its SMs adds up a part of
 // them in slice order and divides by the norms (Eq. 7), so results are bitwise reproducible.
 // With the caller's pivots nothing is selected: first and second read then follow each other within the window.
 //
-// What bounds it: no unit.  16 x 2880 x 4096, 8 pivots (99 us): DRAM 49 % of its peak, L2 40 %, L2 to SM 25 % (8.5 TB/s: every key byte crosses
-// twice), shared-memory wavefronts 32 %, issue slots 46 %, tensor pipe 6 %; the warps wait for values on their way (long scoreboard 4.3
-// of 11.4 cycles per instruction) - the distance between a row's two reads, start and tail.
+// What bounds it: no unit.  32 x 2880 x 4096, 8 pivots (173 us): DRAM 56 % of its peak, L2 41 %, L2 to SM 9.8 TB/s (every key byte crosses
+// twice), shared-memory wavefronts 37 %, issue slots 54 %, tensor pipe 7 %; the warps wait for values on their way (long scoreboard 3.7
+// of 10.7 cycles per instruction) - the distance between a row's two reads, start and tail.
 //
 // Per CTA (768 or 896 threads, one CTA per SM, cooperative launch):
 //   warps 0-3    pivots of the samples this SM has items of: wait for them, fetch the pivot rows' slice (two buffers)
-//   warps 4-7    second pass: mma.sync.m16n8k16, 16 rows each (the tensor pipe is 6 % busy; what the form costs is that every warp
+//   warps 4-7    second pass: mma.sync.m16n8k16, 16 rows each (the tensor pipe is 7 % busy; what the form costs is that every warp
 //                reads the pivot tile from shared memory again, which a tcgen05.mma of 64 rows would do once)
 //   warp 8       producer: TMA tiles of 64 rows x 64 columns (128-byte swizzle), two per ring stage
 //   warps 9-12   combine: count the item, wait for its row group's other slices, add up a part of the shares and write the similarities
